@@ -15,6 +15,7 @@
 #include "smi_box.h"
 #include "smi_fused3d.h"
 #include "smi_internal.h"
+#include "smi_stencil2d.h"
 #include "smi_stencil3d.h"
 
 namespace smi {
@@ -107,6 +108,8 @@ struct Setup {
     bool rho_grad = false;                 // gradient with the density part (parametrisation families)
     bool fused = false;                    // 3D forward / adjoint steps by the single-pass kernel
     bool inline3 = false;                  // 3D two-pass tile kernels with the z / x CPML terms inline
+    bool fast2 = false;                    // 2D steps by the single-launch kernels
+    bool pingpong = false;                 // a step reads one set of state arrays and writes the other
     bool fullmem = false;                  // z / x CPML memory variables as full-size arrays (either of the above)
     long long nrec_total = 0;
     size_t setup_bytes = 0;                // sizes-only set-up: estimated bytes of the set-up arena
@@ -245,6 +248,9 @@ int validate_and_setup(const smi_model *m, const smi_geometry *geo, const smi_wa
     S.fused = o->kernels == SMI_KERNELS_FUSED && fused3d_supported(g);
     S.inline3 = o->kernels == SMI_KERNELS_INLINE && stencil3d_supported(g);
     S.fullmem = S.fused || S.inline3;
+    S.fast2 = o->kernels != SMI_KERNELS_GENERIC && stencil2d_supported(g);
+    S.pingpong = S.fused || S.fast2;
+    if (S.fast2) set_tile_slabs(g);
 
     // boundary bands: v_a on the 2N-1 half nodes straddling each face of the
     // physical domain, over the physical cross-section, stored every dr-th
@@ -334,20 +340,20 @@ int validate_and_setup(const smi_model *m, const smi_geometry *geo, const smi_wa
     const double R = o->cpml_R > 0.0 ? o->cpml_R : 1e-3;
     const double kb = o->kaiser_b > 0.0 ? o->kaiser_b : 4.0;
     for (int a = 0; a < m->ndim; a++) {
-        std::vector<float> tab(4 * (size_t)g.ne[a]);
-        cpml_tables(g.ne[a], o->nb, hh[a], S.vmax, w->fm, R, w->dt, false, tab.data(), tab.data() + g.ne[a]);
-        cpml_tables(g.ne[a], o->nb, hh[a], S.vmax, w->fm, R, w->dt, true, tab.data() + 2 * g.ne[a],
-                    tab.data() + 3 * g.ne[a]);
+        const size_t nt = ((size_t)g.ne[a] + 7) / 8 * 8;    // whole quads, zero past the axis
+        std::vector<float> tab(4 * nt);
+        cpml_tables(g.ne[a], o->nb, hh[a], S.vmax, w->fm, R, w->dt, false, tab.data(), tab.data() + nt);
+        cpml_tables(g.ne[a], o->nb, hh[a], S.vmax, w->fm, R, w->dt, true, tab.data() + 2 * nt, tab.data() + 3 * nt);
         if (a == 0 && g.freesurf)              // the top layer is the image zone: no absorption
             for (int q = 0; q < 4; q++)
-                for (int i = 0; i < g.L[0]; i++) tab[(size_t)q * g.ne[0] + i] = 0.0f;
+                for (int i = 0; i < g.L[0]; i++) tab[(size_t)q * nt + i] = 0.0f;
         float *d = ar.get<float>(tab.size());
         if (!d) return fail(SMI_ERR_NOMEM, "device allocation failed");
         cudaMemcpyAsync(d, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice, st);
         g.cpa[a] = d;
-        g.cpb[a] = d + g.ne[a];
-        g.cva[a] = d + 2 * g.ne[a];
-        g.cvb[a] = d + 3 * g.ne[a];
+        g.cpb[a] = d + nt;
+        g.cva[a] = d + 2 * nt;
+        g.cvb[a] = d + 3 * nt;
     }
     for (int a = m->ndim; a < 3; a++) g.cpa[a] = g.cpb[a] = g.cva[a] = g.cvb[a] = nullptr;
 
@@ -419,7 +425,7 @@ size_t per_shot_bytes(const Setup &S, int kind)
 {
     const Grid &g = S.g;
     const size_t fields = (size_t)(1 + g.ndim) * g.ntot * 4;
-    const int nbuf = S.fused ? 2 : 1;          // the single-pass step reads one state buffer, writes the other
+    const int nbuf = S.pingpong ? 2 : 1;
     size_t slabs = 0;
     for (int a = 0; a < g.ndim; a++) slabs += 2 * (size_t)(S.fullmem && a < 2 ? g.ntot : g.slab_n[a]) * 4;
     long long maxrec = 0;                      // receivers of the largest shot
@@ -430,6 +436,7 @@ size_t per_shot_bytes(const Setup &S, int kind)
         if (kind != 5) {
             b += (size_t)S.nsamp * S.bands.count * band_bytes(S.bands.prec);   // saved bands
             b += (size_t)S.nsamp * 6 * 4;                                  // band scales
+            if (S.fast2) b += (size_t)S.nsamp * 6 * 4;                     // and largest magnitudes
         }
         if (S.dr > 1) b += fields;                                     // state kept during the continuation
         b += (size_t)g.nphys * 4 * (kind == 1 && S.img_norm ? 2 : 1);  // accumulator (+ illumination)
@@ -591,6 +598,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
         int B = (int)std::max<size_t>(1, (size_t)(0.8 * (double)free_b) / per);
         B = std::min(B, S.nshot);
         if (o->max_batch > 0) B = std::min(B, o->max_batch);
+        if (S.fast2) B = std::min(B, 32767);     // two blocks a shot along gridDim.z
         if (kind == 6 && B < S.nshot)
             return fail(SMI_ERR_NOMEM, "a tape keeps every shot's state on the device: %d of %d shots fit", B, S.nshot);
         if (kind == 7) B = S.nshot;
@@ -600,13 +608,15 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
         tm.st = st;
         unsigned *d_flag = ar.get<unsigned>(1);
         unsigned *d_wait = ar.get<unsigned>(1);
-        unsigned *d_absmax = ar.get<unsigned>(6 * (size_t)B);
+        const size_t namax = 6 * (size_t)B * (S.fast2 ? S.nsamp : 1);   // largest band magnitudes (16-bit storage)
+        unsigned *d_absmax = ar.get<unsigned>(namax);
         if (!ar.ok) return fail(SMI_ERR_NOMEM, "device allocation failed");
         launch_zero(lc, d_flag, sizeof(unsigned));
         launch_zero(lc, d_wait, sizeof(unsigned));
         const bool fast3 = o->kernels != SMI_KERNELS_GENERIC && stencil3d_supported(g);
-        const bool fast2 = o->kernels != SMI_KERNELS_GENERIC && stencil2d_supported(g);
-        const bool fused = S.fused;
+        const bool fast2 = S.fast2;
+        const bool fused = S.fused, pp = S.pingpong;
+        const Step2 t2 = fast2 ? step2_tile(g, B) : Step2{};
         const bool inl = S.inline3;            // two-pass 3D kernels with the z / x CPML terms inline
         const bool norm = kind == 1 && S.img_norm;       // normalised RTM image
 
@@ -631,14 +641,14 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             Arena ba(st);
             int *d_roff = ba.get<int>(roff.size());
             long long *d_soff = ba.get<long long>(soff.size());
-            // F, A: the current source-field and adjoint states; with the
-            // single-pass step, F2 and A2 are the buffers it writes (swapped
-            // after every step).  Memory variables of the single-pass step:
+            // F, A: the current source-field and adjoint states; with a
+            // single-pass step (S.pingpong), F2 and A2 are the buffers it writes
+            // (swapped after every step).  Memory variables of the single-pass step:
             // z and x full-size, y in the y-slab layout.
             Fields F{}, A{}, F2{}, A2{};
             auto mem_n = [&](int a) { return (size_t)(S.fullmem && a < 2 ? g.ntot : g.slab_n[a]) * nb_shot; };
             for (Fields *f : {&F, &F2}) {
-                if ((f == &F2 && !fused) || kind == 7) break;
+                if ((f == &F2 && !pp) || kind == 7) break;
                 f->p = ba.get<float>((size_t)g.ntot * nb_shot);
                 for (int a = 0; a < g.ndim; a++) {
                     f->v[a] = ba.get<float>((size_t)g.ntot * nb_shot);
@@ -661,7 +671,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 acc = T.acc;
                 partials = T.partials;
             } else if (kind != 0) {
-                for (int k = 0; k < (fused ? 2 : 1); k++) {   // the adjoint reuses the forward's memory variables
+                for (int k = 0; k < (pp ? 2 : 1); k++) {   // the adjoint reuses the forward's memory variables
                     Fields &a_ = k ? A2 : A;
                     const Fields &f_ = k ? F2 : F;
                     a_.p = ba.get<float>((size_t)g.ntot * nb_shot);
@@ -705,13 +715,19 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                           (kind != 0 && (!make_maps3(mA2, g, A2, nb_shot, true) || !make_maps_fused(fA, g, A, nb_shot) ||
                                          !make_maps_fused(fA2, g, A2, nb_shot)))))
                 return fail(SMI_ERR_CUDA, "tensor map encoding failed");
+            Maps2 m2F{}, m2F2{}, m2A{}, m2A2{};
+            if (fast2 && (!make_maps2(m2F, g, F, nb_shot, t2) || !make_maps2(m2F2, g, F2, nb_shot, t2) ||
+                          (kind != 0 && (!make_maps2(m2A, g, A, nb_shot, t2) || !make_maps2(m2A2, g, A2, nb_shot, t2)))))
+                return fail(SMI_ERR_CUDA, "tensor map encoding failed");
             // after a single-pass step the written buffers become the current ones
             auto swap_F = [&] {
+                std::swap(m2F, m2F2);
                 std::swap(F, F2);
                 std::swap(mF, mF2);
                 std::swap(fF, fF2);
             };
             auto swap_A = [&] {
+                std::swap(m2A, m2A2);
                 std::swap(A, A2);
                 std::swap(mA, mA2);
                 std::swap(fA, fA2);
@@ -727,6 +743,8 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             b.tab_src = S.d_tab_src + (size_t)s0 * (S.nt + 1) * 6;
             b.tab_rec = S.d_tab_rec + (size_t)s0 * (S.nt + 1) * 6;
             b.nt1 = S.nt_fwd + 1;
+            b.h_box_src = S.box_src.data() + 6 * (size_t)s0;
+            b.h_box_rec = S.box_rec.data() + 6 * (size_t)s0;
             // union of the batch's boxes after n steps (bounds the CPML launches)
             auto batch_box = [&](const std::vector<int> &ext, int n, int lo[3], int hi[3]) {
                 for (int a = 0; a < 3; a++) {
@@ -743,7 +761,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 }
             };
             for (const Fields *f : {&F, &F2}) {
-                if ((f == &F2 && !fused) || kind == 7) break;
+                if ((f == &F2 && !pp) || kind == 7) break;
                 launch_zero(lc, f->p, sizeof(float) * g.ntot * nb_shot);
                 for (int a = 0; a < g.ndim; a++) {
                     launch_zero(lc, f->v[a], sizeof(float) * g.ntot * nb_shot);
@@ -758,8 +776,13 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             // reverse loop complete); the state after step nt-1 is kept.
             const size_t fbytes = sizeof(float) * g.ntot * nb_shot;
             const int nsteps = kind == 5 || kind == 7 ? 0 : kind != 0 ? S.nt_fwd : S.nt;
+            if (fast2 && nsteps > 0 && kind != 0) {
+                if (bd.prec != SMI_PREC_F32) launch_zero(lc, d_absmax, sizeof(unsigned) * namax);
+                // interpolation in time reads the whole band, which a step stores inside its box
+                if (S.dr > 1) launch_zero(lc, bd.data, (size_t)nb_shot * S.nsamp * bd.count * band_bytes(bd.prec));
+            }
             for (int it = 0; it < nsteps; it++) {
-                if (kind != 0 && it % S.dr == 0) launch_save_bands(lc, g, b, F, bd, it / S.dr, d_absmax);
+                if (kind != 0 && it % S.dr == 0 && !fast2) launch_save_bands(lc, g, b, F, bd, it / S.dr, d_absmax);
                 tm.begin(0);
                 int blo[3], bhi[3];
                 batch_box(S.box_src, it, blo, bhi);
@@ -774,11 +797,15 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch_free_surface(lc, g, F.v[0], nb_shot, kFsMirrorV);
                     launch3_p(lc, mF, nullptr, g, b, F, it, 0, d_wait, nullptr, 0, nullptr, 0.0f, inl);
                     if (!inl) launch_fwd_corrections(lc, g, b, F, it, false, blo, bhi);
-                } else if (fast2) {                    // CPML and (it < nt) the source inline
-                    launch2_v(lc, g, b, F, it, 0, blo, bhi);
-                    launch_free_surface(lc, g, F.v[0], nb_shot, kFsMirrorV);
-                    launch2_p(lc, g, b, F, it, 0, blo, bhi, nullptr, nullptr, 0, it < S.nt ? S.stf : nullptr,
-                              (float)S.src_scale);
+                } else if (fast2) {                    // CPML, source, boundary saving and samples in one launch
+                    Save2 save{-1, -1, d_absmax};
+                    if (kind != 0 && it % S.dr == 0) save.sample = it / S.dr;
+                    if (kind != 0 && bd.prec != SMI_PREC_F32 && (it + 1) % S.dr == 0 && (it + 1) / S.dr < S.nsamp)
+                        save.next = (it + 1) / S.dr;
+                    const Gather2 ga{seis, d_soff, max_rec > 0 && it <= S.nt ? it - 1 : -1};
+                    launch2_forward(lc, t2, m2F, g, b, F, F2, it, it < S.nt ? S.stf : nullptr, (float)S.src_scale, bd,
+                                    save, ga, d_wait);
+                    swap_F();
                 } else {
                     const long long work = box_points(blo, bhi);
                     launch_fwd_v(lc, g, b, F, it, work);
@@ -787,8 +814,10 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 }
                 tm.end();
                 if (it < S.nt && !fast2) launch_inject_source(lc, g, b, F.p, S.stf, it, (float)S.src_scale);
-                launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
-                if (it < S.nt && max_rec > 0) launch_gather(lc, g, b, F.p, seis, d_soff, S.nt, it);
+                if (!fast2) launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
+                // (a 2D step takes the samples of the step before it)
+                if (max_rec > 0 && (fast2 ? it == nsteps - 1 && it == S.nt - 1 : it < S.nt))
+                    launch_gather(lc, g, b, F.p, seis, d_soff, S.nt, it);
                 for (int s = 0; s < nb_shot; s++) {
                     int lo[3], hi[3];
                     box_bounds(g, S.box_src.data() + 6 * (s0 + s), it, lo, hi);
@@ -846,7 +875,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             }
             // ---- reverse loop ----
             for (const Fields *f : {&A, &A2}) {
-                if (f == &A2 && !fused) break;
+                if (f == &A2 && !pp) break;
                 launch_zero(lc, f->p, sizeof(float) * g.ntot * nb_shot);
                 for (int a = 0; a < g.ndim; a++) {
                     launch_zero(lc, f->v[a], sizeof(float) * g.ntot * nb_shot);
@@ -854,12 +883,20 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch_zero(lc, f->psiv[a], sizeof(float) * mem_n(a));
                 }
             }
+            if (fast2 && kind != 5) {              // the arrays the first reverse step writes: zero outside its box
+                launch_zero(lc, F2.p, fbytes);
+                for (int a = 0; a < g.ndim; a++) launch_zero(lc, F2.v[a], fbytes);
+            }
             if (acc) launch_zero(lc, acc, sizeof(float) * g.nphys * nb_shot * (norm ? 2 : 1));
             if (S.rho_grad)
                 for (int a = 0; a < g.ndim; a++)
                     cudaMemcpyAsync(R.vprev[a], F.v[a], fbytes, cudaMemcpyDeviceToDevice, st);
             // 0: gradient, 1: image, 2: image and source illumination
             const int mode = (kind == 2 || kind == 3 || kind == 7) ? 0 : (norm ? 2 : 1);
+            auto restore = [&](int it) {
+                if (S.dr == 1) launch_restore_bands(lc, g, b, F, bd, it);
+                else launch_restore_bands_interp(lc, g, b, F, bd, time_weights(it, S.dr, S.nsamp));
+            };
             // one reverse step of the source field (reconstruction with the fused
             // imaging / gradient accumulation), then its boundary re-imposed
             auto reconstruct = [&](int it) {
@@ -875,32 +912,45 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                         blo[a] = std::max(blo[a], g.L[a]);
                         bhi[a] = std::min(bhi[a], g.H[a]);
                     }
-                    if (fast2) {
-                        launch2_p(lc, g, b, F, it, 2, blo, bhi, A.p, acc, mode, S.stf, (float)S.src_scale);
-                        launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
-                        launch2_v(lc, g, b, F, it, 2, blo, bhi);
-                    } else {
-                        const long long work = box_points(blo, bhi);
-                        launch_recon_p(lc, g, b, F, A.p, acc, mode, S.stf, it, (float)S.src_scale, work);
-                        launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
-                        launch_recon_v(lc, g, b, F, it, work);
-                    }
+                    const long long work = box_points(blo, bhi);
+                    launch_recon_p(lc, g, b, F, A.p, acc, mode, S.stf, it, (float)S.src_scale, work);
+                    launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
+                    launch_recon_v(lc, g, b, F, it, work);
                 }
                 tm.end();
-                if (S.dr == 1) launch_restore_bands(lc, g, b, F, bd, it);
-                else launch_restore_bands_interp(lc, g, b, F, bd, time_weights(it, S.dr, S.nsamp));
+                restore(it);
+            };
+            // 2D: the adjoint step and the reconstruction share a launch (timed per class: one launch each)
+            auto reverse2 = [&](int it, int mrev) {
+                const int all = kind == 5 ? 1 : 3;
+                for (int part = 0; part < 2; part++) {
+                    const int roles = tm.on ? all & (part == 0 ? 2 : 1) : (part == 0 ? all : 0);
+                    if (!roles) continue;
+                    tm.begin(roles == 2 ? 2 : 1);
+                    launch2_reverse(lc, t2, m2A, m2F, g, b, A, A2, mrev, roles, F, F2, it, acc, mode, S.stf,
+                                    (float)S.src_scale, bd, S.dr == 1, d_wait);
+                    tm.end();
+                }
+                swap_A();
+                if (kind == 5) return;
+                swap_F();
+                if (S.dr > 1) restore(it);
             };
             for (int it = S.nt - 1; it >= 0; it--) {
                 const int mrev = S.nt - 1 - it;
-                if (max_rec > 0) launch_adj_inject(lc, g, b, A.p, res, d_soff, S.nt, it);
+                if (max_rec > 0) {
+                    if (fast2) launch_adj_inject_tile(lc, g, b, A, res, d_soff, it);
+                    else launch_adj_inject(lc, g, b, A.p, res, d_soff, S.nt, it);
+                }
                 // free surface (no-ops without): the transposed p mirror on the
                 // adjoint before anything reads it; p = 0 again at the surface node
                 // of the reversed source field; the transposed v_z mirror between
                 // the two adjoint stages
-                launch_free_surface(lc, g, A.p, nb_shot, kFsFoldP);
+                if (fast2) launch_free_surface_fold_tile(lc, g, A, nb_shot);
+                else launch_free_surface(lc, g, A.p, nb_shot, kFsFoldP);
                 if (kind == 5) launch_src_adjoint(lc, g, b, A.p, part, S.nt, it, S.src_scale);   // wavelet adjoint
-                else reconstruct(it);
-                tm.begin(1);
+                else if (!fast2) reconstruct(it);
+                if (!fast2) tm.begin(1);
                 int blo[3], bhi[3];
                 batch_box(S.box_rec, mrev, blo, bhi);
                 if (fused) {
@@ -912,17 +962,15 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch_free_surface(lc, g, A.v[0], nb_shot, kFsFoldV);
                     if (!inl) launch_adj_corrections(lc, g, b, A, mrev, false, blo, bhi);
                     launch3_p(lc, mA, nullptr, g, b, A, mrev, 1, d_wait, nullptr, 0, nullptr, 0.0f, inl);
-                } else if (fast2) {                    // transposed CPML inline in the 2D kernels
-                    launch2_v(lc, g, b, A, mrev, 1, blo, bhi);
-                    launch_free_surface(lc, g, A.v[0], nb_shot, kFsFoldV);
-                    launch2_p(lc, g, b, A, mrev, 1, blo, bhi, nullptr, nullptr, 0, nullptr, 0.0f);
+                } else if (fast2) {
+                    reverse2(it, mrev);
                 } else {
                     const long long work = box_points(blo, bhi);
                     launch_adj_v(lc, g, b, A, mrev, work);
                     launch_free_surface(lc, g, A.v[0], nb_shot, kFsFoldV);
                     launch_adj_p(lc, g, b, A, mrev, work);
                 }
-                tm.end();
+                if (!fast2) tm.end();
                 if (S.rho_grad) {                      // half nodes touching the physical domain
                     IBox rb;
                     batch_box(S.box_src, it, rb.lo, rb.hi);

@@ -25,6 +25,7 @@ struct Grid {
     long long nphys;       // points of the physical grid
     int S;                 // slab length along its axis: 2*nb + 1
     long long slab_n[3];   // points of the slab array of axis a
+    int zlo, zhi, zp;      // tile kernels' z slabs (smi_slab.h): low slab's quads, first high quad, row length
     float dt;
     float c[3][kMaxHalf];  // a_l / h_a
     double vdt;            // vmax * dt (FP64, for the computing box)
@@ -59,6 +60,7 @@ struct Batch {
     const int *tab_src;     // around the source
     const int *tab_rec;     // around the receivers
     int nt1;                // nt + 1
+    const int *h_box_src, *h_box_rec;   // box_src and box_rec on the host (grid sizes of the launches)
 };
 
 // Wavefields of a batch; shot s of field f is at f + s * ntot, node
@@ -179,6 +181,10 @@ void launch_to_float(const LaunchCtx &lc, const double *a, int n, float *out);
 void launch_dot(const LaunchCtx &lc, const float *a, const float *b, long long n, double *partials, int npart);
 void launch_adj_inject(const LaunchCtx &lc, const Grid &g, const Batch &b, float *lp,
                        const float *res, const long long *seis_off, int nt, int it);
+// The same for the tile kernels' adjoint state, whose CPML operands e hold
+// A lambda_p of the slab nodes (smi_slab.h): e += A times the injected value.
+void launch_adj_inject_tile(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields A, const float *res,
+                            const long long *seis_off, int it);
 void launch_adj_v(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, long long work);
 void launch_adj_p(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, long long work);
 // One piece of the union of the CPML bands: per axis up to two index
@@ -218,14 +224,6 @@ void launch_recon_p(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f
                     float src_scale, long long work);
 void launch_recon_v(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int it, long long work);
 
-// 2D kernels (smi_stencil2d.cu): mode 0 forward, 1 adjoint (both with the
-// CPML terms inline), 2 reconstruction + imaging; [lo, hi] = the batch's box
-// union (for mode 2 within the physical domain).
-bool stencil2d_supported(const Grid &g);
-void launch2_v(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int step, int mode, const int lo[3],
-               const int hi[3]);
-void launch2_p(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int step, int mode, const int lo[3],
-               const int hi[3], const float *lp, float *acc, int img_mode, const float *stf, float src_scale);
 void launch_reduce_shots(const LaunchCtx &lc, const Grid &g, const float *acc, int nshot,
                          float *out, int accumulate);
 // Normalised image: acc holds [nshot][nphys] images then [nshot][nphys]
@@ -260,10 +258,15 @@ void launch_finalize_family(const LaunchCtx &lc, const Grid &g, const float *vp,
 //               value goes to its mirror node (negated for p) and is cleared,
 //               and for p the surface node is cleared.
 enum { kFsMirrorV = 0, kFsMirrorP = 1, kFsFoldV = 2, kFsFoldP = 3 };
+// kFsFoldP on the tile kernels' adjoint state: the pressure and its x and y
+// CPML operands (the z operand is zero at these rows).
+void launch_free_surface_fold_tile(const LaunchCtx &lc, const Grid &g, Fields A, int nshot);
 void launch_free_surface(const LaunchCtx &lc, const Grid &g, float *f, int nshot, int op);
 void launch_nonfinite(const LaunchCtx &lc, const float *x, long long n, unsigned *flag);
 // Sets the padded layout: px, ntot, nphys and the slab sizes (ne, nb, ndim set).
 void set_layout(Grid &g, const int n[3]);
+// Slab sizes of the tile kernels' layout (smi_slab.h; after set_layout).
+void set_tile_slabs(Grid &g);
 
 void launch_box_table(const LaunchCtx &lc, const Grid &g, const int *ext, int n0, int count,
                       int *lo, int *hi);

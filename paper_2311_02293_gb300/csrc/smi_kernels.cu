@@ -15,6 +15,8 @@
 
 #include "smi_internal.h"
 #include "smi_box.h"
+#include "smi_pdl.h"
+#include "smi_slab.h"
 
 namespace smi {
 
@@ -1025,6 +1027,42 @@ __global__ void k_adj_inject(Grid g, Batch b, float *lp, const float *res, const
             }
 }
 
+// The same on the tile kernels' adjoint state (smi_slab.h).
+__global__ void k_adj_inject_tile(Grid g, Batch b, Fields A, const float *res, const long long *seis_off, int it)
+{
+    const int s = blockIdx.y;
+    const int nr = b.rec_off[s + 1] - b.rec_off[s];
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= nr) {
+        if (r == 0) pdl_wait();
+        return;
+    }
+    const Stencil &st = b.rec[b.rec_off[s] + r];
+    const float val = res[seis_off[s] + (long long)it * nr + r];
+    const int n0 = st.cnt[0], n1 = st.cnt[1], n2 = st.cnt[2];
+    pdl_wait();
+    pdl_trigger();
+    for (int a2 = 0; a2 < n2; a2++)
+        for (int a1 = 0; a1 < n1; a1++)
+            for (int a0 = 0; a0 < n0; a0++) {
+                const int z = st.first[0] + a0, x = st.first[1] + a1, y = st.first[2] + a2;
+                const long long k = gidx(g, z, x, y);
+                const float add = g.K[k] * st.w[0][a0] * st.w[1][a1] * st.w[2][a2] * val;
+                atomicAdd(A.p + s * g.ntot + k, add);
+                const int q = zslab_quad(g, z & ~3), jx = slab_row(g, 1, x);
+                if (q >= 0)
+                    atomicAdd(A.psiv[0] + s * g.slab_n[0] + q + (z & 3) + (long long)g.zp * (x + (long long)g.ne[1] * y),
+                              g.cpa[0][z] * add);
+                if (jx >= 0)
+                    atomicAdd(A.psiv[1] + s * g.slab_n[1] + z + (long long)g.px * (jx + (long long)g.S * y),
+                              g.cpa[1][x] * add);
+                const int jy = g.ndim == 3 ? slab_row(g, 2, y) : -1;
+                if (jy >= 0)
+                    atomicAdd(A.psiv[2] + s * g.slab_n[2] + z + (long long)g.px * (x + (long long)g.ne[1] * jy),
+                              g.cpa[2][y] * add);
+            }
+}
+
 // Adjoint of the wavelet samples (the transpose of k_inject_source): the
 // source of step it enters p^{it+1} as dt stf[it] w / dV, so its adjoint is
 // dt / dV sum_w w pbar over the source stencil, with pbar = lambda_p / kappa
@@ -1417,12 +1455,11 @@ __global__ void k_finalize_family(Grid g, const float *vp, const float *rho, con
     }
 }
 
-// Free-surface mirrors and their transposes; thread (j, row, shot), j in
-// 0..N fastest.
-__global__ void k_free_surface(Grid g, float *f, int nshot, int op)
+// Free-surface mirrors and their transposes over the rows of nshot arrays
+// (pitch px, stride floats a shot); thread (j, row, shot), j in 0..N fastest.
+__global__ void k_free_surface(Grid g, float *f, long long rows, long long stride, int nshot, int op)
 {
     const int N = g.N;
-    const long long rows = (long long)g.ne[1] * g.ne[2];
     const long long n = rows * nshot * (N + 1);
     const int L = g.L[0];
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
@@ -1430,7 +1467,7 @@ __global__ void k_free_surface(Grid g, float *f, int nshot, int op)
         const int j = (int)(t % (N + 1));
         const long long r = t / (N + 1);                 // shot * rows + row
         const long long s = r / rows, row = r - s * rows;
-        float *c = f + s * g.ntot + row * g.px;          // the z column of this (x, y)
+        float *c = f + s * stride + row * g.px;          // the z column of this (x, y)
         if (op == kFsMirrorV) {
             if (j < N) c[L - 1 - j] = c[L + j];
         } else if (op == kFsMirrorP) {
@@ -1751,6 +1788,12 @@ void launch_adj_inject(const LaunchCtx &lc, const Grid &g, const Batch &b, float
     ++*lc.launches;
 }
 
+void launch_adj_inject_tile(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields A, const float *res,
+                            const long long *seis_off, int it)
+{
+    launch_pdl(lc, k_adj_inject_tile, dim3((b.max_rec + 127) / 128, b.nshot), 128, 0, g, b, A, res, seis_off, it);
+}
+
 // Band kernels: x = chunks of the largest region, y = region, z = shot.
 static dim3 band_grid(const Bands &bd, int nshot)
 {
@@ -1874,12 +1917,25 @@ void launch_finalize_family(const LaunchCtx &lc, const Grid &g, const float *vp,
     ++*lc.launches;
 }
 
+static void free_surface_rows(const LaunchCtx &lc, const Grid &g, float *f, long long rows, long long stride,
+                              int nshot, int op)
+{
+    const long long n = rows * nshot * (g.N + 1);
+    k_free_surface<<<blocks_for(n), kThreads, 0, S(lc)>>>(g, f, rows, stride, nshot, op);
+    ++*lc.launches;
+}
+
 void launch_free_surface(const LaunchCtx &lc, const Grid &g, float *f, int nshot, int op)
 {
+    if (g.freesurf) free_surface_rows(lc, g, f, (long long)g.ne[1] * g.ne[2], g.ntot, nshot, op);
+}
+
+void launch_free_surface_fold_tile(const LaunchCtx &lc, const Grid &g, Fields A, int nshot)
+{
     if (!g.freesurf) return;
-    const long long n = (long long)g.ne[1] * g.ne[2] * nshot * (g.N + 1);
-    k_free_surface<<<blocks_for(n), kThreads, 0, S(lc)>>>(g, f, nshot, op);
-    ++*lc.launches;
+    launch_free_surface(lc, g, A.p, nshot, kFsFoldP);
+    free_surface_rows(lc, g, A.psiv[1], (long long)g.S * g.ne[2], g.slab_n[1], nshot, kFsFoldP);
+    if (g.ndim == 3) free_surface_rows(lc, g, A.psiv[2], (long long)g.ne[1] * g.S, g.slab_n[2], nshot, kFsFoldP);
 }
 
 void launch_nonfinite(const LaunchCtx &lc, const float *x, long long n, unsigned *flag)

@@ -175,6 +175,17 @@ void set_layout(Grid &g, const int n[3])
     g.slab_n[0] = (long long)g.S * g.ne[1] * g.ne[2];
     g.slab_n[1] = (long long)g.ne[0] * g.S * g.ne[2];
     g.slab_n[2] = g.ndim == 3 ? (long long)g.px * g.ne[1] * g.S : 0;
+    g.zlo = g.zhi = g.zp = 0;
+}
+
+void set_tile_slabs(Grid &g)
+{
+    g.zlo = (g.nb + 3) & ~3;
+    g.zhi = (g.ne[0] - g.nb - 1) & ~3;
+    g.zp = g.zlo + g.px - g.zhi;
+    g.slab_n[0] = (long long)g.zp * g.ne[1] * g.ne[2];
+    g.slab_n[1] = (long long)g.px * g.S * g.ne[2];
+    g.slab_n[2] = g.ndim == 3 ? (long long)g.px * g.ne[1] * g.S : 0;
 }
 
 }  // namespace smi

@@ -979,6 +979,8 @@ bool make_tile_map(CUtensorMap *tm, const Grid &g, const float *base, int nshot,
     return make_map(tm, g, base, nshot, bz, bx);
 }
 
+bool tile_maps_available() { return encoder() != nullptr; }
+
 // The 3D path indexes one shot's arrays with 32-bit offsets.
 void launch_wait_check(const LaunchCtx &lc, unsigned *err, long long polls)
 {

@@ -28,6 +28,9 @@ long long wait_polls_default();
 // the encoder is missing or refuses the map.
 bool make_tile_map(CUtensorMap *tm, const Grid &g, const float *base, int nshot, int bz, int bx);
 
+// True when the tensor-map encoder was found.
+bool tile_maps_available();
+
 // True when the 3D kernels can run (3D, order 4 or 8, tensor-map encoder found).
 bool stencil3d_supported(const Grid &g);
 
