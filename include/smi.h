@@ -68,18 +68,17 @@ extern "C" {
 /* Kernel family (smi_opts.kernels).  Every family computes the same scheme;
  * results agree to FP32 rounding. */
 #define SMI_KERNELS_AUTO 0        /* the fastest measured kernels that support the problem: in 3D the two-pass
-                                     tile kernels (a velocity pass, then a pressure pass) with the z / x CPML
-                                     terms in band kernels over the slabs, in 2D the 2D tile kernels */
+                                     tile kernels (a velocity pass, then a pressure pass, CPML terms inline), in
+                                     2D the single-launch tile steps */
 #define SMI_KERNELS_GENERIC 1     /* the generic grid-stride kernels (CPML inline, 64-bit indexing) that
                                      serve 3D fields of 2^31 points or more and smi_forward_noalloc; for
                                      tests that check them against the oracle on small problems */
-#define SMI_KERNELS_TWOPASS 2     /* 3D: the two-pass tile kernels with the CPML band kernels (what AUTO runs) */
+#define SMI_KERNELS_TWOPASS 2     /* 3D: the two-pass tile kernels (what AUTO runs) */
 #define SMI_KERNELS_FUSED 3       /* 3D forward and adjoint steps: the single-pass kernel (velocity and pressure
                                      in one pass, CPML of all axes inline, state double buffered); no free
                                      surface (falls back to two-pass).  Measured slower than AUTO on GB300 */
-#define SMI_KERNELS_INLINE 4      /* 3D forward and adjoint steps: the two-pass tile kernels launched as an
-                                     interior and a CPML-band tile class, the z / x CPML terms inline in the
-                                     band class (no band kernels).  Measured slower than AUTO on GB300 */
+#define SMI_KERNELS_INLINE 4      /* 3D: the two-pass tile kernels, whose CPML terms are inline (what AUTO runs;
+                                     once a variant of its own) */
 
 /* Storage precision of the saved boundaries (Sec. 4.2). */
 #define SMI_PREC_F32 0

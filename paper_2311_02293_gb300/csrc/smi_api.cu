@@ -107,10 +107,9 @@ struct Setup {
     int img_norm = 0;                      // normalised RTM image
     bool rho_grad = false;                 // gradient with the density part (parametrisation families)
     bool fused = false;                    // 3D forward / adjoint steps by the single-pass kernel
-    bool inline3 = false;                  // 3D two-pass tile kernels with the z / x CPML terms inline
+    bool tile3 = false;                    // 3D forward / adjoint steps by the two-pass tile kernels
     bool fast2 = false;                    // 2D steps by the single-launch kernels
     bool pingpong = false;                 // a step reads one set of state arrays and writes the other
-    bool fullmem = false;                  // z / x CPML memory variables as full-size arrays (either of the above)
     long long nrec_total = 0;
     size_t setup_bytes = 0;                // sizes-only set-up: estimated bytes of the set-up arena
     std::vector<int> rec_offset;
@@ -246,11 +245,10 @@ int validate_and_setup(const smi_model *m, const smi_geometry *geo, const smi_wa
     for (int a = 0; a < 3; a++)
         for (int l = 0; l < kMaxHalf; l++) g.c[a][l] = (a < m->ndim && l < N) ? (float)(coef[l] / hh[a]) : 0.0f;
     S.fused = o->kernels == SMI_KERNELS_FUSED && fused3d_supported(g);
-    S.inline3 = o->kernels == SMI_KERNELS_INLINE && stencil3d_supported(g);
-    S.fullmem = S.fused || S.inline3;
+    S.tile3 = o->kernels != SMI_KERNELS_GENERIC && !S.fused && stencil3d_supported(g);
     S.fast2 = o->kernels != SMI_KERNELS_GENERIC && stencil2d_supported(g);
     S.pingpong = S.fused || S.fast2;
-    if (S.fast2) set_tile_slabs(g);
+    if (S.fast2 || S.tile3) set_tile_slabs(g);
 
     // boundary bands: v_a on the 2N-1 half nodes straddling each face of the
     // physical domain, over the physical cross-section, stored every dr-th
@@ -427,7 +425,7 @@ size_t per_shot_bytes(const Setup &S, int kind)
     const size_t fields = (size_t)(1 + g.ndim) * g.ntot * 4;
     const int nbuf = S.pingpong ? 2 : 1;
     size_t slabs = 0;
-    for (int a = 0; a < g.ndim; a++) slabs += 2 * (size_t)(S.fullmem && a < 2 ? g.ntot : g.slab_n[a]) * 4;
+    for (int a = 0; a < g.ndim; a++) slabs += 2 * (size_t)(S.fused && a < 2 ? g.ntot : g.slab_n[a]) * 4;
     long long maxrec = 0;                      // receivers of the largest shot
     for (int k = 0; k < S.nshot; k++) maxrec = std::max<long long>(maxrec, S.rec_offset[k + 1] - S.rec_offset[k]);
     size_t b = nbuf * (fields + slabs) + (size_t)S.nt * maxrec * 4;
@@ -436,7 +434,7 @@ size_t per_shot_bytes(const Setup &S, int kind)
         if (kind != 5) {
             b += (size_t)S.nsamp * S.bands.count * band_bytes(S.bands.prec);   // saved bands
             b += (size_t)S.nsamp * 6 * 4;                                  // band scales
-            if (S.fast2) b += (size_t)S.nsamp * 6 * 4;                     // and largest magnitudes
+            if (S.fast2 || S.tile3) b += (size_t)S.nsamp * 6 * 4;          // and largest magnitudes
         }
         if (S.dr > 1) b += fields;                                     // state kept during the continuation
         b += (size_t)g.nphys * 4 * (kind == 1 && S.img_norm ? 2 : 1);  // accumulator (+ illumination)
@@ -608,16 +606,20 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
         tm.st = st;
         unsigned *d_flag = ar.get<unsigned>(1);
         unsigned *d_wait = ar.get<unsigned>(1);
-        const size_t namax = 6 * (size_t)B * (S.fast2 ? S.nsamp : 1);   // largest band magnitudes (16-bit storage)
+        const size_t namax = 6 * (size_t)B * (S.fast2 || S.tile3 ? S.nsamp : 1);   // largest band magnitudes (16-bit storage)
         unsigned *d_absmax = ar.get<unsigned>(namax);
         if (!ar.ok) return fail(SMI_ERR_NOMEM, "device allocation failed");
         launch_zero(lc, d_flag, sizeof(unsigned));
         launch_zero(lc, d_wait, sizeof(unsigned));
+        // one work counter per launch of the 3D tile kernels
+        const size_t nctr = g.ndim == 3 ? 2 * (size_t)S.nt_fwd + 4 * (size_t)S.nt : 1;
+        unsigned *d_ctr = ar.get<unsigned>(nctr);
+        if (!d_ctr) return fail(SMI_ERR_NOMEM, "device allocation failed");
         const bool fast3 = o->kernels != SMI_KERNELS_GENERIC && stencil3d_supported(g);
         const bool fast2 = S.fast2;
         const bool fused = S.fused, pp = S.pingpong;
         const Step2 t2 = fast2 ? step2_tile(g, B) : Step2{};
-        const bool inl = S.inline3;            // two-pass 3D kernels with the z / x CPML terms inline
+        const bool tile3 = S.tile3, tiles = fast2 || tile3;   // tiles: the tile kernels' CPML slabs and operands
         const bool norm = kind == 1 && S.img_norm;       // normalised RTM image
 
         size_t batch_peak = 0;                   // largest batch arena (fields, bands, accumulators)
@@ -638,6 +640,8 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 soff = tape_in->soff;
                 max_rec = tape_in->max_rec;
             }
+            launch_zero(lc, d_ctr, sizeof(unsigned) * nctr);
+            unsigned *ctr = d_ctr;               // next launch's counter
             Arena ba(st);
             int *d_roff = ba.get<int>(roff.size());
             long long *d_soff = ba.get<long long>(soff.size());
@@ -646,7 +650,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             // (swapped after every step).  Memory variables of the single-pass step:
             // z and x full-size, y in the y-slab layout.
             Fields F{}, A{}, F2{}, A2{};
-            auto mem_n = [&](int a) { return (size_t)(S.fullmem && a < 2 ? g.ntot : g.slab_n[a]) * nb_shot; };
+            auto mem_n = [&](int a) { return (size_t)(S.fused && a < 2 ? g.ntot : g.slab_n[a]) * nb_shot; };
             for (Fields *f : {&F, &F2}) {
                 if ((f == &F2 && !pp) || kind == 7) break;
                 f->p = ba.get<float>((size_t)g.ntot * nb_shot);
@@ -705,14 +709,14 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 cudaMemcpyAsync(d_soff, soff.data(), sizeof(long long) * soff.size(), cudaMemcpyHostToDevice, st);
             }
             Maps3 mF{}, mA{}, mF2{}, mA2{};
-            if (fast3 && (!make_maps3(mF, g, F, nb_shot, S.fullmem) ||
-                          (kind != 0 && !make_maps3(mA, g, A, nb_shot, S.fullmem))))
+            if (fast3 && (!make_maps3(mF, g, F, nb_shot, tile3) ||
+                          (kind != 0 && !make_maps3(mA, g, A, nb_shot, tile3))))
                 return fail(SMI_ERR_CUDA, "tensor map encoding failed");
             MapsF fF{}, fF2{}, fA{}, fA2{};
             MapsM fM{};
-            if (fused && (!make_maps3(mF2, g, F2, nb_shot, true) || !make_maps_fused(fF, g, F, nb_shot) ||
+            if (fused && (!make_maps3(mF2, g, F2, nb_shot, false) || !make_maps_fused(fF, g, F, nb_shot) ||
                           !make_maps_fused(fF2, g, F2, nb_shot) || !make_maps_model(fM, g) ||
-                          (kind != 0 && (!make_maps3(mA2, g, A2, nb_shot, true) || !make_maps_fused(fA, g, A, nb_shot) ||
+                          (kind != 0 && (!make_maps3(mA2, g, A2, nb_shot, false) || !make_maps_fused(fA, g, A, nb_shot) ||
                                          !make_maps_fused(fA2, g, A2, nb_shot)))))
                 return fail(SMI_ERR_CUDA, "tensor map encoding failed");
             Maps2 m2F{}, m2F2{}, m2A{}, m2A2{};
@@ -776,13 +780,17 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             // reverse loop complete); the state after step nt-1 is kept.
             const size_t fbytes = sizeof(float) * g.ntot * nb_shot;
             const int nsteps = kind == 5 || kind == 7 ? 0 : kind != 0 ? S.nt_fwd : S.nt;
-            if (fast2 && nsteps > 0 && kind != 0) {
+            if (tiles && nsteps > 0 && kind != 0) {
                 if (bd.prec != SMI_PREC_F32) launch_zero(lc, d_absmax, sizeof(unsigned) * namax);
-                // interpolation in time reads the whole band, which a step stores inside its box
-                if (S.dr > 1) launch_zero(lc, bd.data, (size_t)nb_shot * S.nsamp * bd.count * band_bytes(bd.prec));
+                // interpolation in time reads the whole band, which a 2D step stores inside its box
+                if (fast2 && S.dr > 1) launch_zero(lc, bd.data, (size_t)nb_shot * S.nsamp * bd.count * band_bytes(bd.prec));
             }
             for (int it = 0; it < nsteps; it++) {
-                if (kind != 0 && it % S.dr == 0 && !fast2) launch_save_bands(lc, g, b, F, bd, it / S.dr, d_absmax);
+                // (the 2D steps store their bands; the 3D pressure kernel stores those of the next step
+                // in FP32, or finds their largest magnitudes)
+                if (kind != 0 && it % S.dr == 0 && !fast2 && !(tile3 && it > 0 && bd.prec == SMI_PREC_F32))
+                    launch_save_bands(lc, g, b, F, bd, it / S.dr,
+                                      d_absmax + (tile3 ? 6 * (size_t)nb_shot * (it / S.dr) : 0), tile3);
                 tm.begin(0);
                 int blo[3], bhi[3];
                 batch_box(S.box_src, it, blo, bhi);
@@ -791,12 +799,17 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 if (fused) {
                     launch3_fused(lc, fF, fM, g, b, F, F2, it, 0, d_wait);
                     swap_F();
-                } else if (fast3) {
-                    launch3_v(lc, mF, g, b, F, it, 0, d_wait, inl);
-                    if (!inl) launch_fwd_corrections(lc, g, b, F, it, true, blo, bhi);
+                } else if (tile3) {
+                    const Gather3 ga{seis, d_soff, max_rec > 0 && it <= S.nt ? it - 1 : -1};
+                    launch3_v(lc, mF, g, b, F, it, 0, ga, Restore3{bd, {}, -1}, d_wait, ctr++);
                     launch_free_surface(lc, g, F.v[0], nb_shot, kFsMirrorV);
-                    launch3_p(lc, mF, nullptr, g, b, F, it, 0, d_wait, nullptr, 0, nullptr, 0.0f, inl);
-                    if (!inl) launch_fwd_corrections(lc, g, b, F, it, false, blo, bhi);
+                    Save3 save{bd, d_absmax, -1};
+                    if (kind != 0 && (it + 1) % S.dr == 0 && (it + 1) / S.dr < S.nsamp) {
+                        save.sample = (it + 1) / S.dr;
+                        save.amax = d_absmax + 6 * (size_t)nb_shot * save.sample;
+                    }
+                    launch3_p(lc, mF, nullptr, g, b, F, it, 0, d_wait, nullptr, 0, it < S.nt ? S.stf : nullptr,
+                              (float)S.src_scale, save, ctr++);
                 } else if (fast2) {                    // CPML, source, boundary saving and samples in one launch
                     Save2 save{-1, -1, d_absmax};
                     if (kind != 0 && it % S.dr == 0) save.sample = it / S.dr;
@@ -813,10 +826,10 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch_fwd_p(lc, g, b, F, it, work);
                 }
                 tm.end();
-                if (it < S.nt && !fast2) launch_inject_source(lc, g, b, F.p, S.stf, it, (float)S.src_scale);
+                if (it < S.nt && !tiles) launch_inject_source(lc, g, b, F.p, S.stf, it, (float)S.src_scale);
                 if (!fast2) launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
-                // (a 2D step takes the samples of the step before it)
-                if (max_rec > 0 && (fast2 ? it == nsteps - 1 && it == S.nt - 1 : it < S.nt))
+                // (a step of the tile kernels takes the samples of the step before it)
+                if (max_rec > 0 && (tiles ? it == nsteps - 1 && it == S.nt - 1 : it < S.nt))
                     launch_gather(lc, g, b, F.p, seis, d_soff, S.nt, it);
                 for (int s = 0; s < nb_shot; s++) {
                     int lo[3], hi[3];
@@ -902,9 +915,10 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             auto reconstruct = [&](int it) {
                 tm.begin(2);
                 if (fast3) {
-                    launch3_p(lc, mF, &mA, g, b, F, it, 2, d_wait, acc, mode, S.stf, (float)S.src_scale, false);
+                    launch3_p(lc, mF, &mA, g, b, F, it, 2, d_wait, acc, mode, S.stf, (float)S.src_scale,
+                              Save3{bd, nullptr, -1}, ctr++);
                     launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
-                    launch3_v(lc, mF, g, b, F, it, 2, d_wait, false);
+                    launch3_v(lc, mF, g, b, F, it, 2, Gather3{nullptr, nullptr, -1}, Restore3{bd, {}, -1}, d_wait, ctr++);
                 } else {
                     int blo[3], bhi[3];
                     batch_box(S.box_src, it, blo, bhi);
@@ -918,7 +932,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch_recon_v(lc, g, b, F, it, work);
                 }
                 tm.end();
-                restore(it);
+                if (!tile3 || S.dr > 1) restore(it);   // (the 3D adjoint velocity kernel restores a stored step)
             };
             // 2D: the adjoint step and the reconstruction share a launch (timed per class: one launch each)
             auto reverse2 = [&](int it, int mrev) {
@@ -939,14 +953,14 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             for (int it = S.nt - 1; it >= 0; it--) {
                 const int mrev = S.nt - 1 - it;
                 if (max_rec > 0) {
-                    if (fast2) launch_adj_inject_tile(lc, g, b, A, res, d_soff, it);
+                    if (tiles) launch_adj_inject_tile(lc, g, b, A, res, d_soff, it);
                     else launch_adj_inject(lc, g, b, A.p, res, d_soff, S.nt, it);
                 }
                 // free surface (no-ops without): the transposed p mirror on the
                 // adjoint before anything reads it; p = 0 again at the surface node
                 // of the reversed source field; the transposed v_z mirror between
                 // the two adjoint stages
-                if (fast2) launch_free_surface_fold_tile(lc, g, A, nb_shot);
+                if (tiles) launch_free_surface_fold_tile(lc, g, A, nb_shot);
                 else launch_free_surface(lc, g, A.p, nb_shot, kFsFoldP);
                 if (kind == 5) launch_src_adjoint(lc, g, b, A.p, part, S.nt, it, S.src_scale);   // wavelet adjoint
                 else if (!fast2) reconstruct(it);
@@ -956,12 +970,12 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 if (fused) {
                     launch3_fused(lc, fA, fM, g, b, A, A2, mrev, 1, d_wait);
                     swap_A();
-                } else if (fast3) {
-                    if (!inl) launch_adj_corrections(lc, g, b, A, mrev, true, blo, bhi);
-                    launch3_v(lc, mA, g, b, A, mrev, 1, d_wait, inl);
+                } else if (tile3) {
+                    const Restore3 rs{bd, {F.v[0], F.v[1], F.v[2]}, kind != 5 && S.dr == 1 ? it : -1};
+                    launch3_v(lc, mA, g, b, A, mrev, 1, Gather3{nullptr, nullptr, -1}, rs, d_wait, ctr++);
                     launch_free_surface(lc, g, A.v[0], nb_shot, kFsFoldV);
-                    if (!inl) launch_adj_corrections(lc, g, b, A, mrev, false, blo, bhi);
-                    launch3_p(lc, mA, nullptr, g, b, A, mrev, 1, d_wait, nullptr, 0, nullptr, 0.0f, inl);
+                    launch3_p(lc, mA, nullptr, g, b, A, mrev, 1, d_wait, nullptr, 0, nullptr, 0.0f,
+                              Save3{bd, nullptr, -1}, ctr++);
                 } else if (fast2) {
                     reverse2(it, mrev);
                 } else {

@@ -25,7 +25,8 @@ struct Grid {
     long long nphys;       // points of the physical grid
     int S;                 // slab length along its axis: 2*nb + 1
     long long slab_n[3];   // points of the slab array of axis a
-    int zlo, zhi, zp;      // tile kernels' z slabs (smi_slab.h): low slab's quads, first high quad, row length
+    int zlo, zhi, zp;      // tile kernels' z slabs (smi_slab.h): low slab's nodes, first high node, row length
+    int xlo, xhi, xrows;   // and x slabs: low slab's rows, first high row, rows
     float dt;
     float c[3][kMaxHalf];  // a_l / h_a
     double vdt;            // vmax * dt (FP64, for the computing box)
@@ -159,8 +160,9 @@ void launch_inject_source(const LaunchCtx &lc, const Grid &g, const Batch &b, fl
                           const float *stf, int it, float scale);
 void launch_gather(const LaunchCtx &lc, const Grid &g, const Batch &b, const float *p,
                    float *seis, const long long *seis_off, int nt, int it);
+// have_max: absmax_tmp already holds the magnitudes (16-bit storage).
 void launch_save_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f,
-                       Bands bd, int it, unsigned *absmax_tmp);
+                       Bands bd, int it, unsigned *absmax_tmp, bool have_max);
 void launch_restore_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f,
                           Bands bd, int it);
 // Band of a step between stored samples (decimated boundaries).
@@ -187,38 +189,6 @@ void launch_adj_inject_tile(const LaunchCtx &lc, const Grid &g, const Batch &b, 
                             const long long *seis_off, int it);
 void launch_adj_v(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, long long work);
 void launch_adj_p(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, long long work);
-// One piece of the union of the CPML bands: per axis up to two index
-// intervals {start0, len0, start1, len1}; nodes = product of the counts.
-struct Piece {
-    int iv[3][4];
-    int cnt[3];
-    int axis;              // the axis whose band defines the piece
-    int blocks;            // 256-thread blocks of this piece per chunk and shot; 0: empty
-    int chunks;            // chunks along the piece's walk axis
-};
-// Disjoint pieces covering the nodes within w_lo of the low end or w_hi of
-// the high end of axis z or x, clipped to a box (make_pieces); q[a] is the
-// piece of axis a (q[2] unused).
-struct Pieces {
-    int n;                 // non-empty pieces
-    int w_lo, w_hi;
-    Piece q[3];
-};
-// uz: nodes per lane along x in the z piece's kernel.
-Pieces make_pieces(const Grid &g, const int lo[3], const int hi[3], int w_lo, int w_hi, int uz);
-// Transposed z and x CPML terms of the adjoint (vel: velocity part, else
-// pressure part, which in 3D also updates phi_y at its own nodes) over the
-// union of the z and x bands within the box [lo, hi] (union of the batch's
-// receiver boxes after m reverse steps); run before the main kernels (in 3D
-// those apply the y terms).
-void launch_adj_corrections(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, bool vel,
-                            const int lo[3], const int hi[3]);
-// Forward z and x CPML memory-variable updates over the slabs (vel:
-// velocity part, else pressure part) within the box [lo, hi] (union of the
-// batch's source boxes at step it); added to the update of the main kernels
-// (in 3D those apply the y terms).
-void launch_fwd_corrections(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int it, bool vel,
-                            const int lo[3], const int hi[3]);
 void launch_recon_p(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f,
                     const float *lp, float *acc, int mode, const float *stf, int it,
                     float src_scale, long long work);

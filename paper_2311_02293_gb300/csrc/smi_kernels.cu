@@ -15,6 +15,7 @@
 
 #include "smi_internal.h"
 #include "smi_box.h"
+#include "smi_band.h"
 #include "smi_pdl.h"
 #include "smi_slab.h"
 
@@ -23,30 +24,7 @@ namespace smi {
 namespace {
 
 constexpr int kThreads = 256;
-#ifndef SMI_CPML_U
-#define SMI_CPML_U 4
-#endif
-#ifndef SMI_CPML_UZ
-#define SMI_CPML_UZ 2        // adjoint kinds; the forward kinds take twice as many
-#endif
-constexpr int kCpmlChunk = SMI_CPML_U;     // nodes per thread along x, CPML kernel of the x piece
-constexpr int kCpmlChunkZ = SMI_CPML_UZ;   // x lines a unit of the z-piece kernel k_cpml_zp (adjoint kinds)
 constexpr int kMaxBlocksX = 152 * 16;
-#ifndef SMI_CPML_ZP_MINB
-#define SMI_CPML_ZP_MINB 4   // resident 256-thread blocks of k_cpml_zp (its warps loop: fewer are needed)
-#endif
-#ifndef SMI_CPML_XW_U
-#define SMI_CPML_XW_U 4      // nodes a chunk of the walk
-#endif
-#ifndef SMI_CPML_XW_PARTS
-#define SMI_CPML_XW_PARTS 2  // runs a band of k_cpml_xw is cut into (more lines walk at once)
-#endif
-#ifndef SMI_CPML_XW_MINB
-#define SMI_CPML_XW_MINB 4   // resident 256-thread blocks of k_cpml_xw
-#endif
-#ifndef SMI_CPML_MINB_F
-#define SMI_CPML_MINB_F 4
-#endif
 
 __device__ __forceinline__ long long gidx(const Grid &g, int i1, int i2, int i3)
 {
@@ -315,567 +293,6 @@ __global__ void __launch_bounds__(kThreads) k_adj_p(Grid g, Batch b, Fields f, i
 }
 
 // ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
-// CPML terms over the slabs only (Sec. 2.1), added to the interior update of
-// the main 3D kernels, which apply the plain scheme everywhere.
-//
-// Forward (the CPML of Komatitsch & Martin):
-//   FV: psi_a <- Bv_a psi_a + Av_a D_a p;    v_a -= dt b_a psi_a
-//   FP: psi_a <- Bp_a psi_a + Ap_a D_a v_a;  p -= dt kappa sum_a psi_a
-// Adjoint (transpose of one forward step; runs before the interior adjoint
-// kernels; chi / phi are the adjoint memory variables, kept in the psip /
-// psiv slabs):
-//   AV: chi_a <- Bv_a (chi_a + lv_a);  lv_a -= dt b_a D_a[Ap_a (lp + phi_a)]
-//   AP: phi_a <- Bp_a (phi_a + lp);    lp -= dt kappa sum_a D_a[Av_a (lv_a + chi_a)]
-//
-// Every D_a above is sum_l c_l (h(j + o + l) - h(j + o + 1 - l)) over a
-// field h along axis a (o = 0 for the V kinds, -1 for the P kinds), with
-// h = p, v_a, Ap_a (lp + phi_a) or Av_a (lv_a + chi_a), zero outside the
-// grid (and, for the adjoint kinds, outside the slab).
-//
-// The main 3D kernels apply the y terms themselves (their register queue
-// along y holds the operand of D_y; see smi_stencil3d.cu).  The kernels here
-// cover the z and x terms over the union of the z and x bands (nodes within
-// w_lo of the low end or w_hi of the high end of the axis; forward: the
-// slabs; adjoint: every node whose stencil reaches a slab node), cut into
-// two disjoint pieces clipped to the union of the batch's computing boxes
-// (see Pieces).  Each node belongs to one thread, which applies the terms of
-// both axes where both bands hold it, so the kinds that update p / lp (read
-// at the node only) need no ordering between axes.  A thread takes a chunk
-// of consecutive nodes along x and issues all the chunk's loads before its
-// first store (these kernels are bound by memory latency, not bytes).  The
-// adjoint phi_y update needs lp before the step, so the AP kernel makes it
-// at its own nodes of the y slab and the main pressure kernel at the rest.
-enum CpmlKind { kFV = 0, kFP = 1, kAV = 2, kAP = 3 };
-
-__device__ __forceinline__ bool in_band(const Grid &g, const Pieces &P, int a, int j)
-{
-    return j < P.w_lo || j >= g.ne[a] - P.w_hi;
-}
-
-// Offsets inside one shot's arrays are 32-bit: the 3D path requires a
-// field of one shot to hold fewer than 2^31 points.
-__device__ __forceinline__ int gidx32(const Grid &g, int i0, int i1, int i2) { return i0 + g.px * (i1 + g.ne[1] * i2); }
-__device__ __forceinline__ int gstride32(const Grid &g, int a) { return a == 0 ? 1 : (a == 1 ? g.px : g.px * g.ne[1]); }
-
-// Offset and stride of axis a's slab index at node i with i[a] replaced.
-__device__ __forceinline__ void slab_base(const Grid &g, int a, const int i[3], int &base, int &stride)
-{
-    if (a == 0) { base = g.S * (i[1] + g.ne[1] * i[2]); stride = 1; }
-    else if (a == 1) { base = i[0] + g.ne[0] * g.S * i[2]; stride = g.ne[0]; }
-    else { base = i[0] + g.px * i[1]; stride = g.px * g.ne[1]; }
-}
-
-// Arrays of kind KIND along axis A for one shot.
-template <int KIND, int A>
-struct CpmlAxis {
-    static constexpr bool VK = KIND == kFV || KIND == kAV;
-    const float *src;      // h's field: p (FV, AV) or v_a (FP, AP)
-    const float *hmem;     // adjoint kinds: phi_a (AV) or chi_a (AP), the memory variable in h
-    float *mem;            // memory variable updated at the node: psi / chi (V kinds), psi / phi (P kinds)
-    float *fld;            // V kinds: v_a / lv_a
-    int st, ne, sb, ss;    // flat stride, axis length; slab base of the line and slab stride
-    __device__ __forceinline__ CpmlAxis(const Grid &g, const Fields &f, int s, const int i[3])
-    {
-        const long long so = (long long)s * g.ntot, ms = (long long)s * g.slab_n[A];
-        src = VK ? f.p + so : f.v[A] + so;
-        hmem = (KIND == kAV ? f.psiv[A] : f.psip[A]) + ms;
-        mem = (VK ? f.psip[A] : f.psiv[A]) + ms;
-        fld = f.v[A] + so;
-        st = gstride32(g, A);
-        ne = g.ne[A];
-        slab_base(g, A, i, sb, ss);
-    }
-    __device__ __forceinline__ bool slab(const Grid &g, int j) const { return j < g.nb || j >= ne - g.nb - 1; }
-    __device__ __forceinline__ int msi(const Grid &g, int j) const   // slab index of node j (j in the slab)
-    {
-        return sb + (j < g.nb ? j : j - (ne - 2 * g.nb - 1)) * ss;
-    }
-    // h at index j of the line through node k (index ia); zero where the
-    // scheme has none.  Loads depend only on index arithmetic.
-    __device__ __forceinline__ float h(const Grid &g, int k, int ia, int j) const
-    {
-        bool valid = (unsigned)j < (unsigned)ne;
-        if (KIND == kAV || KIND == kAP) valid = valid && slab(g, j);
-        float x = 0.0f;
-        if (valid) {
-            const int kk = k + (j - ia) * st;
-            if (KIND == kFV || KIND == kFP) x = src[kk];
-            else x = __ldg((KIND == kAV ? g.cpa[A] : g.cva[A]) + j) * (src[kk] + hmem[msi(g, j)]);
-        }
-        return x;
-    }
-};
-
-// D_a at a node from its 2N values of h: w[t] = h(ia + o - N + 1 + t).
-template <int N>
-__device__ __forceinline__ float cpml_d(const Grid &g, int a, const float *w)
-{
-    float D = 0.0f;
-#pragma unroll
-    for (int l = 1; l <= N; l++) D += g.c[a][l - 1] * (w[N - 1 + l] - w[N - l]);
-    return D;
-}
-
-// Values of one axis at one node, loaded before any store of the chunk:
-// mem = memory variable (if the node is in the slab), fld = v_a / lv_a (V
-// kinds), rho1 = rho one node up the axis (buoyancy).
-struct CpmlOwn {
-    float mem, fld, rho1;
-};
-
-template <int KIND, int A>
-__device__ __forceinline__ CpmlOwn cpml_own(const Grid &g, const CpmlAxis<KIND, A> &x, int ia, int k, bool sl)
-{
-    CpmlOwn o{0.0f, 0.0f, 0.0f};
-    if (sl) o.mem = x.mem[x.msi(g, ia)];
-    if (CpmlAxis<KIND, A>::VK) {
-        o.fld = x.fld[k];
-        if (ia + 1 < x.ne) o.rho1 = g.rho[k + x.st];
-    }
-    return o;
-}
-
-// Applies the axis-A terms of one node from its preloaded values; the P
-// kinds add their term to acc (p / lp is written once per node).
-template <int KIND, int A>
-__device__ __forceinline__ void cpml_apply(const Grid &g, const CpmlAxis<KIND, A> &x, int ia, int k, bool sl,
-                                           const CpmlOwn &o, float rho0, float lp0, float D, float &acc)
-{
-    if (KIND == kFV || KIND == kAV) {
-        const float b = (ia + 1 < x.ne) ? __fdividef(2.0f, rho0 + o.rho1) : __fdividef(1.0f, rho0);
-        if (KIND == kFV) {
-            const float psi = g.cvb[A][ia] * o.mem + g.cva[A][ia] * D;
-            x.mem[x.msi(g, ia)] = psi;
-            x.fld[k] = o.fld - g.dt * b * psi;
-        } else {
-            if (sl) x.mem[x.msi(g, ia)] = g.cvb[A][ia] * (o.mem + o.fld);   // deferred chi update, lv before this step
-            if (D != 0.0f) x.fld[k] = o.fld - g.dt * b * D;
-        }
-    } else if (KIND == kFP) {
-        const float psi = g.cpb[A][ia] * o.mem + g.cpa[A][ia] * D;
-        x.mem[x.msi(g, ia)] = psi;
-        acc += psi;
-    } else {
-        if (sl) x.mem[x.msi(g, ia)] = g.cpb[A][ia] * (o.mem + lp0);         // phi update, lp before this step
-        acc += D;
-    }
-}
-
-// Band membership of index j on axis a for kind KIND (forward: the slab).
-template <int KIND>
-__device__ __forceinline__ bool cpml_in(const Grid &g, const Pieces &P, int a, int j)
-{
-    return (KIND == kFV || KIND == kFP) ? in_slab(g, a, j) : in_band(g, P, a, j);
-}
-
-__device__ __forceinline__ int iv_map(const int *iv, int c) { return c < iv[1] ? iv[0] + c : iv[2] + c - iv[1]; }
-
-// AP only: phi_y <- Bp_y (phi_y + lp) at nodes of the y slab, with lp
-// before this step (these kernels run before the main pressure kernel,
-// which makes the update at the y-slab nodes outside the z and x bands).
-struct CpmlPhiY {
-    float *ph;             // shot's phi_y slab array at node 0 of the chunk, or null
-    float B;
-    int step;              // offset between consecutive nodes of the chunk
-    __device__ __forceinline__ CpmlPhiY(const Grid &g, const Fields &f, int s, const int i[3], int step_)
-    {
-        ph = nullptr;
-        B = 0.0f;
-        step = step_;
-        const int y = i[2];
-        if (g.ndim == 3 && (y < g.nb || y >= g.ne[2] - g.nb - 1)) {
-            const int js = y < g.nb ? y : y - (g.ne[2] - 2 * g.nb - 1);
-            ph = f.psiv[2] + (long long)s * g.slab_n[2] + i[0] + g.px * (i[1] + g.ne[1] * js);
-            B = g.cpb[2][y];
-        }
-    }
-};
-
-// x piece: a thread takes up to U consecutive nodes along x of one line
-// (fixed z index i0 and y index i2); z is inner there, so the nodes have x
-// terms only.  Phase 1 issues every load of the chunk: the window of h
-// along x shared by the U nodes (U + 2N - 1 values instead of 2N per node)
-// and the nodes' own values.  Phase 2 computes and stores.
-template <int N, int KIND, int U>
-__device__ __forceinline__ void cpml_chunk(const Grid &g, const Fields &f, const Piece &p, int s, int c0, int cr,
-                                           int ch, const int lo[3], const int hi[3])
-{
-    constexpr int W = 1;
-    constexpr bool VK = KIND == kFV || KIND == kAV;
-    constexpr int O = VK ? 0 : -1;
-    int i[3];
-    i[0] = iv_map(p.iv[0], c0);
-    i[2] = iv_map(p.iv[2], cr);
-    if (i[0] < lo[0] || i[0] > hi[0] || i[2] < lo[2] || i[2] > hi[2]) return;
-    const int nc0 = (p.iv[W][1] + U - 1) / U;
-    const int seg = ch < nc0 ? 0 : 1;
-    ch -= seg ? nc0 : 0;
-    const int j0 = p.iv[W][2 * seg] + ch * U;
-    const int jend = min(p.iv[W][2 * seg] + p.iv[W][2 * seg + 1] - 1, hi[W]);
-    i[W] = j0;
-    const int k0 = gidx32(g, i[0], i[1], i[2]);
-    const CpmlAxis<KIND, W> x(g, f, s, i);
-    float *ps = f.p + (long long)s * g.ntot;
-    const CpmlPhiY py(g, f, s, i, g.px);
-
-    // ---- phase 1: loads ----
-    float win[U + 2 * N - 1];
-#pragma unroll
-    for (int q = 0; q < U + 2 * N - 1; q++) win[q] = x.h(g, k0, j0, j0 + O - N + 1 + q);
-    CpmlOwn oW[U];
-    float rho0[U], own_p[U], kap[U], phy[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        const int j = j0 + u, k = k0 + u * x.st;
-        const bool ok = j <= jend && j >= lo[W];
-        rho0[u] = (VK && ok) ? g.rho[k] : 1.0f;
-        own_p[u] = (!VK && ok) ? ps[k] : 0.0f;
-        kap[u] = (!VK && ok) ? g.K[k] : 0.0f;
-        phy[u] = (KIND == kAP && ok && py.ph) ? py.ph[u * py.step] : 0.0f;
-        oW[u] = CpmlOwn{0.0f, 0.0f, 0.0f};
-        if (ok) oW[u] = cpml_own(g, x, j, k, x.slab(g, j));
-    }
-
-    // ---- phase 2: compute and store ----
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        const int j = j0 + u, k = k0 + u * x.st;
-        if (!(j <= jend && j >= lo[W])) continue;
-        float acc = 0.0f;
-        cpml_apply(g, x, j, k, x.slab(g, j), oW[u], rho0[u], own_p[u], cpml_d<N>(g, W, win + u), acc);
-        if (KIND == kFP) ps[k] = own_p[u] - g.dt * kap[u] * acc;
-        if (KIND == kAP) {
-            if (py.ph) py.ph[u * py.step] = py.B * (phy[u] + own_p[u]);
-            if (acc != 0.0f) ps[k] = own_p[u] - g.dt * kap[u] * acc;
-        }
-    }
-}
-
-// x piece, walking: a thread takes one line along x (fixed z index i0 and y
-// index i2) and walks run `part` of one band of it (seg: the low or the high
-// band, cut into nparts runs of whole chunks) in chunks of U nodes.  The
-// window of h along x rolls from chunk to chunk: the last 2N - 1 values of
-// one chunk's window open the next, so each h value is loaded once per run
-// (cpml_chunk loads U + 2N - 1 values for every U nodes).  Same arithmetic as
-// cpml_chunk.
-template <int N, int KIND, int U>
-__device__ __forceinline__ void cpml_xwalk(const Grid &g, const Fields &f, const Piece &p, int s, int c0, int cr,
-                                           int seg, int part, int nparts, const int lo[3], const int hi[3])
-{
-    constexpr int W = 1;
-    constexpr bool VK = KIND == kFV || KIND == kAV;
-    constexpr int O = VK ? 0 : -1;
-    constexpr int NW = U + 2 * N - 1;
-    int i[3];
-    i[0] = iv_map(p.iv[0], c0);
-    i[2] = iv_map(p.iv[2], cr);
-    if (i[0] < lo[0] || i[0] > hi[0] || i[2] < lo[2] || i[2] > hi[2]) return;
-    // the band's chunks, cut into nparts runs of whole chunks; this thread walks run `part`
-    const int jb = max(p.iv[W][2 * seg], lo[W]);
-    const int jl = min(p.iv[W][2 * seg] + p.iv[W][2 * seg + 1] - 1, hi[W]);
-    const int per = ((jl - jb + U) / U + nparts - 1) / nparts * U;
-    const int js = jb + part * per;
-    const int jend = min(jl, js + per - 1);
-    if (js > jend) return;
-    i[W] = js;
-    const int k0 = gidx32(g, i[0], i[1], i[2]);
-    const CpmlAxis<KIND, W> x(g, f, s, i);
-    float *ps = f.p + (long long)s * g.ntot;
-    const CpmlPhiY py(g, f, s, i, g.px);
-
-    float win[NW];
-#pragma unroll
-    for (int q = 0; q < 2 * N - 1; q++) win[q] = x.h(g, k0, js, js + O - N + 1 + q);
-    for (int j0 = js; j0 <= jend; j0 += U) {
-        // ---- loads: the window's U new values and the chunk's own values ----
-#pragma unroll
-        for (int q = 2 * N - 1; q < NW; q++) win[q] = x.h(g, k0, js, j0 + O - N + 1 + q);
-        CpmlOwn oW[U];
-        float rho0[U], own_p[U], kap[U], phy[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int j = j0 + u, k = k0 + (j - js) * x.st;
-            const bool ok = j <= jend;
-            rho0[u] = (VK && ok) ? g.rho[k] : 1.0f;
-            own_p[u] = (!VK && ok) ? ps[k] : 0.0f;
-            kap[u] = (!VK && ok) ? g.K[k] : 0.0f;
-            phy[u] = (KIND == kAP && ok && py.ph) ? py.ph[(j - js) * py.step] : 0.0f;
-            oW[u] = CpmlOwn{0.0f, 0.0f, 0.0f};
-            if (ok) oW[u] = cpml_own(g, x, j, k, x.slab(g, j));
-        }
-        // ---- compute and store ----
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int j = j0 + u, k = k0 + (j - js) * x.st;
-            if (j > jend) continue;
-            float acc = 0.0f;
-            cpml_apply(g, x, j, k, x.slab(g, j), oW[u], rho0[u], own_p[u], cpml_d<N>(g, W, win + u), acc);
-            if (KIND == kFP) ps[k] = own_p[u] - g.dt * kap[u] * acc;
-            if (KIND == kAP) {
-                if (py.ph) py.ph[(j - js) * py.step] = py.B * (phy[u] + own_p[u]);
-                if (acc != 0.0f) ps[k] = own_p[u] - g.dt * kap[u] * acc;
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 2 * N - 1; q++) win[q] = win[q + U];
-    }
-}
-
-// z piece: a warp takes one line segment along z (32 lanes = BW owned nodes
-// plus the 2N - 1 halo nodes of their stencils) times up to U consecutive
-// nodes along x.  Each lane loads h along z at its own position and the z
-// derivatives come from warp shuffles; chunks that reach the x band also
-// load a per-lane window of h along x for the x terms.  Control flow is
-// warp-uniform up to the shuffles.
-template <int N, int KIND, int U>
-__device__ __forceinline__ void cpml_zwarp(const Grid &g, const Fields &f, const Pieces &P, const Piece &p, int s,
-                                           int lane, int zw, int cr, int ch, const int lo[3], const int hi[3])
-{
-    constexpr int W = 1;
-    constexpr bool VK = KIND == kFV || KIND == kAV;
-    constexpr int O = VK ? 0 : -1;
-    constexpr int HL = N - 1 - O, HR = N + O, BW = 32 - HL - HR;
-    const int nz0 = (p.iv[0][1] + BW - 1) / BW;
-    const int cw0 = (p.iv[W][1] + U - 1) / U;
-    int i[3];                                                      // warp-uniform from here to the shuffles
-    i[2] = iv_map(p.iv[2], cr);
-    if (i[2] < lo[2] || i[2] > hi[2]) return;
-    const int zseg = zw < nz0 ? 0 : 1;
-    zw -= zseg ? nz0 : 0;
-    const int zs = p.iv[0][2 * zseg], ze = min(zs + p.iv[0][2 * zseg + 1] - 1, hi[0]);
-    const int z = zs + zw * BW + lane - HL;
-    const bool zown = lane >= HL && lane < 32 - HR && z <= ze && z >= lo[0];
-    const int wseg = ch < cw0 ? 0 : 1;
-    ch -= wseg ? cw0 : 0;
-    const int j0 = p.iv[W][2 * wseg] + ch * U;
-    const int jend = min(p.iv[W][2 * wseg] + p.iv[W][2 * wseg + 1] - 1, hi[W]);
-    const int zc = min(max(z, 0), g.ne[0] - 1);
-    i[0] = zc;
-    i[W] = j0;
-    const int k0 = gidx32(g, i[0], i[1], i[2]);
-    const CpmlAxis<KIND, W> xw(g, f, s, i);
-    float *ps = f.p + (long long)s * g.ntot;
-    // axis-0 arrays: the slab base moves by S per node along x
-    const CpmlAxis<KIND, 0> xz(g, f, s, i);
-    const bool s0 = xz.slab(g, zc);
-    const bool wband = cpml_in<KIND>(g, P, W, j0) || cpml_in<KIND>(g, P, W, j0 + U - 1);   // warp-uniform
-    const CpmlPhiY py(g, f, s, i, g.px);
-
-    // ---- phase 1: loads ----
-    float hz[U], win[U + 2 * N - 1];
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        CpmlAxis<KIND, 0> xu = xz;
-        xu.sb += u * g.S;
-        hz[u] = j0 + u <= jend ? xu.h(g, k0 + u * xw.st, zc, z) : 0.0f;   // no line past the chunk's end
-    }
-#pragma unroll
-    for (int q = 0; q < U + 2 * N - 1; q++) win[q] = (zown && wband) ? xw.h(g, k0, j0, j0 + O - N + 1 + q) : 0.0f;
-    CpmlOwn o0[U], oW[U];
-    float rho0[U], own_p[U], kap[U], phy[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        const int j = j0 + u, k = k0 + u * xw.st;
-        const bool ok = zown && j <= jend && j >= lo[W];
-        rho0[u] = (VK && ok) ? g.rho[k] : 1.0f;
-        own_p[u] = (!VK && ok) ? ps[k] : 0.0f;
-        kap[u] = (!VK && ok) ? g.K[k] : 0.0f;
-        phy[u] = (KIND == kAP && ok && py.ph) ? py.ph[u * py.step] : 0.0f;
-        o0[u] = CpmlOwn{0.0f, 0.0f, 0.0f};
-        oW[u] = CpmlOwn{0.0f, 0.0f, 0.0f};
-        CpmlAxis<KIND, 0> xu = xz;
-        xu.sb += u * g.S;
-        if (ok) o0[u] = cpml_own(g, xu, zc, k, s0);
-        if (ok && wband && cpml_in<KIND>(g, P, W, j)) oW[u] = cpml_own(g, xw, j, k, xw.slab(g, j));
-    }
-
-    // ---- phase 2: compute and store ----
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-        const int j = j0 + u, k = k0 + u * xw.st;
-        if (!(j <= jend && j >= lo[W])) continue;                 // warp-uniform
-        float Dz = 0.0f;
-#pragma unroll
-        for (int l = 1; l <= N; l++)
-            Dz += g.c[0][l - 1] * (__shfl_sync(0xffffffffu, hz[u], lane + O + l) -
-                                   __shfl_sync(0xffffffffu, hz[u], lane + O + 1 - l));
-        if (!zown) continue;
-        float acc = 0.0f;
-        CpmlAxis<KIND, 0> xu = xz;
-        xu.sb += u * g.S;
-        cpml_apply(g, xu, zc, k, s0, o0[u], rho0[u], own_p[u], Dz, acc);
-        if (wband && cpml_in<KIND>(g, P, W, j))
-            cpml_apply(g, xw, j, k, xw.slab(g, j), oW[u], rho0[u], own_p[u], cpml_d<N>(g, W, win + u), acc);
-        if (KIND == kFP) ps[k] = own_p[u] - g.dt * kap[u] * acc;
-        if (KIND == kAP) {
-            if (py.ph) py.ph[u * py.step] = py.B * (phy[u] + own_p[u]);
-            if (acc != 0.0f) ps[k] = own_p[u] - g.dt * kap[u] * acc;
-        }
-    }
-}
-
-// Resident 256-thread blocks per SM that k_cpml_x's register budget must
-// allow (the forward kinds' x piece is load-latency bound: more warps hide
-// more latency).  Measured on the 340^3 RTM step, box off, 30 steps: without
-// a bound (62-95 registers) forward 18.3 ms, with 4 blocks (64 registers)
-// 17.8 ms.
-
-// x piece: block = ZB z indices x 256/ZB y indices (ZB = 64 in 3D, 256 in 2D
-// where y has one index); blockIdx.y = chunk along x, blockIdx.z = shot.
-template <int N, int KIND>
-__global__ void __launch_bounds__(256, SMI_CPML_MINB_F) k_cpml_x(Grid g, Batch b, Fields f, Pieces P, int m)
-{
-    const Piece &p = P.q[1];
-    const int zb = g.ndim == 3 ? 64 : 256;
-    const int nbz = (p.cnt[0] + zb - 1) / zb;
-    const int bz = blockIdx.x % nbz, br = blockIdx.x / nbz;
-    const int c0 = bz * zb + (int)threadIdx.x % zb, cr = br * (256 / zb) + (int)threadIdx.x / zb;
-    if (c0 >= p.cnt[0] || cr >= p.cnt[2]) return;
-    const int s = blockIdx.z;
-    int lo[3], hi[3];
-    box_at((KIND == kFV || KIND == kFP) ? b.tab_src : b.tab_rec, b.nt1, s, m, lo, hi);
-    cpml_chunk<N, KIND, kCpmlChunk>(g, f, p, s, c0, cr, blockIdx.y, lo, hi);
-}
-
-// x piece, walking (cpml_xwalk): block = ZB z indices x 256/ZB y indices
-// as in k_cpml_x; blockIdx.y = band (low, high) x run of the band
-// (SMI_CPML_XW_PARTS runs a band, so that enough lines walk at once),
-// blockIdx.z = shot.
-template <int N, int KIND>
-__global__ void __launch_bounds__(256, SMI_CPML_XW_MINB) k_cpml_xw(Grid g, Batch b, Fields f, Pieces P, int m)
-{
-    const Piece &p = P.q[1];
-    const int zb = g.ndim == 3 ? 64 : 256;
-    const int nbz = (p.cnt[0] + zb - 1) / zb;
-    const int bz = blockIdx.x % nbz, br = blockIdx.x / nbz;
-    const int c0 = bz * zb + (int)threadIdx.x % zb, cr = br * (256 / zb) + (int)threadIdx.x / zb;
-    const int side = blockIdx.y / SMI_CPML_XW_PARTS, part = blockIdx.y % SMI_CPML_XW_PARTS;
-    if (c0 >= p.cnt[0] || cr >= p.cnt[2] || p.iv[1][2 * side + 1] == 0) return;
-    const int s = blockIdx.z;
-    int lo[3], hi[3];
-    box_at((KIND == kFV || KIND == kFP) ? b.tab_src : b.tab_rec, b.nt1, s, m, lo, hi);
-    cpml_xwalk<N, KIND, SMI_CPML_XW_U>(g, f, p, s, c0, cr, side, part, SMI_CPML_XW_PARTS, lo, hi);
-}
-
-// z piece, persistent: blockIdx.y = z warp segment (those of the low band,
-// then those of the high band), blockIdx.z = shot; the warps of a segment
-// walk its units (UZ consecutive x lines at one y, the chunks cpml_zwarp
-// takes) in a strided loop.  What depends on z alone -- the lane's node, its
-// CPML coefficients, slab offsets and box test -- is computed once per warp
-// instead of once per unit.  Units whose x range reaches the x band take
-// cpml_zwarp, which adds the x terms there; the others run the z terms
-// below, the same arithmetic as cpml_apply.
-template <int N, int KIND>
-__global__ void __launch_bounds__(256, SMI_CPML_ZP_MINB) k_cpml_zp(Grid g, Batch b, Fields f, Pieces P, int m)
-{
-    constexpr bool VK = KIND == kFV || KIND == kAV;
-    constexpr bool ADJ = KIND == kAV || KIND == kAP;
-    constexpr int O = VK ? 0 : -1;
-    constexpr int HL = N - 1 - O, HR = N + O, BW = 32 - HL - HR;
-    constexpr int U = ADJ ? kCpmlChunkZ : 2 * kCpmlChunkZ;
-    const Piece &p = P.q[0];
-    const int s = blockIdx.z, lane = threadIdx.x & 31;
-    int lo[3], hi[3];
-    box_at(ADJ ? b.tab_rec : b.tab_src, b.nt1, s, m, lo, hi);
-
-    // ---- per warp: the segment and the lane's node along z ----
-    const int zw = blockIdx.y;
-    const int nz0 = (p.iv[0][1] + BW - 1) / BW;
-    const int zseg = zw < nz0 ? 0 : 1;
-    const int zs = p.iv[0][2 * zseg], ze = min(zs + p.iv[0][2 * zseg + 1] - 1, hi[0]);
-    const int ne = g.ne[0], hib = ne - 2 * g.nb - 1;           // slab index = j, or j - hib in the high slab
-    const int z = zs + (zw - (zseg ? nz0 : 0)) * BW + lane - HL;
-    const bool zown = lane >= HL && lane < 32 - HR && z <= ze && z >= lo[0];
-    const int zc = min(max(z, 0), ne - 1);
-    bool hv = (unsigned)z < (unsigned)ne;                          // h exists at z
-    if (ADJ) hv = hv && (z < g.nb || z >= ne - g.nb - 1);
-    const int hms = z < g.nb ? z : z - hib;
-    const float hca = (ADJ && hv) ? __ldg((KIND == kAV ? g.cpa[0] : g.cva[0]) + z) : 0.0f;
-    const bool sl = zc < g.nb || zc >= ne - g.nb - 1;              // own node in the slab
-    const int oms = zc < g.nb ? zc : zc - hib;
-    const bool up = zc + 1 < ne;
-    const float cb = sl ? (VK ? g.cvb[0][zc] : g.cpb[0][zc]) : 0.0f;
-    const float ca = (!ADJ && sl) ? (VK ? g.cva[0][zc] : g.cpa[0][zc]) : 0.0f;
-
-    const long long so = (long long)s * g.ntot, ms = (long long)s * g.slab_n[0];
-    const float *src = (VK ? f.p : f.v[0]) + so;
-    const float *hmem = (KIND == kAV ? f.psiv[0] : f.psip[0]) + ms;
-    float *mem = (VK ? f.psip[0] : f.psiv[0]) + ms;
-    float *fld = f.v[0] + so;
-    float *ps = f.p + so;
-
-    const int nch = (p.iv[1][1] + U - 1) / U;
-    const int nunit = p.cnt[2] * nch;
-    const int xend = min(p.iv[1][0] + p.iv[1][1] - 1, hi[1]);
-    for (int t = blockIdx.x * 8 + (int)(threadIdx.x >> 5); t < nunit; t += gridDim.x * 8) {   // warp-uniform
-        const int cr = t / nch, ch = t - cr * nch;
-        const int y = iv_map(p.iv[2], cr);
-        if (y < lo[2] || y > hi[2]) continue;
-        const int x0 = p.iv[1][0] + ch * U;
-        if (cpml_in<KIND>(g, P, 1, x0) || cpml_in<KIND>(g, P, 1, x0 + U - 1)) {
-            cpml_zwarp<N, KIND, U>(g, f, P, p, s, lane, zw, cr, ch, lo, hi);
-            continue;
-        }
-        const int kl = gidx32(g, 0, x0, y), sL = g.S * (x0 + g.ne[1] * y);
-        int iz[3] = {zc, x0, y};
-        const CpmlPhiY py(g, f, s, iz, g.px);
-
-        // ---- loads ----
-        float hz[U], rho0[U], rho1[U], fo[U], mo[U], pk[U], kp[U], phy[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int k = kl + u * g.px + zc, mi = sL + u * g.S;
-            const bool ok = zown && x0 + u <= xend && x0 + u >= lo[1];
-            hz[u] = 0.0f;
-            if (hv && x0 + u <= xend) {
-                const int kk = kl + u * g.px + z;
-                hz[u] = ADJ ? hca * (src[kk] + hmem[mi + hms]) : src[kk];
-            }
-            rho0[u] = (VK && ok) ? g.rho[k] : 1.0f;
-            rho1[u] = (VK && ok && up) ? g.rho[k + 1] : 0.0f;
-            fo[u] = (VK && ok) ? fld[k] : 0.0f;
-            mo[u] = (ok && sl) ? mem[mi + oms] : 0.0f;
-            pk[u] = (!VK && ok) ? ps[k] : 0.0f;
-            kp[u] = (!VK && ok) ? g.K[k] : 0.0f;
-            phy[u] = (KIND == kAP && ok && py.ph) ? py.ph[u * py.step] : 0.0f;
-        }
-
-        // ---- compute and store ----
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (!(x0 + u <= xend && x0 + u >= lo[1])) continue;    // warp-uniform
-            float Dz = 0.0f;
-#pragma unroll
-            for (int l = 1; l <= N; l++)
-                Dz += g.c[0][l - 1] * (__shfl_sync(0xffffffffu, hz[u], lane + O + l) -
-                                       __shfl_sync(0xffffffffu, hz[u], lane + O + 1 - l));
-            if (!zown) continue;
-            const int k = kl + u * g.px + zc, mi = sL + u * g.S + oms;
-            if (VK) {
-                const float bb = up ? __fdividef(2.0f, rho0[u] + rho1[u]) : __fdividef(1.0f, rho0[u]);
-                if (KIND == kFV) {
-                    const float psi = cb * mo[u] + ca * Dz;
-                    mem[mi] = psi;
-                    fld[k] = fo[u] - g.dt * bb * psi;
-                } else {
-                    if (sl) mem[mi] = cb * (mo[u] + fo[u]);                // deferred chi update
-                    if (Dz != 0.0f) fld[k] = fo[u] - g.dt * bb * Dz;
-                }
-            } else if (KIND == kFP) {
-                const float psi = cb * mo[u] + ca * Dz;
-                mem[mi] = psi;
-                ps[k] = pk[u] - g.dt * kp[u] * psi;
-            } else {
-                if (sl) mem[mi] = cb * (mo[u] + pk[u]);                    // phi update, lp before this step
-                if (py.ph) py.ph[u * py.step] = py.B * (phy[u] + pk[u]);
-                if (Dz != 0.0f) ps[k] = pk[u] - g.dt * kp[u] * Dz;
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Source-field reconstruction (Sec. 4.2, Algorithm 2 reverse loop) fused with
 // the imaging / gradient accumulation, over the physical nodes of the
 // forward box of step it:
@@ -1054,7 +471,7 @@ __global__ void k_adj_inject_tile(Grid g, Batch b, Fields A, const float *res, c
                     atomicAdd(A.psiv[0] + s * g.slab_n[0] + q + (z & 3) + (long long)g.zp * (x + (long long)g.ne[1] * y),
                               g.cpa[0][z] * add);
                 if (jx >= 0)
-                    atomicAdd(A.psiv[1] + s * g.slab_n[1] + z + (long long)g.px * (jx + (long long)g.S * y),
+                    atomicAdd(A.psiv[1] + s * g.slab_n[1] + z + (long long)g.px * (jx + (long long)g.xrows * y),
                               g.cpa[1][x] * add);
                 const int jy = g.ndim == 3 ? slab_row(g, 2, y) : -1;
                 if (jy >= 0)
@@ -1133,36 +550,6 @@ __global__ void k_dot(const float *a, const float *b, long long n, double *parti
 // 2^31 values (checked at set-up), so offsets are 32-bit.
 constexpr int kBandVals = 4;
 
-struct BandRegion {
-    int a, sd, w0, w1, n, off;
-    const int *lo;
-    unsigned m0, m1;                  // u / w0 and q / w1 by multiply-high (band_divisor)
-    int l0, l1;
-    __device__ __forceinline__ BandRegion(const Bands &bd, int r)
-    {
-        a = r >> 1;
-        sd = r & 1;
-        lo = bd.lo[a][sd];
-        const int *hi = bd.hi[a][sd];
-        w0 = hi[0] - lo[0] + 1;
-        w1 = hi[1] - lo[1] + 1;
-        n = w0 * w1 * (hi[2] - lo[2] + 1);
-        off = (int)bd.off[a][sd];
-        m0 = bd.dm[a][sd][0];
-        l0 = bd.dl[a][sd][0];
-        m1 = bd.dm[a][sd][1];
-        l1 = bd.dl[a][sd][1];
-    }
-    // flat field index of value u of the region
-    __device__ __forceinline__ int node(const Grid &g, int u) const
-    {
-        const unsigned uu = (unsigned)u;
-        const unsigned q = (__umulhi(m0, uu) + uu) >> l0;
-        const unsigned q1 = (__umulhi(m1, q) + q) >> l1;
-        return (lo[0] + u - (int)q * w0) + g.px * ((lo[1] + (int)q - (int)q1 * w1) + g.ne[1] * (lo[2] + (int)q1));
-    }
-};
-
 __global__ void k_band_absmax(Grid g, Fields f, Bands bd, unsigned *amax)
 {
     const BandRegion R(bd, blockIdx.y);
@@ -1182,6 +569,8 @@ __global__ void k_band_absmax(Grid g, Fields f, Bands bd, unsigned *amax)
 __global__ void k_band_save(Grid g, Fields f, Bands bd, int it, const unsigned *amax)
 {
     const BandRegion R(bd, blockIdx.y);
+    pdl_wait();
+    pdl_trigger();
     if (R.a >= g.ndim || R.n <= 0) return;
     const int s = blockIdx.z;
     const float *v = f.v[R.a] + (long long)s * g.ntot;
@@ -1506,11 +895,8 @@ __global__ void k_extend_model(Grid g, const float *vp, const float *rho, int n1
         const int i1 = (int)(t % g.px);
         const int i2 = (int)((t / g.px) % g.ne[1]);
         const int i3 = (int)(t / ((long long)g.px * g.ne[1]));
-        if (i1 >= g.ne[0]) {            // row padding
-            rho_e[t] = 0.0f;
-            K[t] = 0.0f;
-            continue;
-        }
+        // row padding: kappa 0, rho that of the last node (its own neighbour in the buoyancy)
+        const bool pad = i1 >= g.ne[0];
         // free surface: the top layer mirrors the model about the surface node,
         // so that the transposed mirrors of the adjoint take no model ratio
         const int j1 = (g.freesurf && i1 < g.L[0]) ? min(g.L[0] - i1, n1 - 1) : min(max(i1 - g.L[0], 0), n1 - 1);
@@ -1519,7 +905,7 @@ __global__ void k_extend_model(Grid g, const float *vp, const float *rho, int n1
         const long long kp = (long long)j1 + (long long)n1 * ((long long)j2 + (long long)n2 * j3);
         const float r = rho[kp], c = vp[kp];
         rho_e[t] = r;
-        K[t] = r * c * c;
+        K[t] = pad ? 0.0f : r * c * c;
     }
 }
 
@@ -1629,140 +1015,6 @@ void launch_recon_v(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f
     SMI_DISPATCH(k_recon_v, grid, g, b, f, it);
 }
 
-// Pieces of the union of the bands (Sec. 2.1 CPML terms), clipped to the
-// box [lo, hi].  Axis a: band = [0, w_lo) u [ne - w_hi, ne), the rest is
-// "inner"; piece a = band of a x inner of every lower axis x box of every
-// higher axis.  Inactive axes hold the single node 0.
-Pieces make_pieces(const Grid &g, const int lo[3], const int hi[3], int w_lo, int w_hi, int uz)
-{
-    Pieces P{};
-    P.w_lo = w_lo;
-    P.w_hi = w_hi;
-    int band[3][4], inner[3][4], full[3][4];
-    auto clip = [](int x0, int x1, int l, int h, int *out) {
-        const int s = std::max(x0, l), e = std::min(x1, h);
-        out[0] = s;
-        out[1] = e >= s ? e - s + 1 : 0;
-    };
-    for (int a = 0; a < 3; a++) {
-        for (int k = 0; k < 4; k++) band[a][k] = inner[a][k] = full[a][k] = 0;
-        const int ne = g.ne[a];
-        clip(0, ne - 1, lo[a], hi[a], full[a]);
-        if (ne - w_hi <= w_lo) {              // the two bands meet: the whole axis
-            clip(0, ne - 1, lo[a], hi[a], band[a]);
-        } else {
-            clip(0, w_lo - 1, lo[a], hi[a], band[a]);
-            clip(ne - w_hi, ne - 1, lo[a], hi[a], band[a] + 2);
-            clip(w_lo, ne - w_hi - 1, lo[a], hi[a], inner[a]);
-        }
-    }
-    // piece 0: z band x all x x all y; piece 1: x band x inner z x all y
-    for (int a = 0; a < 2; a++) {
-        Piece &p = P.q[a];
-        p.axis = a;
-        long long cnt = 1;
-        for (int b = 0; b < 3; b++) {
-            const int *src = b == a ? band[b] : (b < a ? inner[b] : full[b]);
-            for (int k = 0; k < 4; k++) p.iv[b][k] = src[k];
-            p.cnt[b] = src[1] + src[3];
-            cnt *= p.cnt[b];
-        }
-        if (cnt == 0) continue;
-        P.n++;
-        // x piece: blocks of 64 z x 4 y lines (k_cpml_x: y = chunks along x;
-        // k_cpml_xw: y = band).  z piece: nonzero counts mark the piece as
-        // present (k_cpml_zp sizes its own persistent launch).
-        const int u = a == 0 ? uz : kCpmlChunk;
-        p.chunks = (p.iv[1][1] + u - 1) / u + (p.iv[1][3] + u - 1) / u;
-        if (a == 0) {
-            const int bw = 32 - (2 * g.N - 1);
-            const long long zw = (p.iv[0][1] + bw - 1) / bw + (p.iv[0][3] + bw - 1) / bw;
-            p.blocks = (int)((zw * p.cnt[2] + 7) / 8);
-        } else {
-            const int zb = g.ndim == 3 ? 64 : 256;
-            p.blocks = ((p.cnt[0] + zb - 1) / zb) * ((p.cnt[2] + 256 / zb - 1) / (256 / zb));
-        }
-    }
-    return P;
-}
-
-namespace {
-
-// Persistent z-piece launch: one block column per z warp segment and shot,
-// as many blocks along x as fill the GPU once (at least one unit a warp).
-template <int N, int KIND>
-void zp_launch(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, const Pieces &P, int m)
-{
-    static const int fill = [] {
-        int per = 0, dev = 0, sms = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cpml_zp<N, KIND>, 256, 0);
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        return std::max(1, per) * std::max(1, sms);
-    }();
-    constexpr int BW = 32 - (2 * N - 1);
-    constexpr int U = KIND >= kAV ? kCpmlChunkZ : 2 * kCpmlChunkZ;
-    const Piece &p = P.q[0];
-    const int nseg = (p.iv[0][1] + BW - 1) / BW + (p.iv[0][3] + BW - 1) / BW;
-    const long long nunit = (long long)p.cnt[2] * ((p.iv[1][1] + U - 1) / U);
-    if (nseg == 0 || nunit == 0) return;
-    const long long per_col = (long long)nseg * b.nshot;
-    const long long nblk = std::max(1LL, std::min((fill + per_col - 1) / per_col, (nunit + 7) / 8));
-    k_cpml_zp<N, KIND><<<dim3((unsigned)nblk, nseg, b.nshot), 256, 0, S(lc)>>>(g, b, f, P, m);
-    ++*lc.launches;
-}
-
-template <int N>
-void corr_launch(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, int kind,
-                 const int lo[3], const int hi[3])
-{
-    // adjoint bands: nodes whose stencil reaches a slab node; forward: the slabs
-    const Pieces P = kind >= kAV ? make_pieces(g, lo, hi, g.nb + N, g.nb + N + 1, kCpmlChunkZ)
-                                 : make_pieces(g, lo, hi, g.nb, g.nb + 1, 2 * kCpmlChunkZ);
-    // the two pieces hold disjoint nodes: launches in any order
-    for (int a = 0; a < 2; a++) {
-        const Piece &p = P.q[a];
-        if (p.blocks == 0 || p.chunks == 0) continue;
-        const dim3 grid(p.blocks, p.chunks, b.nshot);
-        if (a == 0) {
-            if (kind == kFV) zp_launch<N, kFV>(lc, g, b, f, P, m);
-            else if (kind == kFP) zp_launch<N, kFP>(lc, g, b, f, P, m);
-            else if (kind == kAV) zp_launch<N, kAV>(lc, g, b, f, P, m);
-            else zp_launch<N, kAP>(lc, g, b, f, P, m);
-            continue;                                     // counts its own launch
-        } else if (kind >= kAV) {                          // measured: the walk pays in the adjoint kinds only
-            const dim3 gw(p.blocks, 2 * SMI_CPML_XW_PARTS, b.nshot);
-            if (kind == kAV) k_cpml_xw<N, kAV><<<gw, 256, 0, S(lc)>>>(g, b, f, P, m);
-            else k_cpml_xw<N, kAP><<<gw, 256, 0, S(lc)>>>(g, b, f, P, m);
-        } else {
-            if (kind == kFV) k_cpml_x<N, kFV><<<grid, 256, 0, S(lc)>>>(g, b, f, P, m);
-            else k_cpml_x<N, kFP><<<grid, 256, 0, S(lc)>>>(g, b, f, P, m);
-        }
-        ++*lc.launches;
-    }
-}
-
-void corr_dispatch(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, int kind,
-                   const int lo[3], const int hi[3])
-{
-    if (g.N == 2) corr_launch<2>(lc, g, b, f, m, kind, lo, hi);
-    else corr_launch<4>(lc, g, b, f, m, kind, lo, hi);
-}
-
-}  // namespace
-
-void launch_adj_corrections(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int m, bool vel,
-                            const int lo[3], const int hi[3])
-{
-    corr_dispatch(lc, g, b, f, m, vel ? kAV : kAP, lo, hi);
-}
-
-void launch_fwd_corrections(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int it, bool vel,
-                            const int lo[3], const int hi[3])
-{
-    corr_dispatch(lc, g, b, f, it, vel ? kFV : kFP, lo, hi);
-}
-
 void launch_inject_source(const LaunchCtx &lc, const Grid &g, const Batch &b, float *p,
                           const float *stf, int it, float scale)
 {
@@ -1808,16 +1060,15 @@ static dim3 band_grid(const Bands &bd, int nshot)
 }
 
 void launch_save_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, Bands bd, int it,
-                       unsigned *absmax_tmp)
+                       unsigned *absmax_tmp, bool have_max)
 {
     const dim3 grid = band_grid(bd, b.nshot);
-    if (bd.prec != SMI_PREC_F32) {
+    if (bd.prec != SMI_PREC_F32 && !have_max) {
         cudaMemsetAsync(absmax_tmp, 0, sizeof(unsigned) * 6 * b.nshot, S(lc));
         k_band_absmax<<<grid, kThreads, 0, S(lc)>>>(g, f, bd, absmax_tmp);
         ++*lc.launches;
     }
-    k_band_save<<<grid, kThreads, 0, S(lc)>>>(g, f, bd, it, absmax_tmp);
-    ++*lc.launches;
+    launch_pdl(lc, k_band_save, grid, kThreads, 0, g, f, bd, it, absmax_tmp);
 }
 
 void launch_restore_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, Bands bd, int it)
@@ -1934,7 +1185,7 @@ void launch_free_surface_fold_tile(const LaunchCtx &lc, const Grid &g, Fields A,
 {
     if (!g.freesurf) return;
     launch_free_surface(lc, g, A.p, nshot, kFsFoldP);
-    free_surface_rows(lc, g, A.psiv[1], (long long)g.S * g.ne[2], g.slab_n[1], nshot, kFsFoldP);
+    free_surface_rows(lc, g, A.psiv[1], (long long)g.xrows * g.ne[2], g.slab_n[1], nshot, kFsFoldP);
     if (g.ndim == 3) free_surface_rows(lc, g, A.psiv[2], (long long)g.ne[1] * g.S, g.slab_n[2], nshot, kFsFoldP);
 }
 

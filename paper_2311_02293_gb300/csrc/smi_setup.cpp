@@ -175,16 +175,21 @@ void set_layout(Grid &g, const int n[3])
     g.slab_n[0] = (long long)g.S * g.ne[1] * g.ne[2];
     g.slab_n[1] = (long long)g.ne[0] * g.S * g.ne[2];
     g.slab_n[2] = g.ndim == 3 ? (long long)g.px * g.ne[1] * g.S : 0;
-    g.zlo = g.zhi = g.zp = 0;
+    g.zlo = g.zhi = g.zp = g.xlo = g.xhi = g.xrows = 0;
 }
 
 void set_tile_slabs(Grid &g)
 {
     g.zlo = (g.nb + 3) & ~3;
     g.zhi = (g.ne[0] - g.nb - 1) & ~3;
+    if (g.zhi - g.zlo < 48) g.zlo = g.zhi = g.px;      // wider than the 40-node window of a tile, else one slab
+    g.xlo = g.nb;
+    g.xhi = g.ne[1] - g.nb - 1;
+    if (g.xhi - g.xlo < 48) g.xlo = g.xhi = g.ne[1];
     g.zp = g.zlo + g.px - g.zhi;
+    g.xrows = g.xlo + g.ne[1] - g.xhi;
     g.slab_n[0] = (long long)g.zp * g.ne[1] * g.ne[2];
-    g.slab_n[1] = (long long)g.px * g.S * g.ne[2];
+    g.slab_n[1] = (long long)g.px * g.xrows * g.ne[2];
     g.slab_n[2] = g.ndim == 3 ? (long long)g.px * g.ne[1] * g.S : 0;
 }
 

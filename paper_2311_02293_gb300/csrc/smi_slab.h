@@ -15,8 +15,10 @@
 //   z: [y][x][js], quads of four z nodes aligned to 16 bytes: the low slab's
 //      nodes 0 .. zlo-1 (zlo = nb rounded up to 4), then the nodes from zhi
 //      (first node of the high slab rounded down to 4) to the row's end;
-//   x: [y][js][z], rows of the field's pitch px, js = x or x - xhi + nb;
+//   x: [y][js][z], rows of the field's pitch px, js = x < xlo or xlo + x - xhi;
 //   y: [js][x][z], the same along y.
+// An axis so short that one tile's stencil window could meet both slabs is
+// stored whole (zlo = px, xlo = ne[1]: one slab).
 #pragma once
 
 #include "smi_internal.h"
@@ -34,9 +36,9 @@ __device__ __forceinline__ int zslab_quad(const Grid &g, int oz)
 // Index of node j inside the slab of axis a (1 or 2), or -1 outside.
 __device__ __forceinline__ int slab_row(const Grid &g, int a, int j)
 {
-    const int hi = g.ne[a] - g.nb - 1;
+    const int lo = a == 1 ? g.xlo : g.nb, hi = a == 1 ? g.xhi : g.ne[a] - g.nb - 1;
     if (j < 0 || j >= g.ne[a]) return -1;
-    return j < g.nb ? j : (j >= hi ? g.nb + j - hi : -1);
+    return j < lo ? j : (j >= hi ? lo + j - hi : -1);
 }
 __device__ __forceinline__ float slab_recur(float B, float m, float A, float x) { return B * m + A * x; }
 #endif

@@ -41,6 +41,7 @@
 
 #include <algorithm>
 
+#include "smi_band.h"
 #include "smi_box.h"
 #include "smi_internal.h"
 #include "smi_pdl.h"
@@ -148,7 +149,7 @@ __device__ __forceinline__ void add_source(const Batch &b, const SrcBox &sb, int
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t0 = oz + r - sb.f0;
-        if (t0 >= 0 && t0 < sb.n0) p[r] += amp * st.w[0][t0] * st.w[1][t1];
+        if (t0 >= 0 && t0 < sb.n0) p[r] += amp * st.w[0][t0] * st.w[1][t1] * st.w[2][0];
     }
 }
 
@@ -200,13 +201,6 @@ __device__ __forceinline__ void band_store(const Bands &bd, const float (&scale)
         }
     }
 }
-__device__ __forceinline__ float band_value(const Bands &bd, long long o, float scale)
-{
-    if (bd.prec == SMI_PREC_F32) return static_cast<const float *>(bd.data)[o];
-    if (bd.prec == SMI_PREC_F16) return __half2float(static_cast<const __half *>(bd.data)[o]) * scale;
-    return __bfloat162float(static_cast<const __nv_bfloat16 *>(bd.data)[o]) * scale;
-}
-
 // One velocity quad of axis A from the tile's pressure: v -= dt b D at the
 // nodes of the box, memory variable m of the v grid, and the operand R that
 // the pressure update differentiates (forward: v; adjoint: v + e).
@@ -791,9 +785,9 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
                 const int s0 = band_side<0>(bd, oz + r, ox), s1 = band_side<1>(bd, oz + r, ox);
                 const bool keep = kx && in_range(oz + r, plo[0], phi[0]);      // zero (and not stored) outside
                 if (s0 >= 0)
-                    vz[r] = keep ? band_value(bd, band_off<0>(bd, s, it, s0, oz + r, ox), s0 ? scale[1] : scale[0]) : 0.0f;
+                    vz[r] = keep ? band_load(bd, band_off<0>(bd, s, it, s0, oz + r, ox), s0 ? scale[1] : scale[0]) : 0.0f;
                 if (s1 >= 0)
-                    vx[r] = keep ? band_value(bd, band_off<1>(bd, s, it, s1, oz + r, ox), s1 ? scale[3] : scale[2]) : 0.0f;
+                    vx[r] = keep ? band_load(bd, band_off<1>(bd, s, it, s1, oz + r, ox), s1 ? scale[3] : scale[2]) : 0.0f;
             }
         }
         if (own) {

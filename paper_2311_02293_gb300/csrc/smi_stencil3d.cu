@@ -2,850 +2,924 @@
 //
 // Two kernels advance one half of a leap-frog step each (Sec. 2.1 update
 // equations): k3_v updates the three velocity components from p, k3_p
-// updates p from the velocities.  They run in two modes:
-//   FWD  the branch-free interior update, applied to every node of the box
-//        for both the forward scheme and the adjoint in "same solver" form;
-//        the CPML terms (forward, and transposed for the adjoint) are added
-//        by slab-only correction kernels (smi_kernels.cu);
+// updates p from the velocities.  Modes:
+//   FWD  forward step on the computing box of the source, with the CPML
+//        memory variables inline (Komatitsch & Martin) and the source;
+//   ADJ  the exact discrete adjoint in "same solver" form on the box of the
+//        receivers: the derivatives act on q + e, the operand of the
+//        transposed CPML terms (smi_slab.h);
 //   REC  source-field reconstruction backwards in time (Sec. 4.2) on the
 //        physical domain, with the imaging / gradient accumulation fused
 //        into the pressure kernel.
 //
 // Work decomposition: persistent CTAs (a fixed multiple of the SM count)
-// walk the work items of the computing box (Sec. 4.1, evaluated on the
-// device from the step counter): 32 (z) x 16 (x) column tiles times chunks
-// of y planes.  A CTA streams its chunk along y.  Plane tiles with their z/x
-// halos arrive by TMA (cp.async.bulk.tensor) into a ring of shared-memory
-// slots guarded by mbarriers; out-of-grid parts of a tile are filled with
-// zeros by the TMA unit, which is exactly the scheme's zero value outside
-// the extended grid.  y-neighbours are kept in a register queue.  Each
-// thread owns 4 consecutive z nodes of one x column: z-derivatives read a
-// 12-float window with three 128-bit shared loads, x-derivatives one 128-bit
-// load per tap.  Every mbarrier wait is bounded; a CTA that gives up sets
-// bit 0 of the error word, drains its own copies (bounded) and returns.
+// draw the work items of the computing box (Sec. 4.1, evaluated on the device
+// from the step counter; see Sched): 32 (z) x 16 (x) column tiles times
+// chunks of y planes.  A CTA streams its chunk along y; a thread owns 4 consecutive
+// z nodes of one x column.  Plane tiles arrive by TMA (cp.async.bulk.tensor;
+// zeros outside the grid are the scheme's values there), issued two planes
+// ahead as one group under one mbarrier:
+//   velocity kernel, plane y: p of plane y+N with its z / x halo (ring of
+//     N+2, since plane y's tile is needed N planes after it served the y
+//     queue), the v tiles of plane y, rho of plane y+1;
+//   pressure kernel, plane y: v_z and v_x with their halos, v_y of plane
+//     y+N-1, p, kappa (and lambda_p) of plane y;
+//   adjoint tiles that meet a z or x slab: e along z and x, halos included,
+//     from the slab arrays (the TMA zero fill outside a slab is e = 0 there).
+// y neighbours are kept in a register queue; z-derivatives read a 12-float
+// window with three 128-bit shared loads, x-derivatives one 128-bit load a
+// tap; multiplies and adds of the x and y derivatives run as packed pairs
+// (f32x2, same rounding).
+//
+// What bounds them: the velocity kernel moves 32 B a point and the pressure
+// kernel 24 (forward, adjoint) plus the halos that miss L2, so large boxes are
+// bound by HBM (about 80 % of the copy rate) and small ones by the latency of
+// a plane iteration.  Both ask for few instructions a point: box tests are
+// folded into per-thread coefficients (a node outside the box has 2 dt = 0),
+// ring positions are counted instead of divided, the last node's density is
+// repeated in memory, one wait and one barrier serve a plane, and the planes
+// without CPML terms run a body without them.  The loop body is not unrolled
+// over planes: both bodies twice cost instruction-cache misses (four times:
+// adjoint 0.88 of the rate).  The CPML terms ride on the tiles in flight
+// instead of in kernels of their own over the slabs, which re-read the fields
+// at half the bandwidth and took 26 % of a forward and 31 % of an adjoint step
+// at 340^3 (50 % at 130^3).  A step of both kernels, GB300, with those kernels
+// and now: 133 x 141 x 127, order 4, forward 77 -> 34 us; 200^3 extended,
+// order 4, box on, 500 steps, forward 107 -> 79 us, adjoint 171 -> 112,
+// reconstruction 67 -> 48; 340^3 extended, order 8, box on, first 600 steps,
+// adjoint 378 -> 297, forward with 16-bit boundary saving 258 -> 230.
+//
+// Every mbarrier wait is bounded; a CTA that gives up issues no more copies,
+// sets bit 0 of the error word, waits once more (bounded) for its copies in
+// flight and returns.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
-#include <type_traits>
 
+#include "smi_band.h"
 #include "smi_box.h"
 #include "smi_internal.h"
+#include "smi_pdl.h"
+#include "smi_slab.h"
 #include "smi_stencil3d.h"
 #include "smi_tile3d.h"
 
 namespace smi {
 namespace s3 {
 
+constexpr int CORE = TZ * TX;
+constexpr int AHEAD = 2;             // planes by which plain loads of a later plane are prefetched into L2
+// Plane groups in flight: two (42 - 53 KB of shared memory a CTA of the
+// velocity kernel, four CTAs a SM); three were within 1 % either way.
+constexpr int DEPTH = 2;
 
-// --- shared-memory slot layouts (floats) ---------------------------------
-// Haloed ring: slots resident while their plane feeds a derivative (N+1
-// planes for the velocity kernel, N for the pressure kernel) plus PFP planes
-// of lead.  Core ring: the pointwise 32 x 16 tiles of one plane, SC slots.
-#ifndef SMI_SC
-#define SMI_SC 3            // core-tile ring depth of the interior kernels
-#endif
-constexpr int PFP = SMI_PFP, SC = SMI_SC, CORE = TZ * TX;
-
-// Tile classes of a launch (template CLS): ALLT every tile column of the box
-// (z / x CPML terms then come from the band kernels), INT the interior
-// columns only, BND the CPML-band columns only, with the z / x CPML terms
-// applied inline from memory-variable tiles that arrive in the core ring
-// (BND core slots: two deep).
-enum { ALLT = 0, INT = 1, BND = 2 };
-
-// Band extras of the velocity kernel's core slot: the p-grid memory
-// variables (adjoint phi_z, phi_x) over the p tile's geometry, and the
-// v-grid ones (forward psi / adjoint chi, z and x) over the core tile.
-template <int N, int CLS = ALLT> struct VLay {
-    static constexpr int PR = TX + 2 * N - 1;            // p tile rows: x0-N+1 .. x0+TX-1+N
-    static constexpr int P_OFF = 0, P_SZ = rup32(ZW * PR);
-    static constexpr int R_OFF = P_SZ, R_SZ = rup32(36 * (TX + 1));   // rho: z0..z0+35, x0..x0+TX
-    static constexpr int SLOT = P_SZ + R_SZ;
-    static constexpr int S = N + 1 + PFP;
-    static constexpr unsigned BYTES = (unsigned)(ZW * PR + 36 * (TX + 1)) * 4u;
-    static constexpr int E_PZ = 3 * CORE, E_PX = E_PZ + P_SZ, E_CZ = E_PX + P_SZ, E_CX = E_CZ + CORE;
-    static constexpr int CSLOT = CLS == BND ? E_CX + CORE : 3 * CORE;   // vz, vx, vy (+ band extras)
-    static constexpr unsigned CBYTES = 3u * CORE * 4u;
-    static constexpr unsigned PBYTES = (unsigned)(ZW * PR) * 4u;        // one p-geometry memory tile
-    static constexpr int NC = CLS == BND ? 2 : SC;
-    static constexpr int SMEM = (S * SLOT + NC * CSLOT) * 4;
+// Shared layouts in floats (every tile starts at a multiple of 128 bytes).
+template <int N, int MODE> struct VLay {
+    static constexpr int PR = TX + 2 * N - 1, PB = ZW * PR, P = rup32(PB), S = N + DEPTH;   // p: x0-N+1 .., z0-4 ..
+    static constexpr int RB = 36 * (TX + 1), R = rup32(RB);                             // rho: x0 .. x0+TX, z0 .. z0+35
+    static constexpr int EZ = ZW * TX, EXB = TZ * PR, EX = rup32(EXB);                  // e_z, e_x on p nodes
+    static constexpr int oV = S * P, oR = oV + DEPTH * 3 * CORE, NR = DEPTH + 1, oE = oR + NR * R;
+    static constexpr int SMEM = (oE + (MODE == ADJ ? DEPTH * (EZ + EX) : 0)) * 4;
 };
-// Band extras of the pressure kernel's core slot: the v-grid memory
-// variables (adjoint chi_z, chi_x) over the v_z / v_x tile geometries, and
-// the p-grid ones (forward psi / adjoint phi, z and x) over the core tile.
-template <int N, int CLS = ALLT> struct PLay {
-    static constexpr int XR = TX + 2 * N - 1;            // vx tile rows: x0-N .. x0+TX-2+N
-    static constexpr int Z_OFF = 0, Z_SZ = rup32(ZW * TX);            // vz: z0-4.., x core
-    static constexpr int X_OFF = Z_SZ, X_SZ = rup32(TZ * XR);         // vx: z core
-    static constexpr int Y_OFF = Z_SZ + X_SZ, Y_SZ = CORE;            // vy: core
-    static constexpr int SLOT = Z_SZ + X_SZ + Y_SZ;
-    static constexpr int S = N + PFP;
-    static constexpr unsigned BYTES = (unsigned)(ZW * TX + TZ * XR + CORE) * 4u;
-    static constexpr int E_HZ = 3 * CORE, E_HX = E_HZ + Z_SZ, E_CZ = E_HX + X_SZ, E_CX = E_CZ + CORE;
-    static constexpr int CSLOT = CLS == BND ? E_CX + CORE : 3 * CORE;   // p, kappa, lambda_p (+ band extras)
-    static constexpr int NC = CLS == BND ? 2 : SC;
-    static constexpr int SMEM = (S * SLOT + NC * CSLOT) * 4;
+template <int N, int MODE> struct PLay {
+    static constexpr int Z = ZW * TX;                                  // v_z: z0-4 .., own x
+    static constexpr int XR = TX + 2 * N - 1, XB = TZ * XR, X = rup32(XB);   // v_x: own z, x0-N ..
+    static constexpr int oX = Z, oY = oX + X, oP = oY + CORE, oK = oP + CORE, oL = oK + CORE;
+    static constexpr int oEZ = oL + (MODE == REC ? CORE : 0), oEX = oEZ + (MODE == ADJ ? Z : 0);
+    static constexpr int G = oEX + (MODE == ADJ ? X : 0);              // one group
+    static constexpr int SMEM = DEPTH * G * 4;
 };
 
+// Quads of FP32 as two packed pairs (each lane rounds like a scalar
+// operation): half the instructions, and a 128-bit load is a quad as it is.
+typedef unsigned long long P2;
+__device__ __forceinline__ P2 pack(float a, float b)
+{
+    P2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack(P2 p, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p)); }
+__device__ __forceinline__ P2 add2(P2 a, P2 b)
+{
+    P2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ P2 sub2(P2 a, P2 b)
+{
+    P2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ P2 mul2(P2 a, P2 b)
+{
+    P2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ P2 fma2(P2 a, P2 b, P2 c)
+{
+    P2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+struct Q4 {
+    P2 a, b;
+};
+__device__ __forceinline__ Q4 ldq(const float *p)
+{
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+    return {t.x, t.y};
+}
+__device__ __forceinline__ void stq(float *p, const Q4 &q) { *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(q.a, q.b); }
+__device__ __forceinline__ Q4 quad(const float (&v)[4]) { return {pack(v[0], v[1]), pack(v[2], v[3])}; }
+__device__ __forceinline__ Q4 zeroq() { return {0ull, 0ull}; }
+__device__ __forceinline__ void split(const Q4 &q, float (&v)[4])
+{
+    unpack(q.a, v[0], v[1]);
+    unpack(q.b, v[2], v[3]);
+}
+__device__ __forceinline__ Q4 addq(const Q4 &x, const Q4 &y) { return {add2(x.a, y.a), add2(x.b, y.b)}; }
+__device__ __forceinline__ Q4 subq(const Q4 &x, const Q4 &y) { return {sub2(x.a, y.a), sub2(x.b, y.b)}; }
+__device__ __forceinline__ Q4 mulq(const Q4 &x, const Q4 &y) { return {mul2(x.a, y.a), mul2(x.b, y.b)}; }
+__device__ __forceinline__ Q4 fmaq(const Q4 &x, const Q4 &y, const Q4 &z) { return {fma2(x.a, y.a, z.a), fma2(x.b, y.b, z.b)}; }
+// D + c (x - y)
+__device__ __forceinline__ Q4 tap(const Q4 &D, float c, const Q4 &x, const Q4 &y)
+{
+    const P2 cc = pack(c, c);
+    return {fma2(cc, sub2(x.a, y.a), D.a), fma2(cc, sub2(x.b, y.b), D.b)};
+}
+// num / (r0 + r1): reciprocal (a few ulp, far below the FP32 scheme error)
+// and product; densities are normal numbers, so it is __fdividef without its
+// range scaling.
+__device__ __forceinline__ float rcpf(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ Q4 buoyq(const Q4 &num, const Q4 &r0, const Q4 &r1)
+{
+    float d[4];
+    split(addq(r0, r1), d);
+#pragma unroll
+    for (int r = 0; r < 4; r++) d[r] = rcpf(d[r]);
+    return mulq(num, quad(d));
+}
+// Brings a line that a later plane reads towards the L2 cache.
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// v - b D: the forward scheme rounds the product first (as it always has).
+template <int MODE> __device__ __forceinline__ Q4 update(const Q4 &v, const Q4 &b, const Q4 &D)
+{
+    return MODE == FWD ? subq(v, mulq(b, D)) : fmaq(b, D, v);
+}
+__device__ __forceinline__ void window(float (&W)[12], const float *row)
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        float v[4];
+        split(ldq(row + 4 * k), v);
+#pragma unroll
+        for (int r = 0; r < 4; r++) W[4 * k + r] = v[r];
+    }
+}
+// D along z of the middle quad of a window, p nodes to v nodes (UP) or back.
+template <int N, bool UP> __device__ __forceinline__ Q4 dz4(const Grid &g, const float (&W)[12])
+{
+    float D[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        float d = 0.f;
+#pragma unroll
+        for (int l = 1; l <= N; l++)
+            d += g.c[0][l - 1] * (UP ? W[4 + r + l] - W[4 + r - l + 1] : W[4 + r + l - 1] - W[4 + r - l]);
+        D[r] = d;
+    }
+    return quad(D);
+}
+
+// CPML coefficients (B, A) of a tile's own nodes along z and x, zero at nodes
+// outside the slabs, the grid or the box of this launch: a memory variable
+// there stays what it is, zero.
+struct alignas(16) Coefs {              // read as quads
+    float zB[TZ], zA[TZ], xB[TX], xA[TX];
+};
+__device__ __forceinline__ void load_coefs(Coefs &c, const float *B0, const float *A0, const float *B1, const float *A1,
+                                           const Item &it)
+{
+    for (int i = threadIdx.x; i < TZ + TX; i += NTHR) {
+        if (i < TZ) {
+            const int z = it.z0 + i;
+            const bool in = in_range(z, it.lo[0], it.hi[0]);
+            c.zB[i] = in ? B0[z] : 0.f;
+            c.zA[i] = in ? A0[z] : 0.f;
+        } else {
+            const int x = it.x0 + i - TZ;
+            const bool in = in_range(x, it.lo[1], it.hi[1]);
+            c.xB[i - TZ] = in ? B1[x] : 0.f;
+            c.xA[i - TZ] = in ? A1[x] : 0.f;
+        }
+    }
+}
+
+// A z slab (low, high) or x slab that the tile's stencil window reaches: its
+// tensor map and the offset of its coordinates, or none.  The slabs of a
+// short axis are one (smi_slab.h), so a window meets at most one.
+struct SlabTile {
+    const CUtensorMap *tm;
+    int c;
+};
+__device__ __forceinline__ SlabTile z_slab_tile(const Grid &g, const CUtensorMap *lo, const CUtensorMap *hi, int z0)
+{
+    if (z0 - 4 < g.zlo) return {lo, z0 - 4};
+    if (z0 + 36 > g.zhi) return {hi, z0 - 4 - g.zhi};
+    return {nullptr, 0};
+}
+__device__ __forceinline__ SlabTile x_slab_tile(const Grid &g, const CUtensorMap *lo, const CUtensorMap *hi, int xs,
+                                                int rows)
+{
+    if (xs < g.xlo) return {lo, xs};
+    if (xs + rows > g.xhi) return {hi, xs - g.xhi};
+    return {nullptr, 0};
+}
+
+// Per-thread position of an item.
+struct Own {
+    int oz, ox;
+    bool act;                  // the quad's column lies in the grid and in the box along x
+    int zq, xq;                // slab offsets of the own quad (-1: none)
+};
+__device__ __forceinline__ Own own_of(const Grid &g, const Item &it, int tzi, int txi)
+{
+    Own o;
+    o.oz = it.z0 + 4 * tzi;
+    o.ox = it.x0 + txi;
+    o.act = o.oz < g.ne[0] && in_range(o.ox, it.lo[1], it.hi[1]);
+    o.zq = o.act ? zslab_quad(g, o.oz) : -1;
+    o.xq = o.act ? slab_row(g, 1, o.ox) : -1;
+    return o;
+}
+// m <- B m + A x over the quad.
+__device__ __forceinline__ void recur4(const float (&B)[4], const float (&A)[4], float (&m)[4], const Q4 &x)
+{
+    float v[4];
+    split(x, v);
+#pragma unroll
+    for (int r = 0; r < 4; r++) m[r] = slab_recur(B[r], m[r], A[r], v[r]);
+}
+__device__ __forceinline__ void recur1(float B, float A, float (&m)[4], const Q4 &x)
+{
+    const float Bq[4] = {B, B, B, B}, Aq[4] = {A, A, A, A};
+    recur4(Bq, Aq, m, x);
+}
+// The forward scheme's z terms: which of the two products is rounded first
+// decides the last bit.  A x enters the multiply-add unrounded, except on x
+// lines whose group of four (from the low end of the launch's boxes) meets an
+// x slab, so that results stay the ones they have always been.
+__device__ __forceinline__ void recur4z(bool xgroup, const float (&B)[4], const float (&A)[4], float (&m)[4], const Q4 &x)
+{
+    float v[4];
+    split(x, v);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+        m[r] = xgroup ? __fmaf_rn(B[r], m[r], __fmul_rn(A[r], v[r])) : __fmaf_rn(A[r], v[r], __fmul_rn(B[r], m[r]));
+}
+__device__ __forceinline__ bool x_group(const Grid &g, int x, int x0)
+{
+    const int first = x0 + ((x - x0) & ~3), hi = g.ne[1] - g.nb - 1;
+    return first < g.nb || first + 3 >= hi;
+}
+// v - b m
+__device__ __forceinline__ Q4 sub_prod(const Q4 &v, const Q4 &b, const float (&m)[4])
+{
+    float x[4], c[4];
+    split(v, x);
+    split(b, c);
+#pragma unroll
+    for (int r = 0; r < 4; r++) x[r] = __fmaf_rn(-c[r], m[r], x[r]);
+    return quad(x);
+}
+// Zero where z.
+__device__ __forceinline__ Q4 clear_if(const Q4 &q, const bool (&z)[4])
+{
+    float x[4];
+    split(q, x);
+#pragma unroll
+    for (int r = 0; r < 4; r++) x[r] = z[r] ? 0.f : x[r];
+    return quad(x);
+}
+
+// How a launch cuts its boxes: planes a chunk, and the boxes' low end along x.
+struct Cut {
+    int chunk, x0;
+};
+
+// Maps of a launch, by the tile they bring.
+struct VMaps {
+    CUtensorMap p, rho, vz, vx, vy, ezl, ezh, exl, exh;
+};
+struct PMaps {
+    CUtensorMap vz, vx, vy, p, K, lp, ezl, ezh, exl, exh;
+};
 
 // ===========================================================================
-// Velocity kernel.  FWD/ADJ: v_a -= dt b_a D_a p (+ CPML terms); REC:
+// Velocity kernel.  FWD / ADJ: v_a -= dt b_a D_a (p with its CPML term); REC:
 // v_a += dt b_a D_a p on L_a+N-1..H_a-N, zero outside the previous box.
-template <int N, int MODE, int CLS>
-__global__ void __launch_bounds__(NTHR, CLS == BND ? 3 : SMI_MINB)
-k3_v(const __grid_constant__ CUtensorMap tm_p, const __grid_constant__ CUtensorMap tm_rho,
-     const __grid_constant__ CUtensorMap tm_vz, const __grid_constant__ CUtensorMap tm_vx,
-     const __grid_constant__ CUtensorMap tm_vy, const __grid_constant__ CUtensorMap tm_pzh,
-     const __grid_constant__ CUtensorMap tm_pxh, const __grid_constant__ CUtensorMap tm_cz,
-     const __grid_constant__ CUtensorMap tm_cx, Grid g, Batch b, Fields f, int step, unsigned *err)
+// Afterwards, by all CTAs: FWD the receivers' samples of p (step ga.it), ADJ
+// the band of the source field from the store (rs.it).
+template <int N, int MODE>
+__global__ void __launch_bounds__(NTHR, SMI_MINB)
+k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, Gather3 ga, Restore3 rs, unsigned *err,
+     unsigned *ctr)
 {
-    using Lay = VLay<N, CLS>;
-    constexpr int S = Lay::S;
-    constexpr int SC = Lay::NC;
+    using La = VLay<N, MODE>;
     extern __shared__ __align__(128) float sm[];
-    float *cbase = sm + S * Lay::SLOT;
-    __shared__ __align__(8) uint64_t bar[S], cbar[SC];
-    __shared__ FTabs tb;
+    float *sv = sm + La::oV, *sr = sm + La::oR, *se = sm + La::oE;
+    __shared__ __align__(8) uint64_t bar[DEPTH];
+    __shared__ Coefs co;
+    __shared__ int next[2];                   // the CTA's next item, in turn
     const int tid = threadIdx.x, tzi = tid & 7, txi = tid >> 3;
     if (tid == 0) {
-        for (int k = 0; k < S; k++) mbar_init(&bar[k], 1);
-        for (int k = 0; k < SC; k++) mbar_init(&cbar[k], 1);
+        for (int k = 0; k < DEPTH; k++) mbar_init(&bar[k], 1);
         mbar_fence_init();
     }
     __syncthreads();
-    unsigned parity = 0;
+    Sched sd;
+    sched_shot(g, b, MODE, step, 0, 0, lc.chunk, sd);   // (the box tables are older than the loop)
+    pdl_wait();
+    pdl_trigger();
+    unsigned phase = 0;                       // bit h: parity of the next completion of bar[h]
+    bool ok = true;
     const float dt = g.dt;
-#ifdef SMI_TIMING
-    long long t_wait = 0, t_sync = 0, t_all = clock64(), n_planes = 0;
-#endif
+    const int plane = g.px * g.ne[1];
 
     Item it;
-    for (long long w = blockIdx.x;
-         CLS == ALLT ? get_item(g, b, MODE, step, w, it) : get_citem(g, b, MODE, step, CLS == BND, w, it);
-         w += gridDim.x) {
+    for (int w = blockIdx.x, par = 0; sched_item(g, b, MODE, step, w, lc.chunk, sd, it); w = next[par], par ^= 1) {
         const int s = it.s, z0 = it.z0, x0 = it.x0, ya = it.ya, yb = it.yb;
-        const int ylast = yb + N;                 // last haloed plane needed
-        const bool zb = CLS == BND && band_z(g, z0), xb = CLS == BND && band_x(g, x0);
-        if (CLS == BND) load_tabs(g, z0, x0, tb);   // published by the barrier after the first waits
-        // band extras of a core slot: bytes and copies (adjoint: p-geometry phi tiles too)
-        const unsigned cbytes = Lay::CBYTES + (zb ? CORE * 4u + (MODE == ADJ ? Lay::PBYTES : 0u) : 0u) +
-                                (xb ? CORE * 4u + (MODE == ADJ ? Lay::PBYTES : 0u) : 0u);
-        auto issue_core = [&](int yy) {
-            const int k = (yy - ya) % SC;
-            float *cs = cbase + k * Lay::CSLOT;
-            mbar_expect(&cbar[k], cbytes);
-            tma4(cs, &tm_vz, z0, x0, yy, s, &cbar[k]);
-            tma4(cs + CORE, &tm_vx, z0, x0, yy, s, &cbar[k]);
-            tma4(cs + 2 * CORE, &tm_vy, z0, x0, yy, s, &cbar[k]);
-            if (CLS == BND) {
-                if (zb) {
-                    if (MODE == ADJ) tma4(cs + Lay::E_PZ, &tm_pzh, z0 - 4, x0 - N + 1, yy, s, &cbar[k]);
-                    tma4(cs + Lay::E_CZ, &tm_cz, z0, x0, yy, s, &cbar[k]);
-                }
-                if (xb) {
-                    if (MODE == ADJ) tma4(cs + Lay::E_PX, &tm_pxh, z0 - 4, x0 - N + 1, yy, s, &cbar[k]);
-                    tma4(cs + Lay::E_CX, &tm_cx, z0, x0, yy, s, &cbar[k]);
-                }
+        const Own me = own_of(g, it, tzi, txi);
+        const int oz = me.oz, ox = me.ox;
+        SlabTile ez{nullptr, 0}, ex{nullptr, 0};
+        unsigned gbytes = (unsigned)(La::PB + 3 * CORE + La::RB) * 4u;
+        if (MODE == ADJ) {
+            ez = z_slab_tile(g, &tm.ezl, &tm.ezh, z0);
+            ex = x_slab_tile(g, &tm.exl, &tm.exh, x0 - N + 1, La::PR);
+            gbytes += (ez.tm ? La::EZ * 4u : 0u) + (ex.tm ? La::EXB * 4u : 0u);
+        }
+        // group of plane y: p(y+N), v(y), rho(y+1), e(y); ph = group slot
+        auto issue = [&](int y, int ph, unsigned extra) {
+            uint64_t *br = &bar[ph];
+            mbar_expect(br, gbytes + extra);
+            tma4(sm + ((y + N - ya) % La::S) * La::P, &tm.p, z0 - 4, x0 - N + 1, y + N, s, br);
+            float *v = sv + ph * 3 * CORE;
+            tma4(v, &tm.vz, z0, x0, y, s, br);
+            tma4(v + CORE, &tm.vx, z0, x0, y, s, br);
+            tma4(v + 2 * CORE, &tm.vy, z0, x0, y, s, br);
+            tma4(sr + ((y + 1 - ya) % La::NR) * La::R, &tm.rho, z0, x0, y + 1, 0, br);
+            if (MODE == ADJ) {
+                float *e = se + ph * (La::EZ + La::EX);
+                if (ez.tm) tma4(e, ez.tm, ez.c, x0, y, s, br);
+                if (ex.tm) tma4(e + La::EZ, ex.tm, z0, ex.c, y, s, br);
             }
         };
-        const int oz = z0 + 4 * tzi, ox = x0 + txi;
-        const bool mem = oz < g.ne[0] && ox < g.ne[1];
+        if (tid == 0 && ok) {
+            issue(ya, 0, (unsigned)(N * La::PB + La::RB) * 4u);
+            for (int l = 0; l < N; l++) tma4(sm + l * La::P, &tm.p, z0 - 4, x0 - N + 1, ya + l, s, &bar[0]);
+            tma4(sr, &tm.rho, z0, x0, ya, 0, &bar[0]);
+            for (int d = 1; d < DEPTH && ya + d <= yb; d++) issue(ya + d, d, 0u);
+            next[par] = (int)(gridDim.x + atomicAdd(ctr, 1u));   // read after the item's last barrier
+        }
         const long long sh = (long long)s * g.ntot;
-        bool mz[4];
+        const unsigned col = (unsigned)(oz + g.px * ox);
+        const bool grid_ok = oz < g.ne[0] && ox < g.ne[1];
+        // y queue of own p: entry l = plane y-N+1+l; adjoint: p + e_y on the y-slab planes
+        Q4 q[2 * N];
 #pragma unroll
-        for (int r = 0; r < 4; r++) mz[r] = in_range(oz + r, it.lo[0], it.hi[0]);
-        const bool mx = in_range(ox, it.lo[1], it.hi[1]);
-        const int own = (txi + N - 1) * ZW + 4 * tzi + 4;   // own nodes in a p tile
-
-        // y queue of own p: entry l = plane y-N+1+l; planes before ya by plain loads
-        float q[2 * N][4];
-#pragma unroll
-        for (int l = 0; l < N - 1; l++) {
+        for (int l = 0; l < 2 * N - 1; l++) {
             const int y = ya - N + 1 + l;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (mem && y >= 0 && y < g.ne[2]) v = *reinterpret_cast<const float4 *>(f.p + sh + gidx(g, oz, ox, y));
-            put(q[l], v);
+            q[l] = grid_ok && y >= 0 && y < g.ne[2] ? ldq(f.p + sh + (col + (unsigned)(y * plane))) : zeroq();
         }
-        Ring hr{ya, min(ylast, ya + S - 1)}, cr{ya, min(yb, ya + SC - 1)};
-        if (tid == 0) {
-            for (int y = ya; y <= hr.issued; y++) {
-                const int k = (y - ya) % S;
-                float *slot = sm + k * Lay::SLOT;
-                mbar_expect(&bar[k], Lay::BYTES);
-                tma4(slot + Lay::P_OFF, &tm_p, z0 - 4, x0 - N + 1, y, s, &bar[k]);
-                tma4(slot + Lay::R_OFF, &tm_rho, z0, x0, y, 0, &bar[k]);
-            }
-            for (int y = ya; y <= cr.issued; y++) issue_core(y);
-        }
-        bool ok = true;
-#pragma unroll
-        for (int l = 0; l < N; l++) {
-            ok &= ring_wait(bar, S, 0, parity, hr, ya + l, ya);
-            put(q[N - 1 + l], lds4(sm + ((l) % S) * Lay::SLOT + Lay::P_OFF + own));
-        }
-        if (MODE == ADJ && mem && mx) {
-            // transposed y CPML: the queue holds lp + Ap_y (lp + phi_y) on y-slab planes
+        if (MODE == ADJ && me.act) {
 #pragma unroll
             for (int l = 0; l < 2 * N - 1; l++) {
-                const int yq = ya - N + 1 + l;
-                if (yq < 0 || yq >= g.ne[2] || !yslab(g, yq)) continue;
-                float ph[4];
-                put(ph, ldg4(f.psiv[2] + yslab_off(g, s, oz, ox, yq)));
-                const float A = g.cpa[2][yq];
-#pragma unroll
-                for (int r = 0; r < 4; r++) q[l][r] += A * (q[l][r] + ph[r]);
+                const int js = slab_row(g, 2, ya - N + 1 + l);
+                if (js >= 0) q[l] = addq(q[l], ldq(f.psiv[2] + s * g.slab_n[2] + (col + (unsigned)(js * plane))));
             }
         }
-        if (__syncthreads_or(!ok)) goto timeout;
-
+        // numerators of the buoyancy: 2 dt at the nodes a component updates, else 0 (adjoint and, along each
+        // component's own range, reconstruction: signed so that the update is one multiply-add)
+        Q4 mz, mx, mh;
+        bool zc[4], hc[4];                    // REC: updated nodes outside the previous box along z and x
+        bool clip = false;                    // REC: the tile has such nodes
         {
-        bool stop = false;
-        int y = ya;
-        auto body = [&](auto kc) {
-            constexpr int kq = decltype(kc)::value;
-#ifdef SMI_TIMING
-            const long long tw0 = clock64();
-#endif
-            // y CPML operands, loaded before the waits: FWD psi_y, ADJ chi_y
-            // of plane y; ADJ phi_y of the plane entering the queue
-            const bool my = in_range(y, it.lo[2], it.hi[2]);
-            const bool ysl = MODE != REC && mem && mx && my && yslab(g, y);
-            const int ye = y + N;
-            const bool yent = MODE == ADJ && mem && mx && ye < g.ne[2] && yslab(g, ye);
-            float ym[4] = {0.f, 0.f, 0.f, 0.f}, yp[4] = {0.f, 0.f, 0.f, 0.f};
-            if (ysl) put(ym, ldg4(f.psip[2] + yslab_off(g, s, oz, ox, y)));
-            if (yent) put(yp, ldg4(f.psiv[2] + yslab_off(g, s, oz, ox, ye)));
-            ok = ring_wait(bar, S, 0, parity, hr, y + N, ya);
-            ok &= ring_wait(cbar, SC, 16, parity, cr, y, ya);
-#ifdef SMI_TIMING
-            t_wait += clock64() - tw0;
-#endif
-            const float *pt = sm + ((y - ya) % S) * Lay::SLOT;
-            const float *rt = pt + Lay::R_OFF;
-            const float *rt1 = sm + ((y + 1 - ya) % S) * Lay::SLOT + Lay::R_OFF;
-            put(q[((2 * N - 1) + kq) % (2 * N)], lds4(sm + ((y + N - ya) % S) * Lay::SLOT + Lay::P_OFF + own));
-            const float *cslot = cbase + ((y - ya) % SC) * Lay::CSLOT;   // this plane's core slot
-            const float *cs = cslot + txi * TZ + 4 * tzi;
-            bool keep[4];
-            if (MODE == REC) {
-                const bool kxy = in_range(ox, it.plo[1], it.phi[1]) && in_range(y, it.plo[2], it.phi[2]);
+            const bool rx = MODE != REC || in_range(ox, g.L[1] + N - 1, g.H[1] - N);
+            const float two = MODE == ADJ ? -2.0f * dt : 2.0f * dt;
+            float a[4], c[4], h4[4];
 #pragma unroll
-                for (int r = 0; r < 4; r++) keep[r] = kxy && in_range(oz + r, it.plo[0], it.phi[0]);
+            for (int r = 0; r < 4; r++) {
+                const bool in = me.act && in_range(oz + r, it.lo[0], it.hi[0]);
+                const bool rz = MODE != REC || in_range(oz + r, g.L[0] + N - 1, g.H[0] - N);
+                a[r] = in && rz ? two : 0.f;
+                c[r] = in && rx ? two : 0.f;
+                h4[r] = in ? two : 0.f;
+                const bool out = MODE == REC && in &&
+                                 !(in_range(oz + r, it.plo[0], it.phi[0]) && in_range(ox, it.plo[1], it.phi[1]));
+                hc[r] = out;
+                zc[r] = out && rz;
+                clip = clip || out;
             }
-            const bool act = mem && mx && my;
-            float rho0[4];
-            put(rho0, lds4(rt + txi * 36 + 4 * tzi));
-            float4 nzv, nxv, nyv;
+            mz = quad(a);
+            mx = quad(c);
+            mh = quad(h4);
+        }
+        const bool rxn = MODE == REC && in_range(ox, g.L[1] + N - 1, g.H[1] - N);
+        if (MODE == REC) clip = __syncthreads_or(clip);
+        if (MODE != REC) {
+            load_coefs(co, g.cvb[0], g.cva[0], g.cvb[1], g.cva[1], it);
+            __syncthreads();
+        }
+        // CPML planes of the item: every plane of a tile that meets a z or x slab, the y-slab planes of the others
+        const bool zxb = MODE != REC && (z_slab_tile(g, &tm.p, &tm.p, z0).tm || x_slab_tile(g, &tm.p, &tm.p, x0 - N + 1, La::PR).tm);
+        const bool xg = MODE == FWD && x_group(g, ox, lc.x0);
+        const bool lastz = oz + 4 >= g.px;
+        const int rxrow = ox + 1 < g.ne[1] ? txi + 1 : txi;        // the last node's neighbour is itself
+        float *const mzp = f.psip[0] + (s * g.slab_n[0] + me.zq + (long long)g.zp * ox);
+        float *const mxp = f.psip[1] + (s * g.slab_n[1] + oz + (long long)g.px * me.xq);
+        const unsigned zpl = (unsigned)(g.zp * g.ne[1]), xpl = (unsigned)(g.px * g.xrows);
+        int h = 0, kp = 0, kq = N % La::S, kr = 0;   // group, ring slots of p(y), p(y+N), rho(y)
 
-            // ---- z component ----
-            {
-                float W[12];
-                {
-                    const float *row = pt + Lay::P_OFF + (txi + N - 1) * ZW + 4 * tzi;
-                    float4 a0 = lds4(row), a1 = lds4(row + 4), a2 = lds4(row + 8);
-                    W[0] = a0.x; W[1] = a0.y; W[2] = a0.z; W[3] = a0.w;
-                    W[4] = a1.x; W[5] = a1.y; W[6] = a1.z; W[7] = a1.w;
-                    W[8] = a2.x; W[9] = a2.y; W[10] = a2.z; W[11] = a2.w;
+        // one plane; BAND: with the CPML terms (REC: with nodes outside the previous box)
+        auto body = [&](auto kc, auto bc, int y) {
+            constexpr int K = decltype(kc)::value;
+            constexpr bool BAND = decltype(bc)::value;
+            const int ys = BAND && MODE != REC ? slab_row(g, 2, y) : -1;
+            const int ye = BAND && MODE == ADJ ? slab_row(g, 2, y + N) : -1;
+            float ym[4], mzv[4], mxv[4];
+            Q4 yp;
+            if (BAND && MODE != REC) {
+                if (ys >= 0 && me.act) put(ym, ldg4(f.psip[2] + s * g.slab_n[2] + (col + (unsigned)(ys * plane))));
+                if (ye >= 0 && me.act) yp = ldq(f.psiv[2] + s * g.slab_n[2] + (col + (unsigned)(ye * plane)));
+                if (me.xq >= 0) put(mxv, ldg4(mxp + (unsigned)y * xpl));
+                if (me.zq >= 0) put(mzv, ldg4(mzp + (unsigned)y * zpl));
+                if (y + AHEAD <= yb) {
+                    if (me.xq >= 0) prefetch_l2(mxp + (unsigned)(y + AHEAD) * xpl);
+                    if (me.zq >= 0) prefetch_l2(mzp + (unsigned)(y + AHEAD) * zpl);
                 }
-                if (MODE == ADJ && CLS == BND && zb && (oz - 4 < g.nb || oz + 7 >= g.ne[0] - g.nb - 1)) {
-                    // transposed CPML operand over the window: lp + Ap (lp + phi) (Ap = 0 off the slab)
-                    const float *ph = cslot + Lay::E_PZ + (txi + N - 1) * ZW + 4 * tzi;
+            }
+            ok = ok && mbar_wait(&bar[h], (phase >> h) & 1u);
+            phase ^= 1u << h;
+            const float *pt = sm + kp * La::P + (txi + N - 1) * ZW + 4 * tzi;      // window of the own quad
+            const int kr1 = kr == La::NR - 1 ? 0 : kr + 1;
+            const float *rt = sr + kr * La::R + 4 * tzi;
+            const float *cs = sv + h * 3 * CORE + txi * TZ + 4 * tzi;
+            Q4 &qn = q[(2 * N - 1 + K) % (2 * N)];
+            qn = ldq(sm + kq * La::P + (txi + N - 1) * ZW + 4 * tzi + 4);
+            if (BAND && ye >= 0 && me.act) qn = addq(qn, yp);
+            const Q4 r0 = ldq(rt + txi * 36);
+            const unsigned o = col + (unsigned)(y * plane);
+            const bool ky = !(BAND && MODE == REC) || in_range(y, it.plo[2], it.phi[2]);
+
+            // ---- y component ----
+            if (MODE != REC || in_range(y, g.L[2] + N - 1, g.H[2] - N)) {
+                Q4 D = zeroq();
 #pragma unroll
-                    for (int i = 0; i < 12; i++) W[i] += tb.z[0][oz - z0 + 4 + i] * (W[i] + ph[i]);
-                }
-                const float r4 = rt[txi * 36 + 4 * tzi + 4];
-                const float rz[5] = {rho0[0], rho0[1], rho0[2], rho0[3], r4};
-                float v[4];
-                put(v, lds4(cs));
-                float D[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int l = 1; l <= N; l++) d += g.c[0][l - 1] * (W[4 + r + l] - W[4 + r - l + 1]);
-                    D[r] = d;
-                }
-                if (CLS == BND && zb && zquad_slab(g, oz) && act) {
-                    // z memory variable at the quad's slab nodes: forward psi <- Bv psi + Av D (added to D);
-                    // adjoint chi <- Bv (chi + lv before this step)
-                    float mz4[4];
-                    put(mz4, lds4(cs + Lay::E_CZ));
+                for (int l = 1; l <= N; l++) D = tap(D, g.c[2][l - 1], q[(N - 1 + l + K) % (2 * N)], q[(N - l + K) % (2 * N)]);
+                const Q4 r1 = ldq((y + 1 < g.ne[2] ? sr + kr1 * La::R : sr + kr * La::R) + txi * 36 + 4 * tzi);
+                const Q4 bb = buoyq(mh, r0, r1);
+                Q4 v = ldq(cs + 2 * CORE);
+                if (BAND && MODE != REC && ys >= 0 && me.act) {
+                    float B[4], A[4], m[4];
+                    split(mh, m);
 #pragma unroll
                     for (int r = 0; r < 4; r++) {
-                        const int t = oz - z0 + 8 + r;
-                        if (!(mz[r] && slab_at(g, 0, oz + r))) continue;
-                        if (MODE == FWD) {
-                            mz4[r] = tb.z[3][t] * mz4[r] + tb.z[2][t] * D[r];
-                            D[r] += mz4[r];
-                        } else {
-                            mz4[r] = tb.z[3][t] * (mz4[r] + v[r]);
-                        }
+                        B[r] = g.cvb[2][y];
+                        A[r] = m[r] != 0.f ? g.cva[2][y] : 0.f;
                     }
-                    stg4(f.psip[0] + sh + gidx(g, oz, ox, y), mz4);
+                    if (MODE == FWD) {
+                        recur4(B, A, ym, D);
+                        D = addq(D, quad(ym));
+                    }
+                    v = update<MODE>(v, bb, D);
+                    if (MODE == ADJ) recur4(B, A, ym, v);
+                    stg4(f.psip[2] + s * g.slab_n[2] + (col + (unsigned)(ys * plane)), ym);
+                } else {
+                    v = update<MODE>(v, bb, D);
                 }
-                float nv[4];
+                if (BAND && MODE == REC) {
+                    float m[4];
+                    bool cl[4];
+                    split(mh, m);
 #pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    const float bz = buoy(rz[r], rz[r + 1], oz + r + 1 >= g.ne[0]);
-                    if (MODE == REC) {
-                        const bool rr = mz[r] && in_range(oz + r, g.L[0] + N - 1, g.H[0] - N);
-                        nv[r] = rr ? (keep[r] ? v[r] + dt * bz * D[r] : 0.f) : v[r];
-                    } else {
-                        nv[r] = mz[r] ? v[r] - dt * bz * D[r] : v[r];
-                    }
+                    for (int r = 0; r < 4; r++) cl[r] = hc[r] || (!ky && m[r] != 0.f);
+                    v = clear_if(v, cl);
                 }
-                nzv = make_float4(nv[0], nv[1], nv[2], nv[3]);
+                if (me.act) stq(f.v[2] + sh + o, v);
             }
+            float W[12];
+            window(W, pt);
             // ---- x component ----
             {
-                float Xr[2 * N][4];
+                Q4 D = zeroq();
+                const float *er = se + h * (La::EZ + La::EX) + La::EZ + (txi + N - 1) * TZ + 4 * tzi;
 #pragma unroll
                 for (int l = 1; l <= N; l++) {
-                    put(Xr[N - 1 + l], lds4(pt + Lay::P_OFF + (txi + N - 1 + l) * ZW + 4 * tzi + 4));
-                    put(Xr[N - l], lds4(pt + Lay::P_OFF + (txi + N - l) * ZW + 4 * tzi + 4));
-                }
-                if (MODE == ADJ && CLS == BND && xb) {
-                    // transposed CPML operand at the taps x - N + 1 + t (Ap = 0 off the slab)
-#pragma unroll
-                    for (int t = 0; t < 2 * N; t++) {
-                        const float A = tb.x[0][txi + t - N + 1 + 8];
-                        if (A != 0.f) {
-                            float ph[4];
-                            put(ph, lds4(cslot + Lay::E_PX + (txi + t) * ZW + 4 * tzi + 4));
-#pragma unroll
-                            for (int r = 0; r < 4; r++) Xr[t][r] += A * (Xr[t][r] + ph[r]);
-                        }
+                    Q4 a = ldq(pt + 4 + l * ZW);
+                    Q4 c = l == 1 ? quad({W[4], W[5], W[6], W[7]}) : ldq(pt + 4 - (l - 1) * ZW);
+                    if (BAND && MODE == ADJ && ex.tm) {
+                        a = addq(a, ldq(er + l * TZ));
+                        c = addq(c, ldq(er - (l - 1) * TZ));
                     }
+                    D = tap(D, g.c[1][l - 1], a, c);
                 }
-                float rx[4], v[4];
-                put(rx, lds4(rt + (txi + 1) * 36 + 4 * tzi));
-                put(v, lds4(cs + CORE));
-                float D[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int l = 1; l <= N; l++) d += g.c[1][l - 1] * (Xr[N - 1 + l][r] - Xr[N - l][r]);
-                    D[r] = d;
+                const Q4 bb = buoyq(mx, r0, ldq(rt + rxrow * 36));
+                Q4 v = update<MODE>(ldq(cs + CORE), bb, D);
+                if (BAND && MODE != REC && me.xq >= 0) {
+                    recur1(co.xB[txi], co.xA[txi], mxv, MODE == FWD ? D : v);
+                    if (MODE == FWD) v = sub_prod(v, bb, mxv);
+                    stg4(mxp + (unsigned)y * xpl, mxv);
                 }
-                if (CLS == BND && xb && ox < g.ne[1] && slab_at(g, 1, ox) && act) {
-                    float mx4[4];
-                    put(mx4, lds4(cs + Lay::E_CX));
-                    const int t = txi + 8;
+                if (BAND && MODE == REC && rxn) {
+                    float m[4];
+                    bool cl[4];
+                    split(mh, m);
 #pragma unroll
-                    for (int r = 0; r < 4; r++) {
-                        if (!mz[r]) continue;
-                        if (MODE == FWD) {
-                            mx4[r] = tb.x[3][t] * mx4[r] + tb.x[2][t] * D[r];
-                            D[r] += mx4[r];
-                        } else {
-                            mx4[r] = tb.x[3][t] * (mx4[r] + v[r]);
-                        }
-                    }
-                    stg4(f.psip[1] + sh + gidx(g, oz, ox, y), mx4);
+                    for (int r = 0; r < 4; r++) cl[r] = hc[r] || (!ky && m[r] != 0.f);
+                    v = clear_if(v, cl);
                 }
-                const bool lastx = ox + 1 >= g.ne[1];
-                const bool rxm = MODE == REC && in_range(ox, g.L[1] + N - 1, g.H[1] - N);
-                float nv[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    const float bx = buoy(rho0[r], rx[r], lastx);
-                    if (MODE == REC) nv[r] = (mz[r] && rxm) ? (keep[r] ? v[r] + dt * bx * D[r] : 0.f) : v[r];
-                    else nv[r] = mz[r] ? v[r] - dt * bx * D[r] : v[r];
-                }
-                nxv = make_float4(nv[0], nv[1], nv[2], nv[3]);
+                if (me.act) stq(f.v[1] + sh + o, v);
             }
-            // ---- y component ----
+            // ---- z component ----
             {
-                if (yent) {                       // entering plane: lp + Ap_y (lp + phi_y)
-                    const float A = g.cpa[2][ye];
+                if (BAND && MODE == ADJ && ez.tm) {
+                    float E[12];
+                    window(E, se + h * (La::EZ + La::EX) + txi * ZW + 4 * tzi);
 #pragma unroll
-                    for (int r = 0; r < 4; r++) {
-                        float &e = q[((2 * N - 1) + kq) % (2 * N)][r];
-                        e += A * (e + yp[r]);
-                    }
+                    for (int i = 0; i < 12; i++) W[i] += E[i];
                 }
-                float ry[4], v[4];
-                put(ry, lds4(rt1 + txi * 36 + 4 * tzi));
-                put(v, lds4(cs + 2 * CORE));
-                float D[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int l = 1; l <= N; l++) d += g.c[2][l - 1] * (q[((N - 1 + l) + kq) % (2 * N)][r] - q[((N - l) + kq) % (2 * N)][r]);
-                    D[r] = d;
+                const Q4 D = dz4<N, true>(g, W);
+                float ra[4];
+                split(r0, ra);
+                const Q4 r1 = quad({ra[1], ra[2], ra[3], lastz ? ra[3] : rt[txi * 36 + 4]});
+                const Q4 bb = buoyq(mz, r0, r1);
+                Q4 v = update<MODE>(ldq(cs), bb, D);
+                if (BAND && MODE != REC && me.zq >= 0) {
+                    float B[4], A[4];
+                    put(B, lds4(co.zB + 4 * tzi));
+                    put(A, lds4(co.zA + 4 * tzi));
+                    if (MODE == FWD) recur4z(xg, B, A, mzv, D);
+                    else recur4(B, A, mzv, v);
+                    if (MODE == FWD) v = sub_prod(v, bb, mzv);
+                    stg4(mzp + (unsigned)y * zpl, mzv);
                 }
-                if (ysl) {
-                    const long long yo = yslab_off(g, s, oz, ox, y);
-                    if (MODE == FWD) {            // psi_y <- Bv psi_y + Av D_y p;  v_y -= dt b (D_y p + psi_y)
-                        const float B = g.cvb[2][y], A = g.cva[2][y];
+                if (BAND && MODE == REC) {
+                    float m[4];
+                    bool cl[4];
+                    split(mz, m);
 #pragma unroll
-                        for (int r = 0; r < 4; r++) {
-                            const float ps = B * ym[r] + A * D[r];
-                            if (mz[r]) {
-                                ym[r] = ps;
-                                D[r] += ps;
-                            }
-                        }
-                    } else {                      // deferred chi_y <- Bv (chi_y + lv_y), lv_y before this step
-                        const float B = g.cvb[2][y];
-#pragma unroll
-                        for (int r = 0; r < 4; r++)
-                            if (mz[r]) ym[r] = B * (ym[r] + v[r]);
-                    }
-                    stg4(f.psip[2] + yo, ym);
+                    for (int r = 0; r < 4; r++) cl[r] = zc[r] || (!ky && m[r] != 0.f);
+                    v = clear_if(v, cl);
                 }
-                const bool lasty = y + 1 >= g.ne[2];
-                const bool rym = MODE == REC && in_range(y, g.L[2] + N - 1, g.H[2] - N);
-                float nv[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    const float by = buoy(rho0[r], ry[r], lasty);
-                    if (MODE == REC) nv[r] = (mz[r] && rym) ? (keep[r] ? v[r] + dt * by * D[r] : 0.f) : v[r];
-                    else nv[r] = mz[r] ? v[r] - dt * by * D[r] : v[r];
-                }
-                nyv = make_float4(nv[0], nv[1], nv[2], nv[3]);
+                if (me.act) stq(f.v[0] + sh + o, v);
             }
-            if (act) {
-                const long long base = sh + gidx(g, oz, ox, y);
-                *reinterpret_cast<float4 *>(f.v[0] + base) = nzv;
-                *reinterpret_cast<float4 *>(f.v[1] + base) = nxv;
-                *reinterpret_cast<float4 *>(f.v[2] + base) = nyv;
-            }
-            // all reads of plane y's slots are done; refill them
-#ifdef SMI_TIMING
-            const long long ts0 = clock64();
-            n_planes++;
-#endif
-            if (__syncthreads_or(!ok)) {
-                stop = true;
-                return;
-            }
-#ifdef SMI_TIMING
-            t_sync += clock64() - ts0;
-#endif
-            if (tid == 0) {
-                if (hr.issued < ylast) {
-                    const int yn = hr.issued + 1;
-                    const int k = (yn - ya) % S;
-                    float *slot = sm + k * Lay::SLOT;
-                    mbar_expect(&bar[k], Lay::BYTES);
-                    tma4(slot + Lay::P_OFF, &tm_p, z0 - 4, x0 - N + 1, yn, s, &bar[k]);
-                    tma4(slot + Lay::R_OFF, &tm_rho, z0, x0, yn, 0, &bar[k]);
-                }
-                if (cr.issued < yb) issue_core(cr.issued + 1);
-            }
-            if (hr.issued < ylast) hr.issued++;
-            if (cr.issued < yb) cr.issued++;
+            kp = kp + 1 == La::S ? 0 : kp + 1;
+            kq = kq + 1 == La::S ? 0 : kq + 1;
+            kr = kr1;
+            __syncthreads();                  // every read of plane y's tiles is done
+            if (tid == 0 && ok && y + DEPTH <= yb) issue(y + DEPTH, h, 0u);
+            h = h + 1 == DEPTH ? 0 : h + 1;
+        };
+        auto one = [&](auto kc, int y) {
+            const bool band = MODE == REC ? clip || !in_range(y, it.plo[2], it.phi[2])
+                                          : zxb || yslab(g, y) || (MODE == ADJ && yslab(g, y + N));
+            if (band) body(kc, std::true_type{}, y);
+            else body(kc, std::false_type{}, y);
         };
         constexpr int G = (2 * N) % SMI_YUNROLL == 0 ? SMI_YUNROLL : 2 * N;
-        while (y <= yb && !stop) {
-            Unroll<0, G>::run(body, y, yb, stop);
+        for (int y = ya; y <= yb; y += G) {
+            unroll_planes<G>(one, y, yb);
             rotate_queue<G>(q);
         }
-        if (stop) goto timeout;
-        }
-        continue;
-    timeout:
+        if (__syncthreads_or(!ok)) break;
+    }
+    if (__syncthreads_or(!ok)) {
         if (tid == 0) atomicOr(err, 1u);
-        ring_drain(bar, S, 0, parity, hr, ya);
-        ring_drain(cbar, SC, 16, parity, cr, ya);
+        for (int k = 0; k < DEPTH; k++) mbar_wait(&bar[k], (phase >> k) & 1u);
         return;
     }
-#ifdef SMI_TIMING
-    if (threadIdx.x == 0 && (blockIdx.x % 97) == 0 && n_planes > 0)
-        printf("T%d blk %d planes %lld all %lld wait %lld (%.0f%%) sync %lld (%.0f%%)\n", MODE, blockIdx.x, n_planes,
-               clock64() - t_all, t_wait, 100.0 * t_wait / (clock64() - t_all), t_sync, 100.0 * t_sync / (clock64() - t_all));
-#endif
+    if (MODE == FWD && ga.it >= 0) gather_tail(g, b, f.p, ga);
+    if (MODE == ADJ && rs.it >= 0) restore_tail(g, b.nshot, rs);
 }
 
 // ===========================================================================
-// Pressure kernel.  FWD/ADJ: p -= dt kappa sum_a D_a v_a (+ CPML terms);
-// REC: acc += lp * (div v | p), p += dt kappa div v - source, zero outside the
-// previous box, on the physical domain.
-template <int N, int MODE, int CLS>
-__global__ void __launch_bounds__(NTHR, CLS == BND ? 3 : SMI_MINB)
-k3_p(const __grid_constant__ CUtensorMap tm_vz, const __grid_constant__ CUtensorMap tm_vx,
-     const __grid_constant__ CUtensorMap tm_vy, const __grid_constant__ CUtensorMap tm_pc,
-     const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_lp,
-     const __grid_constant__ CUtensorMap tm_czh, const __grid_constant__ CUtensorMap tm_cxh,
-     const __grid_constant__ CUtensorMap tm_pzc, const __grid_constant__ CUtensorMap tm_pxc, Grid g, Batch b,
-     Fields f, int step, unsigned *err, float *acc, int img_mode, const float *stf, float src_scale)
+// Pressure kernel.  FWD / ADJ: p -= dt kappa sum_a D_a (v_a with its CPML
+// term), FWD with the source; REC: acc += lp * (div v | p), p += dt kappa div v
+// - source, zero outside the previous box, on the physical domain.
+// Afterwards FWD, by all CTAs: the next stored boundary (or its largest
+// magnitudes, 16-bit storage), from the velocities this kernel only reads.
+template <int N, int MODE>
+__global__ void __launch_bounds__(NTHR, SMI_MINB)
+k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, unsigned *err, float *acc, int img_mode,
+     const float *stf, float src_scale, Save3 sv, unsigned *ctr)
 {
-    using Lay = PLay<N, CLS>;
-    constexpr int S = Lay::S;
-    constexpr int SC = Lay::NC;
-    constexpr unsigned CBYTES = (MODE == REC ? 3u : 2u) * CORE * 4u;
+    using La = PLay<N, MODE>;
     extern __shared__ __align__(128) float sm[];
-    float *cbase = sm + S * Lay::SLOT;
-    __shared__ __align__(8) uint64_t bar[S], cbar[SC];
-    __shared__ FTabs tb;
+    __shared__ __align__(8) uint64_t bar[DEPTH];
+    __shared__ Coefs co;
+    __shared__ int next[2];                   // the CTA's next item, in turn
     const int tid = threadIdx.x, tzi = tid & 7, txi = tid >> 3;
     if (tid == 0) {
-        for (int k = 0; k < S; k++) mbar_init(&bar[k], 1);
-        for (int k = 0; k < SC; k++) mbar_init(&cbar[k], 1);
+        for (int k = 0; k < DEPTH; k++) mbar_init(&bar[k], 1);
         mbar_fence_init();
     }
     __syncthreads();
-    unsigned parity = 0;
+    Sched sd;
+    sched_shot(g, b, MODE, step, 0, 0, lc.chunk, sd);   // (the box tables are older than the loop)
+    pdl_wait();
+    pdl_trigger();
+    unsigned phase = 0;
+    bool ok = true;
     const float dt = g.dt;
-#ifdef SMI_TIMING
-    long long t_wait = 0, t_sync = 0, t_all = clock64(), n_planes = 0;
-#endif
+    const int plane = g.px * g.ne[1];
 
     Item it;
-    for (long long w = blockIdx.x;
-         CLS == ALLT ? get_item(g, b, MODE, step, w, it) : get_citem(g, b, MODE, step, CLS == BND, w, it);
-         w += gridDim.x) {
+    for (int w = blockIdx.x, par = 0; sched_item(g, b, MODE, step, w, lc.chunk, sd, it); w = next[par], par ^= 1) {
         const int s = it.s, z0 = it.z0, x0 = it.x0, ya = it.ya, yb = it.yb;
-        const int ylast = yb + N - 1;
-        const bool zb = CLS == BND && band_z(g, z0), xb = CLS == BND && band_x(g, x0);
-        if (CLS == BND) load_tabs(g, z0, x0, tb);   // published by the barrier after the first waits
-        // band extras of a core slot (adjoint: the chi tiles in the v_z / v_x geometries too)
-        const unsigned cbytes = CBYTES + (zb ? CORE * 4u + (MODE == ADJ ? ZW * TX * 4u : 0u) : 0u) +
-                                (xb ? CORE * 4u + (MODE == ADJ ? TZ * Lay::XR * 4u : 0u) : 0u);
-        auto issue_core = [&](int yy) {
-            const int k = (yy - ya) % SC;
-            float *cs = cbase + k * Lay::CSLOT;
-            mbar_expect(&cbar[k], cbytes);
-            tma4(cs, &tm_pc, z0, x0, yy, s, &cbar[k]);
-            tma4(cs + CORE, &tm_K, z0, x0, yy, 0, &cbar[k]);
-            if (MODE == REC) tma4(cs + 2 * CORE, &tm_lp, z0, x0, yy, s, &cbar[k]);
-            if (CLS == BND) {
-                if (zb) {
-                    if (MODE == ADJ) tma4(cs + Lay::E_HZ, &tm_czh, z0 - 4, x0, yy, s, &cbar[k]);
-                    tma4(cs + Lay::E_CZ, &tm_pzc, z0, x0, yy, s, &cbar[k]);
-                }
-                if (xb) {
-                    if (MODE == ADJ) tma4(cs + Lay::E_HX, &tm_cxh, z0, x0 - N, yy, s, &cbar[k]);
-                    tma4(cs + Lay::E_CX, &tm_pxc, z0, x0, yy, s, &cbar[k]);
-                }
+        const Own me = own_of(g, it, tzi, txi);
+        const int oz = me.oz, ox = me.ox;
+        SlabTile ez{nullptr, 0}, ex{nullptr, 0};
+        unsigned gbytes = (unsigned)(La::Z + La::XB + (MODE == REC ? 4 : 3) * CORE) * 4u;
+        if (MODE == ADJ) {
+            ez = z_slab_tile(g, &tm.ezl, &tm.ezh, z0);
+            ex = x_slab_tile(g, &tm.exl, &tm.exh, x0 - N, La::XR);
+            gbytes += (ez.tm ? La::Z * 4u : 0u) + (ex.tm ? La::XB * 4u : 0u);
+        }
+        auto issue = [&](int y, int ph) {
+            uint64_t *br = &bar[ph];
+            float *t = sm + ph * La::G;
+            mbar_expect(br, gbytes);
+            tma4(t, &tm.vz, z0 - 4, x0, y, s, br);
+            tma4(t + La::oX, &tm.vx, z0, x0 - N, y, s, br);
+            tma4(t + La::oY, &tm.vy, z0, x0, y + N - 1, s, br);
+            tma4(t + La::oP, &tm.p, z0, x0, y, s, br);
+            tma4(t + La::oK, &tm.K, z0, x0, y, 0, br);
+            if (MODE == REC) tma4(t + La::oL, &tm.lp, z0, x0, y, s, br);
+            if (MODE == ADJ) {
+                if (ez.tm) tma4(t + La::oEZ, ez.tm, ez.c, x0, y, s, br);
+                if (ex.tm) tma4(t + La::oEX, ex.tm, z0, ex.c, y, s, br);
             }
         };
-        const int oz = z0 + 4 * tzi, ox = x0 + txi;
-        const bool mem = oz < g.ne[0] && ox < g.ne[1];
+        if (tid == 0 && ok) {
+            issue(ya, 0);
+            for (int d = 1; d < DEPTH && ya + d <= yb; d++) issue(ya + d, d);
+            next[par] = (int)(gridDim.x + atomicAdd(ctr, 1u));
+        }
         const long long sh = (long long)s * g.ntot;
-        bool mz[4];
+        const unsigned col = (unsigned)(oz + g.px * ox);
+        const bool grid_ok = oz < g.ne[0] && ox < g.ne[1];
+        // y queue of own v_y: entry l = plane y-N+l; adjoint: v_y + e_y on the y-slab planes
+        Q4 q[2 * N];
 #pragma unroll
-        for (int r = 0; r < 4; r++) mz[r] = in_range(oz + r, it.lo[0], it.hi[0]);
-        const bool mx = in_range(ox, it.lo[1], it.hi[1]);
-        const int own = txi * TZ + 4 * tzi;           // own nodes in a core tile
-        // REC: whether the source stencil reaches this item's tile column and
-        // y range (the per-node test runs only then)
+        for (int l = 0; l < 2 * N - 1; l++) {
+            const int y = ya - N + l;
+            q[l] = grid_ok && y >= 0 && y < g.ne[2] ? ldq(f.v[2] + sh + (col + (unsigned)(y * plane))) : zeroq();
+        }
+        if (MODE == ADJ && me.act) {
+#pragma unroll
+            for (int l = 0; l < 2 * N - 1; l++) {
+                const int js = slab_row(g, 2, ya - N + l);
+                if (js >= 0) q[l] = addq(q[l], ldq(f.psip[2] + s * g.slab_n[2] + (col + (unsigned)(js * plane))));
+            }
+        }
+        Q4 md;                                // dt at the nodes of the update region, else 0 (adjoint: -dt)
+        bool in[4], out[4];                   // REC: updated nodes, and those outside the previous box along z and x
+        bool clip = false;
+        {
+            float a[4];
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                in[r] = me.act && in_range(oz + r, it.lo[0], it.hi[0]);
+                a[r] = in[r] ? (MODE == ADJ ? -dt : dt) : 0.f;
+                out[r] = MODE == REC && in[r] &&
+                         !(in_range(oz + r, it.plo[0], it.phi[0]) && in_range(ox, it.plo[1], it.phi[1]));
+                clip = clip || out[r];
+            }
+            md = quad(a);
+        }
+        // whether the source stencil reaches this item's tile column and y range
         bool src_col = false;
-        if (MODE == REC) {
+        float amp = 0.f;
+        if (MODE != ADJ && stf) {
             const Stencil &st = b.src[s];
             src_col = st.first[0] <= z0 + TZ - 1 && st.first[0] + st.cnt[0] - 1 >= z0 && st.first[1] <= x0 + TX - 1 &&
                       st.first[1] + st.cnt[1] - 1 >= x0 && st.first[2] <= yb && st.first[2] + st.cnt[2] - 1 >= ya;
+            amp = (MODE == REC ? -src_scale : src_scale) * stf[step];
         }
+        if (MODE == REC) clip = __syncthreads_or(clip);
+        if (MODE != REC) {
+            load_coefs(co, g.cpb[0], g.cpa[0], g.cpb[1], g.cpa[1], it);
+            __syncthreads();
+        }
+        const bool zxb = MODE != REC && (z_slab_tile(g, &tm.p, &tm.p, z0).tm || x_slab_tile(g, &tm.p, &tm.p, x0 - N, La::XR).tm);
+        const bool xg = MODE == FWD && x_group(g, ox, lc.x0);
+        float *const mzp = f.psiv[0] + (s * g.slab_n[0] + me.zq + (long long)g.zp * ox);
+        float *const mxp = f.psiv[1] + (s * g.slab_n[1] + oz + (long long)g.px * me.xq);
+        const unsigned zpl = (unsigned)(g.zp * g.ne[1]), xpl = (unsigned)(g.px * g.xrows);
+        const int n0 = g.H[0] - g.L[0] + 1, n1 = g.H[1] - g.L[1] + 1;
+        const long long acol = (long long)s * g.nphys + (oz - g.L[0]) + (long long)n0 * (ox - g.L[1]);
+        const bool whole = MODE == REC && in[0] && in[3];
+        int h = 0;                            // group slot of plane y
 
-        // y queue of own vy: entry l = plane y-N+l; planes before ya by plain loads
-        float q[2 * N][4];
-#pragma unroll
-        for (int l = 0; l < N; l++) {
-            const int y = ya - N + l;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (mem && y >= 0 && y < g.ne[2]) v = *reinterpret_cast<const float4 *>(f.v[2] + sh + gidx(g, oz, ox, y));
-            put(q[l], v);
-        }
-        Ring hr{ya, min(ylast, ya + S - 1)}, cr{ya, min(yb, ya + SC - 1)};
-        if (tid == 0) {
-            for (int y = ya; y <= hr.issued; y++) {
-                const int k = (y - ya) % S;
-                float *slot = sm + k * Lay::SLOT;
-                mbar_expect(&bar[k], Lay::BYTES);
-                tma4(slot + Lay::Z_OFF, &tm_vz, z0 - 4, x0, y, s, &bar[k]);
-                tma4(slot + Lay::X_OFF, &tm_vx, z0, x0 - N, y, s, &bar[k]);
-                tma4(slot + Lay::Y_OFF, &tm_vy, z0, x0, y, s, &bar[k]);
-            }
-            for (int y = ya; y <= cr.issued; y++) issue_core(y);
-        }
-        bool ok = true;
-#pragma unroll
-        for (int l = 0; l < N - 1; l++) {
-            ok &= ring_wait(bar, S, 0, parity, hr, ya + l, ya);
-            put(q[N + l], lds4(sm + (l % S) * Lay::SLOT + Lay::Y_OFF + own));
-        }
-        if (MODE == ADJ && mem && mx) {
-            // transposed y CPML: the queue holds lv_y + Av_y (lv_y + chi_y) on y-slab planes
-#pragma unroll
-            for (int l = 0; l < 2 * N - 1; l++) {
-                const int yq = ya - N + l;
-                if (yq < 0 || yq >= g.ne[2] || !yslab(g, yq)) continue;
-                float ch[4];
-                put(ch, ldg4(f.psip[2] + yslab_off(g, s, oz, ox, yq)));
-                const float A = g.cva[2][yq];
-#pragma unroll
-                for (int r = 0; r < 4; r++) q[l][r] += A * (q[l][r] + ch[r]);
-            }
-        }
-        // ADJ: nodes whose phi_y update the z / x CPML kernel makes (it reads
-        // lp before that kernel changes it): the adjoint z and x bands
-        bool zxb[4];
-#pragma unroll
-        for (int r = 0; r < 4; r++)
-            zxb[r] = CLS == ALLT && (oz + r < g.nb + N || oz + r >= g.ne[0] - g.nb - N - 1 || ox < g.nb + N ||
-                                     ox >= g.ne[1] - g.nb - N - 1);
-        if (__syncthreads_or(!ok)) goto timeout;
-
-        {
-        bool stop = false;
-        int y = ya;
-        auto body = [&](auto kc) {
-            constexpr int kq = decltype(kc)::value;
-            // accumulator of this plane (REC), loaded before the waits
+        // one plane; BAND: with the CPML terms (REC: with nodes outside the previous box)
+        auto body = [&](auto kc, auto bc, int y) {
+            constexpr int K = decltype(kc)::value;
+            constexpr bool BAND = decltype(bc)::value;
             float accv[4] = {0.f, 0.f, 0.f, 0.f};
             long long accb = 0;
-            bool acc4 = false;                   // the quad as one aligned 16-byte access
-            if (MODE == REC && mem && mx && in_range(y, it.lo[2], it.hi[2])) {
-                const long long n0 = g.H[0] - g.L[0] + 1, n1 = g.H[1] - g.L[1] + 1;
-                accb = (long long)s * g.nphys + (long long)(oz - g.L[0]) +
-                       n0 * ((long long)(ox - g.L[1]) + n1 * (long long)(y - g.L[2]));
-                acc4 = mz[0] && mz[1] && mz[2] && mz[3] && (accb & 3) == 0;
+            bool acc4 = false;                // the quad as one aligned 16-byte access
+            if (MODE == REC && me.act) {
+                accb = acol + (long long)n0 * n1 * (y - g.L[2]);
+                if (y + AHEAD <= yb) prefetch_l2(acc + accb + (long long)n0 * n1 * AHEAD);
+                acc4 = whole && (accb & 3) == 0;
                 if (acc4) {
-                    put(accv, *reinterpret_cast<const float4 *>(acc + accb));
+                    put(accv, ldg4(acc + accb));
                 } else {
 #pragma unroll
                     for (int r = 0; r < 4; r++)
-                        if (mz[r]) accv[r] = acc[accb + r];
+                        if (in[r]) accv[r] = acc[accb + r];
                 }
             }
-#ifdef SMI_TIMING
-            const long long tw0 = clock64();
-#endif
-            // y CPML operands, loaded before the waits: FWD psi_vy, ADJ phi_y
-            // of plane y; ADJ chi_y of the plane entering the queue
-            const bool my = in_range(y, it.lo[2], it.hi[2]);
-            const bool ysl = MODE != REC && mem && mx && my && yslab(g, y);
-            const int ye = y + N - 1;
-            const bool yent = MODE == ADJ && mem && mx && ye < g.ne[2] && yslab(g, ye);
-            float ym[4] = {0.f, 0.f, 0.f, 0.f}, yc[4] = {0.f, 0.f, 0.f, 0.f};
-            if (ysl) put(ym, ldg4(f.psiv[2] + yslab_off(g, s, oz, ox, y)));
-            if (yent) put(yc, ldg4(f.psip[2] + yslab_off(g, s, oz, ox, ye)));
-            ok = ring_wait(bar, S, 0, parity, hr, y + N - 1, ya);
-            ok &= ring_wait(cbar, SC, 16, parity, cr, y, ya);
-#ifdef SMI_TIMING
-            t_wait += clock64() - tw0;
-#endif
-            put(q[((2 * N - 1) + kq) % (2 * N)], lds4(sm + ((y + N - 1 - ya) % S) * Lay::SLOT + Lay::Y_OFF + own));
-            const float *slot = sm + ((y - ya) % S) * Lay::SLOT;
-            const float *cslot = cbase + ((y - ya) % SC) * Lay::CSLOT;   // this plane's core slot
-            const float *cs = cslot + own;
-            const bool act = mem && mx && my;
-            float pv[4], Kv[4];
-            put(pv, lds4(cs));
-            put(Kv, lds4(cs + CORE));
-            float div[4];
-            const bool bact = CLS == BND && act;     // band tile, quad column inside the box
-            // ---- z ----
-            {
-                float W[12];
-                {
-                    const float *row = slot + Lay::Z_OFF + txi * ZW + 4 * tzi;
-                    float4 a0 = lds4(row), a1 = lds4(row + 4), a2 = lds4(row + 8);
-                    W[0] = a0.x; W[1] = a0.y; W[2] = a0.z; W[3] = a0.w;
-                    W[4] = a1.x; W[5] = a1.y; W[6] = a1.z; W[7] = a1.w;
-                    W[8] = a2.x; W[9] = a2.y; W[10] = a2.z; W[11] = a2.w;
+            const int ys = BAND && MODE != REC ? slab_row(g, 2, y) : -1;
+            const int ye = BAND && MODE == ADJ ? slab_row(g, 2, y + N - 1) : -1;
+            float ym[4], mzv[4], mxv[4];
+            Q4 yc;
+            if (BAND && MODE != REC) {
+                if (ys >= 0 && me.act) put(ym, ldg4(f.psiv[2] + s * g.slab_n[2] + (col + (unsigned)(ys * plane))));
+                if (ye >= 0 && me.act) yc = ldq(f.psip[2] + s * g.slab_n[2] + (col + (unsigned)(ye * plane)));
+                if (me.xq >= 0) put(mxv, ldg4(mxp + (unsigned)y * xpl));
+                if (me.zq >= 0) put(mzv, ldg4(mzp + (unsigned)y * zpl));
+                if (y + AHEAD <= yb) {
+                    if (me.xq >= 0) prefetch_l2(mxp + (unsigned)(y + AHEAD) * xpl);
+                    if (me.zq >= 0) prefetch_l2(mzp + (unsigned)(y + AHEAD) * zpl);
                 }
-                if (MODE == ADJ && CLS == BND && zb && (oz - 4 < g.nb || oz + 7 >= g.ne[0] - g.nb - 1)) {
-                    // transposed CPML operand over the v_z window: lv + Av (lv + chi) (Av = 0 off the slab)
-                    const float *ch = cslot + Lay::E_HZ + txi * ZW + 4 * tzi;
+            }
+            ok = ok && mbar_wait(&bar[h], (phase >> h) & 1u);
+            phase ^= 1u << h;
+            const float *t = sm + h * La::G, *own = t + txi * TZ + 4 * tzi;
+            Q4 &qn = q[(2 * N - 1 + K) % (2 * N)];
+            qn = ldq(own + La::oY);
+            if (BAND && ye >= 0 && me.act) qn = addq(qn, yc);
+            // ---- y ----
+            Q4 Dy = zeroq();
 #pragma unroll
-                    for (int i = 0; i < 12; i++) W[i] += tb.z[2][oz - z0 + 4 + i] * (W[i] + ch[i]);
-                }
+            for (int l = 1; l <= N; l++) Dy = tap(Dy, g.c[2][l - 1], q[(N + l - 1 + K) % (2 * N)], q[(N - l + K) % (2 * N)]);
+            float By = 0.f, Ay[4] = {0.f, 0.f, 0.f, 0.f};          // y memory variable
+            if (BAND && MODE != REC && ys >= 0 && me.act) {
+                By = g.cpb[2][y];
 #pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int l = 1; l <= N; l++) d += g.c[0][l - 1] * (W[4 + r + l - 1] - W[4 + r - l]);
-                    div[r] = d;
-                }
-                if (bact && zb && zquad_slab(g, oz)) {
-                    // z memory variable at the quad's slab nodes: forward psi <- Bp psi + Ap D (added);
-                    // adjoint phi <- Bp (phi + lp before this step)
-                    float mz4[4];
-                    put(mz4, lds4(cslot + Lay::E_CZ + own));
-#pragma unroll
-                    for (int r = 0; r < 4; r++) {
-                        const int t = oz - z0 + 8 + r;
-                        if (!(mz[r] && slab_at(g, 0, oz + r))) continue;
-                        if (MODE == FWD) {
-                            mz4[r] = tb.z[1][t] * mz4[r] + tb.z[0][t] * div[r];
-                            div[r] += mz4[r];
-                        } else {
-                            mz4[r] = tb.z[1][t] * (mz4[r] + pv[r]);
-                        }
-                    }
-                    stg4(f.psiv[0] + sh + gidx(g, oz, ox, y), mz4);
+                for (int r = 0; r < 4; r++) Ay[r] = in[r] ? g.cpa[2][y] : 0.f;
+                if (MODE == FWD) {
+                    const float B4[4] = {By, By, By, By};
+                    recur4(B4, Ay, ym, Dy);
+                    Dy = addq(Dy, quad(ym));
                 }
             }
             // ---- x ----
+            Q4 Dx = zeroq();
             {
-                float Xr[2 * N][4];
+                const float *xr = t + La::oX + (txi + N) * TZ + 4 * tzi, *er = t + La::oEX + (txi + N) * TZ + 4 * tzi;
 #pragma unroll
                 for (int l = 1; l <= N; l++) {
-                    put(Xr[N + l - 1], lds4(slot + Lay::X_OFF + (txi + N + l - 1) * TZ + 4 * tzi));
-                    put(Xr[N - l], lds4(slot + Lay::X_OFF + (txi + N - l) * TZ + 4 * tzi));
-                }
-                if (MODE == ADJ && CLS == BND && xb) {
-                    // transposed CPML operand at the taps x - N + t (Av = 0 off the slab)
-#pragma unroll
-                    for (int t = 0; t < 2 * N; t++) {
-                        const float A = tb.x[2][txi + t - N + 8];
-                        if (A != 0.f) {
-                            float ch[4];
-                            put(ch, lds4(cslot + Lay::E_HX + (txi + t) * TZ + 4 * tzi));
-#pragma unroll
-                            for (int r = 0; r < 4; r++) Xr[t][r] += A * (Xr[t][r] + ch[r]);
-                        }
+                    Q4 a = ldq(xr + (l - 1) * TZ), c = ldq(xr - l * TZ);
+                    if (BAND && MODE == ADJ && ex.tm) {
+                        a = addq(a, ldq(er + (l - 1) * TZ));
+                        c = addq(c, ldq(er - l * TZ));
                     }
+                    Dx = tap(Dx, g.c[1][l - 1], a, c);
                 }
-                float D[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int l = 1; l <= N; l++) d += g.c[1][l - 1] * (Xr[N + l - 1][r] - Xr[N - l][r]);
-                    D[r] = d;
-                }
-                if (bact && xb && ox < g.ne[1] && slab_at(g, 1, ox)) {
-                    float mx4[4];
-                    put(mx4, lds4(cslot + Lay::E_CX + own));
-                    const int t = txi + 8;
-#pragma unroll
-                    for (int r = 0; r < 4; r++) {
-                        if (!mz[r]) continue;
-                        if (MODE == FWD) {
-                            mx4[r] = tb.x[1][t] * mx4[r] + tb.x[0][t] * D[r];
-                            D[r] += mx4[r];
-                        } else {
-                            mx4[r] = tb.x[1][t] * (mx4[r] + pv[r]);
-                        }
-                    }
-                    stg4(f.psiv[1] + sh + gidx(g, oz, ox, y), mx4);
-                }
-#pragma unroll
-                for (int r = 0; r < 4; r++) div[r] += D[r];
             }
-            // ---- y ----
+            // ---- z ----
+            Q4 div;
             {
-                if (yent) {                       // entering plane: lv_y + Av_y (lv_y + chi_y)
-                    const float A = g.cva[2][ye];
+                float W[12];
+                window(W, t + txi * ZW + 4 * tzi);
+                if (BAND && MODE == ADJ && ez.tm) {
+                    float E[12];
+                    window(E, t + La::oEZ + txi * ZW + 4 * tzi);
+#pragma unroll
+                    for (int i = 0; i < 12; i++) W[i] += E[i];
+                }
+                div = dz4<N, false>(g, W);
+            }
+            if (BAND && MODE == FWD) {
+                if (me.zq >= 0) {
+                    float B[4], A[4];
+                    put(B, lds4(co.zB + 4 * tzi));
+                    put(A, lds4(co.zA + 4 * tzi));
+                    recur4z(xg, B, A, mzv, div);
+                    stg4(mzp + (unsigned)y * zpl, mzv);
+                }
+                if (me.xq >= 0) {
+                    recur1(co.xB[txi], co.xA[txi], mxv, Dx);
+                    stg4(mxp + (unsigned)y * xpl, mxv);
+                }
+            }
+            div = addq(addq(div, Dx), Dy);
+            const Q4 pv = ldq(own + La::oP), dK = mulq(md, ldq(own + La::oK));
+            Q4 np = update<MODE>(pv, dK, div);
+            if (BAND && MODE == FWD && (me.zq >= 0 || me.xq >= 0)) {
+                // z and x memory variables: their own product, after the plain derivatives'
+                float m[4];
+#pragma unroll
+                for (int r = 0; r < 4; r++) m[r] = (me.zq >= 0 ? mzv[r] : 0.f) + (me.xq >= 0 ? mxv[r] : 0.f);
+                np = sub_prod(np, dK, m);
+            }
+            if (MODE != ADJ && src_col) {
+                const Stencil &st = b.src[s];
+                const int t1 = ox - st.first[1], t2 = y - st.first[2];
+                if (t1 >= 0 && t1 < st.cnt[1] && t2 >= 0 && t2 < st.cnt[2]) {
+                    float x[4];
+                    split(np, x);
 #pragma unroll
                     for (int r = 0; r < 4; r++) {
-                        float &e = q[((2 * N - 1) + kq) % (2 * N)][r];
-                        e += A * (e + yc[r]);
+                        const int t0 = oz + r - st.first[0];
+                        if (t0 >= 0 && t0 < st.cnt[0] && (MODE == FWD || in[r]))
+                            x[r] += amp * (st.w[0][t0] * st.w[1][t1] * st.w[2][t2]);
                     }
+                    np = quad(x);
                 }
-                float D[4];
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    float d = 0.f;
-#pragma unroll
-                    for (int l = 1; l <= N; l++) d += g.c[2][l - 1] * (q[((N + l - 1) + kq) % (2 * N)][r] - q[((N - l) + kq) % (2 * N)][r]);
-                    D[r] = d;
-                }
-                if (ysl) {
-                    if (MODE == FWD) {            // psi_vy <- Bp psi_vy + Ap D_y v_y, added to div v
-                        const float B = g.cpb[2][y], A = g.cpa[2][y];
-#pragma unroll
-                        for (int r = 0; r < 4; r++) {
-                            const float ps = B * ym[r] + A * D[r];
-                            if (mz[r]) {
-                                ym[r] = ps;
-                                D[r] += ps;
-                            }
-                        }
-                    } else {                      // phi_y <- Bp (phi_y + lp), lp before this step
-                        const float B = g.cpb[2][y];
-#pragma unroll
-                        for (int r = 0; r < 4; r++)
-                            if (mz[r] && !zxb[r]) ym[r] = B * (ym[r] + pv[r]);
-                    }
-                    stg4(f.psiv[2] + yslab_off(g, s, oz, ox, y), ym);
-                }
-#pragma unroll
-                for (int r = 0; r < 4; r++) div[r] += D[r];
             }
-            if (act) {
-                float np[4];
-                if (MODE == REC) {
-                    const Stencil &st = b.src[s];
-                    float lpv[4];
-                    put(lpv, lds4(cs + 2 * CORE));
-                    const bool kxy = in_range(ox, it.plo[1], it.phi[1]) && in_range(y, it.plo[2], it.phi[2]);
-                    float na[4];
+            if (MODE == REC) {
+                float lpv[4], dv[4], p4[4];
+                split(ldq(own + La::oL), lpv);
+                split(div, dv);
+                split(pv, p4);
 #pragma unroll
-                    for (int r = 0; r < 4; r++) na[r] = accv[r] + lpv[r] * (img_mode == 0 ? div[r] : pv[r]);
-                    if (acc4) *reinterpret_cast<float4 *>(acc + accb) = make_float4(na[0], na[1], na[2], na[3]);
+                for (int r = 0; r < 4; r++) accv[r] += lpv[r] * (img_mode == 0 ? dv[r] : p4[r]);
+                if (BAND) {
+                    const bool ky = in_range(y, it.plo[2], it.phi[2]);
+                    bool cl[4];
 #pragma unroll
-                    for (int r = 0; r < 4; r++) {
-                        const int z = oz + r;
-                        np[r] = pv[r];
-                        if (!mz[r]) continue;
-                        if (!acc4) acc[accb + r] = na[r];
-                        if (img_mode == 2) acc[(long long)b.nshot * g.nphys + accb + r] += pv[r] * pv[r];   // illumination
-                        float pn = pv[r] + dt * Kv[r] * div[r];
-                        if (src_col) {           // the source stencil reaches this tile column
-                            const int t0 = z - st.first[0], t1 = ox - st.first[1], t2 = y - st.first[2];
-                            if (t0 >= 0 && t0 < st.cnt[0] && t1 >= 0 && t1 < st.cnt[1] && t2 >= 0 && t2 < st.cnt[2])
-                                pn -= src_scale * stf[step] * st.w[0][t0] * st.w[1][t1] * st.w[2][t2];
-                        }
-                        np[r] = (kxy && in_range(z, it.plo[0], it.phi[0])) ? pn : 0.f;
-                    }
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 4; r++) np[r] = mz[r] ? pv[r] - dt * Kv[r] * div[r] : pv[r];
+                    for (int r = 0; r < 4; r++) cl[r] = out[r] || (!ky && in[r]);
+                    np = clear_if(np, cl);
                 }
-                *reinterpret_cast<float4 *>(f.p + sh + gidx(g, oz, ox, y)) = make_float4(np[0], np[1], np[2], np[3]);
-            }
-#ifdef SMI_TIMING
-            const long long ts0 = clock64();
-            n_planes++;
-#endif
-            if (__syncthreads_or(!ok)) {
-                stop = true;
-                return;
-            }
-#ifdef SMI_TIMING
-            t_sync += clock64() - ts0;
-#endif
-            if (tid == 0) {
-                if (hr.issued < ylast) {
-                    const int yn = hr.issued + 1;
-                    const int k = (yn - ya) % S;
-                    float *sl = sm + k * Lay::SLOT;
-                    mbar_expect(&bar[k], Lay::BYTES);
-                    tma4(sl + Lay::Z_OFF, &tm_vz, z0 - 4, x0, yn, s, &bar[k]);
-                    tma4(sl + Lay::X_OFF, &tm_vx, z0, x0 - N, yn, s, &bar[k]);
-                    tma4(sl + Lay::Y_OFF, &tm_vy, z0, x0, yn, s, &bar[k]);
+                if (acc4) {
+                    stg4(acc + accb, accv);
+                } else if (me.act) {
+#pragma unroll
+                    for (int r = 0; r < 4; r++)
+                        if (in[r]) acc[accb + r] = accv[r];
                 }
-                if (cr.issued < yb) issue_core(cr.issued + 1);
+                if (img_mode == 2 && me.act) {                // illumination
+#pragma unroll
+                    for (int r = 0; r < 4; r++)
+                        if (in[r]) acc[(long long)b.nshot * g.nphys + accb + r] += p4[r] * p4[r];
+                }
             }
-            if (hr.issued < ylast) hr.issued++;
-            if (cr.issued < yb) cr.issued++;
+            if (BAND && MODE == ADJ) {
+                if (me.zq >= 0) {
+                    float Bz[4], Az[4];
+                    put(Bz, lds4(co.zB + 4 * tzi));
+                    put(Az, lds4(co.zA + 4 * tzi));
+                    recur4(Bz, Az, mzv, np);
+                    stg4(mzp + (unsigned)y * zpl, mzv);
+                }
+                if (me.xq >= 0) {
+                    recur1(co.xB[txi], co.xA[txi], mxv, np);
+                    stg4(mxp + (unsigned)y * xpl, mxv);
+                }
+                if (ys >= 0 && me.act) {
+                    const float B4[4] = {By, By, By, By};
+                    recur4(B4, Ay, ym, np);
+                }
+            }
+            if (BAND && MODE != REC && ys >= 0 && me.act)
+                stg4(f.psiv[2] + s * g.slab_n[2] + (col + (unsigned)(ys * plane)), ym);
+            if (me.act) stq(f.p + sh + (col + (unsigned)(y * plane)), np);
+            __syncthreads();
+            if (tid == 0 && ok && y + DEPTH <= yb) issue(y + DEPTH, h);
+            h = h + 1 == DEPTH ? 0 : h + 1;
+        };
+        auto one = [&](auto kc, int y) {
+            const bool band = MODE == REC ? clip || !in_range(y, it.plo[2], it.phi[2])
+                                          : zxb || yslab(g, y) || (MODE == ADJ && yslab(g, y + N - 1));
+            if (band) body(kc, std::true_type{}, y);
+            else body(kc, std::false_type{}, y);
         };
         constexpr int G = (2 * N) % SMI_YUNROLL == 0 ? SMI_YUNROLL : 2 * N;
-        while (y <= yb && !stop) {
-            Unroll<0, G>::run(body, y, yb, stop);
+        for (int y = ya; y <= yb; y += G) {
+            unroll_planes<G>(one, y, yb);
             rotate_queue<G>(q);
         }
-        if (stop) goto timeout;
-        }
-        continue;
-    timeout:
+        if (__syncthreads_or(!ok)) break;
+    }
+    if (__syncthreads_or(!ok)) {
         if (tid == 0) atomicOr(err, 1u);
-        ring_drain(bar, S, 0, parity, hr, ya);
-        ring_drain(cbar, SC, 16, parity, cr, ya);
+        for (int k = 0; k < DEPTH; k++) mbar_wait(&bar[k], (phase >> k) & 1u);
         return;
     }
-#ifdef SMI_TIMING
-    if (threadIdx.x == 0 && (blockIdx.x % 97) == 0 && n_planes > 0)
-        printf("T%d blk %d planes %lld all %lld wait %lld (%.0f%%) sync %lld (%.0f%%)\n", MODE, blockIdx.x, n_planes,
-               clock64() - t_all, t_wait, 100.0 * t_wait / (clock64() - t_all), t_sync, 100.0 * t_sync / (clock64() - t_all));
-#endif
+    if (MODE == FWD && sv.sample >= 0) save_tail(g, b.nshot, f, sv);
 }
 
 // Give-up path of the bounded waits: one warp waits, with the tile kernels'
@@ -909,6 +983,21 @@ bool make_map(CUtensorMap *tm, const Grid &g, const float *base, int nshot, int 
     return r == CUDA_SUCCESS;
 }
 
+// 4D map over a slab array (n0, n1, n2, shot) with strides in floats.
+bool make_slab_map(CUtensorMap *tm, const float *base, int n0, int n1, int n2, int nshot, long long s1, long long s2,
+                   long long sshot, int b0, int b1)
+{
+    EncodeFn fn = encoder();
+    if (!fn) return false;
+    cuuint64_t dims[4] = {(cuuint64_t)n0, (cuuint64_t)n1, (cuuint64_t)n2, (cuuint64_t)nshot};
+    cuuint64_t strides[3] = {(cuuint64_t)s1 * 4, (cuuint64_t)s2 * 4, (cuuint64_t)sshot * 4};
+    cuuint32_t box[4] = {(cuuint32_t)b0, (cuuint32_t)b1, 1, 1};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float *>(base), dims, strides, box, es,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <class K> int grid_for(K kernel, int smem)
 {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -920,56 +1009,81 @@ template <class K> int grid_for(K kernel, int smem)
     return std::max(1, per) * std::max(1, sms);
 }
 
-template <int N, int MODE, int CLS>
-void run_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, Fields f, int step, unsigned *err)
+// Planes a chunk of a launch over `cols` tile columns (all shots) of ylen
+// planes.  Large launches: 8 planes (more when that makes over eight items a
+// CTA), so that the sweep stays local (see Sched).  Small ones, whose items
+// run at once: the chunk between 8 and 24 planes that finishes first when an
+// item costs its planes plus a start of about 7, and an SM runs three items
+// as fast as one (measured on 133 x 141 x 127 points, order 4, a step: 22
+// planes 44 us, 15 planes 33, 12 planes 37, 8 planes 34).
+int pick_chunk(long long cols, int ylen, int grid, int sms)
 {
-    constexpr int smem = s3::VLay<N, CLS>::SMEM;
-    static const int grid = grid_for(s3::k3_v<N, MODE, CLS>, smem);
-    s3::k3_v<N, MODE, CLS><<<grid, s3::NTHR, smem, static_cast<cudaStream_t>(lc.stream)>>>(
-        m.p_halo, m.rho_v, m.vz_core, m.vx_core, m.vy_core, m.pz_halo, m.px_halo, m.cz_core, m.cx_core, g, b, f,
-        step, err);
-    ++*lc.launches;
-}
-
-template <int N, int MODE, int CLS>
-void run_p(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g, const Batch &b, Fields f, int step,
-           unsigned *err, float *acc, int img_mode, const float *stf, float src_scale)
-{
-    constexpr int smem = s3::PLay<N, CLS>::SMEM;
-    static const int grid = grid_for(s3::k3_p<N, MODE, CLS>, smem);
-    s3::k3_p<N, MODE, CLS><<<grid, s3::NTHR, smem, static_cast<cudaStream_t>(lc.stream)>>>(
-        m.vz_halo, m.vx_halo, m.vy_core, m.p_core, m.K_core, lpm ? lpm->p_core : m.p_core, m.cz_vhalo, m.cx_vhalo,
-        m.pz_core, m.px_core, g, b, f, step, err, acc, img_mode, stf, src_scale);
-    ++*lc.launches;
-}
-
-// One forward / adjoint stencil half-step: every tile column in one launch
-// (inl = false: the z / x CPML terms come from the band kernels), or the
-// interior columns and then the CPML-band columns with the terms inline.
-// The two classes update disjoint nodes and, within a half-step, read only
-// what the other does not write.
-template <int N, int MODE>
-void run_v_cls(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, Fields f, int step,
-               unsigned *err, bool inl)
-{
-    if (!inl) {
-        run_v<N, MODE, s3::ALLT>(lc, m, g, b, f, step, err);
-        return;
+    if (cols <= 0 || ylen <= 0) return 1;
+    const long long items8 = cols * ((ylen + 7) / 8);
+    if (items8 >= 4LL * grid) return (int)std::max<long long>(8, cols * ylen / (8LL * grid));
+    if (items8 >= 2LL * grid) return 12;
+    long long best = -1;
+    int cy = ylen;
+    for (int n = (ylen + 23) / 24; n <= std::max(1, ylen / 8); n++) {
+        const int c = (ylen + n - 1) / n;
+        const long long items = cols * ((ylen + c - 1) / c);
+        const long long cost = (c + 7) * std::max<long long>(3, (items + sms - 1) / sms);
+        if (best < 0 || cost <= best) {
+            best = cost;
+            cy = c;
+        }
     }
-    run_v<N, MODE, s3::BND>(lc, m, g, b, f, step, err);
-    run_v<N, MODE, s3::INT>(lc, m, g, b, f, step, err);
+    return cy;
+}
+
+// The cut of a launch from the boxes of its shots.
+s3::Cut launch_cut(const Grid &g, const Batch &b, int mode, int step, int grid)
+{
+    long long cols = 0;
+    int ylen = 0, x0 = g.ne[1];
+    for (int s = 0; s < b.nshot; s++) {
+        int lo[3], hi[3];
+        box_bounds(g, (mode == s3::ADJ ? b.h_box_rec : b.h_box_src) + 6 * s, step, lo, hi);
+        if (mode == s3::REC)
+            for (int a = 0; a < 3; a++) {
+                lo[a] = std::max(lo[a], g.L[a]);
+                hi[a] = std::min(hi[a], g.H[a]);
+            }
+        if (hi[0] < lo[0] || hi[1] < lo[1]) continue;
+        cols += (long long)((hi[0] - (lo[0] & ~31)) / s3::TZ + 1) * ((hi[1] - lo[1]) / s3::TX + 1);
+        ylen = std::max(ylen, hi[2] - lo[2] + 1);
+        x0 = std::min(x0, lo[1]);
+    }
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return std::max(1, n);
+    }();
+    return {pick_chunk(cols, ylen, grid, sms), x0};
 }
 
 template <int N, int MODE>
-void run_p_cls(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g, const Batch &b, Fields f,
-               int step, unsigned *err, float *acc, int img_mode, const float *stf, float src_scale, bool inl)
+void run_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, const Fields &f, int step, const Gather3 &ga,
+           const Restore3 &rs, unsigned *err, unsigned *ctr)
 {
-    if (!inl) {
-        run_p<N, MODE, s3::ALLT>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale);
-        return;
-    }
-    run_p<N, MODE, s3::BND>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale);
-    run_p<N, MODE, s3::INT>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale);
+    constexpr int smem = s3::VLay<N, MODE>::SMEM;
+    static const int grid = grid_for(s3::k3_v<N, MODE>, smem);
+    const s3::VMaps tm{m.p_halo, m.rho_v, m.vz_core, m.vx_core, m.vy_core, m.ezl_p, m.ezh_p, m.exl_p, m.exh_p};
+    launch_pdl(lc, s3::k3_v<N, MODE>, dim3(grid), s3::NTHR, smem, tm, g, b, f, step, launch_cut(g, b, MODE, step, grid), ga,
+               rs, err, ctr);
+}
+
+template <int N, int MODE>
+void run_p(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g, const Batch &b, const Fields &f, int step,
+           unsigned *err, float *acc, int img_mode, const float *stf, float src_scale, const Save3 &sv, unsigned *ctr)
+{
+    constexpr int smem = s3::PLay<N, MODE>::SMEM;
+    static const int grid = grid_for(s3::k3_p<N, MODE>, smem);
+    const s3::PMaps tm{m.vz_halo, m.vx_halo, m.vy_core, m.p_core, m.K_core, lpm ? lpm->p_core : m.p_core,
+                       m.ezl_v, m.ezh_v, m.exl_v, m.exh_v};
+    launch_pdl(lc, s3::k3_p<N, MODE>, dim3(grid), s3::NTHR, smem, tm, g, b, f, step,
+               launch_cut(g, b, MODE, step, grid), err, acc, img_mode, stf, src_scale, sv, ctr);
 }
 
 }  // namespace
@@ -995,60 +1109,70 @@ bool stencil3d_supported(const Grid &g)
     return g.ndim == 3 && (g.N == 2 || g.N == 4) && g.ntot < (1LL << 31) && encoder() != nullptr;
 }
 
-bool make_maps3(Maps3 &m, const Grid &g, const Fields &f, int nshot, bool fullmem)
+bool make_maps3(Maps3 &m, const Grid &g, const Fields &f, int nshot, bool slabs)
 {
     const int R = s3::TX + 2 * g.N - 1;
+    Grid gr = g;                              // rho: the row padding repeats the last node (k_extend_model)
+    gr.ne[0] = g.px;
     bool ok = make_map(&m.p_halo, g, f.p, nshot, s3::ZW, R) && make_map(&m.p_core, g, f.p, nshot, s3::TZ, s3::TX) &&
               make_map(&m.vz_core, g, f.v[0], nshot, s3::TZ, s3::TX) &&
               make_map(&m.vx_core, g, f.v[1], nshot, s3::TZ, s3::TX) &&
               make_map(&m.vy_core, g, f.v[2], nshot, s3::TZ, s3::TX) &&
               make_map(&m.vz_halo, g, f.v[0], nshot, s3::ZW, s3::TX) &&
               make_map(&m.vx_halo, g, f.v[1], nshot, s3::TZ, R) &&
-              make_map(&m.rho_v, g, g.rho, 1, 36, s3::TX + 1) && make_map(&m.K_core, g, g.K, 1, s3::TZ, s3::TX);
+              make_map(&m.rho_v, gr, g.rho, 1, 36, s3::TX + 1) && make_map(&m.K_core, g, g.K, 1, s3::TZ, s3::TX);
     if (!ok) return false;
-    if (!fullmem) {
-        // compressed CPML slabs: the band maps are never read (the band kernels apply the terms)
-        m.pz_halo = m.px_halo = m.p_halo;
-        m.cz_core = m.cx_core = m.pz_core = m.px_core = m.p_core;
-        m.cz_vhalo = m.vz_halo;
-        m.cx_vhalo = m.vx_halo;
+    if (!slabs) {
+        m.ezl_p = m.ezh_p = m.exl_p = m.exh_p = m.ezl_v = m.ezh_v = m.exl_v = m.exh_v = m.p_core;   // never read
         return true;
     }
-    return make_map(&m.pz_halo, g, f.psiv[0], nshot, s3::ZW, R) && make_map(&m.px_halo, g, f.psiv[1], nshot, s3::ZW, R) &&
-           make_map(&m.cz_core, g, f.psip[0], nshot, s3::TZ, s3::TX) &&
-           make_map(&m.cx_core, g, f.psip[1], nshot, s3::TZ, s3::TX) &&
-           make_map(&m.cz_vhalo, g, f.psip[0], nshot, s3::ZW, s3::TX) &&
-           make_map(&m.cx_vhalo, g, f.psip[1], nshot, s3::TZ, R) &&
-           make_map(&m.pz_core, g, f.psiv[0], nshot, s3::TZ, s3::TX) &&
-           make_map(&m.px_core, g, f.psiv[1], nshot, s3::TZ, s3::TX);
+    // z slab arrays [y][x][zp]: low and high part; x slab arrays [y][row][px]
+    auto zmap = [&](CUtensorMap *lo, CUtensorMap *hi, const float *a) {
+        const int nhi = g.zp - g.zlo;
+        return make_slab_map(lo, a, g.zlo, g.ne[1], g.ne[2], nshot, g.zp, (long long)g.zp * g.ne[1], g.slab_n[0], s3::ZW,
+                             s3::TX) &&
+               (nhi > 0 ? make_slab_map(hi, a + g.zlo, nhi, g.ne[1], g.ne[2], nshot, g.zp, (long long)g.zp * g.ne[1],
+                                        g.slab_n[0], s3::ZW, s3::TX)
+                        : (*hi = *lo, true));
+    };
+    auto xmap = [&](CUtensorMap *lo, CUtensorMap *hi, const float *a) {
+        const int nhi = g.xrows - g.xlo;
+        return make_slab_map(lo, a, g.px, g.xlo, g.ne[2], nshot, g.px, (long long)g.px * g.xrows, g.slab_n[1], s3::TZ, R) &&
+               (nhi > 0 ? make_slab_map(hi, a + (long long)g.xlo * g.px, g.px, nhi, g.ne[2], nshot, g.px,
+                                        (long long)g.px * g.xrows, g.slab_n[1], s3::TZ, R)
+                        : (*hi = *lo, true));
+    };
+    return zmap(&m.ezl_p, &m.ezh_p, f.psiv[0]) && xmap(&m.exl_p, &m.exh_p, f.psiv[1]) &&
+           zmap(&m.ezl_v, &m.ezh_v, f.psip[0]) && xmap(&m.exl_v, &m.exh_v, f.psip[1]);
 }
 
 void launch3_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, Fields f, int step, int mode,
-               unsigned *err, bool inl)
+               Gather3 ga, Restore3 rs, unsigned *err,
+     unsigned *ctr)
 {
-    // the adjoint's interior update is the forward scheme; only its box differs
     if (g.N == 2) {
-        if (mode == 0) run_v_cls<2, 0>(lc, m, g, b, f, step, err, inl);
-        else if (mode == 1) run_v_cls<2, 1>(lc, m, g, b, f, step, err, inl);
-        else run_v<2, 2, s3::ALLT>(lc, m, g, b, f, step, err);
+        if (mode == 0) run_v<2, 0>(lc, m, g, b, f, step, ga, rs, err, ctr);
+        else if (mode == 1) run_v<2, 1>(lc, m, g, b, f, step, ga, rs, err, ctr);
+        else run_v<2, 2>(lc, m, g, b, f, step, ga, rs, err, ctr);
     } else {
-        if (mode == 0) run_v_cls<4, 0>(lc, m, g, b, f, step, err, inl);
-        else if (mode == 1) run_v_cls<4, 1>(lc, m, g, b, f, step, err, inl);
-        else run_v<4, 2, s3::ALLT>(lc, m, g, b, f, step, err);
+        if (mode == 0) run_v<4, 0>(lc, m, g, b, f, step, ga, rs, err, ctr);
+        else if (mode == 1) run_v<4, 1>(lc, m, g, b, f, step, ga, rs, err, ctr);
+        else run_v<4, 2>(lc, m, g, b, f, step, ga, rs, err, ctr);
     }
 }
 
 void launch3_p(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g, const Batch &b, Fields f,
-               int step, int mode, unsigned *err, float *acc, int img_mode, const float *stf, float src_scale, bool inl)
+               int step, int mode, unsigned *err, float *acc, int img_mode, const float *stf, float src_scale, Save3 sv,
+               unsigned *ctr)
 {
     if (g.N == 2) {
-        if (mode == 0) run_p_cls<2, 0>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, inl);
-        else if (mode == 1) run_p_cls<2, 1>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, inl);
-        else run_p<2, 2, s3::ALLT>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale);
+        if (mode == 0) run_p<2, 0>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, sv, ctr);
+        else if (mode == 1) run_p<2, 1>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, sv, ctr);
+        else run_p<2, 2>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, sv, ctr);
     } else {
-        if (mode == 0) run_p_cls<4, 0>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, inl);
-        else if (mode == 1) run_p_cls<4, 1>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, inl);
-        else run_p<4, 2, s3::ALLT>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale);
+        if (mode == 0) run_p<4, 0>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, sv, ctr);
+        else if (mode == 1) run_p<4, 1>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, sv, ctr);
+        else run_p<4, 2>(lc, m, lpm, g, b, f, step, err, acc, img_mode, stf, src_scale, sv, ctr);
     }
 }
 

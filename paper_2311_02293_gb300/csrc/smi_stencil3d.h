@@ -8,13 +8,35 @@
 namespace smi {
 
 // Tensor maps of one batch's fields (haloed plane tiles and 32 x 16 core
-// tiles) and of the model arrays.
+// tiles), of the model arrays, and of the CPML slab arrays of the adjoint's
+// operands (low and high slab; _p: on the p nodes, psiv, in the velocity
+// kernel's geometry; _v: on the v nodes, psip, in the pressure kernel's).
 struct Maps3 {
     CUtensorMap p_halo, p_core, vz_core, vx_core, vy_core, vz_halo, vx_halo, rho_v, K_core;
-    // full-size z / x CPML memory variables (inline band terms): the p-grid ones
-    // (psiv) in the p tile geometry and core, the v-grid ones (psip) core and in
-    // the v_z / v_x tile geometries
-    CUtensorMap pz_halo, px_halo, pz_core, px_core, cz_core, cx_core, cz_vhalo, cx_vhalo;
+    CUtensorMap ezl_p, ezh_p, exl_p, exh_p, ezl_v, ezh_v, exl_v, exh_v;
+};
+
+// What the forward velocity kernel also does: receivers' samples of the
+// pressure it reads, which is the pressure after step `it` (it < 0: none).
+struct Gather3 {
+    float *seis;
+    const long long *off;
+    int it;
+};
+// What the adjoint velocity kernel also does: the boundary of the source
+// field v from the store's sample `it` (it < 0: none).
+struct Restore3 {
+    Bands bd;
+    float *v[3];
+    int it;
+};
+// What the forward pressure kernel also does: the velocities it reads become
+// stored sample `sample` (FP32 storage), or their largest magnitudes per
+// (shot, axis, side) go into amax (16-bit storage; zeroed).  sample < 0: none.
+struct Save3 {
+    Bands bd;
+    unsigned *amax;
+    int sample;
 };
 
 // One warp waits with the tile kernels' bounded-wait helper on an mbarrier
@@ -34,21 +56,19 @@ bool tile_maps_available();
 // True when the 3D kernels can run (3D, order 4 or 8, tensor-map encoder found).
 bool stencil3d_supported(const Grid &g);
 
-// Builds the maps for fields f of a batch of nshot shots (fullmem: the z / x
-// memory variables are full-size arrays, whose maps the inline band terms
-// read); false on failure.
-bool make_maps3(Maps3 &m, const Grid &g, const Fields &f, int nshot, bool fullmem);
+// Builds the maps for fields f of a batch of nshot shots (slabs: the CPML
+// slab arrays too, in the tile kernels' layout); false on failure.
+bool make_maps3(Maps3 &m, const Grid &g, const Fields &f, int nshot, bool slabs);
 
 // mode 0: forward, 1: adjoint (step = reverse steps elapsed), 2: reconstruction.
-// err: device word, bit 0 set if a bounded wait gave up.
-// inl (modes 0 and 1): the z / x CPML terms inline (interior and band tile
-// classes; full-size memory variables); else they are left to the band
-// kernels (launch_fwd_corrections / launch_adj_corrections).
+// err: device word, bit 0 set if a bounded wait gave up; ctr: a zeroed device
+// word of this launch (its work counter).
 void launch3_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, Fields f, int step, int mode,
-               unsigned *err, bool inl);
+               Gather3 ga, Restore3 rs, unsigned *err, unsigned *ctr);
 // lpm: maps of the adjoint fields, whose pressure the reconstruction mode
-// correlates with (mode 2 only).
+// correlates with (mode 2 only).  stf null: no source.
 void launch3_p(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g, const Batch &b, Fields f,
-               int step, int mode, unsigned *err, float *acc, int img_mode, const float *stf, float src_scale, bool inl);
+               int step, int mode, unsigned *err, float *acc, int img_mode, const float *stf, float src_scale, Save3 sv,
+               unsigned *ctr);
 
 }  // namespace smi

@@ -11,9 +11,6 @@
 
 #include <cstdint>
 #include <type_traits>
-#ifdef SMI_TIMING
-#include <cstdio>
-#endif
 
 #include "smi_box.h"
 #include "smi_internal.h"
@@ -31,7 +28,7 @@ namespace s3 {
 #define SMI_MINB 4
 #endif
 #ifndef SMI_YUNROLL
-#define SMI_YUNROLL 2        // y planes per unrolled group (divides 2N)
+#define SMI_YUNROLL 1        // y planes per unrolled group (divides 2N)
 #endif
 constexpr int TZ = 32, TX = SMI_TX, NTHR = 8 * TX;
 constexpr int ZW = 40;                 // z extent of haloed tiles: [z0-4, z0+36)
@@ -122,80 +119,6 @@ __device__ __forceinline__ void item_box(const Grid &g, const Batch &b, int mode
     }
 }
 
-struct Decomp {
-    int nzt, nxt, nyc, cy, zb;
-};
-
-// Column tiles x y-chunks of a box.  Long chunks: each chunk pays a
-// pipeline start-up of about 2N planes, so a box is split into
-// min(ylen / 16, grid / columns) chunks a column, one wave of the persistent
-// grid.  When that wave leaves more than a tenth of the CTAs idle (the
-// 340^3 box makes 242 columns for a 608-CTA grid: 2 chunks fill 80 %), the
-// chunk count grows to the smallest that fills the waves to 90 % (5 there:
-// 99.5 %).
-__device__ __forceinline__ Decomp decomp(const int lo[3], const int hi[3], int grid)
-{
-    Decomp d;
-    d.zb = lo[0] & ~31;
-    d.nzt = hi[0] >= lo[0] ? (hi[0] - d.zb) / TZ + 1 : 0;
-    d.nxt = hi[1] >= lo[1] ? (hi[1] - lo[1]) / TX + 1 : 0;
-    const int ylen = hi[2] - lo[2] + 1;
-    if (d.nzt == 0 || d.nxt == 0 || ylen <= 0) {
-        d.nzt = d.nxt = d.nyc = 0;
-        d.cy = 1;
-        return d;
-    }
-    const long long cols = (long long)d.nzt * d.nxt;
-    const int cmax = max(1, ylen / 16);
-    auto fill = [&](int c) {
-        const long long items = cols * c;
-        return (float)items / (float)(((items + grid - 1) / grid) * grid);
-    };
-    int chunks = max(1, min(cmax, (int)(grid / cols)));
-    if (fill(chunks) < 0.9f) {
-        for (int c = chunks + 1; c <= min(cmax, 4 * chunks + 4); c++) {
-            if (fill(c) >= 0.9f) {
-                chunks = c;
-                break;
-            }
-        }
-    }
-    d.cy = (ylen + chunks - 1) / chunks;
-    d.nyc = (ylen + d.cy - 1) / d.cy;
-    return d;
-}
-
-// Item w of the launch (shots in order), false past the end.
-__device__ __forceinline__ bool get_item(const Grid &g, const Batch &b, int mode, int step, long long w, Item &it)
-{
-    const int target = (int)gridDim.x;
-    for (int s = 0; s < b.nshot; s++) {
-        int lo[3], hi[3], plo[3] = {0, 0, 0}, phi[3] = {-1, -1, -1};
-        item_box(g, b, mode, s, step, lo, hi, plo, phi);
-        const Decomp d = decomp(lo, hi, target);
-        const long long n = (long long)d.nzt * d.nxt * d.nyc;
-        if (w < n) {
-            const int zi = (int)(w % d.nzt);
-            const int xi = (int)((w / d.nzt) % d.nxt);
-            const int ci = (int)(w / ((long long)d.nzt * d.nxt));
-            it.s = s;
-            it.z0 = d.zb + TZ * zi;
-            it.x0 = lo[1] + TX * xi;
-            it.ya = lo[2] + ci * d.cy;
-            it.yb = min(hi[2], it.ya + d.cy - 1);
-            for (int a = 0; a < 3; a++) {
-                it.lo[a] = lo[a];
-                it.hi[a] = hi[a];
-                it.plo[a] = plo[a];
-                it.phi[a] = phi[a];
-            }
-            return true;
-        }
-        w -= n;
-    }
-    return false;
-}
-
 __device__ __forceinline__ bool in_range(int v, int lo, int hi) { return v >= lo && v <= hi; }
 
 // ===========================================================================
@@ -246,6 +169,16 @@ template <int M> struct Unroll<M, M> {
     template <class F> __device__ __forceinline__ static void run(F &, int &, int, const bool &) {}
 };
 
+// Planes y .. y+G-1 (those up to yb) of a loop body f(step, plane).
+template <int G, int K = 0, class F> __device__ __forceinline__ void unroll_planes(F &f, int y, int yb)
+{
+    if constexpr (K < G) {
+        if (y + K > yb) return;
+        f(std::integral_constant<int, K>{}, y + K);
+        unroll_planes<G, K + 1>(f, y, yb);
+    }
+}
+
 // After a group of G planes the logical entry l sits at (l + G) % L: move
 // it back to l so the next group starts at step 0 (fewer unrolled copies of
 // the loop body keep the code inside the instruction cache).
@@ -262,6 +195,15 @@ __device__ __forceinline__ void rotate_queue(float (&q)[L][4])
     for (int l = 0; l < L; l++)
 #pragma unroll
         for (int r = 0; r < 4; r++) q[l][r] = t[l][r];
+}
+template <int G, class T, int L> __device__ __forceinline__ void rotate_queue(T (&q)[L])
+{
+    if (G % L == 0) return;
+    T t[L];
+#pragma unroll
+    for (int l = 0; l < L; l++) t[l] = q[(l + G) % L];
+#pragma unroll
+    for (int l = 0; l < L; l++) q[l] = t[l];
 }
 
 __device__ __forceinline__ float buoy(float r0, float r1, bool last)
@@ -420,6 +362,69 @@ __device__ __forceinline__ bool get_citem(const Grid &g, const Batch &b, int mod
         w -= n;
     }
     return false;
+}
+
+// Work list of a two-pass launch: chunks of y planes in order, within a chunk
+// the 32 x 16 tile columns, z fastest.  CTAs start with the item of their
+// index and then draw from a counter, so a slow item (CPML terms) delays one
+// CTA, and the CTAs sweep through the box together: what one reads as a halo
+// its neighbours have just read or written, in L2.  Short chunks (pick_chunk
+// in smi_stencil3d.cu) keep the sweep local, although a chunk reads 2N - 1
+// planes beyond its own and starts with a pipeline bubble.  Measured on 170 x
+// 340 x 340 points, adjoint velocity / pressure kernel: three items a CTA of
+// at least 24 planes, the columns with CPML terms first, 210 / 157 us (672 +
+// 633 MB read); 8-planes items in this order 166 / 131 us (505 + 500 MB).
+struct Sched {
+    int lo[3], hi[3], plo[3], phi[3];
+    int zbase, nzt, nxt, cy;   // tile columns, planes a chunk
+    int base, count;           // list positions of the shot's items
+    int s;
+};
+__device__ __forceinline__ void sched_shot(const Grid &g, const Batch &b, int mode, int step, int s, int base, int chunk,
+                                           Sched &d)
+{
+    d.s = s;
+    d.base = base;
+    d.plo[0] = d.plo[1] = d.plo[2] = 0;
+    d.phi[0] = d.phi[1] = d.phi[2] = -1;
+    item_box(g, b, mode, s, step, d.lo, d.hi, d.plo, d.phi);
+    d.count = 0;
+    d.cy = 1;
+    d.zbase = d.lo[0] & ~31;
+    const int ylen = d.hi[2] - d.lo[2] + 1;
+    d.nzt = d.hi[0] >= d.lo[0] ? (d.hi[0] - d.zbase) / TZ + 1 : 0;
+    d.nxt = d.hi[1] >= d.lo[1] ? (d.hi[1] - d.lo[1]) / TX + 1 : 0;
+    if (d.nzt == 0 || d.nxt == 0 || ylen <= 0) return;
+    const int nyc = (ylen + chunk - 1) / chunk;
+    d.cy = (ylen + nyc - 1) / nyc;
+    d.count = d.nzt * d.nxt * ((ylen + d.cy - 1) / d.cy);
+}
+
+// Item w of the launch (w grows from call to call); false past the end.
+__device__ __forceinline__ bool sched_item(const Grid &g, const Batch &b, int mode, int step, int w, int chunk, Sched &d,
+                                           Item &it)
+{
+    while (w >= d.base + d.count) {
+        if (d.s + 1 >= b.nshot) return false;
+        sched_shot(g, b, mode, step, d.s + 1, d.base + d.count, chunk, d);
+    }
+    int k = w - d.base;
+    const int nc = d.nzt * d.nxt, ci = k / nc;
+    k -= ci * nc;
+    const int xi = k / d.nzt, zi = k - xi * d.nzt;
+    it.s = d.s;
+    it.z0 = d.zbase + TZ * zi;
+    it.x0 = d.lo[1] + TX * xi;
+    it.ya = d.lo[2] + ci * d.cy;
+    it.yb = min(d.hi[2], it.ya + d.cy - 1);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        it.lo[a] = d.lo[a];
+        it.hi[a] = d.hi[a];
+        it.plo[a] = d.plo[a];
+        it.phi[a] = d.phi[a];
+    }
+    return true;
 }
 
 }  // namespace s3
