@@ -5,6 +5,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/smi.h"
@@ -118,6 +119,24 @@ void cpml_tables(int ne, int nb, double h, double vmax, double fm, double R, dou
 // Kaiser-windowed sinc stencil of a position (metres) on the extended grid;
 // false if it leaves the physical domain or its stencil leaves the grid.
 bool make_stencil(const Grid &g, const double pos[3], double kaiser_b, Stencil *st);
+// The same for the many positions of one call: the window's normalisation is
+// evaluated once, and the weights of a coordinate between nodes once however
+// many receivers (a line's depth, a carpet's rows, every shot) share it -- a
+// Bessel function a tap otherwise took 0.3 us a receiver, 4 us between nodes.
+class StencilMaker {
+public:
+    StencilMaker(const Grid &g, double kaiser_b);
+    bool make(const double pos[3], Stencil *st);
+
+private:
+    struct Taps {
+        float w[kMaxTaps];
+    };
+    bool taps(int ax, int first, double x, Taps &t) const;
+    const Grid &g_;
+    double b_, i0b_;
+    std::unordered_map<double, Taps> seen_[3];    // by extended-grid coordinate
+};
 
 // Decimated boundaries (Sec. 4.2): the band of step k*dr is stored for
 // k = 0..nsamp-1, and the band of step it is a Kaiser-windowed sinc (radius

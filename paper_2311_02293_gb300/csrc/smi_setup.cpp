@@ -82,62 +82,81 @@ void cpml_tables(int ne, int nb, double h, double vmax, double fm, double R, dou
 // (weight 1; sinc vanishes on every other node).  The nominal extent of a
 // stencil, used by the computing box, is base-ri+1 .. base+ri with base the
 // node (on a node) or floor(x) (off the nodes).
-bool make_stencil(const Grid &g, const double pos[3], double kaiser_b, Stencil *st)
+bool StencilMaker::make(const double pos[3], Stencil *st)
 {
-    const double i0b = std::cyl_bessel_i(0.0, kaiser_b);
     for (int ax = 0; ax < 3; ax++) {
         for (int k = 0; k < kMaxTaps; k++) st->w[ax][k] = 0.0f;
-        if (ax >= g.ndim) {
+        if (ax >= g_.ndim) {
             st->first[ax] = 0;
             st->cnt[ax] = 1;
             st->w[ax][0] = 1.0f;
             continue;
         }
-        const double rel = pos[ax] / g.h[ax];        // physical grid units
-        const int nphys = g.H[ax] - g.L[ax] + 1;
+        const double rel = pos[ax] / g_.h[ax];       // physical grid units
+        const int nphys = g_.H[ax] - g_.L[ax] + 1;
         if (!(rel >= -1e-6 && rel <= nphys - 1 + 1e-6)) return false;
-        const double x = rel + g.nb;
+        const double x = rel + g_.nb;
         const double nearest = std::nearbyint(x);
         const bool on_node = std::fabs(x - nearest) <= 1e-6;
         const int base = on_node ? (int)nearest : (int)std::floor(x);
         // the nominal 2*ri-node stencil must fit in the extended grid
-        if (base - g.ri + 1 < 0 || base + g.ri > g.ne[ax] - 1) return false;
-        // free surface on the top face (image-source form of Hicks 2002): a
-        // weight above the surface node L folds, negated, onto its mirror
-        // node 2L - i, and the weight at L is dropped (p = 0 there)
-        const bool fold = ax == 0 && g.freesurf;
+        if (base - g_.ri + 1 < 0 || base + g_.ri > g_.ne[ax] - 1) return false;
         if (on_node) {
+            // free surface: the weight at the surface node is dropped (p = 0 there)
             st->first[ax] = base;
             st->cnt[ax] = 1;
-            st->w[ax][0] = (fold && base == g.L[0]) ? 0.0f : 1.0f;
-        } else {
-            st->first[ax] = base - g.ri + 1;
-            st->cnt[ax] = 2 * g.ri;
-            double wd[kMaxTaps] = {0};
-            for (int k = 0; k < 2 * g.ri; k++) {
-                const double u = (st->first[ax] + k) - x;
-                const double sinc = std::sin(M_PI * u) / (M_PI * u);
-                const double q = u / g.ri;
-                const double arg = 1.0 - q * q;
-                const double win = arg > 0.0 ? std::cyl_bessel_i(0.0, kaiser_b * std::sqrt(arg)) / i0b : 0.0;
-                wd[k] = sinc * win;
-            }
-            if (fold) {
-                for (int k = 0; k < 2 * g.ri; k++) {
-                    const int node = st->first[ax] + k;
-                    if (node >= g.L[0]) continue;
-                    const int km = 2 * g.L[0] - node - st->first[ax];
-                    if (km >= 2 * g.ri) return false;
-                    wd[km] -= wd[k];
-                    wd[k] = 0.0;
-                }
-                const int k0 = g.L[0] - st->first[ax];
-                if (k0 >= 0 && k0 < 2 * g.ri) wd[k0] = 0.0;
-            }
-            for (int k = 0; k < 2 * g.ri; k++) st->w[ax][k] = (float)wd[k];
+            st->w[ax][0] = (ax == 0 && g_.freesurf && base == g_.L[0]) ? 0.0f : 1.0f;
+            continue;
         }
+        st->first[ax] = base - g_.ri + 1;
+        st->cnt[ax] = 2 * g_.ri;
+        auto hit = seen_[ax].find(x);
+        if (hit == seen_[ax].end()) {
+            Taps t;
+            if (!taps(ax, st->first[ax], x, t)) return false;
+            hit = seen_[ax].emplace(x, t).first;
+        }
+        for (int k = 0; k < 2 * g_.ri; k++) st->w[ax][k] = hit->second.w[k];
     }
     return true;
+}
+
+// Off-node weights along one axis.
+bool StencilMaker::taps(int ax, int first, double x, Taps &t) const
+{
+    double wd[kMaxTaps] = {0};
+    for (int k = 0; k < 2 * g_.ri; k++) {
+        const double u = (first + k) - x;
+        const double sinc = std::sin(M_PI * u) / (M_PI * u);
+        const double q = u / g_.ri;
+        const double arg = 1.0 - q * q;
+        const double win = arg > 0.0 ? std::cyl_bessel_i(0.0, b_ * std::sqrt(arg)) / i0b_ : 0.0;
+        wd[k] = sinc * win;
+    }
+    // free surface on the top face (image-source form of Hicks 2002): a
+    // weight above the surface node L folds, negated, onto its mirror
+    // node 2L - i, and the weight at L is dropped (p = 0 there)
+    if (ax == 0 && g_.freesurf) {
+        for (int k = 0; k < 2 * g_.ri; k++) {
+            const int node = first + k;
+            if (node >= g_.L[0]) continue;
+            const int km = 2 * g_.L[0] - node - first;
+            if (km >= 2 * g_.ri) return false;
+            wd[km] -= wd[k];
+            wd[k] = 0.0;
+        }
+        const int k0 = g_.L[0] - first;
+        if (k0 >= 0 && k0 < 2 * g_.ri) wd[k0] = 0.0;
+    }
+    for (int k = 0; k < 2 * g_.ri; k++) t.w[k] = (float)wd[k];
+    return true;
+}
+
+StencilMaker::StencilMaker(const Grid &g, double kaiser_b) : g_(g), b_(kaiser_b), i0b_(std::cyl_bessel_i(0.0, kaiser_b)) {}
+
+bool make_stencil(const Grid &g, const double pos[3], double kaiser_b, Stencil *st)
+{
+    return StencilMaker(g, kaiser_b).make(pos, st);
 }
 
 TimeWeights time_weights(int it, int dr, int nsamp)
