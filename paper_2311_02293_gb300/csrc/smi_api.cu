@@ -153,6 +153,7 @@ struct Setup {
     bool fused = false;                    // 3D forward / adjoint steps by the single-pass kernel
     bool tile3 = false;                    // 3D forward / adjoint steps by the two-pass tile kernels
     bool fast2 = false;                    // 2D steps by the single-launch kernels
+    bool padacc = false;                   // image accumulators in the fields' padded layout (tile kernels)
     bool pingpong = false;                 // a step reads one set of state arrays and writes the other
     long long nrec_total = 0;
     size_t setup_bytes = 0;                // sizes-only set-up: estimated bytes of the set-up arena
@@ -292,6 +293,7 @@ int validate_and_setup(const smi_model *m, const smi_geometry *geo, const smi_wa
     S.tile3 = o->kernels != SMI_KERNELS_GENERIC && !S.fused && stencil3d_supported(g);
     S.fast2 = o->kernels != SMI_KERNELS_GENERIC && stencil2d_supported(g);
     S.pingpong = S.fused || S.fast2;
+    S.padacc = S.fast2 || S.fused || S.tile3;
     if (S.fast2 || S.tile3) set_tile_slabs(g);
 
     // boundary bands: v_a on the 2N-1 half nodes straddling each face of the
@@ -482,7 +484,7 @@ size_t per_shot_bytes(const Setup &S, int kind)
             if (S.fast2 || S.tile3) b += (size_t)S.nsamp * 6 * 4;          // and largest magnitudes
         }
         if (S.dr > 1) b += fields;                                     // state kept during the continuation
-        b += (size_t)g.nphys * 4 * (kind == 1 && S.img_norm ? 2 : 1);  // accumulator (+ illumination)
+        b += (size_t)(g.nphys + (S.padacc ? g.ntot : 0)) * 4 * (kind == 1 && S.img_norm ? 2 : 1);  // accumulator (+ illumination)
         if (S.rho_grad) b += (size_t)g.ndim * g.ntot * 4;              // velocities of the previous step
         b += (size_t)S.nt * maxrec * 4 * 2;                            // seis + residual
     }
@@ -716,7 +718,9 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             float *seis = out_seis ? d_seis_out + (size_t)S.nt * S.rec_offset[s0]
                                    : ba.get<float>(std::max<long long>(1, batch_seis));
             Bands bd = S.bands;
-            float *res = nullptr, *acc = nullptr, *keep = nullptr;
+            float *res = nullptr, *acc = nullptr, *keep = nullptr, *accc = nullptr;
+            const size_t nacc = (size_t)nb_shot * (norm ? 2 : 1);      // accumulators: [images | illuminations]
+            const size_t acc_n = S.padacc ? (size_t)g.ntot : (size_t)g.nphys;   // floats of each
             unsigned *norm_mx = nullptr;
             double *partials = nullptr, *part = nullptr;
             const int npart = 256;
@@ -726,6 +730,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 bd = T.bd;
                 res = T.res;
                 acc = T.acc;
+                if (S.padacc) accc = ba.get<float>((size_t)g.nphys * nacc);
                 partials = T.partials;
             } else if (kind != 0) {
                 for (int k = 0; k < (pp ? 2 : 1); k++) {   // the adjoint reuses the forward's memory variables
@@ -742,7 +747,8 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     bd.data = ba.raw((size_t)nb_shot * S.nsamp * bd.count * band_bytes(bd.prec));
                     bd.scale = ba.get<float>((size_t)nb_shot * S.nsamp * 6);
                     if (S.dr > 1) keep = ba.get<float>((size_t)(1 + g.ndim) * g.ntot * nb_shot);
-                    acc = ba.get<float>((size_t)g.nphys * nb_shot * (norm ? 2 : 1));   // [images | illuminations]
+                    acc = ba.get<float>(acc_n * nacc);
+                    if (S.padacc && kind != 6) accc = ba.get<float>((size_t)g.nphys * nacc);   // the physical nodes alone
                 } else {
                     part = ba.get<double>((size_t)nb_shot * S.nt);
                 }
@@ -953,7 +959,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 launch_zero(lc, F2.p, fbytes);
                 for (int a = 0; a < g.ndim; a++) launch_zero(lc, F2.v[a], fbytes);
             }
-            if (acc) launch_zero(lc, acc, sizeof(float) * g.nphys * nb_shot * (norm ? 2 : 1));
+            if (acc) launch_zero(lc, acc, sizeof(float) * acc_n * nacc);
             if (S.rho_grad)
                 for (int a = 0; a < g.ndim; a++)
                     cudaMemcpyAsync(R.vprev[a], F.v[a], fbytes, cudaMemcpyDeviceToDevice, st);
@@ -1063,6 +1069,10 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             if (kind == 5) {
                 launch_sum_series(lc, part, nb_shot, S.nt, d_series, s0 > 0);
                 continue;
+            }
+            if (S.padacc) {
+                launch_unpad(lc, g, acc, nacc, accc);
+                acc = accc;
             }
             launch_nonfinite(lc, acc, g.nphys * nb_shot, d_flag);
             if (per_shot)

@@ -213,6 +213,8 @@ void launch_recon_p(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f
                     float src_scale, long long work);
 void launch_recon_v(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, int it, long long work);
 
+// The physical nodes of n arrays in the fields' padded layout: out[n][nphys].
+void launch_unpad(const LaunchCtx &lc, const Grid &g, const float *a, size_t n, float *out);
 void launch_reduce_shots(const LaunchCtx &lc, const Grid &g, const float *acc, int nshot,
                          float *out, int accumulate);
 // Normalised image: acc holds [nshot][nphys] images then [nshot][nphys]

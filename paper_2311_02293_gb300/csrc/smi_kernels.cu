@@ -696,6 +696,18 @@ __global__ void k_sum_partials(const double *partials, int n, double *out)
     *out += s;
 }
 
+// out[k] = the physical nodes of array k in the fields' padded layout.
+__global__ void k_unpad(Grid g, const float *a, long long n, float *out)
+{
+    const int n0 = g.H[0] - g.L[0] + 1, n1 = g.H[1] - g.L[1] + 1;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n * g.nphys;
+         t += (long long)gridDim.x * blockDim.x) {
+        const long long k = t / g.nphys, u = t - k * g.nphys, q = u / n0;
+        const int i0 = (int)(u - q * n0), i1 = (int)(q % n1), i2 = (int)(q / n1);
+        out[t] = a[k * g.ntot + gidx(g, g.L[0] + i0, g.L[1] + i1, g.L[2] + i2)];
+    }
+}
+
 // out[x] (+)= sum_s acc[s][x], shots added in order (deterministic).
 __global__ void k_reduce_shots(const float *acc, long long n, int nshot, float *out, int accumulate)
 {
@@ -1121,6 +1133,12 @@ void launch_dot(const LaunchCtx &lc, const float *a, const float *b, long long n
 void launch_sum_partials(const LaunchCtx &lc, const double *partials, int npart, double *out)
 {
     k_sum_partials<<<1, 32, 0, S(lc)>>>(partials, npart, out);
+    ++*lc.launches;
+}
+
+void launch_unpad(const LaunchCtx &lc, const Grid &g, const float *a, size_t n, float *out)
+{
+    k_unpad<<<blocks_for(g.nphys * (long long)n), kThreads, 0, S(lc)>>>(g, a, (long long)n, out);
     ++*lc.launches;
 }
 

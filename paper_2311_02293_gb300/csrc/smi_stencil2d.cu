@@ -28,8 +28,11 @@
 // velocity and a pressure pass move 36, and a step is one launch instead of
 // four to nine.  Against the two-pass kernels with their own launches for
 // sources, receivers and bands (GB300): 201 x 201 order 4 forward, one shot,
-// 16.9 -> 3.7 us a step; 257 x 903 order 8 gradient, one shot, 16-bit
-// boundaries, 69.5 -> 20.6 us a step pair; 301 x 1001, 40 shots, 315 -> 223.
+// 16.9 -> 3.2 us a step; 257 x 903 order 8 gradient, one shot, 16-bit
+// boundaries, 69.5 -> 18.6 us a step pair; 301 x 1001, 40 shots, 315 -> 165.
+// Most tiles of a survey meet no slab, box edge, band or source: they run a
+// body without tests or memory variables, in packed pairs (40 shots, whole
+// grid: forward 172 -> 153 us, reverse 353 -> 273).
 //
 // Rows are padded to px (a multiple of 8), the padding of the fields holds
 // zeros and TMA fills zeros outside the grid: the scheme's zero values.
@@ -44,6 +47,7 @@
 #include "smi_band.h"
 #include "smi_box.h"
 #include "smi_internal.h"
+#include "smi_pack.h"
 #include "smi_pdl.h"
 #include "smi_slab.h"
 #include "smi_stencil2d.h"
@@ -62,6 +66,15 @@ using s3::mbar_wait;
 using s3::put;
 using s3::tma4;
 
+// Resident blocks a SM that the register budget allows.  Wide tiles (many
+// shots): enough blocks to hide the load phase of one behind another's
+// arithmetic, 3 forward and 4 reverse (80 and 64 registers, some spilled; 40
+// shots 301 x 1001, 800 steps: reverse at 3 / 4 / 5 blocks 140 / 132 / 139 ms;
+// six-shot forward line at 3 / 4 / 5 blocks 8.1 / 8.9 / 10.2 ms).  Narrow tiles
+// (small launches) are alone on their SM: no spills.
+constexpr int fwd_blocks(int tx) { return tx == 32 ? 3 : 4; }
+constexpr int rev_blocks(int) { return 4; }
+
 enum { FWD = 0, ADJ = 1 };
 
 // Shared tiles (floats).  Forward / adjoint: pressure rows x0-2N+1 ..
@@ -79,52 +92,51 @@ template <int N, int TX> struct Lay {
     static constexpr int MAXF = FA > REC ? FA : REC;
 };
 
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ void st4(float *p, const float (&a)[4])
+// rho of the quad one node up the z axis from r0 = rho of the quad (the row
+// padding repeats the last node: 2 / (rho + rho) = 1 / rho there).
+__device__ __forceinline__ Q4 rho_up(const Grid &g, int oz, int k, const Q4 &r0)
 {
-    *reinterpret_cast<float4 *>(p) = make_float4(a[0], a[1], a[2], a[3]);
+    float a[4];
+    split(r0, a);
+    return quad({a[1], a[2], a[3], oz + 4 < g.px ? g.rho[k + 4] : a[3]});
 }
-__device__ __forceinline__ void window(float (&W)[12], const float *row)
+// v where the quad's nodes lie in [lo, hi] along z (and x in), else 0.
+__device__ __forceinline__ Q4 masked(float v, int oz, bool x_in, int lo, int hi)
 {
+    float a[4];
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const float4 a = ld4(row + 4 * k);
-        W[4 * k] = a.x;
-        W[4 * k + 1] = a.y;
-        W[4 * k + 2] = a.z;
-        W[4 * k + 3] = a.w;
+    for (int r = 0; r < 4; r++) a[r] = x_in && in_range(oz + r, lo, hi) ? v : 0.0f;
+    return quad(a);
+}
+// CPML coefficients of a quad along z, 0 where m is 0.
+__device__ __forceinline__ void zcoefs(const float *tab, int oz, const Q4 &m, float (&c)[4])
+{
+    float a[4];
+    split(m, a);
+    put(c, s3::ldg4(tab + oz));
+#pragma unroll
+    for (int r = 0; r < 4; r++) c[r] = a[r] != 0.0f ? c[r] : 0.0f;
+}
+__device__ __forceinline__ void xcoefs(float v, const Q4 &m, float (&c)[4])
+{
+    float a[4];
+    split(m, a);
+#pragma unroll
+    for (int r = 0; r < 4; r++) c[r] = a[r] != 0.0f ? v : 0.0f;
+}
+// v - b D (forward) or, b negative, v + b D (adjoint).
+template <int MODE> __device__ __forceinline__ Q4 update(const Q4 &v, const Q4 &b, const Q4 &D)
+{
+    if (MODE == FWD) {
+        float x[4], c[4], d[4];
+        split(v, x);
+        split(b, c);
+        split(D, d);
+#pragma unroll
+        for (int r = 0; r < 4; r++) x[r] = __fmaf_rn(-c[r], d[r], x[r]);
+        return quad(x);
     }
-}
-// Derivative along z of the quad in the middle of a 12-value window, p nodes
-// to v nodes (UP) or back.
-template <int N, bool UP> __device__ __forceinline__ void dz4(const Grid &g, const float (&W)[12], float (&D)[4])
-{
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-        float d = 0.0f;
-#pragma unroll
-        for (int l = 1; l <= N; l++)
-            d += g.c[0][l - 1] * (UP ? W[4 + r + l] - W[4 + r - l + 1] : W[4 + r + l - 1] - W[4 + r - l]);
-        D[r] = d;
-    }
-}
-__device__ __forceinline__ void buoy4(const float (&r0)[4], const float (&r1)[4], float (&b)[4])
-{
-    // fast reciprocal-based division: a few ulp, far below the FP32 scheme error
-#pragma unroll
-    for (int r = 0; r < 4; r++) b[r] = __fdividef(2.0f, r0[r] + r1[r]);
-}
-// rho of the quad and of the quad one node up the axis (the last node's
-// neighbour is itself: 2 / (rho + rho) = 1 / rho).
-__device__ __forceinline__ void rho_z(const Grid &g, int oz, int k, float (&r0)[4], float (&r1)[4])
-{
-    put(r0, ld4(g.rho + k));
-    const float up = oz + 4 < g.ne[0] ? g.rho[k + 4] : r0[3];
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const float nx = r < 3 ? r0[r + 1] : up;
-        r1[r] = oz + r + 1 < g.ne[0] ? nx : r0[r];
-    }
+    return fmaq(b, D, v);
 }
 
 // The block's share of a step.
@@ -141,16 +153,24 @@ __device__ __forceinline__ SrcBox src_box(const Batch &b, int s)
     const Stencil &st = b.src[s];
     return {st.first[0], st.first[1], st.cnt[0], st.cnt[1]};
 }
-__device__ __forceinline__ void add_source(const Batch &b, const SrcBox &sb, int s, int oz, int ox, float amp, float (&p)[4])
+// Whether the stencil meets nodes [z0, z1] x [x0, x1].
+__device__ __forceinline__ bool src_near(const SrcBox &sb, int z0, int z1, int x0, int x1)
+{
+    return sb.f0 <= z1 && sb.f0 + sb.n0 - 1 >= z0 && sb.f1 <= x1 && sb.f1 + sb.n1 - 1 >= x0;
+}
+__device__ __forceinline__ void add_source(const Batch &b, const SrcBox &sb, int s, int oz, int ox, float amp, Q4 &q)
 {
     const int t1 = ox - sb.f1;
     if (t1 < 0 || t1 >= sb.n1 || oz + 3 < sb.f0 || oz >= sb.f0 + sb.n0) return;
+    float p[4];
+    split(q, p);
     const Stencil &st = b.src[s];
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int t0 = oz + r - sb.f0;
         if (t0 >= 0 && t0 < sb.n0) p[r] += amp * st.w[0][t0] * st.w[1][t1] * st.w[2][0];
     }
+    q = quad(p);
 }
 
 // Boundary regions of axis A at node (z, x): side 0 / 1, or -1.
@@ -184,8 +204,10 @@ template <int TX> __device__ __forceinline__ bool band_tile(const Bands &bd, int
 // maps to 2^14 (FP16) or 1 (BF16).
 template <int A>
 __device__ __forceinline__ void band_store(const Bands &bd, const float (&scale)[4], int s, int it, int oz, int x,
-                                           const float (&v)[4])
+                                           const Q4 &q)
 {
+    float v[4];
+    split(q, v);
 #pragma unroll
     for (int r = 0; r < 4; r++) {
         const int sd = band_side<A>(bd, oz + r, x);
@@ -201,33 +223,30 @@ __device__ __forceinline__ void band_store(const Bands &bd, const float (&scale)
         }
     }
 }
-// One velocity quad of axis A from the tile's pressure: v -= dt b D at the
-// nodes of the box, memory variable m of the v grid, and the operand R that
-// the pressure update differentiates (forward: v; adjoint: v + e).
-// D: derivative of the axis; B, Av: the quad's CPML coefficients.
+// One velocity quad: v -+ b D, the memory variable m of the v grid (B, A: its
+// coefficients), and the operand that the pressure update differentiates
+// (forward: v; adjoint: v + e), returned.
 template <int MODE>
-__device__ __forceinline__ void vel_quad(float dt, const float (&D)[4], const float (&b)[4], const bool (&in)[4],
-                                         bool slab, const float (&B)[4], const float (&Av)[4], float (&m)[4],
-                                         float (&v)[4], float (&R)[4])
+__device__ __forceinline__ Q4 vel_quad(const Q4 &b, Q4 D, bool slab, const float (&B)[4], const float (&A)[4], float (&m)[4],
+                                       Q4 &v)
 {
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-        float d = D[r];
-        if (MODE == FWD && slab && in[r]) {
-            m[r] = slab_recur(B[r], m[r], Av[r], d);
-            d += m[r];
-        }
-        if (in[r]) v[r] -= dt * b[r] * d;
-        R[r] = v[r];
-        if (MODE == ADJ && slab) {
-            if (in[r]) m[r] = slab_recur(B[r], m[r], Av[r], v[r]);
-            R[r] += m[r];
-        }
+    if (MODE == FWD && slab) {
+        recur4(B, A, m, D);
+        D = addq(D, quad(m));
     }
+    v = update<MODE>(v, b, D);
+    if (MODE == ADJ && slab) {
+        recur4(B, A, m, v);
+        return addq(v, quad(m));
+    }
+    return v;
 }
 
-// Forward or adjoint step of one tile.  sm: the block's shared tiles.
-template <int N, int MODE, int TX>
+// Forward or adjoint step of one tile.  sm: the block's shared tiles.  FAST:
+// a tile whose nodes and halo lie inside the box and away from the slabs, the
+// free surface, the source and the bands (tile_fast): no tests, no memory
+// variables.
+template <int N, int MODE, int TX, bool FAST>
 __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g, const Batch &b, const Fields &c,
                                           const Fields &n, const Tile &t, int step, const float *stf, float src_scale,
                                           const Bands &bd, const Save2 &save, float *sm, uint64_t *bar,
@@ -239,10 +258,10 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
     const int tid = threadIdx.x, tzi = tid & 7, txi = tid >> 3;
     const int s = t.s, z0 = t.z0, x0 = t.x0;
     const int oz = z0 + 4 * tzi, ox = x0 + txi, k = oz + g.px * ox;
-    const bool own = oz < g.ne[0] && ox < g.ne[1];
+    const bool own = FAST || (oz < g.ne[0] && ox < g.ne[1]);
     const long long sh = (long long)s * g.ntot;
     const long long so0 = (long long)s * g.slab_n[0], so1 = (long long)s * g.slab_n[1];
-    const float dt = g.dt;
+    const float dt2 = MODE == ADJ ? -2.0f * g.dt : 2.0f * g.dt;
 
     // extra velocity quads of the halo: threads below 2 TX take v_z on either
     // side along z, the next 8 (2N - 1) take v_x on either side along x
@@ -258,38 +277,35 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
         ex = rr < N ? x0 - N + rr : x0 + TX + rr - N;
         extra = true;
     }
-    const bool ein = extra && ez >= 0 && ez < g.ne[0] && ex >= 0 && ex < g.ne[1];
+    const bool ein = extra && (FAST || (ez >= 0 && ez < g.ne[0] && ex >= 0 && ex < g.ne[1]));
     const int ke = ez + g.px * ex;
 
     // ---- what no earlier step writes: model, coefficients, source stencil ----
-    float bz[4], bx[4], be[4], Kv[4];
-    {
-        float r0[4] = {1.0f, 1.0f, 1.0f, 1.0f}, r1[4] = {1.0f, 1.0f, 1.0f, 1.0f};
-        if (own) rho_z(g, oz, k, r0, r1);
-        buoy4(r0, r1, bz);
-        if (own && ox + 1 < g.ne[1]) put(r1, ld4(g.rho + k + g.px));
-        else for (int r = 0; r < 4; r++) r1[r] = r0[r];
-        buoy4(r0, r1, bx);
-        for (int r = 0; r < 4; r++) Kv[r] = 0.0f;
-        if (own) put(Kv, ld4(g.K + k));
-        if (ein) {
-            if (exz) {
-                rho_z(g, ez, ke, r0, r1);
-            } else {
-                put(r0, ld4(g.rho + ke));
-                if (ex + 1 < g.ne[1]) put(r1, ld4(g.rho + ke + g.px));
-                else for (int r = 0; r < 4; r++) r1[r] = r0[r];
-            }
-        }
-        buoy4(r0, r1, be);
+    // buoyancies: 2 dt / (rho + rho') at the nodes of the box, else 0
+    const Q4 two = quad({dt2, dt2, dt2, dt2});
+    Q4 in = two, ie = two;
+    if (!FAST) {
+        in = masked(dt2, oz, own && in_range(ox, t.lo[1], t.hi[1]), t.lo[0], t.hi[0]);
+        ie = masked(dt2, ez, ein && in_range(ex, t.lo[1], t.hi[1]), t.lo[0], t.hi[0]);
     }
-    const int zq = own ? zslab_quad(g, oz) : -1, xq = own ? slab_row(g, 1, ox) : -1;
-    const int eq = ein ? (exz ? zslab_quad(g, ez) : slab_row(g, 1, ex)) : -1;
+    Q4 bz = zeroq(), bx = zeroq(), be = zeroq(), Kv = zeroq();
+    if (own) {
+        const Q4 r0 = ldq(g.rho + k);
+        bz = buoyq(in, r0, rho_up(g, oz, k, r0));
+        bx = buoyq(in, r0, FAST || ox + 1 < g.ne[1] ? ldq(g.rho + k + g.px) : r0);
+        Kv = ldq(g.K + k);
+    }
+    if (ein) {
+        const Q4 r0 = ldq(g.rho + ke);
+        be = buoyq(ie, r0, exz ? rho_up(g, ez, ke, r0) : (FAST || ex + 1 < g.ne[1] ? ldq(g.rho + ke + g.px) : r0));
+    }
+    const int zq = !FAST && own ? zslab_quad(g, oz) : -1, xq = !FAST && own ? slab_row(g, 1, ox) : -1;
+    const int eq = !FAST && ein ? (exz ? zslab_quad(g, ez) : slab_row(g, 1, ex)) : -1;
     const long long zo = so0 + zq + (long long)g.zp * ox, xo = so1 + (long long)g.px * xq + oz;
     const long long eo = exz ? so0 + eq + (long long)g.zp * ex : so1 + (long long)g.px * eq + ez;
     SrcBox sb{0, 0, 0, 0};
     float amp = 0.0f;
-    if (MODE == FWD && stf) {
+    if (!FAST && MODE == FWD && stf) {
         sb = src_box(b, s);
         amp = src_scale * stf[step];
     }
@@ -303,24 +319,27 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
         tma4(sp, tm_p, z0 - 8, x0 - HX, 0, s, bar);
     }
     // ---- the old state ----
-    float vz[4] = {}, vx[4] = {}, ve[4] = {}, mz[4] = {}, mx[4] = {}, me[4] = {}, pz[4] = {}, px[4] = {};
+    Q4 vz = zeroq(), vx = zeroq(), ve = zeroq();
+    float mz[4] = {}, mx[4] = {}, me[4] = {}, pz[4] = {}, px[4] = {};
     if (own) {
-        put(vz, ld4(c.v[0] + sh + k));
-        put(vx, ld4(c.v[1] + sh + k));
+        vz = ldq(c.v[0] + sh + k);
+        vx = ldq(c.v[1] + sh + k);
     }
-    if (ein) put(ve, ld4((exz ? c.v[0] : c.v[1]) + sh + ke));
-    if (zq >= 0) {
-        put(mz, ld4(c.psip[0] + zo));
-        put(pz, ld4(c.psiv[0] + zo));
+    if (ein) ve = ldq((exz ? c.v[0] : c.v[1]) + sh + ke);
+    if (!FAST) {
+        if (zq >= 0) {
+            put(mz, s3::ldg4(c.psip[0] + zo));
+            put(pz, s3::ldg4(c.psiv[0] + zo));
+        }
+        if (xq >= 0) {
+            put(mx, s3::ldg4(c.psip[1] + xo));
+            put(px, s3::ldg4(c.psiv[1] + xo));
+        }
+        if (eq >= 0) put(me, s3::ldg4((exz ? c.psip[0] : c.psip[1]) + eo));
     }
-    if (xq >= 0) {
-        put(mx, ld4(c.psip[1] + xo));
-        put(px, ld4(c.psiv[1] + xo));
-    }
-    if (eq >= 0) put(me, ld4((exz ? c.psip[0] : c.psip[1]) + eo));
 
-    const bool first = blockIdx.x == 0 && blockIdx.y == 0;      // writes the shot's scales
-    if (MODE == FWD && save.sample >= 0 && (first || band_tile<TX>(bd, z0, x0))) {
+    const bool first = t.z0 == (t.lo[0] & ~3) && t.x0 == t.lo[1];      // writes the shot's scales
+    if (MODE == FWD && save.sample >= 0 && (first || (!FAST && band_tile<TX>(bd, z0, x0)))) {
         float scale[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         if (bd.prec != SMI_PREC_F32) {
 #pragma unroll
@@ -330,7 +349,7 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
                 if (first && tid == q) bd.scale[((long long)s * bd.nt + save.sample) * 6 + q] = scale[q];
             }
         }
-        if (own) {
+        if (!FAST && own) {
             band_store<0>(bd, scale, s, save.sample, oz, ox, vz);
             band_store<1>(bd, scale, s, save.sample, oz, ox, vx);
         }
@@ -340,105 +359,73 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
         if (tid == 0) atomicOr(err, 1u);
         mbar_wait(bar, 0);
     }
+    float *const pz_own = svz + txi * La::VW + 4 * tzi + 4, *const px_own = svx + (txi + N) * 32 + 4 * tzi;
 
     // ---- velocities: own quads, then the halo's ----
-    const bool inx = in_range(ox, t.lo[1], t.hi[1]);
-    bool in[4];
-#pragma unroll
-    for (int r = 0; r < 4; r++) in[r] = inx && in_range(oz + r, t.lo[0], t.hi[0]);
-    auto z_deriv = [&](int qz, int qx, float (&D)[4]) {
+    auto z_deriv = [&](int qz, int qx) {
         float W[12];
         window(W, sp + (qx - x0 + HX) * La::PW + (qz - z0) + 4);
-        if (MODE == ADJ && (qz - 4 < g.zlo || qz + 7 >= g.zhi) && qx >= 0 && qx < g.ne[1]) {
+        if (!FAST && MODE == ADJ && (qz - 4 < g.zlo || qz + 7 >= g.zhi) && qx >= 0 && qx < g.ne[1]) {
 #pragma unroll
             for (int q = 0; q < 3; q++) {
                 const int e = zslab_quad(g, qz - 4 + 4 * q);
                 if (e < 0) continue;
                 float a[4];
-                put(a, ld4(c.psiv[0] + so0 + e + (long long)g.zp * qx));
+                put(a, s3::ldg4(c.psiv[0] + so0 + e + (long long)g.zp * qx));
 #pragma unroll
                 for (int r = 0; r < 4; r++) W[4 * q + r] += a[r];
             }
         }
-        dz4<N, true>(g, W, D);
+        return dz4<N, true>(g, W);
     };
-    auto x_deriv = [&](int qz, int qx, float (&D)[4]) {
-#pragma unroll
-        for (int r = 0; r < 4; r++) D[r] = 0.0f;
-        const bool near = MODE == ADJ && (qx - N + 1 < g.nb || qx + N >= g.ne[1] - g.nb - 1);
+    auto x_deriv = [&](int qz, int qx) {
+        Q4 D = zeroq();
+        const bool near = !FAST && MODE == ADJ && (qx - N + 1 < g.xlo || qx + N >= g.xhi) && qz < g.ne[0];
+        const float *row = sp + (qx - x0 + HX) * La::PW + (qz - z0) + 8;
 #pragma unroll
         for (int l = 1; l <= N; l++) {
-            float a[4], d[4];
-            const float *row = sp + (qx - x0 + HX) * La::PW + (qz - z0) + 8;
-            put(a, ld4(row + l * La::PW));
-            put(d, ld4(row - (l - 1) * La::PW));
-            if (near && qz < g.ne[0]) {
+            Q4 a = ldq(row + l * La::PW), d = ldq(row - (l - 1) * La::PW);
+            if (near) {
                 const int ja = slab_row(g, 1, qx + l), jd = slab_row(g, 1, qx - l + 1);
-                float e[4];
-                if (ja >= 0) {
-                    put(e, ld4(c.psiv[1] + so1 + (long long)g.px * ja + qz));
-#pragma unroll
-                    for (int r = 0; r < 4; r++) a[r] += e[r];
-                }
-                if (jd >= 0) {
-                    put(e, ld4(c.psiv[1] + so1 + (long long)g.px * jd + qz));
-#pragma unroll
-                    for (int r = 0; r < 4; r++) d[r] += e[r];
-                }
+                if (ja >= 0) a = addq(a, ldq(c.psiv[1] + so1 + (long long)g.px * ja + qz));
+                if (jd >= 0) d = addq(d, ldq(c.psiv[1] + so1 + (long long)g.px * jd + qz));
             }
-#pragma unroll
-            for (int r = 0; r < 4; r++) D[r] += g.c[1][l - 1] * (a[r] - d[r]);
+            D = tap(D, g.c[1][l - 1], a, d);
         }
+        return D;
     };
     {
-        float D[4], R[4], B[4] = {}, Av[4] = {};
-        z_deriv(oz, ox, D);
-        if (zq >= 0) {
-            put(B, ld4(g.cvb[0] + oz));
-            put(Av, ld4(g.cva[0] + oz));
+        float B[4] = {}, A[4] = {};
+        if (!FAST && zq >= 0) {
+            zcoefs(g.cvb[0], oz, in, B);
+            zcoefs(g.cva[0], oz, in, A);
         }
-        vel_quad<MODE>(dt, D, bz, in, zq >= 0, B, Av, mz, vz, R);
-        st4(svz + txi * La::VW + 4 * tzi + 4, R);
-        x_deriv(oz, ox, D);
-        if (xq >= 0) {
-            const float bb = g.cvb[1][ox], aa = g.cva[1][ox];
-#pragma unroll
-            for (int r = 0; r < 4; r++) {
-                B[r] = bb;
-                Av[r] = aa;
-            }
+        stq(pz_own, vel_quad<MODE>(bz, z_deriv(oz, ox), zq >= 0, B, A, mz, vz));
+        if (!FAST && xq >= 0) {
+            xcoefs(g.cvb[1][ox], in, B);
+            xcoefs(g.cva[1][ox], in, A);
         }
-        vel_quad<MODE>(dt, D, bx, in, xq >= 0, B, Av, mx, vx, R);
-        st4(svx + (txi + N) * 32 + 4 * tzi, R);
+        stq(px_own, vel_quad<MODE>(bx, x_deriv(oz, ox), xq >= 0, B, A, mx, vx));
     }
     if (extra) {
-        float D[4], R[4], B[4] = {}, Av[4] = {};
-        bool ie[4];
-        const bool iex = in_range(ex, t.lo[1], t.hi[1]);
-#pragma unroll
-        for (int r = 0; r < 4; r++) ie[r] = iex && in_range(ez + r, t.lo[0], t.hi[0]);
+        float B[4] = {}, A[4] = {};
+        float *const pe = exz ? svz + (ex - x0) * La::VW + (ez - z0 + 4) : svx + (ex - x0 + N) * 32 + (ez - z0);
         if (exz) {
-            z_deriv(ez, ex, D);
-            if (eq >= 0) {
-                put(B, ld4(g.cvb[0] + ez));
-                put(Av, ld4(g.cva[0] + ez));
+            if (!FAST && eq >= 0) {
+                zcoefs(g.cvb[0], ez, ie, B);
+                zcoefs(g.cva[0], ez, ie, A);
             }
+            stq(pe, vel_quad<MODE>(be, z_deriv(ez, ex), eq >= 0, B, A, me, ve));
         } else {
-            x_deriv(ez, ex, D);
-            if (eq >= 0) {
-#pragma unroll
-                for (int r = 0; r < 4; r++) {
-                    B[r] = g.cvb[1][ex];
-                    Av[r] = g.cva[1][ex];
-                }
+            if (!FAST && eq >= 0) {
+                xcoefs(g.cvb[1][ex], ie, B);
+                xcoefs(g.cva[1][ex], ie, A);
             }
+            stq(pe, vel_quad<MODE>(be, x_deriv(ez, ex), eq >= 0, B, A, me, ve));
         }
-        vel_quad<MODE>(dt, D, be, ie, eq >= 0, B, Av, me, ve, R);
-        if (exz) st4(svz + (ex - x0) * La::VW + (ez - z0 + 4), R);
-        else st4(svx + (ex - x0 + N) * 32 + (ez - z0), R);
     }
     __syncthreads();
-    if (g.freesurf && z0 - 4 < g.L[0]) {
+    if (!FAST && g.freesurf && z0 - 4 < g.L[0]) {
         // free surface (image method): half node L-1-j mirrors L+j; the adjoint folds it there.  The box
         // starts at L-N or below the image rows, so a tile that holds an image row holds its mirror; the
         // memory variables of these rows are zero (no absorption at the top).
@@ -455,105 +442,87 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
             }
         }
         __syncthreads();
-        if (oz < L + N) put(vz, ld4(svz + txi * La::VW + 4 * tzi + 4));
+        if (oz < L + N) vz = ldq(pz_own);
     }
 
     // ---- pressure ----
-    float pv[4], div[4];
-    put(pv, ld4(sp + (txi + HX) * La::PW + 4 * tzi + 8));
+    Q4 pv = ldq(sp + (txi + HX) * La::PW + 4 * tzi + 8);
     {
-        float W[12], D[4];
+        float W[12], B[4], A[4];
         window(W, svz + txi * La::VW + 4 * tzi);
-        dz4<N, false>(g, W, D);
-        if (MODE == FWD && zq >= 0) {
-            float B[4], A[4];
-            put(B, ld4(g.cpb[0] + oz));
-            put(A, ld4(g.cpa[0] + oz));
+        Q4 Dz = dz4<N, false>(g, W), Dx = zeroq();
 #pragma unroll
-            for (int r = 0; r < 4; r++)
-                if (in[r]) {
-                    pz[r] = slab_recur(B[r], pz[r], A[r], D[r]);
-                    D[r] += pz[r];
-                }
+        for (int l = 1; l <= N; l++)
+            Dx = tap(Dx, g.c[1][l - 1], ldq(svx + (txi + N + l - 1) * 32 + 4 * tzi), ldq(svx + (txi + N - l) * 32 + 4 * tzi));
+        if (!FAST && MODE == FWD && zq >= 0) {
+            zcoefs(g.cpb[0], oz, in, B);
+            zcoefs(g.cpa[0], oz, in, A);
+            recur4(B, A, pz, Dz);
+            Dz = addq(Dz, quad(pz));
         }
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            div[r] = D[r];
-            D[r] = 0.0f;
+        if (!FAST && MODE == FWD && xq >= 0) {
+            xcoefs(g.cpb[1][ox], in, B);
+            xcoefs(g.cpa[1][ox], in, A);
+            recur4(B, A, px, Dx);
+            Dx = addq(Dx, quad(px));
         }
-#pragma unroll
-        for (int l = 1; l <= N; l++) {
-            float a[4], d[4];
-            put(a, ld4(svx + (txi + N + l - 1) * 32 + 4 * tzi));
-            put(d, ld4(svx + (txi + N - l) * 32 + 4 * tzi));
-#pragma unroll
-            for (int r = 0; r < 4; r++) D[r] += g.c[1][l - 1] * (a[r] - d[r]);
+        const float sg = MODE == ADJ ? -g.dt : g.dt;
+        const Q4 dts = FAST ? quad({sg, sg, sg, sg})
+                            : masked(sg, oz, own && in_range(ox, t.lo[1], t.hi[1]), t.lo[0], t.hi[0]);
+        pv = update<MODE>(pv, mulq(dts, Kv), addq(Dz, Dx));
+        if (!FAST && MODE == ADJ && zq >= 0) {
+            zcoefs(g.cpb[0], oz, in, B);
+            zcoefs(g.cpa[0], oz, in, A);
+            recur4(B, A, pz, pv);
         }
-        if (MODE == FWD && xq >= 0) {
-            const float B = g.cpb[1][ox], A = g.cpa[1][ox];
-#pragma unroll
-            for (int r = 0; r < 4; r++)
-                if (in[r]) {
-                    px[r] = slab_recur(B, px[r], A, D[r]);
-                    D[r] += px[r];
-                }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            div[r] += D[r];
-            if (in[r]) pv[r] -= dt * Kv[r] * div[r];
-        }
-        if (MODE == ADJ && zq >= 0) {
-            float B[4], A[4];
-            put(B, ld4(g.cpb[0] + oz));
-            put(A, ld4(g.cpa[0] + oz));
-#pragma unroll
-            for (int r = 0; r < 4; r++)
-                if (in[r]) pz[r] = slab_recur(B[r], pz[r], A[r], pv[r]);
-        }
-        if (MODE == ADJ && xq >= 0) {
-            const float B = g.cpb[1][ox], A = g.cpa[1][ox];
-#pragma unroll
-            for (int r = 0; r < 4; r++)
-                if (in[r]) px[r] = slab_recur(B, px[r], A, pv[r]);
+        if (!FAST && MODE == ADJ && xq >= 0) {
+            xcoefs(g.cpb[1][ox], in, B);
+            xcoefs(g.cpa[1][ox], in, A);
+            recur4(B, A, px, pv);
         }
     }
-    if (MODE == FWD && stf) add_source(b, sb, s, oz, ox, amp, pv);
-    if (MODE == FWD && g.freesurf && z0 <= g.L[0] + N) {
+    if (!FAST && MODE == FWD && stf) add_source(b, sb, s, oz, ox, amp, pv);
+    if (!FAST && MODE == FWD && g.freesurf && z0 <= g.L[0] + N) {
         // p = 0 on the surface row L, -p mirrored above it (the own pressures of the tile's centre)
-        st4(sp + (txi + HX) * La::PW + 4 * tzi + 8, pv);
+        stq(sp + (txi + HX) * La::PW + 4 * tzi + 8, pv);
         __syncthreads();
         const int L = g.L[0];
+        float p4[4];
+        split(pv, p4);
 #pragma unroll
         for (int r = 0; r < 4; r++) {
             const int z = oz + r, zm = 2 * L - z - z0;
-            if (z == L) pv[r] = 0.0f;
-            else if (z < L && z >= L - N && zm < 32) pv[r] = -sp[(txi + HX) * La::PW + zm + 8];
+            if (z == L) p4[r] = 0.0f;
+            else if (z < L && z >= L - N && zm < 32) p4[r] = -sp[(txi + HX) * La::PW + zm + 8];
         }
+        pv = quad(p4);
     }
     if (own) {
-        st4(n.v[0] + sh + k, vz);
-        st4(n.v[1] + sh + k, vx);
-        st4(n.p + sh + k, pv);
-        if (zq >= 0) {
-            st4(n.psip[0] + zo, mz);
-            st4(n.psiv[0] + zo, pz);
+        stq(n.v[0] + sh + k, vz);
+        stq(n.v[1] + sh + k, vx);
+        stq(n.p + sh + k, pv);
+        if (!FAST && zq >= 0) {
+            s3::stg4(n.psip[0] + zo, mz);
+            s3::stg4(n.psiv[0] + zo, pz);
         }
-        if (xq >= 0) {
-            st4(n.psip[1] + xo, mx);
-            st4(n.psiv[1] + xo, px);
+        if (!FAST && xq >= 0) {
+            s3::stg4(n.psip[1] + xo, mx);
+            s3::stg4(n.psiv[1] + xo, px);
         }
     }
-    if (MODE == FWD && save.next >= 0 && band_tile<TX>(bd, z0, x0)) {
+    if (!FAST && MODE == FWD && save.next >= 0 && band_tile<TX>(bd, z0, x0)) {
         // largest magnitude per (axis, side) of the velocities the next sample stores
         if (tid < 4) smax[tid] = 0u;
         __syncthreads();
         if (own) {
+            float a[4], d[4];
+            split(vz, a);
+            split(vx, d);
 #pragma unroll
             for (int r = 0; r < 4; r++) {
                 const int s0 = band_side<0>(bd, oz + r, ox), s1 = band_side<1>(bd, oz + r, ox);
-                if (s0 >= 0 && vz[r] != 0.0f) atomicMax(smax + s0, __float_as_uint(fabsf(vz[r])));
-                if (s1 >= 0 && vx[r] != 0.0f) atomicMax(smax + 2 + s1, __float_as_uint(fabsf(vx[r])));
+                if (s0 >= 0 && a[r] != 0.0f) atomicMax(smax + s0, __float_as_uint(fabsf(a[r])));
+                if (s1 >= 0 && d[r] != 0.0f) atomicMax(smax + 2 + s1, __float_as_uint(fabsf(d[r])));
             }
         }
         __syncthreads();
@@ -561,34 +530,71 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
     }
 }
 
+// Whether the tile and its halo lie inside the box of the step and away from
+// every special case (uniform over the block).
+template <int N, int MODE, int TX>
+__device__ __forceinline__ bool tile_fast(const Grid &g, const Batch &b, const Tile &t, bool src, const Bands &bd, bool bands)
+{
+    const int zl = t.z0 - 8, zh = t.z0 + 39, xl = t.x0 - 2 * N + 1, xh = t.x0 + TX + 2 * N - 2;
+    bool f = t.z0 - 4 >= t.lo[0] && t.z0 + 35 <= t.hi[0] && t.x0 - N >= t.lo[1] && t.x0 + TX + N - 2 <= t.hi[1] &&
+             zl >= g.zlo && zh < g.zhi && xl >= g.xlo && xh < g.xhi && !(g.freesurf && t.z0 - 4 <= g.L[0] + N);
+    if (MODE == FWD && f && src) f = !src_near(src_box(b, t.s), t.z0, t.z0 + 31, t.x0, t.x0 + TX - 1);
+    return f && !(bands && band_tile<TX>(bd, t.z0, t.x0));
+}
+
 template <int N, int TX>
-__global__ void __launch_bounds__(8 * TX, TX == 32 ? 3 : 6)
+__global__ void __launch_bounds__(8 * TX, fwd_blocks(TX))
 k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fields n, int step, const float *stf,
-       float src_scale, Bands bd, Save2 save, Gather2 ga, int nxt, unsigned *err)
+       float src_scale, Bands bd, Save2 save, Gather2 ga, int ng, unsigned *err)
 {
     __shared__ __align__(128) float sm[Lay<N, TX>::FA];
     __shared__ __align__(8) uint64_t bar;
     __shared__ unsigned smax[4];
     Tile t;
     t.s = blockIdx.z;
-    if ((int)blockIdx.y >= nxt) {              // receivers: samples of the pressure before the step
+    if ((int)blockIdx.y < ng) {                // receivers: samples of the pressure before the step
+        const int nr = b.rec_off[t.s + 1] - b.rec_off[t.s];
+        const int r = (blockIdx.y * gridDim.x + blockIdx.x) * (8 * TX) + threadIdx.x;
+        const bool have = r < nr;
+        const Stencil &st = b.rec[b.rec_off[t.s] + (have ? r : 0)];
+        const float *ps = c.p + t.s * g.ntot + (have ? st.first[0] + g.px * st.first[1] : 0);
+        const int n0 = have ? st.cnt[0] : 0, n1 = have ? st.cnt[1] : 0;
+        float w0[2 * N], w1[2 * N];
+#pragma unroll
+        for (int a = 0; a < 2 * N; a++) {
+            w0[a] = a < n0 ? st.w[0][a] : 0.0f;
+            w1[a] = a < n1 ? st.w[1][a] : 0.0f;
+        }
         pdl_wait();
         pdl_trigger();
-        const int nr = b.rec_off[t.s + 1] - b.rec_off[t.s];
-        const int r = ((blockIdx.y - nxt) * gridDim.x + blockIdx.x) * (8 * TX) + threadIdx.x;
-        if (r >= nr) return;
-        const Stencil &st = b.rec[b.rec_off[t.s] + r];
-        const float *ps = c.p + t.s * g.ntot;
+        if (!have) return;
         float sum = 0.0f;
-        for (int a1 = 0; a1 < st.cnt[1]; a1++)
-            for (int a0 = 0; a0 < st.cnt[0]; a0++)
-                sum += st.w[0][a0] * st.w[1][a1] * st.w[2][0] * ps[st.first[0] + a0 + g.px * (st.first[1] + a1)];
+        if (n0 == 2 * N && n1 == 2 * N) {      // every tap: four rows of loads in flight
+#pragma unroll
+            for (int h = 0; h < 2 * N; h += 4) {
+                float x[4][2 * N];
+#pragma unroll
+                for (int a1 = 0; a1 < 4; a1++)
+#pragma unroll
+                    for (int a0 = 0; a0 < 2 * N; a0++) x[a1][a0] = ps[a0 + g.px * (h + a1)];
+#pragma unroll
+                for (int a1 = 0; a1 < 4; a1++)
+#pragma unroll
+                    for (int a0 = 0; a0 < 2 * N; a0++) sum += w0[a0] * w1[h + a1] * x[a1][a0];
+            }
+        } else {
+#pragma unroll
+            for (int a1 = 0; a1 < 2 * N; a1++)
+#pragma unroll
+                for (int a0 = 0; a0 < 2 * N; a0++)
+                    if (a0 < n0 && a1 < n1) sum += w0[a0] * w1[a1] * ps[a0 + g.px * a1];
+        }
         ga.seis[ga.off[t.s] + (long long)ga.it * nr + r] = sum;
         return;
     }
     box_at(b.tab_src, b.nt1, t.s, step, t.lo, t.hi);
     t.z0 = (t.lo[0] & ~3) + 32 * blockIdx.x;
-    t.x0 = t.lo[1] + TX * blockIdx.y;
+    t.x0 = t.lo[1] + TX * ((int)blockIdx.y - ng);
     if (t.z0 > t.hi[0] || t.x0 > t.hi[1]) {
         if (blockIdx.x + blockIdx.y + blockIdx.z == 0) pdl_wait();   // one block of a launch always waits
         return;
@@ -598,15 +604,21 @@ k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fiel
         mbar_fence_init();
     }
     __syncthreads();
-    tile_step<N, FWD, TX>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, sm, &bar, smax, err);
+    if (tile_fast<N, FWD, TX>(g, b, t, stf != nullptr, bd, save.sample >= 0 || save.next >= 0))
+        tile_step<N, FWD, TX, true>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, sm, &bar, smax, err);
+    else
+        tile_step<N, FWD, TX, false>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, sm, &bar, smax, err);
 }
 
 // Reconstruction of one tile.  Own nodes: the physical domain and the
 // boundary bands inside the box of step it + 1 (so that nodes which left the
-// box are written as zeros into both sets of arrays).
-template <int N, int TX>
+// box are written as zeros into both sets of arrays).  FAST: a tile whose
+// nodes and halo lie inside the box of the step before, the range that every
+// velocity component updates, and away from the source and the bands.
+template <int N, int TX, bool FAST>
 __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtensorMap *tm_vx, const Grid &g,
-                                         const Batch &b, const Fields &c, const Fields &n, const Tile &t, int it,
+                                         const Batch &b, const Fields &c, const Fields &n, const Tile &t, const int (&lo)[2],
+                                         const int (&hi)[2], const int (&plo)[3], const int (&phi)[3], int it,
                                          const float *lp, float *acc, int img_mode, const float *stf, float src_scale,
                                          const Bands &bd, bool restore, float *sm, uint64_t *bar, unsigned *err)
 {
@@ -616,25 +628,13 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
     const int tid = threadIdx.x, tzi = tid & 7, txi = tid >> 3;
     const int s = t.s, z0 = t.z0, x0 = t.x0;
     const int oz = z0 + 4 * tzi, ox = x0 + txi, k = oz + g.px * ox;
-    const bool own = oz < g.ne[0] && ox < g.ne[1];
+    const bool own = FAST || (oz < g.ne[0] && ox < g.ne[1]);
     const long long sh = (long long)s * g.ntot;
     const float dt = g.dt;
     if (tid == 0) {
         mbar_expect(bar, (unsigned)(La::RZB + La::RXB) * 4u);
         tma4(tz, tm_vz, z0 - 8, x0 - N + 1, 0, s, bar);
         tma4(tx, tm_vx, z0 - 4, x0 - HX, 0, s, bar);
-    }
-    // update region (box of the step within the physical domain), previous box
-    int plo[3], phi[3], lo[2], hi[2];
-    box_at(b.tab_src, b.nt1, s, it - 1, plo, phi);
-    {
-        int bl[3], bh[3];
-        box_at(b.tab_src, b.nt1, s, it, bl, bh);
-#pragma unroll
-        for (int a = 0; a < 2; a++) {
-            lo[a] = max(bl[a], g.L[a]);
-            hi[a] = min(bh[a], g.H[a]);
-        }
     }
     int ez = 0, ex = 0;                       // extra pressure quads of the halo
     bool extra = tid < 2 * TX;
@@ -647,47 +647,39 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
         ex = rr < N - 1 ? x0 - N + 1 + rr : x0 + TX + rr - (N - 1);
         extra = true;
     }
-    const bool ein = extra && ez >= 0 && ez < g.ne[0] && ex >= 0 && ex < g.ne[1];
+    const bool ein = extra && (FAST || (ez >= 0 && ez < g.ne[0] && ex >= 0 && ex < g.ne[1]));
     const int ke = ez + g.px * ex;
 
-    float bz[4], bx[4], Kv[4] = {}, Ke[4] = {}, pv[4] = {}, pe[4] = {}, lpv[4] = {};
-    {
-        float r0[4] = {1.0f, 1.0f, 1.0f, 1.0f}, r1[4] = {1.0f, 1.0f, 1.0f, 1.0f};
-        if (own) rho_z(g, oz, k, r0, r1);
-        buoy4(r0, r1, bz);
-        if (own && ox + 1 < g.ne[1]) put(r1, ld4(g.rho + k + g.px));
-        else for (int r = 0; r < 4; r++) r1[r] = r0[r];
-        buoy4(r0, r1, bx);
-    }
+    const Q4 one = quad({dt, dt, dt, dt}), two = quad({2.0f * dt, 2.0f * dt, 2.0f * dt, 2.0f * dt});
+    // dt (or 2 dt) at the nodes that the pressure and each velocity component update, else 0
+    const bool inx = FAST || in_range(ox, lo[1], hi[1]);
+    const Q4 dp = FAST ? one : masked(dt, oz, inx, lo[0], hi[0]);
+    const Q4 de = FAST ? one : masked(dt, ez, ein && in_range(ex, lo[1], hi[1]), lo[0], hi[0]);
+    const Q4 dz = FAST ? two : masked(2.0f * dt, oz, inx, max(lo[0], g.L[0] + N - 1), min(hi[0], g.H[0] - N));
+    const Q4 dx = FAST ? two : masked(2.0f * dt, oz, inx && in_range(ox, g.L[1] + N - 1, g.H[1] - N), lo[0], hi[0]);
+    Q4 bz = zeroq(), bx = zeroq(), Kv = zeroq(), Ke = zeroq(), pv = zeroq(), pe = zeroq(), lpv = zeroq(), av = zeroq();
     if (own) {
-        put(Kv, ld4(g.K + k));
-        put(pv, ld4(c.p + sh + k));
-        put(lpv, ld4(lp + sh + k));
+        const Q4 r0 = ldq(g.rho + k);
+        bz = buoyq(dz, r0, rho_up(g, oz, k, r0));
+        bx = buoyq(dx, r0, FAST || ox + 1 < g.ne[1] ? ldq(g.rho + k + g.px) : r0);
+        Kv = ldq(g.K + k);
+        pv = ldq(c.p + sh + k);
+        lpv = ldq(lp + sh + k);
+        av = ldq(acc + sh + k);
     }
     if (ein) {
-        put(Ke, ld4(g.K + ke));
-        put(pe, ld4(c.p + sh + ke));
+        Ke = ldq(g.K + ke);
+        pe = ldq(c.p + sh + ke);
     }
-    const SrcBox sb = src_box(b, s);
-    const float amp = -src_scale * stf[it];
-    // image / gradient accumulator of the quad: one 16-byte access where it is whole and aligned
-    bool in[4];
-    const bool inx = in_range(ox, lo[1], hi[1]);
-#pragma unroll
-    for (int r = 0; r < 4; r++) in[r] = inx && in_range(oz + r, lo[0], hi[0]);
-    const long long ka = (long long)s * g.nphys + (oz - g.L[0]) + (long long)(g.H[0] - g.L[0] + 1) * (ox - g.L[1]);
-    const bool acc4 = in[0] && in[3] && (ka & 3) == 0;
-    float av[4] = {};
-    if (acc4) {
-        put(av, ld4(acc + ka));
-    } else {
-#pragma unroll
-        for (int r = 0; r < 4; r++)
-            if (in[r]) av[r] = acc[ka + r];
+    SrcBox sb{0, 0, 0, 0};
+    float amp = 0.0f;
+    if (!FAST) {
+        sb = src_box(b, s);
+        amp = -src_scale * stf[it];
     }
-    const bool bands = band_tile<TX>(bd, z0, x0);
+    const bool bands = !FAST && band_tile<TX>(bd, z0, x0);
     float scale[4] = {1.0f, 1.0f, 1.0f, 1.0f};
-    if (restore && bands && bd.prec != SMI_PREC_F32) {
+    if (!FAST && restore && bands && bd.prec != SMI_PREC_F32) {
 #pragma unroll
         for (int q = 0; q < 4; q++) scale[q] = bd.scale[((long long)s * bd.nt + it) * 6 + q];
     }
@@ -695,112 +687,105 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
         if (tid == 0) atomicOr(err, 1u);
         mbar_wait(bar, 0);
     }
+    // nodes of the update region d (not 0) that the previous box leaves out
+    auto clear_left = [&](Q4 &q, const Q4 &d, int qz, int qx) {
+        float m[4];
+        bool cl[4];
+        split(d, m);
+        const bool kx = in_range(qx, plo[1], phi[1]);
+#pragma unroll
+        for (int r = 0; r < 4; r++) cl[r] = m[r] != 0.0f && !(kx && in_range(qz + r, plo[0], phi[0]));
+        q = clear_if(q, cl);
+    };
 
     // ---- pressures: p + dt kappa div v - source, zero outside the previous box ----
-    auto press = [&](int qz, int qx, const float (&K4)[4], float (&p)[4], float (&dv)[4]) {
-        float W[12], D[4];
+    auto div_at = [&](int qz, int qx) {
+        float W[12];
         window(W, tz + (qx - x0 + N - 1) * La::PW + (qz - z0) + 4);
-        dz4<N, false>(g, W, dv);
-#pragma unroll
-        for (int r = 0; r < 4; r++) D[r] = 0.0f;
+        const Q4 Dz = dz4<N, false>(g, W);
+        Q4 Dx = zeroq();
         const float *row = tx + (qx - x0 + HX) * La::VW + (qz - z0) + 4;
 #pragma unroll
-        for (int l = 1; l <= N; l++) {
-            float a[4], d[4];
-            put(a, ld4(row + (l - 1) * La::VW));
-            put(d, ld4(row - l * La::VW));
-#pragma unroll
-            for (int r = 0; r < 4; r++) D[r] += g.c[1][l - 1] * (a[r] - d[r]);
-        }
-        float q[4];
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            dv[r] += D[r];
-            q[r] = p[r] + dt * K4[r] * dv[r];
-        }
-        add_source(b, sb, s, qz, qx, amp, q);
-        const bool ix = in_range(qx, lo[1], hi[1]), kx = in_range(qx, plo[1], phi[1]);
+        for (int l = 1; l <= N; l++) Dx = tap(Dx, g.c[1][l - 1], ldq(row + (l - 1) * La::VW), ldq(row - l * La::VW));
+        return addq(Dz, Dx);
+    };
+    auto press = [&](int qz, int qx, const Q4 &d, const Q4 &K4, const Q4 &p, const Q4 &dv) {
+        Q4 q = fmaq(mulq(d, K4), dv, p);
+        if (FAST) return q;
+        Q4 w = q;
+        add_source(b, sb, s, qz, qx, amp, w);
+        float m[4], a[4], e[4];
+        split(d, m);
+        split(q, a);
+        split(w, e);
 #pragma unroll
         for (int r = 0; r < 4; r++) {
-            if (!(ix && in_range(qz + r, lo[0], hi[0]))) continue;
-            p[r] = (kx && in_range(qz + r, plo[0], phi[0]) && !(g.freesurf && qz + r == g.L[0])) ? q[r] : 0.0f;
+            if (m[r] != 0.0f) a[r] = e[r];
+            if (m[r] != 0.0f && g.freesurf && qz + r == g.L[0]) a[r] = 0.0f;
         }
+        q = quad(a);
+        clear_left(q, d, qz, qx);
+        return q;
     };
     {
-        float dv[4], np[4];
-#pragma unroll
-        for (int r = 0; r < 4; r++) np[r] = pv[r];
-        press(oz, ox, Kv, np, dv);
-        st4(spn + (txi + N - 1) * La::VW + 4 * tzi + 4, np);
-        if (own) st4(n.p + sh + k, np);
-#pragma unroll
-        for (int r = 0; r < 4; r++) av[r] += lpv[r] * (img_mode == 0 ? dv[r] : pv[r]);
-        if (acc4) {
-            st4(acc + ka, av);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 4; r++)
-                if (in[r]) acc[ka + r] = av[r];
-        }
-        if (img_mode == 2) {                   // illumination
-#pragma unroll
-            for (int r = 0; r < 4; r++)
-                if (in[r]) acc[(long long)b.nshot * g.nphys + ka + r] += pv[r] * pv[r];
+        const Q4 dv = div_at(oz, ox), np = press(oz, ox, dp, Kv, pv, dv);
+        stq(spn + (txi + N - 1) * La::VW + 4 * tzi + 4, np);
+        if (own) {
+            stq(n.p + sh + k, np);
+            // (nodes outside the physical domain gather values that nobody reads)
+            stq(acc + sh + k, fmaq(lpv, img_mode == 0 ? dv : pv, av));
+            if (img_mode == 2) {               // illumination
+                float *ill = acc + (long long)b.nshot * g.ntot + sh + k;
+                stq(ill, fmaq(pv, pv, ldq(ill)));
+            }
         }
     }
-    if (extra) {
-        float dv[4];
-        press(ez, ex, Ke, pe, dv);
-        st4(spn + (ex - x0 + N - 1) * La::VW + (ez - z0) + 4, pe);
-    }
-    float vz[4] = {}, vx[4] = {};
-    put(vz, ld4(tz + (txi + N - 1) * La::PW + 4 * tzi + 8));
-    put(vx, ld4(tx + (txi + HX) * La::VW + 4 * tzi + 4));
+    if (extra) stq(spn + (ex - x0 + N - 1) * La::VW + (ez - z0) + 4, press(ez, ex, de, Ke, pe, div_at(ez, ex)));
+    Q4 vz = ldq(tz + (txi + N - 1) * La::PW + 4 * tzi + 8), vx = ldq(tx + (txi + HX) * La::VW + 4 * tzi + 4);
     __syncthreads();
 
     // ---- velocities: v_a + dt b_a D_a p on L_a+N-1 .. H_a-N, the bands from the store ----
-    {
-        float W[12], D[4], X[4] = {};
-        window(W, spn + (txi + N - 1) * La::VW + 4 * tzi);
-        dz4<N, true>(g, W, D);
+    float W[12];
+    window(W, spn + (txi + N - 1) * La::VW + 4 * tzi);
+    const Q4 D = dz4<N, true>(g, W);
+    Q4 X = zeroq();
 #pragma unroll
-        for (int l = 1; l <= N; l++) {
-            float a[4], d[4];
-            put(a, ld4(spn + (txi + N - 1 + l) * La::VW + 4 * tzi + 4));
-            put(d, ld4(spn + (txi + N - l) * La::VW + 4 * tzi + 4));
-#pragma unroll
-            for (int r = 0; r < 4; r++) X[r] += g.c[1][l - 1] * (a[r] - d[r]);
-        }
-        const bool kx = in_range(ox, plo[1], phi[1]), rx = in_range(ox, g.L[1] + N - 1, g.H[1] - N);
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            const int z = oz + r;
-            const bool keep = kx && in_range(z, plo[0], phi[0]);
-            if (in[r] && in_range(z, g.L[0] + N - 1, g.H[0] - N)) vz[r] = keep ? vz[r] + dt * bz[r] * D[r] : 0.0f;
-            if (in[r] && rx) vx[r] = keep ? vx[r] + dt * bx[r] * X[r] : 0.0f;
-        }
+    for (int l = 1; l <= N; l++)
+        X = tap(X, g.c[1][l - 1], ldq(spn + (txi + N - 1 + l) * La::VW + 4 * tzi + 4),
+                ldq(spn + (txi + N - l) * La::VW + 4 * tzi + 4));
+    vz = fmaq(bz, D, vz);
+    vx = fmaq(bx, X, vx);
+    if (!FAST) {
+        clear_left(vz, dz, oz, ox);
+        clear_left(vx, dx, oz, ox);
         if (restore && bands) {
+            float a[4], d[4];
+            split(vz, a);
+            split(vx, d);
+            const bool kx = in_range(ox, plo[1], phi[1]);
 #pragma unroll
             for (int r = 0; r < 4; r++) {
                 const int s0 = band_side<0>(bd, oz + r, ox), s1 = band_side<1>(bd, oz + r, ox);
                 const bool keep = kx && in_range(oz + r, plo[0], phi[0]);      // zero (and not stored) outside
                 if (s0 >= 0)
-                    vz[r] = keep ? band_load(bd, band_off<0>(bd, s, it, s0, oz + r, ox), s0 ? scale[1] : scale[0]) : 0.0f;
+                    a[r] = keep ? band_load(bd, band_off<0>(bd, s, it, s0, oz + r, ox), s0 ? scale[1] : scale[0]) : 0.0f;
                 if (s1 >= 0)
-                    vx[r] = keep ? band_load(bd, band_off<1>(bd, s, it, s1, oz + r, ox), s1 ? scale[3] : scale[2]) : 0.0f;
+                    d[r] = keep ? band_load(bd, band_off<1>(bd, s, it, s1, oz + r, ox), s1 ? scale[3] : scale[2]) : 0.0f;
             }
+            vz = quad(a);
+            vx = quad(d);
         }
-        if (own) {
-            st4(n.v[0] + sh + k, vz);
-            st4(n.v[1] + sh + k, vx);
-        }
+    }
+    if (own) {
+        stq(n.v[0] + sh + k, vz);
+        stq(n.v[1] + sh + k, vx);
     }
 }
 
 // roles 1: adjoint, 2: reconstruction (blockIdx.z = shot), 3: both
 // (blockIdx.z = 2 shot + role, 0 adjoint, 1 reconstruction).
 template <int N, int TX>
-__global__ void __launch_bounds__(8 * TX, TX == 32 ? 3 : 6)
+__global__ void __launch_bounds__(8 * TX, rev_blocks(TX))
 k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtensorMap tm_vz,
        const __grid_constant__ CUtensorMap tm_vx, Grid g, Batch b, Fields ac, Fields an, int mrev, int roles, Fields fc,
        Fields fn, int it, float *acc, int img_mode, const float *stf, float src_scale, Bands bd, int restore,
@@ -834,12 +819,33 @@ k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtens
     __syncthreads();
     pdl_wait();
     pdl_trigger();
-    if (role)
-        tile_rec<N, TX>(&tm_vz, &tm_vx, g, b, fc, fn, t, it, ac.p, acc, img_mode, stf, src_scale, bd, restore != 0, sm,
-                        &bar, err);
-    else
-        tile_step<N, ADJ, TX>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, sm, &bar,
-                              nullptr, err);
+    if (role) {
+        // update region (box of the step within the physical domain), previous box
+        int lo[2], hi[2], plo[3], phi[3], bl[3], bh[3];
+        box_at(b.tab_src, b.nt1, t.s, it - 1, plo, phi);
+        box_at(b.tab_src, b.nt1, t.s, it, bl, bh);
+        bool fast = !band_tile<TX>(bd, t.z0, t.x0) &&
+                    !src_near(src_box(b, t.s), t.z0 - 4, t.z0 + 35, t.x0 - N + 1, t.x0 + TX - 1 + N);
+#pragma unroll
+        for (int a = 0; a < 2; a++) {
+            lo[a] = max(bl[a], g.L[a]);
+            hi[a] = min(bh[a], g.H[a]);
+            const int l = a == 0 ? t.z0 - 4 : t.x0 - N + 1, h = a == 0 ? t.z0 + 35 : t.x0 + TX - 1 + N;
+            fast = fast && l >= max(lo[a], max(plo[a], g.L[a] + N - 1)) && h <= min(hi[a], min(phi[a], g.H[a] - N));
+        }
+        if (fast)
+            tile_rec<N, TX, true>(&tm_vz, &tm_vx, g, b, fc, fn, t, lo, hi, plo, phi, it, ac.p, acc, img_mode, stf,
+                                  src_scale, bd, restore != 0, sm, &bar, err);
+        else
+            tile_rec<N, TX, false>(&tm_vz, &tm_vx, g, b, fc, fn, t, lo, hi, plo, phi, it, ac.p, acc, img_mode, stf,
+                                   src_scale, bd, restore != 0, sm, &bar, err);
+    } else if (tile_fast<N, ADJ, TX>(g, b, t, false, bd, false)) {
+        tile_step<N, ADJ, TX, true>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, sm, &bar,
+                                    nullptr, err);
+    } else {
+        tile_step<N, ADJ, TX, false>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, sm, &bar,
+                                     nullptr, err);
+    }
 }
 
 // Most tiles of a shot of the batch along z and x, for boxes [lo, hi] clipped
@@ -892,7 +898,7 @@ void run_fwd(const LaunchCtx &lc, const Maps2 &mc, const Grid &g, const Batch &b
     const int ng = ga.it >= 0 ? (b.max_rec + per - 1) / per : 0;
     if (e.nx + ng == 0) return;
     launch_pdl(lc, k2_fwd<N, TX>, dim3(std::max(1, e.nz), e.nx + ng, b.nshot), 8 * TX, 0, mc.p, g, b, c, n, step, stf,
-               src_scale, bd, save, ga, e.nx, err);
+               src_scale, bd, save, ga, ng, err);
 }
 
 template <int N, int TX>

@@ -61,6 +61,7 @@
 #include "smi_band.h"
 #include "smi_box.h"
 #include "smi_internal.h"
+#include "smi_pack.h"
 #include "smi_pdl.h"
 #include "smi_slab.h"
 #include "smi_stencil3d.h"
@@ -91,115 +92,6 @@ template <int N, int MODE> struct PLay {
     static constexpr int G = oEX + (MODE == ADJ ? X : 0);              // one group
     static constexpr int SMEM = DEPTH * G * 4;
 };
-
-// Quads of FP32 as two packed pairs (each lane rounds like a scalar
-// operation): half the instructions, and a 128-bit load is a quad as it is.
-typedef unsigned long long P2;
-__device__ __forceinline__ P2 pack(float a, float b)
-{
-    P2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack(P2 p, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p)); }
-__device__ __forceinline__ P2 add2(P2 a, P2 b)
-{
-    P2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ P2 sub2(P2 a, P2 b)
-{
-    P2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ P2 mul2(P2 a, P2 b)
-{
-    P2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ P2 fma2(P2 a, P2 b, P2 c)
-{
-    P2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-struct Q4 {
-    P2 a, b;
-};
-__device__ __forceinline__ Q4 ldq(const float *p)
-{
-    const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
-    return {t.x, t.y};
-}
-__device__ __forceinline__ void stq(float *p, const Q4 &q) { *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(q.a, q.b); }
-__device__ __forceinline__ Q4 quad(const float (&v)[4]) { return {pack(v[0], v[1]), pack(v[2], v[3])}; }
-__device__ __forceinline__ Q4 zeroq() { return {0ull, 0ull}; }
-__device__ __forceinline__ void split(const Q4 &q, float (&v)[4])
-{
-    unpack(q.a, v[0], v[1]);
-    unpack(q.b, v[2], v[3]);
-}
-__device__ __forceinline__ Q4 addq(const Q4 &x, const Q4 &y) { return {add2(x.a, y.a), add2(x.b, y.b)}; }
-__device__ __forceinline__ Q4 subq(const Q4 &x, const Q4 &y) { return {sub2(x.a, y.a), sub2(x.b, y.b)}; }
-__device__ __forceinline__ Q4 mulq(const Q4 &x, const Q4 &y) { return {mul2(x.a, y.a), mul2(x.b, y.b)}; }
-__device__ __forceinline__ Q4 fmaq(const Q4 &x, const Q4 &y, const Q4 &z) { return {fma2(x.a, y.a, z.a), fma2(x.b, y.b, z.b)}; }
-// D + c (x - y)
-__device__ __forceinline__ Q4 tap(const Q4 &D, float c, const Q4 &x, const Q4 &y)
-{
-    const P2 cc = pack(c, c);
-    return {fma2(cc, sub2(x.a, y.a), D.a), fma2(cc, sub2(x.b, y.b), D.b)};
-}
-// num / (r0 + r1): reciprocal (a few ulp, far below the FP32 scheme error)
-// and product; densities are normal numbers, so it is __fdividef without its
-// range scaling.
-__device__ __forceinline__ float rcpf(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ Q4 buoyq(const Q4 &num, const Q4 &r0, const Q4 &r1)
-{
-    float d[4];
-    split(addq(r0, r1), d);
-#pragma unroll
-    for (int r = 0; r < 4; r++) d[r] = rcpf(d[r]);
-    return mulq(num, quad(d));
-}
-// Brings a line that a later plane reads towards the L2 cache.
-__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-// v - b D: the forward scheme rounds the product first (as it always has).
-template <int MODE> __device__ __forceinline__ Q4 update(const Q4 &v, const Q4 &b, const Q4 &D)
-{
-    return MODE == FWD ? subq(v, mulq(b, D)) : fmaq(b, D, v);
-}
-__device__ __forceinline__ void window(float (&W)[12], const float *row)
-{
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-        float v[4];
-        split(ldq(row + 4 * k), v);
-#pragma unroll
-        for (int r = 0; r < 4; r++) W[4 * k + r] = v[r];
-    }
-}
-// D along z of the middle quad of a window, p nodes to v nodes (UP) or back.
-template <int N, bool UP> __device__ __forceinline__ Q4 dz4(const Grid &g, const float (&W)[12])
-{
-    float D[4];
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-        float d = 0.f;
-#pragma unroll
-        for (int l = 1; l <= N; l++)
-            d += g.c[0][l - 1] * (UP ? W[4 + r + l] - W[4 + r - l + 1] : W[4 + r + l - 1] - W[4 + r - l]);
-        D[r] = d;
-    }
-    return quad(D);
-}
 
 // CPML coefficients (B, A) of a tile's own nodes along z and x, zero at nodes
 // outside the slabs, the grid or the box of this launch: a memory variable
@@ -262,18 +154,10 @@ __device__ __forceinline__ Own own_of(const Grid &g, const Item &it, int tzi, in
     o.xq = o.act ? slab_row(g, 1, o.ox) : -1;
     return o;
 }
-// m <- B m + A x over the quad.
-__device__ __forceinline__ void recur4(const float (&B)[4], const float (&A)[4], float (&m)[4], const Q4 &x)
+// v - b D: the forward scheme rounds the product first (as it always has).
+template <int MODE> __device__ __forceinline__ Q4 update(const Q4 &v, const Q4 &b, const Q4 &D)
 {
-    float v[4];
-    split(x, v);
-#pragma unroll
-    for (int r = 0; r < 4; r++) m[r] = slab_recur(B[r], m[r], A[r], v[r]);
-}
-__device__ __forceinline__ void recur1(float B, float A, float (&m)[4], const Q4 &x)
-{
-    const float Bq[4] = {B, B, B, B}, Aq[4] = {A, A, A, A};
-    recur4(Bq, Aq, m, x);
+    return MODE == FWD ? subq(v, mulq(b, D)) : fmaq(b, D, v);
 }
 // The forward scheme's z terms: which of the two products is rounded first
 // decides the last bit.  A x enters the multiply-add unrounded, except on x
@@ -292,26 +176,6 @@ __device__ __forceinline__ bool x_group(const Grid &g, int x, int x0)
     const int first = x0 + ((x - x0) & ~3), hi = g.ne[1] - g.nb - 1;
     return first < g.nb || first + 3 >= hi;
 }
-// v - b m
-__device__ __forceinline__ Q4 sub_prod(const Q4 &v, const Q4 &b, const float (&m)[4])
-{
-    float x[4], c[4];
-    split(v, x);
-    split(b, c);
-#pragma unroll
-    for (int r = 0; r < 4; r++) x[r] = __fmaf_rn(-c[r], m[r], x[r]);
-    return quad(x);
-}
-// Zero where z.
-__device__ __forceinline__ Q4 clear_if(const Q4 &q, const bool (&z)[4])
-{
-    float x[4];
-    split(q, x);
-#pragma unroll
-    for (int r = 0; r < 4; r++) x[r] = z[r] ? 0.f : x[r];
-    return quad(x);
-}
-
 // How a launch cuts its boxes: planes a chunk, and the boxes' low end along x.
 struct Cut {
     int chunk, x0;
@@ -726,29 +590,17 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
         float *const mzp = f.psiv[0] + (s * g.slab_n[0] + me.zq + (long long)g.zp * ox);
         float *const mxp = f.psiv[1] + (s * g.slab_n[1] + oz + (long long)g.px * me.xq);
         const unsigned zpl = (unsigned)(g.zp * g.ne[1]), xpl = (unsigned)(g.px * g.xrows);
-        const int n0 = g.H[0] - g.L[0] + 1, n1 = g.H[1] - g.L[1] + 1;
-        const long long acol = (long long)s * g.nphys + (oz - g.L[0]) + (long long)n0 * (ox - g.L[1]);
-        const bool whole = MODE == REC && in[0] && in[3];
         int h = 0;                            // group slot of plane y
 
         // one plane; BAND: with the CPML terms (REC: with nodes outside the previous box)
         auto body = [&](auto kc, auto bc, int y) {
             constexpr int K = decltype(kc)::value;
             constexpr bool BAND = decltype(bc)::value;
-            float accv[4] = {0.f, 0.f, 0.f, 0.f};
-            long long accb = 0;
-            bool acc4 = false;                // the quad as one aligned 16-byte access
+            const unsigned o = col + (unsigned)(y * plane);
+            Q4 accv = zeroq();
             if (MODE == REC && me.act) {
-                accb = acol + (long long)n0 * n1 * (y - g.L[2]);
-                if (y + AHEAD <= yb) prefetch_l2(acc + accb + (long long)n0 * n1 * AHEAD);
-                acc4 = whole && (accb & 3) == 0;
-                if (acc4) {
-                    put(accv, ldg4(acc + accb));
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 4; r++)
-                        if (in[r]) accv[r] = acc[accb + r];
-                }
+                if (y + AHEAD <= yb) prefetch_l2(acc + sh + (o + (unsigned)(AHEAD * plane)));
+                accv = ldq(acc + sh + o);
             }
             const int ys = BAND && MODE != REC ? slab_row(g, 2, y) : -1;
             const int ye = BAND && MODE == ADJ ? slab_row(g, 2, y + N - 1) : -1;
@@ -851,30 +703,18 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
                 }
             }
             if (MODE == REC) {
-                float lpv[4], dv[4], p4[4];
-                split(ldq(own + La::oL), lpv);
-                split(div, dv);
-                split(pv, p4);
-#pragma unroll
-                for (int r = 0; r < 4; r++) accv[r] += lpv[r] * (img_mode == 0 ? dv[r] : p4[r]);
+                // (nodes of the quad outside the physical domain gather values that nobody reads)
+                if (me.act) stq(acc + sh + o, fmaq(ldq(own + La::oL), img_mode == 0 ? div : pv, accv));
+                if (img_mode == 2 && me.act) {                // illumination
+                    float *ill = acc + (long long)b.nshot * g.ntot + sh + o;
+                    stq(ill, fmaq(pv, pv, ldq(ill)));
+                }
                 if (BAND) {
                     const bool ky = in_range(y, it.plo[2], it.phi[2]);
                     bool cl[4];
 #pragma unroll
                     for (int r = 0; r < 4; r++) cl[r] = out[r] || (!ky && in[r]);
                     np = clear_if(np, cl);
-                }
-                if (acc4) {
-                    stg4(acc + accb, accv);
-                } else if (me.act) {
-#pragma unroll
-                    for (int r = 0; r < 4; r++)
-                        if (in[r]) acc[accb + r] = accv[r];
-                }
-                if (img_mode == 2 && me.act) {                // illumination
-#pragma unroll
-                    for (int r = 0; r < 4; r++)
-                        if (in[r]) acc[(long long)b.nshot * g.nphys + accb + r] += p4[r] * p4[r];
                 }
             }
             if (BAND && MODE == ADJ) {
@@ -896,7 +736,7 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
             }
             if (BAND && MODE != REC && ys >= 0 && me.act)
                 stg4(f.psiv[2] + s * g.slab_n[2] + (col + (unsigned)(ys * plane)), ym);
-            if (me.act) stq(f.p + sh + (col + (unsigned)(y * plane)), np);
+            if (me.act) stq(f.p + sh + o, np);
             __syncthreads();
             if (tid == 0 && ok && y + DEPTH <= yb) issue(y + DEPTH, h);
             h = h + 1 == DEPTH ? 0 : h + 1;
