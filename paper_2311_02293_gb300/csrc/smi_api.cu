@@ -870,7 +870,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch3_p(lc, mF, nullptr, g, b, F, it, 0, d_wait, nullptr, 0, it < S.nt ? S.stf : nullptr,
                               (float)S.src_scale, save, ctr++);
                 } else if (fast2) {                    // CPML, source, boundary saving and samples in one launch
-                    Save2 save{-1, -1, d_absmax};
+                    Save2 save{-1, -1, kind != 0 ? d_absmax : nullptr};
                     if (kind != 0 && it % S.dr == 0) save.sample = it / S.dr;
                     if (kind != 0 && bd.prec != SMI_PREC_F32 && (it + 1) % S.dr == 0 && (it + 1) / S.dr < S.nsamp)
                         save.next = (it + 1) / S.dr;
@@ -993,15 +993,42 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 tm.end();
                 if (!tile3 || S.dr > 1) restore(it);   // (the 3D adjoint velocity kernel restores a stored step)
             };
-            // 2D: the adjoint step and the reconstruction share a launch (timed per class: one launch each)
+            // 2D: receivers of each shot by cells of 32 columns, for the step kernels' adjoint source
+            Inject2 ij{res, d_soff, nullptr, nullptr, (g.ne[1] + 31) / 32, -1};
+            if (fast2 && max_rec > 0) {
+                std::vector<int> cell((size_t)nb_shot * (ij.ncell + 1), 0), ids;
+                ids.reserve(2 * (size_t)roff[nb_shot]);
+                std::vector<std::vector<int>> in(ij.ncell);
+                for (int s = 0; s < nb_shot; s++) {
+                    for (auto &v : in) v.clear();
+                    for (int r = 0; r < roff[s + 1] - roff[s]; r++) {
+                        const Stencil &q = S.rec_st[(size_t)S.rec_offset[s0] + roff[s] + r];
+                        for (int c = q.first[1] >> 5; c <= (q.first[1] + q.cnt[1] - 1) >> 5; c++) in[c].push_back(r);
+                    }
+                    int *co = cell.data() + (size_t)s * (ij.ncell + 1);
+                    co[0] = (int)ids.size();
+                    for (int c = 0; c < ij.ncell; c++) {
+                        ids.insert(ids.end(), in[c].begin(), in[c].end());
+                        co[c + 1] = (int)ids.size();
+                    }
+                }
+                int *dc = ba.get<int>(cell.size()), *di = ba.get<int>(std::max<size_t>(1, ids.size()));
+                if (!dc || !di) return fail(SMI_ERR_NOMEM, "device allocation failed");
+                cudaMemcpyAsync(dc, cell.data(), sizeof(int) * cell.size(), cudaMemcpyHostToDevice, st);
+                if (!ids.empty()) cudaMemcpyAsync(di, ids.data(), sizeof(int) * ids.size(), cudaMemcpyHostToDevice, st);
+                ij.cell = dc;
+                ij.ids = di;
+            }
+            // the adjoint step and the reconstruction share a launch (timed per class: one launch each)
             auto reverse2 = [&](int it, int mrev) {
                 const int all = kind == 5 ? 1 : 3;
+                ij.it = max_rec > 0 ? it - 1 : -1;
                 for (int part = 0; part < 2; part++) {
                     const int roles = tm.on ? all & (part == 0 ? 2 : 1) : (part == 0 ? all : 0);
                     if (!roles) continue;
                     tm.begin(roles == 2 ? 2 : 1);
                     launch2_reverse(lc, t2, m2A, m2F, g, b, A, A2, mrev, roles, F, F2, it, acc, mode, S.stf,
-                                    (float)S.src_scale, bd, S.dr == 1, d_wait);
+                                    (float)S.src_scale, bd, S.dr == 1, ij, d_wait);
                     tm.end();
                 }
                 swap_A();
@@ -1012,7 +1039,9 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             for (int it = S.nt - 1; it >= 0; it--) {
                 const int mrev = S.nt - 1 - it;
                 if (max_rec > 0) {
-                    if (tiles) launch_adj_inject_tile(lc, g, b, A, res, d_soff, it);
+                    if (fast2 && it < S.nt - 1) {
+                        // (the step before has added it)
+                    } else if (tiles) launch_adj_inject_tile(lc, g, b, A, res, d_soff, it);
                     else launch_adj_inject(lc, g, b, A.p, res, d_soff, S.nt, it);
                 }
                 // free surface (no-ops without): the transposed p mirror on the

@@ -173,20 +173,34 @@ __device__ __forceinline__ void add_source(const Batch &b, const SrcBox &sb, int
     q = quad(p);
 }
 
-// Boundary regions of axis A at node (z, x): side 0 / 1, or -1.
-template <int A> __device__ __forceinline__ int band_side(const Bands &bd, int z, int x)
-{
+// Where the quad at (oz, ox) meets the boundary regions: bit r of z[sd] for
+// node r in the z band of side sd (2N - 1 half nodes across the face, over the
+// physical x), xs = side of the x band that holds the column (-1: none) with
+// bit r of x for the physical z; and the offsets of node 0 in the stored step.
+template <int N> struct BandQuad {
+    unsigned z[2], x;
+    int xs, zo[2], xo;
+    __device__ __forceinline__ BandQuad(const Grid &g, const Bands &bd, int oz, int ox, bool own)
+    {
+        constexpr unsigned W = 2 * N - 2;              // last index across a face
+        const bool px = own && in_range(ox, g.L[1], g.H[1]);
+        const int t0 = oz - (g.L[0] - N), t1 = oz - (g.H[0] - N + 1);
+        const unsigned u0 = (unsigned)(ox - (g.L[1] - N)), u1 = (unsigned)(ox - (g.H[1] - N + 1));
+        z[0] = z[1] = x = 0u;
 #pragma unroll
-    for (int sd = 0; sd < 2; sd++)
-        if (in_range(z, bd.lo[A][sd][0], bd.hi[A][sd][0]) && in_range(x, bd.lo[A][sd][1], bd.hi[A][sd][1])) return sd;
-    return -1;
-}
-template <int A> __device__ __forceinline__ long long band_off(const Bands &bd, int s, int it, int sd, int z, int x)
-{
-    const int w0 = bd.hi[A][sd][0] - bd.lo[A][sd][0] + 1;
-    return ((long long)s * bd.nt + it) * bd.count + bd.off[A][sd] + (z - bd.lo[A][sd][0]) +
-           (long long)w0 * (x - bd.lo[A][sd][1]);
-}
+        for (int r = 0; r < 4; r++) {
+            z[0] |= (px && (unsigned)(t0 + r) <= W) ? 1u << r : 0u;
+            z[1] |= (px && (unsigned)(t1 + r) <= W) ? 1u << r : 0u;
+            x |= (own && in_range(oz + r, g.L[0], g.H[0])) ? 1u << r : 0u;
+        }
+        xs = u0 <= W ? 0 : (u1 <= W ? 1 : -1);
+        if (xs < 0) x = 0u;
+        zo[0] = (int)bd.off[0][0] + t0 + (int)(W + 1) * (ox - g.L[1]);
+        zo[1] = (int)bd.off[0][1] + t1 + (int)(W + 1) * (ox - g.L[1]);
+        xo = (int)(xs == 1 ? bd.off[1][1] : bd.off[1][0]) + (oz - g.L[0]) +
+             (g.H[0] - g.L[0] + 1) * (int)(xs == 1 ? u1 : u0);
+    }
+};
 // Whether the block's own nodes meet a band of either axis (uniform).
 template <int TX> __device__ __forceinline__ bool band_tile(const Bands &bd, int z0, int x0)
 {
@@ -201,28 +215,52 @@ template <int TX> __device__ __forceinline__ bool band_tile(const Bands &bd, int
 }
 
 // 16-bit storage is scaled per (step, axis, side): the largest magnitude
-// maps to 2^14 (FP16) or 1 (BF16).
-template <int A>
-__device__ __forceinline__ void band_store(const Bands &bd, const float (&scale)[4], int s, int it, int oz, int x,
-                                           const Q4 &q)
+// maps to 2^14 (FP16) or 1 (BF16).  Stores the quad's nodes in mask at
+// o .. o+3 of the step that starts at base.
+__device__ __forceinline__ void band_store(const Bands &bd, float scale, long long base, int o, unsigned mask, const Q4 &q)
+{
+    float v[4];
+    split(q, v);
+    if (bd.prec == SMI_PREC_F32) {
+        float *d = static_cast<float *>(bd.data) + base + o;
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+            if (mask >> r & 1u) d[r] = v[r];
+        return;
+    }
+    // one reciprocal a quad; early steps, whose scale is so small that it would overflow, divide
+    const bool tiny = scale < 1e-36f;
+    const float inv = tiny ? 0.0f : __frcp_rn(scale);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        if (!(mask >> r & 1u)) continue;
+        float y = v[r] * inv;
+        if (tiny) y = scale > 0.0f ? v[r] / scale : 0.0f;
+        if (bd.prec == SMI_PREC_F16) static_cast<__half *>(bd.data)[base + o + r] = __float2half_rn(y);
+        else static_cast<__nv_bfloat16 *>(bd.data)[base + o + r] = __float2bfloat16_rn(y);
+    }
+}
+// The stored values into the quad's nodes in mask, 0 where keep lacks them.
+__device__ __forceinline__ void band_restore(const Bands &bd, float scale, long long base, int o, unsigned mask, unsigned keep,
+                                             Q4 &q)
 {
     float v[4];
     split(q, v);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const int sd = band_side<A>(bd, oz + r, x);
-        if (sd < 0) continue;
-        const long long o = band_off<A>(bd, s, it, sd, oz + r, x);
-        if (bd.prec == SMI_PREC_F32) {
-            static_cast<float *>(bd.data)[o] = v[r];
-        } else {
-            const float sc = sd == 0 ? scale[2 * A] : scale[2 * A + 1];
-            const float y = sc > 0.0f ? v[r] / sc : 0.0f;
-            if (bd.prec == SMI_PREC_F16) static_cast<__half *>(bd.data)[o] = __float2half_rn(y);
-            else static_cast<__nv_bfloat16 *>(bd.data)[o] = __float2bfloat16_rn(y);
-        }
-    }
+    for (int r = 0; r < 4; r++)
+        if (mask >> r & 1u) v[r] = keep >> r & 1u ? band_load(bd, base + o + r, scale) : 0.0f;
+    q = quad(v);
 }
+// Largest magnitude of the quad's nodes in mask, over the warp.
+__device__ __forceinline__ unsigned warp_max(const Q4 &q, unsigned mask)
+{
+    float v[4], m = 0.0f;
+    split(q, v);
+#pragma unroll
+    for (int r = 0; r < 4; r++) m = mask >> r & 1u ? fmaxf(m, fabsf(v[r])) : m;
+    return __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+}
+
 // One velocity quad: v -+ b D, the memory variable m of the v grid (B, A: its
 // coefficients), and the operand that the pressure update differentiates
 // (forward: v; adjoint: v + e), returned.
@@ -246,11 +284,11 @@ __device__ __forceinline__ Q4 vel_quad(const Q4 &b, Q4 D, bool slab, const float
 // a tile whose nodes and halo lie inside the box and away from the slabs, the
 // free surface, the source and the bands (tile_fast): no tests, no memory
 // variables.
-template <int N, int MODE, int TX, bool FAST>
+template <int N, int MODE, int TX, bool FAST, bool SAVE>
 __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g, const Batch &b, const Fields &c,
                                           const Fields &n, const Tile &t, int step, const float *stf, float src_scale,
-                                          const Bands &bd, const Save2 &save, float *sm, uint64_t *bar,
-                                          unsigned *smax, unsigned *err)
+                                          const Bands &bd, const Save2 &save, const float *inj, float *sm,
+                                          uint64_t *bar, unsigned *err)
 {
     using La = Lay<N, TX>;
     constexpr int HX = 2 * N - 1, NT = 8 * TX;
@@ -338,20 +376,18 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
         if (eq >= 0) put(me, s3::ldg4((exz ? c.psip[0] : c.psip[1]) + eo));
     }
 
-    const bool first = t.z0 == (t.lo[0] & ~3) && t.x0 == t.lo[1];      // writes the shot's scales
-    if (MODE == FWD && save.sample >= 0 && (first || (!FAST && band_tile<TX>(bd, z0, x0)))) {
-        float scale[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (bd.prec != SMI_PREC_F32) {
+    // scales of the sample this step stores (at the end, from the old arrays)
+    const bool saves = !FAST && SAVE && save.sample >= 0 && band_tile<TX>(bd, z0, x0);
+    float scale[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (SAVE && save.sample >= 0 && bd.prec != SMI_PREC_F32) {
+        const bool first = t.z0 == (t.lo[0] & ~3) && t.x0 == t.lo[1];      // writes the shot's scales
+        if (saves || first) {
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 scale[q] = __uint_as_float(save.amax[((long long)save.sample * b.nshot + s) * 6 + q]) /
                            (bd.prec == SMI_PREC_F16 ? 16384.0f : 1.0f);
                 if (first && tid == q) bd.scale[((long long)s * bd.nt + save.sample) * 6 + q] = scale[q];
             }
-        }
-        if (!FAST && own) {
-            band_store<0>(bd, scale, s, save.sample, oz, ox, vz);
-            band_store<1>(bd, scale, s, save.sample, oz, ox, vx);
         }
     }
 
@@ -470,6 +506,7 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
         const Q4 dts = FAST ? quad({sg, sg, sg, sg})
                             : masked(sg, oz, own && in_range(ox, t.lo[1], t.hi[1]), t.lo[0], t.hi[0]);
         pv = update<MODE>(pv, mulq(dts, Kv), addq(Dz, Dx));
+        if (MODE == ADJ && inj) pv = fmaq(Kv, ldq(inj + txi * 32 + 4 * tzi), pv);   // the next step's adjoint source
         if (!FAST && MODE == ADJ && zq >= 0) {
             zcoefs(g.cpb[0], oz, in, B);
             zcoefs(g.cpa[0], oz, in, A);
@@ -510,23 +547,27 @@ __device__ __forceinline__ void tile_step(const CUtensorMap *tm_p, const Grid &g
             s3::stg4(n.psiv[1] + xo, px);
         }
     }
-    if (!FAST && MODE == FWD && save.next >= 0 && band_tile<TX>(bd, z0, x0)) {
-        // largest magnitude per (axis, side) of the velocities the next sample stores
-        if (tid < 4) smax[tid] = 0u;
-        __syncthreads();
-        if (own) {
-            float a[4], d[4];
-            split(vz, a);
-            split(vx, d);
-#pragma unroll
-            for (int r = 0; r < 4; r++) {
-                const int s0 = band_side<0>(bd, oz + r, ox), s1 = band_side<1>(bd, oz + r, ox);
-                if (s0 >= 0 && a[r] != 0.0f) atomicMax(smax + s0, __float_as_uint(fabsf(a[r])));
-                if (s1 >= 0 && d[r] != 0.0f) atomicMax(smax + 2 + s1, __float_as_uint(fabsf(d[r])));
+    if (!FAST && SAVE && (save.sample >= 0 || save.next >= 0) && band_tile<TX>(bd, z0, x0)) {
+        const BandQuad<N> bq(g, bd, oz, ox, own);
+        if (saves && (bq.z[0] | bq.z[1] | bq.x)) {
+            const Q4 vz_old = ldq(c.v[0] + sh + k), vx_old = ldq(c.v[1] + sh + k);
+            const long long base = ((long long)s * bd.nt + save.sample) * bd.count;
+            if (bq.z[0]) band_store(bd, scale[0], base, bq.zo[0], bq.z[0], vz_old);
+            if (bq.z[1]) band_store(bd, scale[1], base, bq.zo[1], bq.z[1], vz_old);
+            if (bq.x) band_store(bd, bq.xs ? scale[3] : scale[2], base, bq.xo, bq.x, vx_old);
+        }
+        if (save.next >= 0) {
+            // largest magnitude per (axis, side) of the velocities the next sample stores
+            unsigned *am = save.amax + ((long long)save.next * b.nshot + s) * 6;
+            const unsigned m0 = warp_max(vz, bq.z[0]), m1 = warp_max(vz, bq.z[1]);
+            const unsigned m2 = warp_max(vx, bq.xs == 0 ? bq.x : 0u), m3 = warp_max(vx, bq.xs == 1 ? bq.x : 0u);
+            if ((tid & 31) == 0) {
+                if (m0) atomicMax(am, m0);
+                if (m1) atomicMax(am + 1, m1);
+                if (m2) atomicMax(am + 2, m2);
+                if (m3) atomicMax(am + 3, m3);
             }
         }
-        __syncthreads();
-        if (tid < 4 && smax[tid]) atomicMax(save.amax + ((long long)save.next * b.nshot + s) * 6 + tid, smax[tid]);
     }
 }
 
@@ -542,14 +583,14 @@ __device__ __forceinline__ bool tile_fast(const Grid &g, const Batch &b, const T
     return f && !(bands && band_tile<TX>(bd, t.z0, t.x0));
 }
 
-template <int N, int TX>
+// SAVE: boundary saving (a call that reverses the field later).
+template <int N, int TX, bool SAVE>
 __global__ void __launch_bounds__(8 * TX, fwd_blocks(TX))
 k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fields n, int step, const float *stf,
        float src_scale, Bands bd, Save2 save, Gather2 ga, int ng, unsigned *err)
 {
     __shared__ __align__(128) float sm[Lay<N, TX>::FA];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ unsigned smax[4];
     Tile t;
     t.s = blockIdx.z;
     if ((int)blockIdx.y < ng) {                // receivers: samples of the pressure before the step
@@ -604,10 +645,10 @@ k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fiel
         mbar_fence_init();
     }
     __syncthreads();
-    if (tile_fast<N, FWD, TX>(g, b, t, stf != nullptr, bd, save.sample >= 0 || save.next >= 0))
-        tile_step<N, FWD, TX, true>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, sm, &bar, smax, err);
+    if (tile_fast<N, FWD, TX>(g, b, t, stf != nullptr, bd, SAVE && (save.sample >= 0 || save.next >= 0)))
+        tile_step<N, FWD, TX, true, SAVE>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, nullptr, sm, &bar, err);
     else
-        tile_step<N, FWD, TX, false>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, sm, &bar, smax, err);
+        tile_step<N, FWD, TX, false, SAVE>(&tm_p, g, b, c, n, t, step, stf, src_scale, bd, save, nullptr, sm, &bar, err);
 }
 
 // Reconstruction of one tile.  Own nodes: the physical domain and the
@@ -758,22 +799,16 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
     if (!FAST) {
         clear_left(vz, dz, oz, ox);
         clear_left(vx, dx, oz, ox);
-        if (restore && bands) {
-            float a[4], d[4];
-            split(vz, a);
-            split(vx, d);
+        if (restore && bands) {                // zero (and not stored) outside the previous box
+            const BandQuad<N> bq(g, bd, oz, ox, own);
+            const long long base = ((long long)s * bd.nt + it) * bd.count;
             const bool kx = in_range(ox, plo[1], phi[1]);
+            unsigned keep = 0u;
 #pragma unroll
-            for (int r = 0; r < 4; r++) {
-                const int s0 = band_side<0>(bd, oz + r, ox), s1 = band_side<1>(bd, oz + r, ox);
-                const bool keep = kx && in_range(oz + r, plo[0], phi[0]);      // zero (and not stored) outside
-                if (s0 >= 0)
-                    a[r] = keep ? band_load(bd, band_off<0>(bd, s, it, s0, oz + r, ox), s0 ? scale[1] : scale[0]) : 0.0f;
-                if (s1 >= 0)
-                    d[r] = keep ? band_load(bd, band_off<1>(bd, s, it, s1, oz + r, ox), s1 ? scale[3] : scale[2]) : 0.0f;
-            }
-            vz = quad(a);
-            vx = quad(d);
+            for (int r = 0; r < 4; r++) keep |= kx && in_range(oz + r, plo[0], phi[0]) ? 1u << r : 0u;
+            if (bq.z[0]) band_restore(bd, scale[0], base, bq.zo[0], bq.z[0], keep, vz);
+            if (bq.z[1]) band_restore(bd, scale[1], base, bq.zo[1], bq.z[1], keep, vz);
+            if (bq.x) band_restore(bd, bq.xs ? scale[3] : scale[2], base, bq.xo, bq.x, keep, vx);
         }
     }
     if (own) {
@@ -789,9 +824,10 @@ __global__ void __launch_bounds__(8 * TX, rev_blocks(TX))
 k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtensorMap tm_vz,
        const __grid_constant__ CUtensorMap tm_vx, Grid g, Batch b, Fields ac, Fields an, int mrev, int roles, Fields fc,
        Fields fn, int it, float *acc, int img_mode, const float *stf, float src_scale, Bands bd, int restore,
-       unsigned *err)
+       Inject2 ij, unsigned *err)
 {
     __shared__ __align__(128) float sm[Lay<N, TX>::MAXF];
+    __shared__ __align__(16) float sinj[32 * TX];
     __shared__ __align__(8) uint64_t bar;
     const bool role = roles == 3 ? blockIdx.z & 1 : roles == 2;
     Tile t;
@@ -815,6 +851,36 @@ k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtens
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         mbar_fence_init();
+    }
+    // The adjoint source of the reverse step after this one, sum over receivers of weight times residual at
+    // the tile's nodes: it enters the adjoint pressure as this step writes it (nothing here is written by an
+    // earlier step, so it is done before the wait).  Receivers are listed by cells of 32 columns.
+    const float *inj = nullptr;
+    if (!role && ij.it >= 0) {
+        const int *e = b.box_rec + 6 * t.s;
+        if (e[0] <= t.z0 + 31 && e[3] >= t.z0 && e[1] <= t.x0 + TX - 1 && e[4] >= t.x0) {
+            for (int i = threadIdx.x; i < 32 * TX; i += 8 * TX) sinj[i] = 0.0f;
+            __syncthreads();
+            const int nr = b.rec_off[t.s + 1] - b.rec_off[t.s];
+            const float *res = ij.res + ij.off[t.s] + (long long)ij.it * nr;
+            const int c1 = min((t.x0 + TX - 1) >> 5, ij.ncell - 1);
+            for (int c = t.x0 >> 5; c <= c1; c++) {
+                const int *co = ij.cell + (long long)t.s * (ij.ncell + 1) + c;
+                for (int i = co[0] + threadIdx.x; i < co[1]; i += 8 * TX) {
+                    const int r = ij.ids[i];
+                    const Stencil &st = b.rec[b.rec_off[t.s] + r];
+                    const float val = res[r];
+                    const int xa = max(st.first[1], max(t.x0, c << 5));
+                    const int xb = min(st.first[1] + st.cnt[1] - 1, min(t.x0 + TX - 1, (c << 5) + 31));
+                    const int za = max(st.first[0], t.z0), zb = min(st.first[0] + st.cnt[0] - 1, t.z0 + 31);
+                    for (int x = xa; x <= xb; x++)
+                        for (int z = za; z <= zb; z++)
+                            atomicAdd(sinj + (x - t.x0) * 32 + z - t.z0,
+                                      st.w[0][z - st.first[0]] * st.w[1][x - st.first[1]] * st.w[2][0] * val);
+                }
+            }
+            inj = sinj;
+        }
     }
     __syncthreads();
     pdl_wait();
@@ -840,11 +906,11 @@ k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtens
             tile_rec<N, TX, false>(&tm_vz, &tm_vx, g, b, fc, fn, t, lo, hi, plo, phi, it, ac.p, acc, img_mode, stf,
                                    src_scale, bd, restore != 0, sm, &bar, err);
     } else if (tile_fast<N, ADJ, TX>(g, b, t, false, bd, false)) {
-        tile_step<N, ADJ, TX, true>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, sm, &bar,
-                                    nullptr, err);
+        tile_step<N, ADJ, TX, true, false>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, inj, sm,
+                                    &bar, err);
     } else {
-        tile_step<N, ADJ, TX, false>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, sm, &bar,
-                                     nullptr, err);
+        tile_step<N, ADJ, TX, false, false>(&tm_lp, g, b, ac, an, t, mrev, nullptr, 0.0f, bd, Save2{-1, -1, nullptr}, inj,
+                                     sm, &bar, err);
     }
 }
 
@@ -897,14 +963,15 @@ void run_fwd(const LaunchCtx &lc, const Maps2 &mc, const Grid &g, const Batch &b
     const int per = std::max(1, e.nz) * 8 * TX;
     const int ng = ga.it >= 0 ? (b.max_rec + per - 1) / per : 0;
     if (e.nx + ng == 0) return;
-    launch_pdl(lc, k2_fwd<N, TX>, dim3(std::max(1, e.nz), e.nx + ng, b.nshot), 8 * TX, 0, mc.p, g, b, c, n, step, stf,
+    auto *kernel = save.amax ? k2_fwd<N, TX, true> : k2_fwd<N, TX, false>;
+    launch_pdl(lc, kernel, dim3(std::max(1, e.nz), e.nx + ng, b.nshot), 8 * TX, 0, mc.p, g, b, c, n, step, stf,
                src_scale, bd, save, ga, ng, err);
 }
 
 template <int N, int TX>
 void run_rev(const LaunchCtx &lc, const Maps2 &mac, const Maps2 &mfc, const Grid &g, const Batch &b, const Fields &ac,
              const Fields &an, int mrev, int roles, const Fields &fc, const Fields &fn, int it, float *acc, int img_mode,
-             const float *stf, float src_scale, const Bands &bd, bool restore, unsigned *err)
+             const float *stf, float src_scale, const Bands &bd, bool restore, const Inject2 &ij, unsigned *err)
 {
     Extent2 e;
     for (int s = 0; s < b.nshot; s++) {
@@ -923,7 +990,7 @@ void run_rev(const LaunchCtx &lc, const Maps2 &mac, const Maps2 &mfc, const Grid
     }
     if (e.nx == 0) return;
     launch_pdl(lc, k2_rev<N, TX>, dim3(e.nz, e.nx, b.nshot * (roles == 3 ? 2 : 1)), 8 * TX, 0, mac.p, mfc.vz, mfc.vx, g, b, ac,
-               an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore ? 1 : 0, err);
+               an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore ? 1 : 0, ij, err);
 }
 
 }  // namespace
@@ -941,16 +1008,16 @@ void launch2_forward(const LaunchCtx &lc, const Step2 &t, const Maps2 &mc, const
 void launch2_reverse(const LaunchCtx &lc, const Step2 &t, const Maps2 &mac, const Maps2 &mfc, const Grid &g,
                      const Batch &b, Fields ac, Fields an, int mrev, int roles, Fields fc, Fields fn, int it,
                      float *acc, int img_mode, const float *stf, float src_scale, const Bands &bd, bool restore,
-                     unsigned *err)
+                     Inject2 ij, unsigned *err)
 {
     if (g.N == 2 && t.tx == 16)
-        run_rev<2, 16>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, err);
+        run_rev<2, 16>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
     else if (g.N == 2)
-        run_rev<2, 32>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, err);
+        run_rev<2, 32>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
     else if (t.tx == 16)
-        run_rev<4, 16>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, err);
+        run_rev<4, 16>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
     else
-        run_rev<4, 32>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, err);
+        run_rev<4, 32>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
 }
 
 }  // namespace smi

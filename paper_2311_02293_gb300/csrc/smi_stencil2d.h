@@ -28,10 +28,22 @@ struct Gather2 {
 // sample `sample` (negative: none); 16-bit storage scales by amax[sample]
 // (device array [nsamp][nshot][6] of the largest magnitudes, zeroed before
 // the first step), which the step before has filled; a step fills
-// amax[next] (negative: none) with the velocities it writes.
+// amax[next] (negative: none) with the velocities it writes.  amax null: a
+// call that saves nothing.
 struct Save2 {
     int sample, next;
     unsigned *amax;
+};
+
+// Adjoint source of the next reverse step (it: its step, negative: none), for
+// the step kernel to add to the adjoint pressure it writes: residuals res at
+// off[shot] + it nrec + r, and per shot the receivers whose stencils meet each
+// cell of 32 columns (cell: [nshot][ncell + 1] positions in ids).
+struct Inject2 {
+    const float *res;
+    const long long *off;
+    const int *cell, *ids;
+    int ncell, it;
 };
 
 bool stencil2d_supported(const Grid &g);
@@ -51,6 +63,6 @@ void launch2_forward(const LaunchCtx &lc, const Step2 &t, const Maps2 &mc, const
 void launch2_reverse(const LaunchCtx &lc, const Step2 &t, const Maps2 &mac, const Maps2 &mfc, const Grid &g,
                      const Batch &b, Fields ac, Fields an, int mrev, int roles, Fields fc, Fields fn, int it,
                      float *acc, int img_mode, const float *stf, float src_scale, const Bands &bd, bool restore,
-                     unsigned *err);
+                     Inject2 ij, unsigned *err);
 
 }  // namespace smi
