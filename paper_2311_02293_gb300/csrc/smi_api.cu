@@ -779,8 +779,8 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                                          !make_maps_fused(fA2, g, A2, nb_shot)))))
                 return fail(SMI_ERR_CUDA, "tensor map encoding failed");
             Maps2 m2F{}, m2F2{}, m2A{}, m2A2{};
-            if (fast2 && (!make_maps2(m2F, g, F, nb_shot, t2) || !make_maps2(m2F2, g, F2, nb_shot, t2) ||
-                          (kind != 0 && (!make_maps2(m2A, g, A, nb_shot, t2) || !make_maps2(m2A2, g, A2, nb_shot, t2)))))
+            if (fast2 && (!make_maps2(m2F, g, F, nb_shot, t2, false) || !make_maps2(m2F2, g, F2, nb_shot, t2, false) ||
+                          (kind != 0 && (!make_maps2(m2A, g, A, nb_shot, t2, true) || !make_maps2(m2A2, g, A2, nb_shot, t2, true)))))
                 return fail(SMI_ERR_CUDA, "tensor map encoding failed");
             // after a single-pass step the written buffers become the current ones
             auto swap_F = [&] {

@@ -66,14 +66,20 @@ using s3::mbar_wait;
 using s3::put;
 using s3::tma4;
 
-// Resident blocks a SM that the register budget allows.  Wide tiles (many
-// shots): enough blocks to hide the load phase of one behind another's
-// arithmetic, 3 forward and 4 reverse (80 and 64 registers, some spilled; 40
-// shots 301 x 1001, 800 steps: reverse at 3 / 4 / 5 blocks 140 / 132 / 139 ms;
-// six-shot forward line at 3 / 4 / 5 blocks 8.1 / 8.9 / 10.2 ms).  Narrow tiles
-// (small launches) are alone on their SM: no spills.
-constexpr int fwd_blocks(int tx) { return tx == 32 ? 3 : 4; }
-constexpr int rev_blocks(int) { return 4; }
+// Tile widths and register budgets, by the 32 x 32 tiles of a launch over the
+// whole grid (all shots).  Below kMany a launch hardly fills the GPU: narrow
+// tiles (more, shorter blocks) and the registers a thread wants (4 blocks of
+// 128 threads a SM, no spills).  Above, the blocks hide each other's load
+// phases: forward 6 narrow blocks a SM (85 registers), reverse 4 wide ones (64,
+// some spilled).  Measured (us a step, or a step pair): forward 201 x 601, 4
+// shots, order 8: narrow 4.3, narrow with 6 blocks 4.9, wide 5.2; 40 shots
+// 301 x 1001 gradient with the forward narrow / 4 blocks 172, narrow / 6 166,
+// wide / 3 169, and the reverse wide / 3 175, wide / 4 165, wide / 5 174, narrow
+// 211; reverse at 8 shots 201 x 601 (1344 tiles) wide 17.7, narrow 18.6, at 4
+// shots wide 12.5, narrow 12.1.
+constexpr int kMany = 1200;
+constexpr int kFwdTX = 16;
+constexpr int kRevBlocks = 4;
 
 enum { FWD = 0, ADJ = 1 };
 
@@ -584,11 +590,12 @@ __device__ __forceinline__ bool tile_fast(const Grid &g, const Batch &b, const T
 }
 
 // SAVE: boundary saving (a call that reverses the field later).
-template <int N, int TX, bool SAVE>
-__global__ void __launch_bounds__(8 * TX, fwd_blocks(TX))
+template <int N, int BLOCKS, bool SAVE>
+__global__ void __launch_bounds__(8 * kFwdTX, BLOCKS)
 k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fields n, int step, const float *stf,
        float src_scale, Bands bd, Save2 save, Gather2 ga, int ng, unsigned *err)
 {
+    constexpr int TX = kFwdTX;
     __shared__ __align__(128) float sm[Lay<N, TX>::FA];
     __shared__ __align__(8) uint64_t bar;
     Tile t;
@@ -820,7 +827,7 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
 // roles 1: adjoint, 2: reconstruction (blockIdx.z = shot), 3: both
 // (blockIdx.z = 2 shot + role, 0 adjoint, 1 reconstruction).
 template <int N, int TX>
-__global__ void __launch_bounds__(8 * TX, rev_blocks(TX))
+__global__ void __launch_bounds__(8 * TX, kRevBlocks)
 k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtensorMap tm_vz,
        const __grid_constant__ CUtensorMap tm_vx, Grid g, Batch b, Fields ac, Fields an, int mrev, int roles, Fields fc,
        Fields fn, int it, float *acc, int img_mode, const float *stf, float src_scale, Bands bd, int restore,
@@ -933,27 +940,27 @@ bool stencil2d_supported(const Grid &g)
     return g.ndim == 2 && (g.N == 2 || g.N == 4) && g.ntot < (1LL << 31) && tile_maps_available();
 }
 
-// Narrow tiles when the wide ones would not give every SM two blocks: the
-// step is then bound by latency, and more, smaller blocks shorten it.
 Step2 step2_tile(const Grid &g, int nshot)
 {
     const long long tiles = (long long)((g.ne[0] + 31) / 32) * ((g.ne[1] + 31) / 32) * nshot;
-    return Step2{tiles < 2 * 152 ? 16 : 32};
+    return Step2{tiles >= kMany};
 }
 
-bool make_maps2(Maps2 &m, const Grid &g, const Fields &f, int nshot, const Step2 &t)
+bool make_maps2(Maps2 &m, const Grid &g, const Fields &f, int nshot, const Step2 &t, bool adjoint)
 {
-    const int pr = t.tx + 4 * g.N - 2, xr = t.tx + 2 * g.N - 1;
-    return make_tile_map(&m.p, g, f.p, nshot, 48, pr) && make_tile_map(&m.vz, g, f.v[0], nshot, 48, xr) &&
-           make_tile_map(&m.vx, g, f.v[1], nshot, 40, pr);
+    const int rev = t.many ? 32 : 16, step = adjoint ? rev : kFwdTX;
+    return make_tile_map(&m.p, g, f.p, nshot, 48, step + 4 * g.N - 2) &&
+           make_tile_map(&m.vz, g, f.v[0], nshot, 48, rev + 2 * g.N - 1) &&
+           make_tile_map(&m.vx, g, f.v[1], nshot, 40, rev + 4 * g.N - 2);
 }
 
 namespace {
 
-template <int N, int TX>
+template <int N, int BLOCKS>
 void run_fwd(const LaunchCtx &lc, const Maps2 &mc, const Grid &g, const Batch &b, const Fields &c, const Fields &n, int step,
              const float *stf, float src_scale, const Bands &bd, const Save2 &save, const Gather2 &ga, unsigned *err)
 {
+    constexpr int TX = kFwdTX;
     Extent2 e;
     for (int s = 0; s < b.nshot; s++) {
         int lo[3], hi[3];
@@ -963,7 +970,7 @@ void run_fwd(const LaunchCtx &lc, const Maps2 &mc, const Grid &g, const Batch &b
     const int per = std::max(1, e.nz) * 8 * TX;
     const int ng = ga.it >= 0 ? (b.max_rec + per - 1) / per : 0;
     if (e.nx + ng == 0) return;
-    auto *kernel = save.amax ? k2_fwd<N, TX, true> : k2_fwd<N, TX, false>;
+    auto *kernel = save.amax ? k2_fwd<N, BLOCKS, true> : k2_fwd<N, BLOCKS, false>;
     launch_pdl(lc, kernel, dim3(std::max(1, e.nz), e.nx + ng, b.nshot), 8 * TX, 0, mc.p, g, b, c, n, step, stf,
                src_scale, bd, save, ga, ng, err);
 }
@@ -999,10 +1006,10 @@ void launch2_forward(const LaunchCtx &lc, const Step2 &t, const Maps2 &mc, const
                      Fields n, int step, const float *stf, float src_scale, const Bands &bd, Save2 save, Gather2 ga,
                      unsigned *err)
 {
-    if (g.N == 2 && t.tx == 16) run_fwd<2, 16>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
-    else if (g.N == 2) run_fwd<2, 32>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
-    else if (t.tx == 16) run_fwd<4, 16>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
-    else run_fwd<4, 32>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
+    if (g.N == 2 && !t.many) run_fwd<2, 4>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
+    else if (g.N == 2) run_fwd<2, 6>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
+    else if (!t.many) run_fwd<4, 4>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
+    else run_fwd<4, 6>(lc, mc, g, b, c, n, step, stf, src_scale, bd, save, ga, err);
 }
 
 void launch2_reverse(const LaunchCtx &lc, const Step2 &t, const Maps2 &mac, const Maps2 &mfc, const Grid &g,
@@ -1010,11 +1017,11 @@ void launch2_reverse(const LaunchCtx &lc, const Step2 &t, const Maps2 &mac, cons
                      float *acc, int img_mode, const float *stf, float src_scale, const Bands &bd, bool restore,
                      Inject2 ij, unsigned *err)
 {
-    if (g.N == 2 && t.tx == 16)
+    if (g.N == 2 && !t.many)
         run_rev<2, 16>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
     else if (g.N == 2)
         run_rev<2, 32>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
-    else if (t.tx == 16)
+    else if (!t.many)
         run_rev<4, 16>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);
     else
         run_rev<4, 32>(lc, mac, mfc, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore, ij, err);

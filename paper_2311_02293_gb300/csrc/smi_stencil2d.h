@@ -12,10 +12,10 @@ namespace smi {
 struct Maps2 {
     CUtensorMap p, vz, vx;
 };
-// Tile width along x of a batch: chosen once a call by step2_tile, from the
+// How a batch's steps are cut, chosen once a call by step2_tile from the
 // points of a launch.
 struct Step2 {
-    int tx;                // 16 or 32
+    bool many;             // enough tiles to fill the GPU several times
 };
 // Receivers' samples read by a forward step: p before the step is the
 // pressure after step `it` (it < 0: none).
@@ -48,7 +48,8 @@ struct Inject2 {
 
 bool stencil2d_supported(const Grid &g);
 Step2 step2_tile(const Grid &g, int nshot);
-bool make_maps2(Maps2 &m, const Grid &g, const Fields &f, int nshot, const Step2 &t);
+// adjoint: maps of the adjoint fields (else of the source field).
+bool make_maps2(Maps2 &m, const Grid &g, const Fields &f, int nshot, const Step2 &t, bool adjoint);
 
 // One time step in one launch, from state c into state n (the same arrays'
 // second set; memory variables included).  step = steps elapsed (the box).
