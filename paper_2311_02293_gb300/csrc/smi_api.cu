@@ -324,6 +324,7 @@ int validate_and_setup(const smi_model *m, const smi_geometry *geo, const smi_wa
             long long c = 1;
             for (int b = 0; b < 3; b++) c *= bd.hi[a][sd][b] - bd.lo[a][sd][b] + 1;
             bd.count += c;
+            for (int b = 0; b < 2; b++) bd.sw[a][sd][b] = bd.hi[a][sd][b] - bd.lo[a][sd][b] + 1;
             for (int b = 0; b < 2; b++)
                 band_divisor((unsigned)(bd.hi[a][sd][b] - bd.lo[a][sd][b] + 1), bd.dm[a][sd][b], bd.dl[a][sd][b]);
         }
@@ -841,13 +842,14 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             const int nsteps = kind == 5 || kind == 7 ? 0 : kind != 0 ? S.nt_fwd : S.nt;
             if (tiles && nsteps > 0 && kind != 0) {
                 if (bd.prec != SMI_PREC_F32) launch_zero(lc, d_absmax, sizeof(unsigned) * namax);
-                // interpolation in time reads the whole band, which a 2D step stores inside its box
-                if (fast2 && S.dr > 1) launch_zero(lc, bd.data, (size_t)nb_shot * S.nsamp * bd.count * band_bytes(bd.prec));
+                // interpolation in time reads more of a sample than its step's box, where alone it is stored
+                if (S.dr > 1) launch_zero(lc, bd.data, (size_t)nb_shot * S.nsamp * bd.count * band_bytes(bd.prec));
             }
             for (int it = 0; it < nsteps; it++) {
-                // (the 2D steps store their bands; the 3D pressure kernel stores those of the next step
-                // in FP32, or finds their largest magnitudes)
-                if (kind != 0 && it % S.dr == 0 && !fast2 && !(tile3 && it > 0 && bd.prec == SMI_PREC_F32))
+                // (the 2D steps store their bands; the 3D pressure kernel stores those of the next step,
+                // or with 16-bit storage and a free surface finds their largest magnitudes)
+                if (kind != 0 && it % S.dr == 0 && !fast2 &&
+                    !(tile3 && it > 0 && (bd.prec == SMI_PREC_F32 || !g.freesurf)))
                     launch_save_bands(lc, g, b, F, bd, it / S.dr,
                                       d_absmax + (tile3 ? 6 * (size_t)nb_shot * (it / S.dr) : 0), tile3);
                 tm.begin(0);
@@ -860,13 +862,18 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     swap_F();
                 } else if (tile3) {
                     const Gather3 ga{seis, d_soff, max_rec > 0 && it <= S.nt ? it - 1 : -1};
-                    launch3_v(lc, mF, g, b, F, it, 0, ga, Restore3{bd, {}, -1}, d_wait, ctr++);
-                    launch_free_surface(lc, g, F.v[0], nb_shot, kFsMirrorV);
-                    Save3 save{bd, d_absmax, -1};
+                    Save3 save{bd, nullptr, -1, false};
                     if (kind != 0 && (it + 1) % S.dr == 0 && (it + 1) / S.dr < S.nsamp) {
+                        int nlo[3], nhi[3];
+                        batch_box(S.box_src, it + 1, nlo, nhi);
+                        save.bd = clip_bands(bd, g.ndim, nlo, nhi);
                         save.sample = (it + 1) / S.dr;
-                        save.amax = d_absmax + 6 * (size_t)nb_shot * save.sample;
+                        if (bd.prec != SMI_PREC_F32) save.amax = d_absmax + 6 * (size_t)nb_shot * save.sample;
+                        save.find = g.freesurf && bd.prec != SMI_PREC_F32;
                     }
+                    launch3_v(lc, mF, g, b, F, it, 0, ga, Restore3{bd, {}, -1}, save.find ? nullptr : save.amax, d_wait,
+                              ctr++);
+                    launch_free_surface(lc, g, F.v[0], nb_shot, kFsMirrorV);
                     launch3_p(lc, mF, nullptr, g, b, F, it, 0, d_wait, nullptr, 0, it < S.nt ? S.stf : nullptr,
                               (float)S.src_scale, save, ctr++);
                 } else if (fast2) {                    // CPML, source, boundary saving and samples in one launch
@@ -967,7 +974,13 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             const int mode = (kind == 2 || kind == 3 || kind == 7) ? 0 : (norm ? 2 : 1);
             auto restore = [&](int it) {
                 if (S.dr == 1) launch_restore_bands(lc, g, b, F, bd, it);
-                else launch_restore_bands_interp(lc, g, b, F, bd, time_weights(it, S.dr, S.nsamp));
+                else {
+                    // zero in every sample of the window outside the box of its last step
+                    const TimeWeights tw = time_weights(it, S.dr, S.nsamp);
+                    int nlo[3], nhi[3];
+                    batch_box(S.box_src, std::min((tw.first + 2 * kTimeR - 1) * S.dr, S.nt_fwd - 1), nlo, nhi);
+                    launch_restore_bands_interp(lc, g, b, F, clip_bands(bd, g.ndim, nlo, nhi), tw);
+                }
             };
             // one reverse step of the source field (reconstruction with the fused
             // imaging / gradient accumulation), then its boundary re-imposed
@@ -975,9 +988,9 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 tm.begin(2);
                 if (fast3) {
                     launch3_p(lc, mF, &mA, g, b, F, it, 2, d_wait, acc, mode, S.stf, (float)S.src_scale,
-                              Save3{bd, nullptr, -1}, ctr++);
+                              Save3{bd, nullptr, -1, false}, ctr++);
                     launch_free_surface(lc, g, F.p, nb_shot, kFsMirrorP);
-                    launch3_v(lc, mF, g, b, F, it, 2, Gather3{nullptr, nullptr, -1}, Restore3{bd, {}, -1}, d_wait, ctr++);
+                    launch3_v(lc, mF, g, b, F, it, 2, Gather3{nullptr, nullptr, -1}, Restore3{bd, {}, -1}, nullptr, d_wait, ctr++);
                 } else {
                     int blo[3], bhi[3];
                     batch_box(S.box_src, it, blo, bhi);
@@ -1059,11 +1072,16 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     launch3_fused(lc, fA, fM, g, b, A, A2, mrev, 1, d_wait);
                     swap_A();
                 } else if (tile3) {
-                    const Restore3 rs{bd, {F.v[0], F.v[1], F.v[2]}, kind != 5 && S.dr == 1 ? it : -1};
-                    launch3_v(lc, mA, g, b, A, mrev, 1, Gather3{nullptr, nullptr, -1}, rs, d_wait, ctr++);
+                    Restore3 rs{bd, {F.v[0], F.v[1], F.v[2]}, kind != 5 && S.dr == 1 ? it : -1};
+                    if (rs.it >= 0) {          // outside the step's box the source field is zero already
+                        int nlo[3], nhi[3];
+                        batch_box(S.box_src, it, nlo, nhi);
+                        rs.bd = clip_bands(bd, g.ndim, nlo, nhi);
+                    }
+                    launch3_v(lc, mA, g, b, A, mrev, 1, Gather3{nullptr, nullptr, -1}, rs, nullptr, d_wait, ctr++);
                     launch_free_surface(lc, g, A.v[0], nb_shot, kFsFoldV);
                     launch3_p(lc, mA, nullptr, g, b, A, mrev, 1, d_wait, nullptr, 0, nullptr, 0.0f,
-                              Save3{bd, nullptr, -1}, ctr++);
+                              Save3{bd, nullptr, -1, false}, ctr++);
                 } else if (fast2) {
                     reverse2(it, mrev);
                 } else {

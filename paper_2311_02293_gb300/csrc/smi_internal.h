@@ -80,6 +80,7 @@ struct Bands {
     long long count;             // values per shot per step
     long long off[3][2];         // start of (axis, side) within one step
     int lo[3][2][3], hi[3][2][3];  // region of (axis, side): inclusive bounds per axis
+    int sw[3][2][2];               // widths of the stored region along z and x (a clipped region keeps them)
     int prec;                    // SMI_PREC_*
     void *data;                  // [nshot][nt][count] of float / half / bf16
     float *scale;                // [nshot][nt][3][2] (16-bit storage only)
@@ -97,6 +98,29 @@ inline void band_divisor(unsigned d, unsigned &m, int &l)
     l = 0;
     while ((1ull << l) < d) l++;
     m = (unsigned)(((1ull << 32) * ((1ull << l) - d)) / d + 1);
+}
+
+// The parts of the bands inside a box [lo, hi], at their places in the store.
+inline Bands clip_bands(const Bands &b, int ndim, const int *lo, const int *hi)
+{
+    Bands c = b;
+    for (int a = 0; a < ndim; a++)
+        for (int sd = 0; sd < 2; sd++) {
+            int from[3];
+            for (int e = 0; e < 3; e++) {
+                const int l = e < ndim && lo[e] > b.lo[a][sd][e] ? lo[e] : b.lo[a][sd][e];
+                const int h = e < ndim && hi[e] < b.hi[a][sd][e] ? hi[e] : b.hi[a][sd][e];
+                from[e] = l - b.lo[a][sd][e];
+                c.lo[a][sd][e] = l;
+                c.hi[a][sd][e] = h;
+            }
+            c.off[a][sd] += from[0] + (long long)b.sw[a][sd][0] * (from[1] + (long long)b.sw[a][sd][1] * from[2]);
+            for (int e = 0; e < 2; e++) {
+                const int w = c.hi[a][sd][e] - c.lo[a][sd][e] + 1;
+                if (w > 0) band_divisor((unsigned)w, c.dm[a][sd][e], c.dl[a][sd][e]);
+            }
+        }
+    return c;
 }
 
 // ---------------------------------------------------------------------------
@@ -185,6 +209,7 @@ void launch_save_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Field
 void launch_restore_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f,
                           Bands bd, int it);
 // Band of a step between stored samples (decimated boundaries).
+// (bd: the parts to restore)
 void launch_restore_bands_interp(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, Bands bd,
                                  const TimeWeights &tw);
 void launch_residual(const LaunchCtx &lc, const float *seis, const float *dobs, long long n,

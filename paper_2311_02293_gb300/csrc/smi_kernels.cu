@@ -560,7 +560,10 @@ __global__ void k_band_absmax(Grid g, Fields f, Bands bd, unsigned *amax)
 #pragma unroll
     for (int q = 0; q < kBandVals; q++) {
         const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-        if (u < R.n) m = fmaxf(m, fabsf(v[R.node(g, u)]));
+        if (u >= R.n) continue;
+        int node, place;
+        R.at(g, u, node, place);
+        m = fmaxf(m, fabsf(v[node]));
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(amax + s * 6 + blockIdx.y, __float_as_uint(m));
@@ -568,100 +571,77 @@ __global__ void k_band_absmax(Grid g, Fields f, Bands bd, unsigned *amax)
 
 __global__ void k_band_save(Grid g, Fields f, Bands bd, int it, const unsigned *amax)
 {
-    const BandRegion R(bd, blockIdx.y);
     pdl_wait();
     pdl_trigger();
+    const BandRegion R(bd, blockIdx.y);
     if (R.a >= g.ndim || R.n <= 0) return;
     const int s = blockIdx.z;
     const float *v = f.v[R.a] + (long long)s * g.ntot;
-    const long long o0 = ((long long)s * bd.nt + it) * bd.count + R.off;
-    float x[kBandVals];
-#pragma unroll
-    for (int q = 0; q < kBandVals; q++) {
-        const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-        x[q] = u < R.n ? v[R.node(g, u)] : 0.0f;
-    }
-    // 16-bit storage scaled per (step, axis, side): the largest magnitude
-    // maps to 2^14 (FP16) or 1 (BF16).
-    float inv = 1.0f;
+    const long long b0 = (long long)s * bd.nt + it;
+    float scale = 1.0f;
     if (bd.prec != SMI_PREC_F32) {
-        const float m = __uint_as_float(amax[s * 6 + blockIdx.y]);
-        const float scale = m > 0.0f ? m / (bd.prec == SMI_PREC_F16 ? 16384.0f : 1.0f) : 0.0f;
-        if (blockIdx.x == 0 && threadIdx.x == 0) bd.scale[((long long)s * bd.nt + it) * 6 + blockIdx.y] = scale;
-        inv = scale;
+        scale = band_scale(bd, amax[s * 6 + blockIdx.y]);
+        if (blockIdx.x == 0 && threadIdx.x == 0) bd.scale[b0 * 6 + blockIdx.y] = scale;
+    }
+    const float inv = band_inv(scale);
+    float x[kBandVals];
+    int place[kBandVals];
+#pragma unroll
+    for (int q = 0; q < kBandVals; q++) {
+        const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
+        int node;
+        R.at(g, min(u, R.n - 1), node, place[q]);
+        x[q] = v[node];
     }
 #pragma unroll
     for (int q = 0; q < kBandVals; q++) {
         const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-        if (u >= R.n) continue;
-        if (bd.prec == SMI_PREC_F32) {
-            static_cast<float *>(bd.data)[o0 + u] = x[q];
-        } else {
-            const float y = inv > 0.0f ? x[q] / inv : 0.0f;
-            if (bd.prec == SMI_PREC_F16) static_cast<__half *>(bd.data)[o0 + u] = __float2half_rn(y);
-            else static_cast<__nv_bfloat16 *>(bd.data)[o0 + u] = __float2bfloat16_rn(y);
-        }
+        if (u < R.n) band_put(bd, b0 * bd.count + place[q], x[q], scale, inv);
     }
 }
 
-__global__ void k_band_restore(Grid g, Fields f, Bands bd, int it)
+// Band of step it: sum_q w_q sample[first+q] over the samples that exist
+// (before sample 0 the field is zero), or with one weight that sample alone.
+// A thread takes kBandVals values and has the loads of all their samples in
+// flight: a step reads 16 stored steps, which L2 holds from the step before.
+template <int NT>
+__global__ void k_band_restore(Grid g, Fields f, Bands bd, TimeWeights tw)
 {
+    pdl_wait();
+    pdl_trigger();
     const BandRegion R(bd, blockIdx.y);
     if (R.a >= g.ndim || R.n <= 0) return;
     const int s = blockIdx.z;
     float *v = f.v[R.a] + (long long)s * g.ntot;
-    const long long o0 = ((long long)s * bd.nt + it) * bd.count + R.off;
-    const float scale = bd.prec == SMI_PREC_F32 ? 1.0f : bd.scale[((long long)s * bd.nt + it) * 6 + blockIdx.y];
-    float x[kBandVals];
+    int node[kBandVals], place[kBandVals];
 #pragma unroll
     for (int q = 0; q < kBandVals; q++) {
         const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-        x[q] = 0.0f;
-        if (u < R.n) {
-            if (bd.prec == SMI_PREC_F32) x[q] = static_cast<const float *>(bd.data)[o0 + u];
-            else if (bd.prec == SMI_PREC_F16) x[q] = __half2float(static_cast<const __half *>(bd.data)[o0 + u]) * scale;
-            else x[q] = __bfloat162float(static_cast<const __nv_bfloat16 *>(bd.data)[o0 + u]) * scale;
+        R.at(g, min(u, R.n - 1), node[q], place[q]);
+    }
+    float x[kBandVals] = {};
+#pragma unroll
+    for (int t0 = 0; t0 < NT; t0 += 8) {
+        constexpr int M = NT < 8 ? NT : 8;
+        float y[M][kBandVals], wt[M];
+#pragma unroll
+        for (int t = 0; t < M; t++) {
+            const int k = tw.first + t0 + t, kc = min(max(k, 0), tw.nsamp - 1);
+            const long long b0 = (long long)s * bd.nt + kc;
+            wt[t] = k == kc ? tw.w[t0 + t] : 0.0f;
+            if (bd.prec != SMI_PREC_F32) wt[t] *= bd.scale[b0 * 6 + blockIdx.y];
+#pragma unroll
+            for (int q = 0; q < kBandVals; q++) y[t][q] = band_load(bd, b0 * bd.count + place[q], 1.0f);
         }
+#pragma unroll
+        for (int t = 0; t < M; t++)
+#pragma unroll
+            for (int q = 0; q < kBandVals; q++) x[q] = NT == 1 ? wt[t] * y[t][q] : x[q] + wt[t] * y[t][q];
     }
 #pragma unroll
     for (int q = 0; q < kBandVals; q++) {
         const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-        if (u < R.n) v[R.node(g, u)] = x[q];
-    }
-}
-
-// Band of a step between stored samples: sum_q w_q sample[first+q] over the
-// samples that exist (before sample 0 the field is zero).
-__global__ void k_band_restore_interp(Grid g, Fields f, Bands bd, TimeWeights tw)
-{
-    const BandRegion R(bd, blockIdx.y);
-    if (R.a >= g.ndim || R.n <= 0) return;
-    const int s = blockIdx.z;
-    float *v = f.v[R.a] + (long long)s * g.ntot;
-    float x[kBandVals];
-#pragma unroll
-    for (int q = 0; q < kBandVals; q++) x[q] = 0.0f;
-#pragma unroll
-    for (int t = 0; t < 2 * kTimeR; t++) {
-        const int k = tw.first + t;
-        if (k < 0 || k >= tw.nsamp || tw.w[t] == 0.0f) continue;
-        const long long o0 = ((long long)s * bd.nt + k) * bd.count + R.off;
-        const float wt = bd.prec == SMI_PREC_F32 ? tw.w[t] : tw.w[t] * bd.scale[((long long)s * bd.nt + k) * 6 + blockIdx.y];
-#pragma unroll
-        for (int q = 0; q < kBandVals; q++) {
-            const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-            if (u >= R.n) continue;
-            float y;
-            if (bd.prec == SMI_PREC_F32) y = static_cast<const float *>(bd.data)[o0 + u];
-            else if (bd.prec == SMI_PREC_F16) y = __half2float(static_cast<const __half *>(bd.data)[o0 + u]);
-            else y = __bfloat162float(static_cast<const __nv_bfloat16 *>(bd.data)[o0 + u]);
-            x[q] += wt * y;
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < kBandVals; q++) {
-        const int u = (blockIdx.x * kBandVals + q) * blockDim.x + threadIdx.x;
-        if (u < R.n) v[R.node(g, u)] = x[q];
+        if (u < R.n) v[node[q]] = x[q];
     }
 }
 
@@ -1083,19 +1063,22 @@ void launch_save_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Field
     launch_pdl(lc, k_band_save, grid, kThreads, 0, g, f, bd, it, absmax_tmp);
 }
 
-void launch_restore_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, Bands bd, int it)
-{
-    const dim3 grid = band_grid(bd, b.nshot);
-    k_band_restore<<<grid, kThreads, 0, S(lc)>>>(g, f, bd, it);
-    ++*lc.launches;
-}
-
 void launch_restore_bands_interp(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, Bands bd,
                                  const TimeWeights &tw)
 {
-    const dim3 grid = band_grid(bd, b.nshot);
-    k_band_restore_interp<<<grid, kThreads, 0, S(lc)>>>(g, f, bd, tw);
-    ++*lc.launches;
+    bool one = true;                           // a step on a stored sample
+    for (int q = 1; q < 2 * kTimeR; q++) one = one && tw.w[q] == 0.0f;
+    if (one) launch_pdl(lc, k_band_restore<1>, band_grid(bd, b.nshot), kThreads, 0, g, f, bd, tw);
+    else launch_pdl(lc, k_band_restore<2 * kTimeR>, band_grid(bd, b.nshot), kThreads, 0, g, f, bd, tw);
+}
+
+void launch_restore_bands(const LaunchCtx &lc, const Grid &g, const Batch &b, Fields f, Bands bd, int it)
+{
+    TimeWeights tw{};
+    tw.first = it;
+    tw.nsamp = bd.nt;
+    tw.w[0] = 1.0f;
+    launch_restore_bands_interp(lc, g, b, f, bd, tw);
 }
 
 void launch_residual(const LaunchCtx &lc, const float *seis, const float *dobs, long long n, int mode,

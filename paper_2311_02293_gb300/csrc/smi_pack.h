@@ -146,4 +146,14 @@ __device__ __forceinline__ Q4 clear_if(const Q4 &q, const bool (&z)[4])
     return quad(x);
 }
 
+// Largest magnitude of the quad's nodes in mask, over the warp.
+__device__ __forceinline__ unsigned warp_max(const Q4 &q, unsigned mask)
+{
+    float v[4], m = 0.0f;
+    split(q, v);
+#pragma unroll
+    for (int r = 0; r < 4; r++) m = mask >> r & 1u ? fmaxf(m, fabsf(v[r])) : m;
+    return __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+}
+
 }  // namespace smi

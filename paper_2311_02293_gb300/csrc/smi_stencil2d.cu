@@ -257,16 +257,6 @@ __device__ __forceinline__ void band_restore(const Bands &bd, float scale, long 
         if (mask >> r & 1u) v[r] = keep >> r & 1u ? band_load(bd, base + o + r, scale) : 0.0f;
     q = quad(v);
 }
-// Largest magnitude of the quad's nodes in mask, over the warp.
-__device__ __forceinline__ unsigned warp_max(const Q4 &q, unsigned mask)
-{
-    float v[4], m = 0.0f;
-    split(q, v);
-#pragma unroll
-    for (int r = 0; r < 4; r++) m = mask >> r & 1u ? fmaxf(m, fabsf(v[r])) : m;
-    return __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-}
-
 // One velocity quad: v -+ b D, the memory variable m of the v grid (B, A: its
 // coefficients), and the operand that the pressure update differentiates
 // (forward: v; adjoint: v + e), returned.

@@ -192,24 +192,27 @@ struct PMaps {
 // ===========================================================================
 // Velocity kernel.  FWD / ADJ: v_a -= dt b_a D_a (p with its CPML term); REC:
 // v_a += dt b_a D_a p on L_a+N-1..H_a-N, zero outside the previous box.
+// MAG (FWD): the largest band magnitudes of the new velocities go into amax.
 // Afterwards, by all CTAs: FWD the receivers' samples of p (step ga.it), ADJ
 // the band of the source field from the store (rs.it).
-template <int N, int MODE>
+template <int N, int MODE, bool MAG>
 __global__ void __launch_bounds__(NTHR, SMI_MINB)
-k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, Gather3 ga, Restore3 rs, unsigned *err,
-     unsigned *ctr)
+k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, Gather3 ga, Restore3 rs,
+     unsigned *amax, unsigned *err, unsigned *ctr)
 {
     using La = VLay<N, MODE>;
     extern __shared__ __align__(128) float sm[];
     float *sv = sm + La::oV, *sr = sm + La::oR, *se = sm + La::oE;
     __shared__ __align__(8) uint64_t bar[DEPTH];
     __shared__ Coefs co;
+    __shared__ unsigned smx[6];               // largest band magnitudes of the item (FWD with amax)
     __shared__ int next[2];                   // the CTA's next item, in turn
     const int tid = threadIdx.x, tzi = tid & 7, txi = tid >> 3;
     if (tid == 0) {
         for (int k = 0; k < DEPTH; k++) mbar_init(&bar[k], 1);
         mbar_fence_init();
     }
+    if (tid < 6) smx[tid] = 0u;
     __syncthreads();
     Sched sd;
     sched_shot(g, b, MODE, step, 0, 0, lc.chunk, sd);   // (the box tables are older than the loop)
@@ -307,6 +310,28 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
         // CPML planes of the item: every plane of a tile that meets a z or x slab, the y-slab planes of the others
         const bool zxb = MODE != REC && (z_slab_tile(g, &tm.p, &tm.p, z0).tm || x_slab_tile(g, &tm.p, &tm.p, x0 - N + 1, La::PR).tm);
         const bool xg = MODE == FWD && x_group(g, ox, lc.x0);
+        // boundary bands (2N - 1 half nodes across each face): the quad's nodes per side of z, the side of x
+        // that holds the column, the physical nodes; a plane's part is decided per plane
+        unsigned bz0 = 0u, bz1 = 0u, bph = 0u;
+        int bxs = -1;
+        bool bzt = false, bxt = false;         // the tile meets a z band, an x band
+        if (MAG) {
+            constexpr unsigned W = 2 * N - 2;
+            const bool px = me.act && in_range(ox, g.L[1], g.H[1]);
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                bz0 |= px && (unsigned)(oz + r - g.L[0] + N) <= W ? 1u << r : 0u;
+                bz1 |= px && (unsigned)(oz + r - g.H[0] + N - 1) <= W ? 1u << r : 0u;
+                bph |= me.act && in_range(oz + r, g.L[0], g.H[0]) ? 1u << r : 0u;
+            }
+            bxs = (unsigned)(ox - g.L[1] + N) <= W ? 0 : ((unsigned)(ox - g.H[1] + N - 1) <= W ? 1 : -1);
+            bzt = (z0 <= g.L[0] + N - 2 && z0 + TZ - 1 >= g.L[0] - N) || (z0 <= g.H[0] + N - 1 && z0 + TZ - 1 >= g.H[0] - N + 1);
+            bxt = (x0 <= g.L[1] + N - 2 && x0 + TX - 1 >= g.L[1] - N) || (x0 <= g.H[1] + N - 1 && x0 + TX - 1 >= g.H[1] - N + 1);
+        }
+        auto note = [&](int k, const Q4 &v, unsigned mask) {      // uniform call
+            const unsigned u = warp_max(v, mask);
+            if ((tid & 31) == 0 && u) atomicMax(&smx[k], u);
+        };
         const bool lastz = oz + 4 >= g.px;
         const int rxrow = ox + 1 < g.ne[1] ? txi + 1 : txi;        // the last node's neighbour is itself
         float *const mzp = f.psip[0] + (s * g.slab_n[0] + me.zq + (long long)g.zp * ox);
@@ -380,6 +405,11 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
                     v = clear_if(v, cl);
                 }
                 if (me.act) stq(f.v[2] + sh + o, v);
+                if (BAND && MAG) {
+                    const unsigned in = in_range(ox, g.L[1], g.H[1]) ? bph : 0u;
+                    if ((unsigned)(y - g.L[2] + N) <= 2 * N - 2) note(4, v, in);
+                    if ((unsigned)(y - g.H[2] + N - 1) <= 2 * N - 2) note(5, v, in);
+                }
             }
             float W[12];
             window(W, pt);
@@ -413,6 +443,10 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
                     v = clear_if(v, cl);
                 }
                 if (me.act) stq(f.v[1] + sh + o, v);
+                if (BAND && MAG && bxt && in_range(y, g.L[2], g.H[2])) {
+                    note(2, v, bxs == 0 ? bph : 0u);
+                    note(3, v, bxs == 1 ? bph : 0u);
+                }
             }
             // ---- z component ----
             {
@@ -446,6 +480,10 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
                     v = clear_if(v, cl);
                 }
                 if (me.act) stq(f.v[0] + sh + o, v);
+                if (BAND && MAG && bzt && in_range(y, g.L[2], g.H[2])) {
+                    note(0, v, bz0);
+                    note(1, v, bz1);
+                }
             }
             kp = kp + 1 == La::S ? 0 : kp + 1;
             kq = kq + 1 == La::S ? 0 : kq + 1;
@@ -456,7 +494,10 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
         };
         auto one = [&](auto kc, int y) {
             const bool band = MODE == REC ? clip || !in_range(y, it.plo[2], it.phi[2])
-                                          : zxb || yslab(g, y) || (MODE == ADJ && yslab(g, y + N));
+                                          : zxb || yslab(g, y) || (MODE == ADJ && yslab(g, y + N)) ||
+                                                (MAG &&
+                                                 (bzt || bxt || (unsigned)(y - g.L[2] + N) <= 2 * N - 2 ||
+                                                  (unsigned)(y - g.H[2] + N - 1) <= 2 * N - 2));
             if (band) body(kc, std::true_type{}, y);
             else body(kc, std::false_type{}, y);
         };
@@ -466,6 +507,10 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
             rotate_queue<G>(q);
         }
         if (__syncthreads_or(!ok)) break;
+        if (MAG && tid < 6 && smx[tid]) {         // (the next item notes nothing before its barrier)
+            atomicMax(amax + s * 6 + tid, smx[tid]);
+            smx[tid] = 0u;
+        }
     }
     if (__syncthreads_or(!ok)) {
         if (tid == 0) atomicOr(err, 1u);
@@ -481,7 +526,7 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
 // term), FWD with the source; REC: acc += lp * (div v | p), p += dt kappa div v
 // - source, zero outside the previous box, on the physical domain.
 // Afterwards FWD, by all CTAs: the next stored boundary (or its largest
-// magnitudes, 16-bit storage), from the velocities this kernel only reads.
+// magnitudes), from the velocities this kernel only reads.
 template <int N, int MODE>
 __global__ void __launch_bounds__(NTHR, SMI_MINB)
 k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, unsigned *err, float *acc, int img_mode,
@@ -905,13 +950,15 @@ s3::Cut launch_cut(const Grid &g, const Batch &b, int mode, int step, int grid)
 
 template <int N, int MODE>
 void run_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, const Fields &f, int step, const Gather3 &ga,
-           const Restore3 &rs, unsigned *err, unsigned *ctr)
+           const Restore3 &rs, unsigned *amax, unsigned *err, unsigned *ctr)
 {
     constexpr int smem = s3::VLay<N, MODE>::SMEM;
-    static const int grid = grid_for(s3::k3_v<N, MODE>, smem);
+    constexpr bool M = MODE == s3::FWD;
+    auto *kernel = amax ? s3::k3_v<N, MODE, M> : s3::k3_v<N, MODE, false>;
+    static const int grid = std::min(grid_for(s3::k3_v<N, MODE, M>, smem), grid_for(s3::k3_v<N, MODE, false>, smem));
     const s3::VMaps tm{m.p_halo, m.rho_v, m.vz_core, m.vx_core, m.vy_core, m.ezl_p, m.ezh_p, m.exl_p, m.exh_p};
-    launch_pdl(lc, s3::k3_v<N, MODE>, dim3(grid), s3::NTHR, smem, tm, g, b, f, step, launch_cut(g, b, MODE, step, grid), ga,
-               rs, err, ctr);
+    launch_pdl(lc, kernel, dim3(grid), s3::NTHR, smem, tm, g, b, f, step, launch_cut(g, b, MODE, step, grid), ga,
+               rs, amax, err, ctr);
 }
 
 template <int N, int MODE>
@@ -987,17 +1034,16 @@ bool make_maps3(Maps3 &m, const Grid &g, const Fields &f, int nshot, bool slabs)
 }
 
 void launch3_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, Fields f, int step, int mode,
-               Gather3 ga, Restore3 rs, unsigned *err,
-     unsigned *ctr)
+               Gather3 ga, Restore3 rs, unsigned *amax, unsigned *err, unsigned *ctr)
 {
     if (g.N == 2) {
-        if (mode == 0) run_v<2, 0>(lc, m, g, b, f, step, ga, rs, err, ctr);
-        else if (mode == 1) run_v<2, 1>(lc, m, g, b, f, step, ga, rs, err, ctr);
-        else run_v<2, 2>(lc, m, g, b, f, step, ga, rs, err, ctr);
+        if (mode == 0) run_v<2, 0>(lc, m, g, b, f, step, ga, rs, amax, err, ctr);
+        else if (mode == 1) run_v<2, 1>(lc, m, g, b, f, step, ga, rs, amax, err, ctr);
+        else run_v<2, 2>(lc, m, g, b, f, step, ga, rs, amax, err, ctr);
     } else {
-        if (mode == 0) run_v<4, 0>(lc, m, g, b, f, step, ga, rs, err, ctr);
-        else if (mode == 1) run_v<4, 1>(lc, m, g, b, f, step, ga, rs, err, ctr);
-        else run_v<4, 2>(lc, m, g, b, f, step, ga, rs, err, ctr);
+        if (mode == 0) run_v<4, 0>(lc, m, g, b, f, step, ga, rs, amax, err, ctr);
+        else if (mode == 1) run_v<4, 1>(lc, m, g, b, f, step, ga, rs, amax, err, ctr);
+        else run_v<4, 2>(lc, m, g, b, f, step, ga, rs, amax, err, ctr);
     }
 }
 

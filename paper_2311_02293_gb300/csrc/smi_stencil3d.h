@@ -31,12 +31,15 @@ struct Restore3 {
     int it;
 };
 // What the forward pressure kernel also does: the velocities it reads become
-// stored sample `sample` (FP32 storage), or their largest magnitudes per
-// (shot, axis, side) go into amax (16-bit storage; zeroed).  sample < 0: none.
+// stored sample `sample` within bd's regions (16-bit storage scaled by the
+// magnitudes in amax, which the velocity kernel has found), or, with find,
+// their largest magnitudes per (shot, axis, side) go into amax (zeroed).
+// sample < 0: none.
 struct Save3 {
     Bands bd;
     unsigned *amax;
     int sample;
+    bool find;
 };
 
 // One warp waits with the tile kernels' bounded-wait helper on an mbarrier
@@ -62,9 +65,10 @@ bool make_maps3(Maps3 &m, const Grid &g, const Fields &f, int nshot, bool slabs)
 
 // mode 0: forward, 1: adjoint (step = reverse steps elapsed), 2: reconstruction.
 // err: device word, bit 0 set if a bounded wait gave up; ctr: a zeroed device
-// word of this launch (its work counter).
+// word of this launch (its work counter).  amax (forward, may be null): takes
+// the largest magnitude per (shot, axis, side) of the band's velocities.
 void launch3_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, Fields f, int step, int mode,
-               Gather3 ga, Restore3 rs, unsigned *err, unsigned *ctr);
+               Gather3 ga, Restore3 rs, unsigned *amax, unsigned *err, unsigned *ctr);
 // lpm: maps of the adjoint fields, whose pressure the reconstruction mode
 // correlates with (mode 2 only).  stf null: no source.
 void launch3_p(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g, const Batch &b, Fields f,
