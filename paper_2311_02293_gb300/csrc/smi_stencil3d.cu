@@ -935,7 +935,9 @@ s3::Cut launch_cut(const Grid &g, const Batch &b, int mode, int step, int grid)
                 hi[a] = std::min(hi[a], g.H[a]);
             }
         if (hi[0] < lo[0] || hi[1] < lo[1]) continue;
-        cols += (long long)((hi[0] - (lo[0] & ~31)) / s3::TZ + 1) * ((hi[1] - lo[1]) / s3::TX + 1);
+        int base, rows;
+        s3::tile_rows(lo[0], hi[0], base, rows);
+        cols += (long long)rows * ((hi[1] - lo[1]) / s3::TX + 1);
         ylen = std::max(ylen, hi[2] - lo[2] + 1);
         x0 = std::min(x0, lo[1]);
     }

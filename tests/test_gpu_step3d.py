@@ -31,6 +31,7 @@ CASES = [
     (61, 62, 19, 8, 4, False, {"dr": 3}),              # two slabs an axis, one each a tile
     (70, 40, 25, 8, 9, True, {"dr": 2, "shell_prec": "bf16"}),
     (33, 30, 28, 8, 8, False, {"freesurf": True}),
+    (28, 40, 20, 8, 6, True, {}),                      # the physical box needs one row of tiles, not two
     (41, 64, 22, 4, 5, True, {"freesurf": True, "use_box": False}),
 ]
 
