@@ -745,12 +745,21 @@ __global__ void k_finalize_grad(long long n, const float *vp, float dt, float *g
 // 4 and the box's z width a multiple of 4 (the host widens the box; G is
 // read only on the half nodes next to the physical domain, which the
 // widened box always covers).
-template <int NDIM>
-__global__ void __launch_bounds__(kThreads) k_rho_acc(Grid g, int nshot, Fields F, Fields A, RhoAcc r, IBox box)
+// Bound by the latency of its loads: one axis per blockIdx.y and the loads of
+// two shots in flight at 4 blocks a SM (60 registers).  All axes in a thread
+// ran in two and a half waves of fewer blocks; 6 and 8 blocks are slower (92.8,
+// 93.3 ms), and so is a dependent launch (93.2).  90 x 110 x 100 + 10 layers, 2
+// shots, 300 steps: a gradient 93.9 -> 91.2 ms.
+__global__ void __launch_bounds__(kThreads, 4) k_rho_acc(Grid g, int nshot, Fields F, Fields A, RhoAcc r, IBox box)
 {
     const int wq = (box.hi[0] - box.lo[0] + 1) >> 2;
     const int w1 = box.hi[1] - box.lo[1] + 1;
     const long long vol = (long long)wq * w1 * (box.hi[2] - box.lo[2] + 1);
+    const int a = blockIdx.y;              // (selected, not indexed: an index would put the pointers on the stack)
+    const float *const fv = a == 0 ? F.v[0] : (a == 1 ? F.v[1] : F.v[2]);
+    const float *const av = a == 0 ? A.v[0] : (a == 1 ? A.v[1] : A.v[2]);
+    float *const pr = a == 0 ? r.vprev[0] : (a == 1 ? r.vprev[1] : r.vprev[2]);
+    float *const gr = a == 0 ? r.G[0] : (a == 1 ? r.G[1] : r.G[2]);
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < vol;
          q += (long long)gridDim.x * blockDim.x) {
         int iq, i1, i2;
@@ -766,37 +775,37 @@ __global__ void __launch_bounds__(kThreads) k_rho_acc(Grid g, int nshot, Fields 
             i2 = (int)(rr / w1);
         }
         const long long k = gidx(g, box.lo[0] + 4 * iq, box.lo[1] + i1, box.lo[2] + i2);
-        float4 c[NDIM];
-#pragma unroll
-        for (int a = 0; a < NDIM; a++) c[a] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (int s = 0; s < nshot; s++) {
-            const long long kk = s * g.ntot + k;
-            float4 v[NDIM], l[NDIM], pv[NDIM];
-#pragma unroll
-            for (int a = 0; a < NDIM; a++) {
-                v[a] = *reinterpret_cast<const float4 *>(F.v[a] + kk);
-                l[a] = *reinterpret_cast<const float4 *>(A.v[a] + kk);
-                pv[a] = *reinterpret_cast<const float4 *>(r.vprev[a] + kk);
-            }
-#pragma unroll
-            for (int a = 0; a < NDIM; a++) {
-                c[a].x += l[a].x * (pv[a].x - v[a].x);
-                c[a].y += l[a].y * (pv[a].y - v[a].y);
-                c[a].z += l[a].z * (pv[a].z - v[a].z);
-                c[a].w += l[a].w * (pv[a].w - v[a].w);
-                *reinterpret_cast<float4 *>(r.vprev[a] + kk) = v[a];
-            }
+        float4 *const G = reinterpret_cast<float4 *>(gr + k);
+        float4 t = *G;
+        float4 c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        auto add = [&](const float4 &v, const float4 &l, const float4 &pv) {
+            c.x += l.x * (pv.x - v.x);
+            c.y += l.y * (pv.y - v.y);
+            c.z += l.z * (pv.z - v.z);
+            c.w += l.w * (pv.w - v.w);
+        };
+        auto ld = [](const float *x, long long i) { return *reinterpret_cast<const float4 *>(x + i); };
+        int s = 0;
+        for (; s + 2 <= nshot; s += 2) {
+            const long long k0 = s * g.ntot + k, k1 = k0 + g.ntot;
+            const float4 v0 = ld(fv, k0), l0 = ld(av, k0), p0 = ld(pr, k0);
+            const float4 v1 = ld(fv, k1), l1 = ld(av, k1), p1 = ld(pr, k1);
+            add(v0, l0, p0);
+            add(v1, l1, p1);
+            *reinterpret_cast<float4 *>(pr + k0) = v0;
+            *reinterpret_cast<float4 *>(pr + k1) = v1;
         }
-#pragma unroll
-        for (int a = 0; a < NDIM; a++) {
-            float4 *G = reinterpret_cast<float4 *>(r.G[a] + k);
-            float4 t = *G;
-            t.x += c[a].x;
-            t.y += c[a].y;
-            t.z += c[a].z;
-            t.w += c[a].w;
-            *G = t;
+        if (s < nshot) {
+            const long long k0 = s * g.ntot + k;
+            const float4 v0 = ld(fv, k0);
+            add(v0, ld(av, k0), ld(pr, k0));
+            *reinterpret_cast<float4 *>(pr + k0) = v0;
         }
+        t.x += c.x;
+        t.y += c.y;
+        t.z += c.z;
+        t.w += c.w;
+        *G = t;
     }
 }
 
@@ -1157,8 +1166,7 @@ void launch_rho_acc(const LaunchCtx &lc, const Grid &g, int nshot, Fields F, Fie
     box.hi[0] |= 3;
     const long long quads = (long long)((box.hi[0] - box.lo[0] + 1) >> 2) * (box.hi[1] - box.lo[1] + 1) *
                             (box.hi[2] - box.lo[2] + 1);
-    if (g.ndim == 3) k_rho_acc<3><<<blocks_for(quads), kThreads, 0, S(lc)>>>(g, nshot, F, A, r, box);
-    else k_rho_acc<2><<<blocks_for(quads), kThreads, 0, S(lc)>>>(g, nshot, F, A, r, box);
+    k_rho_acc<<<dim3(blocks_for(quads), g.ndim), kThreads, 0, S(lc)>>>(g, nshot, F, A, r, box);
     ++*lc.launches;
 }
 

@@ -385,7 +385,7 @@ struct Sched {
 // multiples of 32 (whole 128-byte lines), unless starting at the box's own quad
 // saves a row of tiles (160 physical nodes from 20: 5 rows, not 6; TMA needs the
 // multiple of 4).  300^3 RTM 371 -> 365 ms, 160^3 RTM with 3 shots 117.1 -> 115.7 ms,
-// 4-parameter gradient 96.4 -> 95.1 ms; forward runs unchanged.
+// two-parameter gradient 96.4 -> 95.1 ms; forward runs unchanged.
 __host__ __device__ __forceinline__ void tile_rows(int lo, int hi, int &base, int &n)
 {
     base = lo & ~31;
