@@ -485,7 +485,9 @@ size_t per_shot_bytes(const Setup &S, int kind)
             if (S.fast2 || S.tile3) b += (size_t)S.nsamp * 6 * 4;          // and largest magnitudes
         }
         if (S.dr > 1) b += fields;                                     // state kept during the continuation
-        b += (size_t)(g.nphys + (S.padacc ? g.ntot : 0)) * 4 * (kind == 1 && S.img_norm ? 2 : 1);  // accumulator (+ illumination)
+        const bool norm = kind == 1 && S.img_norm;                         // accumulator (+ illumination), and the
+        b += (size_t)(S.padacc ? g.ntot : g.nphys) * 4 * (norm ? 2 : 1);   // physical nodes of both
+        if (S.padacc && norm) b += (size_t)g.nphys * 4 * 2;
         if (S.rho_grad) b += (size_t)g.ndim * g.ntot * 4;              // velocities of the previous step
         b += (size_t)S.nt * maxrec * 4 * 2;                            // seis + residual
     }
@@ -731,7 +733,6 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 bd = T.bd;
                 res = T.res;
                 acc = T.acc;
-                if (S.padacc) accc = ba.get<float>((size_t)g.nphys * nacc);
                 partials = T.partials;
             } else if (kind != 0) {
                 for (int k = 0; k < (pp ? 2 : 1); k++) {   // the adjoint reuses the forward's memory variables
@@ -749,7 +750,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                     bd.scale = ba.get<float>((size_t)nb_shot * S.nsamp * 6);
                     if (S.dr > 1) keep = ba.get<float>((size_t)(1 + g.ndim) * g.ntot * nb_shot);
                     acc = ba.get<float>(acc_n * nacc);
-                    if (S.padacc && kind != 6) accc = ba.get<float>((size_t)g.nphys * nacc);   // the physical nodes alone
+                    if (S.padacc && norm) accc = ba.get<float>((size_t)g.nphys * nacc);   // the physical nodes of both
                 } else {
                     part = ba.get<double>((size_t)nb_shot * S.nt);
                 }
@@ -1117,7 +1118,8 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 launch_sum_series(lc, part, nb_shot, S.nt, d_series, s0 > 0);
                 continue;
             }
-            if (S.padacc) {
+            if (S.padacc) {                       // the source pressure is not needed any more
+                if (!accc) accc = F.p;
                 launch_unpad(lc, g, acc, nacc, accc);
                 acc = accc;
             }
