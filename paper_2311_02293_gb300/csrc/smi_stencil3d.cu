@@ -896,7 +896,12 @@ template <class K> int grid_for(K kernel, int smem)
 
 // Planes a chunk of a launch over `cols` tile columns (all shots) of ylen
 // planes.  Large launches: 8 planes (more when that makes over eight items a
-// CTA), so that the sweep stays local (see Sched).  Small ones, whose items
+// CTA), so that the sweep stays local (see Sched).  Launches of one to four
+// 8-plane items a CTA: four items a CTA, of 5 planes or more -- items differ in
+// cost (CPML planes, cut tiles), and the CTAs that draw cheap ones take over
+// (12 planes, or 8 planes in a wave and a part, before: 160^3 migration order 4
+// 115.9 -> 107.5 ms, 131 x 243 x 205 162.2 -> 157.9, 93 x 101 x 87 forward 13.18 ->
+// 12.72; three items a CTA 108.7, 158.4, 12.92).  Smaller ones, whose items
 // run at once: the chunk between 8 and 24 planes that finishes first when an
 // item costs its planes plus a start of about 7, and an SM runs three items
 // as fast as one (measured on 133 x 141 x 127 points, order 4, a step: 22
@@ -906,7 +911,10 @@ int pick_chunk(long long cols, int ylen, int grid, int sms)
     if (cols <= 0 || ylen <= 0) return 1;
     const long long items8 = cols * ((ylen + 7) / 8);
     if (items8 >= 4LL * grid) return (int)std::max<long long>(8, cols * ylen / (8LL * grid));
-    if (items8 >= 2LL * grid) return 12;
+    if (items8 >= grid) {
+        const long long n = 4LL * grid / cols;
+        return (int)std::max<long long>(5, (ylen + n - 1) / n);
+    }
     long long best = -1;
     int cy = ylen;
     for (int n = (ylen + 23) / 24; n <= std::max(1, ylen / 8); n++) {
