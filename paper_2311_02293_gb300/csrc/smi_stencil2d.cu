@@ -29,7 +29,7 @@
 // four to nine.  Against the two-pass kernels with their own launches for
 // sources, receivers and bands (GB300): 201 x 201 order 4 forward, one shot,
 // 16.9 -> 3.2 us a step; 257 x 903 order 8 gradient, one shot, 16-bit
-// boundaries, 69.5 -> 18.6 us a step pair; 301 x 1001, 40 shots, 315 -> 165.
+// boundaries, 69.5 -> 14.6 us a step pair; 301 x 1001, 40 shots, 315 -> 165.
 // Most tiles of a survey meet no slab, box edge, band or source: they run a
 // body without tests or memory variables, in packed pairs (40 shots, whole
 // grid: forward 172 -> 153 us, reverse 353 -> 273).

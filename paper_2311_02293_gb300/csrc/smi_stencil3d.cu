@@ -44,10 +44,10 @@
 // instead of in kernels of their own over the slabs, which re-read the fields
 // at half the bandwidth and took 26 % of a forward and 31 % of an adjoint step
 // at 340^3 (50 % at 130^3).  A step of both kernels, GB300, with those kernels
-// and now: 133 x 141 x 127, order 4, forward 77 -> 34 us; 200^3 extended,
-// order 4, box on, 500 steps, forward 107 -> 79 us, adjoint 171 -> 112,
-// reconstruction 67 -> 48; 340^3 extended, order 8, box on, first 600 steps,
-// adjoint 378 -> 297, forward with 16-bit boundary saving 258 -> 230.
+// and now: 133 x 141 x 127, order 4, forward 77 -> 32 us; 200^3 extended,
+// order 4, box on, 500 steps, forward 107 -> 77 us, adjoint 171 -> 98,
+// reconstruction 67 -> 46; 340^3 extended, order 8, box on, first 600 steps,
+// adjoint 378 -> 279, forward with 16-bit boundary saving 258 -> 179.
 //
 // Every mbarrier wait is bounded; a CTA that gives up issues no more copies,
 // sets bit 0 of the error word, waits once more (bounded) for its copies in

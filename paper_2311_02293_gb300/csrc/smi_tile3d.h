@@ -21,9 +21,6 @@ namespace s3 {
 #ifndef SMI_TX
 #define SMI_TX 16
 #endif
-#ifndef SMI_PFP
-#define SMI_PFP 1
-#endif
 #ifndef SMI_MINB
 #define SMI_MINB 4
 #endif
