@@ -805,9 +805,9 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
             b.rec = S.d_rec + S.rec_offset[s0];
             b.rec_off = d_roff;
             b.max_rec = max_rec;
-            b.tab_src = S.d_tab_src + (size_t)s0 * (S.nt + 1) * 6;
-            b.tab_rec = S.d_tab_rec + (size_t)s0 * (S.nt + 1) * 6;
             b.nt1 = S.nt_fwd + 1;
+            b.tab_src = S.d_tab_src + (size_t)s0 * b.nt1 * 6;
+            b.tab_rec = S.d_tab_rec + (size_t)s0 * b.nt1 * 6;
             b.h_box_src = S.box_src.data() + 6 * (size_t)s0;
             b.h_box_rec = S.box_rec.data() + 6 * (size_t)s0;
             // union of the batch's boxes after n steps (bounds the CPML launches)
