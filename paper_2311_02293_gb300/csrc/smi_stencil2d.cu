@@ -778,8 +778,16 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
         stq(spn + (txi + N - 1) * La::VW + 4 * tzi + 4, np);
         if (own) {
             stq(n.p + sh + k, np);
-            // (nodes outside the physical domain gather values that nobody reads)
-            stq(acc + sh + k, fmaq(lpv, img_mode == 0 ? dv : pv, av));
+            Q4 t = img_mode == 0 ? dv : pv;
+            if (!FAST && img_mode == 0) {      // div v reaches past the box (p does not)
+                float m[4];
+                bool out[4];
+                split(dp, m);
+#pragma unroll
+                for (int r = 0; r < 4; r++) out[r] = m[r] == 0.0f;
+                t = clear_if(t, out);
+            }
+            stq(acc + sh + k, fmaq(lpv, t, av));
             if (img_mode == 2) {               // illumination
                 float *ill = acc + (long long)b.nshot * g.ntot + sh + k;
                 stq(ill, fmaq(pv, pv, ldq(ill)));

@@ -748,8 +748,11 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
                 }
             }
             if (MODE == REC) {
-                // (nodes of the quad outside the physical domain gather values that nobody reads)
-                if (me.act) stq(acc + sh + o, fmaq(ldq(own + La::oL), img_mode == 0 ? div : pv, accv));
+                // (div v reaches past the box, p does not; outside the physical domain p gathers what nobody reads)
+                bool off[4];
+#pragma unroll
+                for (int r = 0; r < 4; r++) off[r] = !in[r];
+                if (me.act) stq(acc + sh + o, fmaq(ldq(own + La::oL), img_mode == 0 ? clear_if(div, off) : pv, accv));
                 if (img_mode == 2 && me.act) {                // illumination
                     float *ill = acc + (long long)b.nshot * g.ntot + sh + o;
                     stq(ill, fmaq(pv, pv, ldq(ill)));
