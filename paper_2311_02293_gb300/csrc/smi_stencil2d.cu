@@ -79,6 +79,7 @@ using s3::tma4;
 // shots wide 12.5, narrow 12.1.
 constexpr int kMany = 1200;
 constexpr int kFwdTX = 16;
+constexpr int kMaxRows = 65535;    // gridDim.y of a launch: longer models take several a step
 constexpr int kRevBlocks = 4;
 
 enum { FWD = 0, ADJ = 1 };
@@ -579,20 +580,22 @@ __device__ __forceinline__ bool tile_fast(const Grid &g, const Batch &b, const T
     return f && !(bands && band_tile<TX>(bd, t.z0, t.x0));
 }
 
-// SAVE: boundary saving (a call that reverses the field later).
+// SAVE: boundary saving (a call that reverses the field later).  Rows of
+// blocks y0 .. y0 + gridDim.y - 1 of the step: ng of receivers, then tiles.
 template <int N, int BLOCKS, bool SAVE>
 __global__ void __launch_bounds__(8 * kFwdTX, BLOCKS)
 k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fields n, int step, const float *stf,
-       float src_scale, Bands bd, Save2 save, Gather2 ga, int ng, unsigned *err)
+       float src_scale, Bands bd, Save2 save, Gather2 ga, int ng, int y0, unsigned *err)
 {
     constexpr int TX = kFwdTX;
     __shared__ __align__(128) float sm[Lay<N, TX>::FA];
     __shared__ __align__(8) uint64_t bar;
     Tile t;
     t.s = blockIdx.z;
-    if ((int)blockIdx.y < ng) {                // receivers: samples of the pressure before the step
+    const int row = (int)blockIdx.y + y0;
+    if (row < ng) {                // receivers: samples of the pressure before the step
         const int nr = b.rec_off[t.s + 1] - b.rec_off[t.s];
-        const int r = (blockIdx.y * gridDim.x + blockIdx.x) * (8 * TX) + threadIdx.x;
+        const int r = (row * gridDim.x + blockIdx.x) * (8 * TX) + threadIdx.x;
         const bool have = r < nr;
         const Stencil &st = b.rec[b.rec_off[t.s] + (have ? r : 0)];
         const float *ps = c.p + t.s * g.ntot + (have ? st.first[0] + g.px * st.first[1] : 0);
@@ -632,7 +635,7 @@ k2_fwd(const __grid_constant__ CUtensorMap tm_p, Grid g, Batch b, Fields c, Fiel
     }
     box_at(b.tab_src, b.nt1, t.s, step, t.lo, t.hi);
     t.z0 = (t.lo[0] & ~3) + 32 * blockIdx.x;
-    t.x0 = t.lo[1] + TX * ((int)blockIdx.y - ng);
+    t.x0 = t.lo[1] + TX * (row - ng);
     if (t.z0 > t.hi[0] || t.x0 > t.hi[1]) {
         if (blockIdx.x + blockIdx.y + blockIdx.z == 0) pdl_wait();   // one block of a launch always waits
         return;
@@ -823,13 +826,13 @@ __device__ __forceinline__ void tile_rec(const CUtensorMap *tm_vz, const CUtenso
 }
 
 // roles 1: adjoint, 2: reconstruction (blockIdx.z = shot), 3: both
-// (blockIdx.z = 2 shot + role, 0 adjoint, 1 reconstruction).
+// (blockIdx.z = 2 shot + role, 0 adjoint, 1 reconstruction).  Tile rows from y0.
 template <int N, int TX>
 __global__ void __launch_bounds__(8 * TX, kRevBlocks)
 k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtensorMap tm_vz,
        const __grid_constant__ CUtensorMap tm_vx, Grid g, Batch b, Fields ac, Fields an, int mrev, int roles, Fields fc,
        Fields fn, int it, float *acc, int img_mode, const float *stf, float src_scale, Bands bd, int restore,
-       Inject2 ij, unsigned *err)
+       Inject2 ij, int y0, unsigned *err)
 {
     __shared__ __align__(128) float sm[Lay<N, TX>::MAXF];
     __shared__ __align__(16) float sinj[32 * TX];
@@ -848,7 +851,7 @@ k2_rev(const __grid_constant__ CUtensorMap tm_lp, const __grid_constant__ CUtens
         box_at(b.tab_rec, b.nt1, t.s, mrev, t.lo, t.hi);
     }
     t.z0 = (t.lo[0] & ~3) + 32 * blockIdx.x;
-    t.x0 = t.lo[1] + TX * blockIdx.y;
+    t.x0 = t.lo[1] + TX * ((int)blockIdx.y + y0);
     if (t.z0 > t.hi[0] || t.x0 > t.hi[1]) {
         if (blockIdx.x + blockIdx.y + blockIdx.z == 0) pdl_wait();
         return;
@@ -968,10 +971,10 @@ void run_fwd(const LaunchCtx &lc, const Maps2 &mc, const Grid &g, const Batch &b
     }
     const int per = std::max(1, e.nz) * 8 * TX;
     const int ng = ga.it >= 0 ? (b.max_rec + per - 1) / per : 0;
-    if (e.nx + ng == 0) return;
     auto *kernel = save.amax ? k2_fwd<N, BLOCKS, true> : k2_fwd<N, BLOCKS, false>;
-    launch_pdl(lc, kernel, dim3(std::max(1, e.nz), e.nx + ng, b.nshot), 8 * TX, 0, mc.p, g, b, c, n, step, stf,
-               src_scale, bd, save, ga, ng, err);
+    for (int y0 = 0; y0 < e.nx + ng; y0 += kMaxRows)
+        launch_pdl(lc, kernel, dim3(std::max(1, e.nz), std::min(kMaxRows, e.nx + ng - y0), b.nshot), 8 * TX, 0, mc.p, g, b,
+                   c, n, step, stf, src_scale, bd, save, ga, ng, y0, err);
     // the few steps in which a deep source's box grows through the rows next to the surface; starting
     // every step's tiles at the image rows instead cost all launches 40 ns (201 x 201: 3.25 -> 3.29 us)
     if (images) launch_free_surface(lc, g, n.p, b.nshot, kFsMirrorP);
@@ -997,9 +1000,10 @@ void run_rev(const LaunchCtx &lc, const Maps2 &mac, const Maps2 &mfc, const Grid
         }
         e.add(TX, lo, hi);
     }
-    if (e.nx == 0) return;
-    launch_pdl(lc, k2_rev<N, TX>, dim3(e.nz, e.nx, b.nshot * (roles == 3 ? 2 : 1)), 8 * TX, 0, mac.p, mfc.vz, mfc.vx, g, b, ac,
-               an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd, restore ? 1 : 0, ij, err);
+    for (int y0 = 0; y0 < e.nx; y0 += kMaxRows)
+        launch_pdl(lc, k2_rev<N, TX>, dim3(e.nz, std::min(kMaxRows, e.nx - y0), b.nshot * (roles == 3 ? 2 : 1)), 8 * TX, 0,
+                   mac.p, mfc.vz, mfc.vx, g, b, ac, an, mrev, roles, fc, fn, it, acc, img_mode, stf, src_scale, bd,
+                   restore ? 1 : 0, ij, y0, err);
 }
 
 }  // namespace
