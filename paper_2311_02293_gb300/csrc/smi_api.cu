@@ -654,9 +654,10 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
         int B = (int)std::max<size_t>(1, (size_t)(0.8 * (double)free_b) / per);
         B = std::min(B, S.nshot);
         if (o->max_batch > 0) B = std::min(B, o->max_batch);
-        if (S.fast2) B = std::min(B, 32767);     // two blocks a shot along gridDim.z
+        B = std::min(B, 65535);                  // shots lie along a grid's second or third dimension
         if (kind == 6 && B < S.nshot)
-            return fail(SMI_ERR_NOMEM, "a tape keeps every shot's state on the device: %d of %d shots fit", B, S.nshot);
+            return fail(SMI_ERR_NOMEM, "a tape keeps every shot's state on the device in one batch: %d of %d shots fit", B,
+                        S.nshot);
         if (kind == 7) B = S.nshot;
 
         Timer tm;
@@ -1033,12 +1034,14 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
                 ij.cell = dc;
                 ij.ids = di;
             }
-            // the adjoint step and the reconstruction share a launch (timed per class: one launch each)
+            // the adjoint step and the reconstruction share a launch (one launch each when timed per class, and
+            // for more shots than half of gridDim.z)
+            const bool apart = tm.on || nb_shot > 65535 / 2;
             auto reverse2 = [&](int it, int mrev) {
                 const int all = kind == 5 ? 1 : 3;
                 ij.it = max_rec > 0 ? it - 1 : -1;
                 for (int part = 0; part < 2; part++) {
-                    const int roles = tm.on ? all & (part == 0 ? 2 : 1) : (part == 0 ? all : 0);
+                    const int roles = apart ? all & (part == 0 ? 2 : 1) : (part == 0 ? all : 0);
                     if (!roles) continue;
                     tm.begin(roles == 2 ? 2 : 1);
                     launch2_reverse(lc, t2, m2A, m2F, g, b, A, A2, mrev, roles, F, F2, it, acc, mode, S.stf,

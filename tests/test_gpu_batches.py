@@ -48,3 +48,28 @@ def test_decimated_boundaries_in_several_batches(ndim, order, dr, kernels):
     for cut in (3, 1):
         for a, b in zip(out[cut], out[0]):
             assert rel(a, b) <= tol
+
+
+def test_tape_of_more_shots_than_half_a_grid_dimension():
+    """33000 small 2D shots in one batch: the adjoint and the reconstruction
+    no longer share a launch along gridDim.z.  Only three shots have an
+    adjoint source, so the gradient is that of the three alone."""
+    from paper_2311_02293_gb300 import smi
+    nshot, n, nt, h = 33000, 9, 30, 10.0
+    some = [0, 32767, nshot - 1]
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(3)
+    vp = 1800.0 + 600.0 * torch.rand((n, n), generator=gen, device=dev)
+    rho = torch.full((n, n), 1500.0, device=dev)
+    stf = torch.ones(nt, device=dev)
+    srcs = np.stack([3.0 + np.arange(nshot) % 3, 4.0 + np.arange(nshot) % 2, np.zeros(nshot)], 1) * h
+    recs = [np.array([[5.0, 2.0 + s % 5, 0.0]]) * h for s in range(nshot)]
+    prob = smi.Problem((h, h), nt, 1e-3, 0.0, order=4, nb=2)
+    u, tape = smi.smi_forward_tape(vp, rho, prob, srcs, recs, stf)
+    adj = torch.zeros_like(u).reshape(nshot, nt)
+    adj[some] = u.reshape(nshot, nt)[some]
+    g = tape.vjp(adj.reshape(-1))
+    tape.free()
+    alone = smi.smi_forward_vjp(vp, rho, prob, srcs[some], [recs[s] for s in some], stf, adj[some].reshape(-1).contiguous())
+    assert float(alone.abs().max()) > 0
+    assert rel(g, alone) <= 4 * nt * 2.0 ** -24
