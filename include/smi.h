@@ -386,6 +386,14 @@ void smi_server_destroy(smi_server *s);
  * kernel's duration.  stream: cudaStream_t or NULL. */
 int smi_wait_check(void *stream, long long polls, double *ms);
 
+/* Gives the working memory that the library keeps mapped between calls on the
+ * current device back to it.  While at least half of the device's memory is free, up to 1/64 of
+ * it (4.5 GB) stays with the library when a call ends, so that the next call
+ * need not map it again; a call that finds less free keeps nothing.  For
+ * callers that want the rest for other allocations.  Tapes and running calls
+ * keep theirs. */
+int smi_release_memory(void);
+
 /* Measurements of the calling thread's last smi_forward / smi_rtm /
  * smi_fwi_gradient call. */
 int smi_last_stats(smi_stats *st);

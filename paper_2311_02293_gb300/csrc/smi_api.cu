@@ -68,12 +68,14 @@ int check_same_device(const void *p, const char *name)
 }
 
 // The device's pool of working memory, created with the first call on it.
-// Stream-ordered allocations return to it when a call ends and it keeps up to
-// 1/64 of the device's memory mapped for the next call (any thread, any
-// stream); what exceeds that goes back to the device at the call's last
-// synchronisation, as everything did without it (mapping costs about 2 ms a
-// GB: 301 x 1001, 40 shots, 800 steps 180 -> 172 ms; 300^3 migration, 600
-// steps, 420 -> 408 ms).  The rest goes back when an allocation fails.
+// Stream-ordered allocations return to it when a call ends, and while at least
+// half of the device's memory is free it keeps up to 1/64 of it mapped for the
+// next call (any thread, any stream); what exceeds that goes back to the
+// device at the call's last synchronisation, as everything did without it
+// (mapping costs about 2 ms a GB: 301 x 1001, 40 shots, 800 steps 180 -> 172 ms;
+// 300^3 migration, 600 steps, 420 -> 408 ms).  The rest goes back with
+// smi_release_memory, with a call that finds less than half of the memory
+// free, and when an allocation fails.
 cudaMemPool_t device_pool()
 {
     static std::mutex mu;
@@ -88,16 +90,29 @@ cudaMemPool_t device_pool()
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
     cudaMemPool_t pool = nullptr;
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
         cudaGetLastError();
         pool = nullptr;                        // the device's default pool then
-    } else {
-        unsigned long long keep = total_b / 64;
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
     pools[dev] = pool;
     return pool;
+}
+
+// Memory free to a call: the device's, and what the pool keeps and no call
+// uses.  Decides what the pool may keep when the call ends.
+size_t free_memory()
+{
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+    if (cudaMemPool_t pool = device_pool()) {
+        unsigned long long held = 0, used = 0;
+        if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+            cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && held > used)
+            free_b += (size_t)(held - used);
+        unsigned long long keep = free_b >= total_b / 2 ? total_b / 64 : 0;
+        if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+    }
+    return free_b;
 }
 
 // Stream-ordered device allocations of one call, released in the destructor.
@@ -641,15 +656,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
         if (!ar.ok) return fail(SMI_ERR_NOMEM, "device allocation of outputs failed");
 
         // batch size by device memory
-        size_t free_b = 0, total_b = 0;
-        cudaMemGetInfo(&free_b, &total_b);
-        if (cudaMemPool_t pool = device_pool()) {   // what the pool keeps and no call uses is free to this call
-            unsigned long long held = 0, used = 0;
-            if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
-                cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && held > used)
-                free_b += (size_t)(held - used);
-            else cudaGetLastError();
-        }
+        const size_t free_b = free_memory();
         const size_t per = std::max<size_t>(per_shot_bytes(S, kind), 1);
         int B = (int)std::max<size_t>(1, (size_t)(0.8 * (double)free_b) / per);
         B = std::min(B, S.nshot);
@@ -1185,6 +1192,8 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
 // Error message of the calling thread, for entry points in other files.
 void record_error(const char *msg) { t_err = msg; }
 
+size_t free_device_memory() { return free_memory(); }
+
 }  // namespace smi
 
 using namespace smi;
@@ -1436,6 +1445,18 @@ int smi_wait_check(void *stream, long long polls, double *ms)
     }
     int rc2 = finish_stream(st);
     return rc ? rc : rc2;
+}
+
+int smi_release_memory(void)
+{
+    t_err.clear();
+    cudaMemPool_t pool = device_pool();       // (calls return after their frees)
+    const cudaError_t e = pool ? cudaMemPoolTrimTo(pool, 0) : cudaSuccess;
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(SMI_ERR_CUDA, "CUDA error: %s", cudaGetErrorString(e));
+    }
+    return SMI_OK;
 }
 
 int smi_last_stats(smi_stats *st)

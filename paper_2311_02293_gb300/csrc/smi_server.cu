@@ -29,6 +29,10 @@
 
 #include "../../include/smi.h"
 
+namespace smi {
+size_t free_device_memory();            // smi_api.cu: with what the library keeps between calls
+}
+
 namespace {
 
 using Clock = std::chrono::steady_clock;
@@ -265,9 +269,7 @@ smi_server *smi_server_create(size_t budget_bytes, int slots)
     if (slots < 1) slots = 1;
     auto *s = new smi_server();
     if (budget_bytes == 0) {
-        size_t free_b = 0, total_b = 0;
-        cudaMemGetInfo(&free_b, &total_b);
-        budget_bytes = (size_t)(0.8 * (double)free_b);
+        budget_bytes = (size_t)(0.8 * (double)smi::free_device_memory());
     }
     cudaGetDevice(&s->device);
     s->budget = budget_bytes;

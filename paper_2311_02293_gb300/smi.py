@@ -83,7 +83,7 @@ EXPORTS = ["smi_opts_default", "smi_forward", "smi_rtm", "smi_fwi_gradient", "sm
            "smi_box_table", "smi_last_stats", "smi_last_error", "smi_version", "smi_forward_noalloc",
            "smi_forward_vjp", "smi_server_create", "smi_submit", "smi_wait", "smi_poll", "smi_cancel",
            "smi_server_info", "smi_server_merges", "smi_server_destroy", "smi_fwi_gradient_family", "smi_wait_check",
-           "smi_forward_adjoint", "smi_dot", "smi_forward_tape", "smi_tape_vjp", "smi_tape_free"]
+           "smi_forward_adjoint", "smi_dot", "smi_forward_tape", "smi_tape_vjp", "smi_tape_free", "smi_release_memory"]
 KERNELS = {"auto": 0, "generic": 1, "twopass": 2, "fused": 3, "inline": 4}
 
 
@@ -117,7 +117,8 @@ def _load():
     L.smi_version.restype = ctypes.c_char_p
     for name in ("smi_forward", "smi_rtm", "smi_fwi_gradient", "smi_query", "smi_footprint", "smi_box_table",
                  "smi_last_stats", "smi_forward_noalloc", "smi_forward_vjp", "smi_fwi_gradient_family",
-                 "smi_wait_check", "smi_forward_adjoint", "smi_dot", "smi_forward_tape", "smi_tape_vjp"):
+                 "smi_wait_check", "smi_forward_adjoint", "smi_dot", "smi_forward_tape", "smi_tape_vjp",
+                 "smi_release_memory"):
         getattr(L, name).restype = c_int
     return L
 
@@ -522,6 +523,14 @@ def smi_wait_check(polls: int = -1, stream=None):
     ms = ctypes.c_double()
     rc = _lib.smi_wait_check(stream, int(polls), ctypes.byref(ms))
     return rc, ms.value
+
+
+def smi_release_memory(device=None) -> None:
+    """Gives the working memory that the library keeps mapped between calls on
+    a device (the current one by default) back to it."""
+    import contextlib
+    with torch.cuda.device(device) if device is not None else contextlib.nullcontext():
+        _check(_lib.smi_release_memory())
 
 
 def smi_last_stats() -> dict:
