@@ -657,11 +657,21 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
 
         // batch size by device memory
         const size_t free_b = free_memory();
-        const size_t per = std::max<size_t>(per_shot_bytes(S, kind), 1);
-        int B = (int)std::max<size_t>(1, (size_t)(0.8 * (double)free_b) / per);
-        B = std::min(B, S.nshot);
-        if (o->max_batch > 0) B = std::min(B, o->max_batch);
-        B = std::min(B, 65535);                  // shots lie along a grid's second or third dimension
+        auto batch_size = [&] {
+            const size_t per = std::max<size_t>(per_shot_bytes(S, kind), 1);
+            int n = (int)std::min<size_t>(S.nshot, std::max<size_t>(1, (size_t)(0.8 * (double)free_b) / per));
+            if (o->max_batch > 0) n = std::min(n, o->max_batch);
+            return std::min(n, 65535);           // shots lie along a grid's second or third dimension
+        };
+        int B = batch_size();
+        // The tile kernels' state is larger (2D: two copies; 3D: padded accumulators): a tape, or a shot, that
+        // fits only without that runs the generic kernels.
+        if ((S.fast2 || S.tile3) && kind != 7 &&
+            (kind == 6 ? B < S.nshot && (o->max_batch <= 0 || o->max_batch >= S.nshot) : per_shot_bytes(S, kind) > free_b)) {
+            S.fast2 = S.tile3 = S.pingpong = S.padacc = false;
+            set_layout(S.g, S.n);
+            B = batch_size();
+        }
         if (kind == 6 && B < S.nshot)
             return fail(SMI_ERR_NOMEM, "a tape keeps every shot's state on the device in one batch: %d of %d shots fit", B,
                         S.nshot);
@@ -681,7 +691,7 @@ int run(int kind, const smi_model *m, const smi_geometry *geo, const smi_wavelet
         const size_t nctr = g.ndim == 3 ? 2 * (size_t)S.nt_fwd + 4 * (size_t)S.nt : 1;
         unsigned *d_ctr = ar.get<unsigned>(nctr);
         if (!d_ctr) return fail(SMI_ERR_NOMEM, "device allocation failed");
-        const bool fast3 = o->kernels != SMI_KERNELS_GENERIC && stencil3d_supported(g);
+        const bool fast3 = S.tile3 || S.fused;
         const bool fast2 = S.fast2;
         const bool fused = S.fused, pp = S.pingpong;
         const Step2 t2 = fast2 ? step2_tile(g, B) : Step2{};
