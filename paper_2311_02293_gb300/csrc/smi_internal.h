@@ -140,13 +140,12 @@ double points_per_wavelength(int ndim, const double *h, double vmin, double fm);
 void cpml_tables(int ne, int nb, double h, double vmax, double fm, double R, double dt,
                  bool vgrid, float *a, float *b);
 
-// Kaiser-windowed sinc stencil of a position (metres) on the extended grid;
-// false if it leaves the physical domain or its stencil leaves the grid.
-bool make_stencil(const Grid &g, const double pos[3], double kaiser_b, Stencil *st);
-// The same for the many positions of one call: the window's normalisation is
-// evaluated once, and the weights of a coordinate between nodes once however
-// many receivers (a line's depth, a carpet's rows, every shot) share it -- a
-// Bessel function a tap otherwise took 0.3 us a receiver, 4 us between nodes.
+// Kaiser-windowed sinc stencils of the positions (metres) of one call on the
+// extended grid; make returns false if a position leaves the physical domain
+// or its stencil leaves the grid.  The window's normalisation is evaluated
+// once, and the weights of a coordinate between nodes once however many
+// receivers (a line's depth, a carpet's rows, every shot) share it -- a Bessel
+// function a tap otherwise took 0.3 us a receiver, 4 us between nodes.
 class StencilMaker {
 public:
     StencilMaker(const Grid &g, double kaiser_b);

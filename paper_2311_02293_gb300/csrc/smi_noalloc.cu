@@ -279,10 +279,11 @@ int forward_noalloc(const smi_model *m, const smi_geometry *geo, const smi_wavel
     for (int a = 0; a < m->ndim; a++) dV *= hh[a];
     const float src_scale = (float)(w->dt / dV);
 
+    StencilMaker maker(g, kb);               // host memory alone
     for (int s = 0; s < geo->nshot; s++) {
         const int r0 = geo->rec_offset[s], nr = geo->rec_offset[s + 1] - r0;
         Stencil sst;
-        if (!make_stencil(g, geo->src + 3 * s, kb, &sst))
+        if (!maker.make(geo->src + 3 * s, &sst))
             return err(SMI_ERR_ARG, "source %d lies outside the model or its stencil leaves the grid", s);
         int box[12], lo[3], hi[3];
         extent_of(g, sst, lo, hi);
@@ -297,7 +298,7 @@ int forward_noalloc(const smi_model *m, const smi_geometry *geo, const smi_wavel
             Stencil chunk[kStencilChunk];
             const int k = std::min(kStencilChunk, nr - r);
             for (int j = 0; j < k; j++) {
-                if (!make_stencil(g, geo->rec + 3 * (size_t)(r0 + r + j), kb, &chunk[j]))
+                if (!maker.make(geo->rec + 3 * (size_t)(r0 + r + j), &chunk[j]))
                     return err(SMI_ERR_ARG, "receiver %d lies outside the model or its stencil leaves the grid", r0 + r + j);
                 extent_of(g, chunk[j], lo, hi);
                 for (int a = 0; a < 3; a++) {

@@ -154,11 +154,6 @@ bool StencilMaker::taps(int ax, int first, double x, Taps &t) const
 
 StencilMaker::StencilMaker(const Grid &g, double kaiser_b) : g_(g), b_(kaiser_b), i0b_(std::cyl_bessel_i(0.0, kaiser_b)) {}
 
-bool make_stencil(const Grid &g, const double pos[3], double kaiser_b, Stencil *st)
-{
-    return StencilMaker(g, kaiser_b).make(pos, st);
-}
-
 TimeWeights time_weights(int it, int dr, int nsamp)
 {
     TimeWeights tw{};
