@@ -161,8 +161,9 @@ template <int MODE> __device__ __forceinline__ Q4 update(const Q4 &v, const Q4 &
 }
 // The forward scheme's z terms: which of the two products is rounded first
 // decides the last bit.  A x enters the multiply-add unrounded, except on x
-// lines whose group of four (from the low end of the launch's boxes) meets an
-// x slab, so that results stay the ones they have always been.
+// lines whose group of four (from the low end of the shot's box) meets an x
+// slab: a shot's bits are the same whichever shots it is launched with, and
+// those of earlier kernels.
 __device__ __forceinline__ void recur4z(bool xgroup, const float (&B)[4], const float (&A)[4], float (&m)[4], const Q4 &x)
 {
     float v[4];
@@ -176,11 +177,6 @@ __device__ __forceinline__ bool x_group(const Grid &g, int x, int x0)
     const int first = x0 + ((x - x0) & ~3), hi = g.ne[1] - g.nb - 1;
     return first < g.nb || first + 3 >= hi;
 }
-// How a launch cuts its boxes: planes a chunk, and the boxes' low end along x.
-struct Cut {
-    int chunk, x0;
-};
-
 // Maps of a launch, by the tile they bring.
 struct VMaps {
     CUtensorMap p, rho, vz, vx, vy, ezl, ezh, exl, exh;
@@ -197,7 +193,7 @@ struct PMaps {
 // the band of the source field from the store (rs.it).
 template <int N, int MODE, bool MAG>
 __global__ void __launch_bounds__(NTHR, SMI_MINB)
-k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, Gather3 ga, Restore3 rs,
+k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, int chunk, Gather3 ga, Restore3 rs,
      unsigned *amax, unsigned *err, unsigned *ctr)
 {
     using La = VLay<N, MODE>;
@@ -215,7 +211,7 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
     if (tid < 6) smx[tid] = 0u;
     __syncthreads();
     Sched sd;
-    sched_shot(g, b, MODE, step, 0, 0, lc.chunk, sd);   // (the box tables are older than the loop)
+    sched_shot(g, b, MODE, step, 0, 0, chunk, sd);   // (the box tables are older than the loop)
     pdl_wait();
     pdl_trigger();
     unsigned phase = 0;                       // bit h: parity of the next completion of bar[h]
@@ -224,7 +220,7 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
     const int plane = g.px * g.ne[1];
 
     Item it;
-    for (int w = blockIdx.x, par = 0; sched_item(g, b, MODE, step, w, lc.chunk, sd, it); w = next[par], par ^= 1) {
+    for (int w = blockIdx.x, par = 0; sched_item(g, b, MODE, step, w, chunk, sd, it); w = next[par], par ^= 1) {
         const int s = it.s, z0 = it.z0, x0 = it.x0, ya = it.ya, yb = it.yb;
         const Own me = own_of(g, it, tzi, txi);
         const int oz = me.oz, ox = me.ox;
@@ -309,7 +305,7 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
         }
         // CPML planes of the item: every plane of a tile that meets a z or x slab, the y-slab planes of the others
         const bool zxb = MODE != REC && (z_slab_tile(g, &tm.p, &tm.p, z0).tm || x_slab_tile(g, &tm.p, &tm.p, x0 - N + 1, La::PR).tm);
-        const bool xg = MODE == FWD && x_group(g, ox, lc.x0);
+        const bool xg = MODE == FWD && x_group(g, ox, it.lo[1]);
         // boundary bands (2N - 1 half nodes across each face): the quad's nodes per side of z, the side of x
         // that holds the column, the physical nodes; a plane's part is decided per plane
         unsigned bz0 = 0u, bz1 = 0u, bph = 0u;
@@ -529,7 +525,7 @@ k3_v(const __grid_constant__ VMaps tm, Grid g, Batch b, Fields f, int step, Cut 
 // magnitudes), from the velocities this kernel only reads.
 template <int N, int MODE>
 __global__ void __launch_bounds__(NTHR, SMI_MINB)
-k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut lc, unsigned *err, float *acc, int img_mode,
+k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, int chunk, unsigned *err, float *acc, int img_mode,
      const float *stf, float src_scale, Save3 sv, unsigned *ctr)
 {
     using La = PLay<N, MODE>;
@@ -544,7 +540,7 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
     }
     __syncthreads();
     Sched sd;
-    sched_shot(g, b, MODE, step, 0, 0, lc.chunk, sd);   // (the box tables are older than the loop)
+    sched_shot(g, b, MODE, step, 0, 0, chunk, sd);   // (the box tables are older than the loop)
     pdl_wait();
     pdl_trigger();
     unsigned phase = 0;
@@ -553,7 +549,7 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
     const int plane = g.px * g.ne[1];
 
     Item it;
-    for (int w = blockIdx.x, par = 0; sched_item(g, b, MODE, step, w, lc.chunk, sd, it); w = next[par], par ^= 1) {
+    for (int w = blockIdx.x, par = 0; sched_item(g, b, MODE, step, w, chunk, sd, it); w = next[par], par ^= 1) {
         const int s = it.s, z0 = it.z0, x0 = it.x0, ya = it.ya, yb = it.yb;
         const Own me = own_of(g, it, tzi, txi);
         const int oz = me.oz, ox = me.ox;
@@ -631,7 +627,7 @@ k3_p(const __grid_constant__ PMaps tm, Grid g, Batch b, Fields f, int step, Cut 
             __syncthreads();
         }
         const bool zxb = MODE != REC && (z_slab_tile(g, &tm.p, &tm.p, z0).tm || x_slab_tile(g, &tm.p, &tm.p, x0 - N, La::XR).tm);
-        const bool xg = MODE == FWD && x_group(g, ox, lc.x0);
+        const bool xg = MODE == FWD && x_group(g, ox, it.lo[1]);
         float *const mzp = f.psiv[0] + (s * g.slab_n[0] + me.zq + (long long)g.zp * ox);
         float *const mxp = f.psiv[1] + (s * g.slab_n[1] + oz + (long long)g.px * me.xq);
         const unsigned zpl = (unsigned)(g.zp * g.ne[1]), xpl = (unsigned)(g.px * g.xrows);
@@ -932,11 +928,11 @@ int pick_chunk(long long cols, int ylen, int grid, int sms)
     return cy;
 }
 
-// The cut of a launch from the boxes of its shots.
-s3::Cut launch_cut(const Grid &g, const Batch &b, int mode, int step, int grid)
+// Planes a chunk of a launch, from the boxes of its shots.
+int launch_chunk(const Grid &g, const Batch &b, int mode, int step, int grid)
 {
     long long cols = 0;
-    int ylen = 0, x0 = g.ne[1];
+    int ylen = 0;
     for (int s = 0; s < b.nshot; s++) {
         int lo[3], hi[3];
         box_bounds(g, (mode == s3::ADJ ? b.h_box_rec : b.h_box_src) + 6 * s, step, lo, hi);
@@ -950,7 +946,6 @@ s3::Cut launch_cut(const Grid &g, const Batch &b, int mode, int step, int grid)
         s3::tile_rows(lo[0], hi[0], base, rows);
         cols += (long long)rows * ((hi[1] - lo[1]) / s3::TX + 1);
         ylen = std::max(ylen, hi[2] - lo[2] + 1);
-        x0 = std::min(x0, lo[1]);
     }
     static const int sms = [] {
         int dev = 0, n = 0;
@@ -958,7 +953,7 @@ s3::Cut launch_cut(const Grid &g, const Batch &b, int mode, int step, int grid)
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         return std::max(1, n);
     }();
-    return {pick_chunk(cols, ylen, grid, sms), x0};
+    return pick_chunk(cols, ylen, grid, sms);
 }
 
 template <int N, int MODE>
@@ -970,7 +965,7 @@ void run_v(const LaunchCtx &lc, const Maps3 &m, const Grid &g, const Batch &b, c
     auto *kernel = amax ? s3::k3_v<N, MODE, M> : s3::k3_v<N, MODE, false>;
     static const int grid = std::min(grid_for(s3::k3_v<N, MODE, M>, smem), grid_for(s3::k3_v<N, MODE, false>, smem));
     const s3::VMaps tm{m.p_halo, m.rho_v, m.vz_core, m.vx_core, m.vy_core, m.ezl_p, m.ezh_p, m.exl_p, m.exh_p};
-    launch_pdl(lc, kernel, dim3(grid), s3::NTHR, smem, tm, g, b, f, step, launch_cut(g, b, MODE, step, grid), ga,
+    launch_pdl(lc, kernel, dim3(grid), s3::NTHR, smem, tm, g, b, f, step, launch_chunk(g, b, MODE, step, grid), ga,
                rs, amax, err, ctr);
 }
 
@@ -983,7 +978,7 @@ void run_p(const LaunchCtx &lc, const Maps3 &m, const Maps3 *lpm, const Grid &g,
     const s3::PMaps tm{m.vz_halo, m.vx_halo, m.vy_core, m.p_core, m.K_core, lpm ? lpm->p_core : m.p_core,
                        m.ezl_v, m.ezh_v, m.exl_v, m.exh_v};
     launch_pdl(lc, s3::k3_p<N, MODE>, dim3(grid), s3::NTHR, smem, tm, g, b, f, step,
-               launch_cut(g, b, MODE, step, grid), err, acc, img_mode, stf, src_scale, sv, ctr);
+               launch_chunk(g, b, MODE, step, grid), err, acc, img_mode, stf, src_scale, sv, ctr);
 }
 
 }  // namespace

@@ -73,3 +73,20 @@ def test_tape_of_more_shots_than_half_a_grid_dimension():
     alone = smi.smi_forward_vjp(vp, rho, prob, srcs[some], [recs[s] for s in some], stf, adj[some].reshape(-1).contiguous())
     assert float(alone.abs().max()) > 0
     assert rel(g, alone) <= 4 * nt * 2.0 ** -24
+
+
+@pytest.mark.parametrize("order,nb,nx", [(8, 8, 150), (4, 6, 141), (8, 10, 170)])
+def test_3d_shots_are_the_same_bits_alone(order, nb, nx):
+    """Two shots far apart in x, whose boxes start at different nodes: their
+    seismograms in one batch and one after the other."""
+    from paper_2311_02293_gb300 import smi
+    w = synth.tiny_3d(nz=40, nx=nx, ny=34, nt=60, order=order, nb=nb)
+    h = w.d[0]
+    srcs = np.repeat(w.srcs, 2, 0)
+    srcs[:, 1] = [3 * h, (nx - 4) * h]
+    recs = [w.recs[0], w.recs[0]]
+    dev = torch.device("cuda:0")
+    vp, rho, stf = (torch.from_numpy(a).to(dev) for a in (w.vp, w.rho, w.stf))
+    u = [smi.smi_forward(vp, rho, smi.Problem(w.d, w.nt, w.dt, w.fm, order=order, nb=nb, max_batch=k), srcs, recs, stf,
+                         flat=True) for k in (0, 1)]
+    assert float(u[0].abs().max()) > 0 and torch.equal(u[0], u[1])
