@@ -223,8 +223,10 @@ def other_workloads(smi, synth, torch, dev, peak: float, args) -> dict:
         order 8, nt 3000, corner source, 200 x 200 receivers;
       - 2D FWI gradient: 301 x 1001 + 20 layers, order 8, nt 3000, 40 shots
         in one batch, observed data from the true model.
-    Each reports grid-point updates/s (box points) and the roofline of its
-    dominant stencil class (algorithmic bytes / that class's event time)."""
+    Each reports grid-point updates/s (box points) of a plain call, and from a
+    call with an event pair around every step (which splits the 2D reverse
+    step's launch) the roofline of its dominant stencil class (algorithmic
+    bytes / that class's event time)."""
     out = {}
 
     def roof(st):
@@ -246,10 +248,12 @@ def other_workloads(smi, synth, torch, dev, peak: float, args) -> dict:
 
     w = synth.random_smooth_3d(nt=args.other_nt3)
     vp, rho, stf = (torch.from_numpy(a).to(dev) for a in (w.vp, w.rho, w.stf))
-    prob = smi.Problem(w.d, w.nt, w.dt, w.fm, order=w.order, nb=w.nb, profile=True)
+    prob = smi.Problem(w.d, w.nt, w.dt, w.fm, order=w.order, nb=w.nb)
     warm = smi.Problem(w.d, min(w.nt, 200), w.dt, w.fm, order=w.order, nb=w.nb)
     smi.smi_forward(vp, rho, warm, w.srcs, w.recs, stf[:warm.nt].contiguous())
     ms = timed(lambda: smi.smi_forward(vp, rho, prob, w.srcs, w.recs, stf))
+    prob.profile = True                 # the classes: a call of its own, with events around every step
+    smi.smi_forward(vp, rho, prob, w.srcs, w.recs, stf)
     st = smi.smi_last_stats()
     out["forward_3d_random_400x400x200_nt%d" % w.nt] = {
         "gpts": st["point_updates"] / (ms * 1e6), "ms": ms, "roofline": roof(st),
@@ -258,10 +262,12 @@ def other_workloads(smi, synth, torch, dev, peak: float, args) -> dict:
 
     w = synth.layered_fault_2d(nt=args.other_nt2, nshot=40)
     vp, rho, stf, vpt = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (w.vp, w.rho, w.stf, w.vp_true))
-    prob = smi.Problem(w.d, w.nt, w.dt, w.fm, order=w.order, nb=w.nb, profile=True)
+    prob = smi.Problem(w.d, w.nt, w.dt, w.fm, order=w.order, nb=w.nb)
     dobs = smi.smi_forward(vpt, rho, prob, w.srcs, w.recs, stf, flat=True)
     smi.smi_fwi_gradient(vp, rho, prob, w.srcs[:2], w.recs[:2], stf, dobs[: 2 * w.nt * len(w.recs[0])])
     ms = timed(lambda: smi.smi_fwi_gradient(vp, rho, prob, w.srcs, w.recs, stf, dobs))
+    prob.profile = True
+    smi.smi_fwi_gradient(vp, rho, prob, w.srcs, w.recs, stf, dobs)
     st = smi.smi_last_stats()
     out["gradient_2d_layered_301x1001_40shots_nt%d" % w.nt] = {
         "gpts": st["point_updates"] / (ms * 1e6), "ms": ms, "shots_per_s": 40 / (ms / 1e3), "roofline": roof(st)}
@@ -520,9 +526,10 @@ def run_profile_grad2d(args, torch, synth, smi, dev):
 
 def run_table(args):
     """One JSON line per workload for the results table: the GPU rate of the
-    workload's call (CUDA events after a warm-up call; grid-point updates
-    inside the computing box, and over the full grid) with the dominant
-    stencil class's roofline fraction, and the FP64 oracle's per-step rate on
+    workload's plain call (CUDA events after a warm-up call; grid-point updates
+    inside the computing box, and over the full grid), the dominant stencil
+    class's roofline fraction from a call with an event pair around every step
+    (which splits the 2D reverse step's launch), and the FP64 oracle's per-step rate on
     all of this host's cores and on one core (a few time steps of one shot
     with the box off, set-up and each loop's first step excluded)."""
     import torch
@@ -544,7 +551,7 @@ def run_table(args):
         return {"gpts": k * (2 * ext + phys) / (phase[0] + phase[1]) / 1e9, "threads": nthreads or O.max_threads(),
                 "steps_timed": k}
 
-    def gpu(call, st_scale=1.0):
+    def gpu(call, prob):
         call()
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -553,6 +560,8 @@ def run_table(args):
         e1.record()
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1)
+        prob.profile = True
+        call()
         st = smi.smi_last_stats()
         cms, cby = np.array(st["ms"]), np.array(st["bytes"])
         dom = int(np.argmax(cms))
@@ -568,7 +577,7 @@ def run_table(args):
         vp, rho, stf = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (w.vp, w.rho, w.stf))
         line = {"table": name}
         for shell in (["f32", "f16"] if kind == "rtm" else ["f32"]):
-            prob = smi.Problem(w.d, w.nt, w.dt, w.fm, order=w.order, nb=w.nb, profile=True, shell_prec=shell)
+            prob = smi.Problem(w.d, w.nt, w.dt, w.fm, order=w.order, nb=w.nb, shell_prec=shell)
             if kind == "forward":
                 call = lambda: smi.smi_forward(vp, rho, prob, w.srcs, w.recs, stf, flat=True)
                 props = 1
@@ -581,7 +590,7 @@ def run_table(args):
                 else:
                     call = lambda: smi.smi_fwi_gradient(vp, rho, prob, w.srcs, w.recs, stf, dobs)
                 props = 3
-            ms, st, roof = gpu(call)
+            ms, st, roof = gpu(call, prob)
             ext = float(np.prod([n + 2 * w.nb for n in w.n]))
             phys = float(np.prod(w.n))
             full = (ext if props == 1 else 2 * ext + phys) * w.nt * len(w.srcs)

@@ -69,9 +69,10 @@ __device__ __forceinline__ Q4 tap(const Q4 &D, float c, const Q4 &x, const Q4 &y
     const P2 cc = pack(c, c);
     return {fma2(cc, sub2(x.a, y.a), D.a), fma2(cc, sub2(x.b, y.b), D.b)};
 }
-// num / (r0 + r1): reciprocal (a few ulp, far below the FP32 scheme error)
-// and product; densities are normal numbers, so it is __fdividef without its
-// range scaling.
+// num / (r0 + r1) as reciprocal and product.  The reciprocal is PTX's
+// rcp.approx.ftz.f32, which the PTX ISA documents to within 1 ulp; with the
+// product about 1.5 ulp, far below the FP32 scheme error.  Its operand is a sum
+// of two densities, positive normal numbers.
 __device__ __forceinline__ float rcpf(float x)
 {
     float r;

@@ -70,8 +70,8 @@ using s3::tma4;
 // whole grid (all shots).  Below kMany a launch hardly fills the GPU: narrow
 // tiles (more, shorter blocks) and the registers a thread wants (4 blocks of
 // 128 threads a SM, no spills).  Above, the blocks hide each other's load
-// phases: forward 6 narrow blocks a SM (85 registers), reverse 4 wide ones (64,
-// some spilled).  Measured (us a step, or a step pair): forward 201 x 601, 4
+// phases: forward 6 narrow blocks a SM (80 registers, 60 - 160 bytes spilled),
+// reverse 4 wide ones (64 registers, 0.4 KB spilled).  Measured (us a step, or a step pair): forward 201 x 601, 4
 // shots, order 8: narrow 4.3, narrow with 6 blocks 4.9, wide 5.2; 40 shots
 // 301 x 1001 gradient with the forward narrow / 4 blocks 172, narrow / 6 166,
 // wide / 3 169, and the reverse wide / 3 175, wide / 4 165, wide / 5 174, narrow

@@ -148,8 +148,6 @@ __device__ __forceinline__ void ring_drain(uint64_t *bars, int nslots, int bitba
     }
 }
 
-// Buoyancy on a half node: 2 / (rho_i + rho_{i+1}), 1/rho at the last node
-// (fast reciprocal-based division: a few ulp, far below the FP32 scheme error).
 // y-loop unrolled in groups of G planes: step K of a group sees logical
 // queue entry l at physical index (l + K) % 2N, so inside a group the queue
 // rotates by renaming registers; rotate_queue moves it back between groups.
@@ -203,6 +201,8 @@ template <int G, class T, int L> __device__ __forceinline__ void rotate_queue(T 
     for (int l = 0; l < L; l++) q[l] = t[l];
 }
 
+// Buoyancy on a half node: 2 / (rho_i + rho_{i+1}), 1/rho at the last node
+// (__fdividef: 2 ulp, far below the FP32 scheme error).
 __device__ __forceinline__ float buoy(float r0, float r1, bool last)
 {
     return last ? __fdividef(1.0f, r0) : __fdividef(2.0f, r0 + r1);
