@@ -140,7 +140,8 @@ typedef struct {
                                  SMI_ERR_ARG */
     int per_shot;             /* 1: smi_rtm and smi_fwi_gradient return each shot's result instead of the sum
                                  over shots: image / gradient [nshot][n3][n2][n1] and misfit [nshot],
-                                 shot s equal to a call with shot s alone (the shots of a batch share
+                                 shot s equal to a call with shot s alone up to the order of the FP32
+                                 sums over receivers that share nodes (the shots of a batch share
                                  launches).  Not with img_norm, the family gradients or the tape calls
                                  (SMI_ERR_ARG); no effect on smi_forward.  0: sums (default) */
 } smi_opts;
