@@ -835,19 +835,17 @@ using EncodeFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, vo
 
 EncodeFn encoder()
 {
-    static EncodeFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    // initialised once, by the first thread; others wait (the server's slots start together)
+    static const EncodeFn fn = []() -> EncodeFn {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeFn>(p);
-        else
-            cudaGetLastError();
-    }
+            return reinterpret_cast<EncodeFn>(p);
+        cudaGetLastError();
+        return nullptr;
+    }();
     return fn;
 }
 
